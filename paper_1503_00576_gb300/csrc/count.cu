@@ -91,8 +91,6 @@ __device__ __forceinline__ uint32_t table_slots(int32_t len, uint32_t capacity) 
 
 // Read-only view of the forward lists and partner groups.
 struct Lists {
-  const int32_t *__restrict__ off;   // node array (rank space): list lengths
-  const int32_t *__restrict__ voff;  // node array of col4, in 16-byte words (even)
   const int32_t *__restrict__ col4;  // forward lists, sorted, each padded with -1 to whole 32-byte blocks
   const int32_t *__restrict__ goff;  // partner-group offsets
   const int32_t *__restrict__ part;   // partners
@@ -491,7 +489,7 @@ struct CtaShared {
   unsigned long long groupsum;
 };
 
-// Groups of `list` counted by the whole CTA: N+(h) hashed once, warps claim
+// Groups list[0], list[step], ... counted by the whole CTA: N+(h) hashed once, warps claim
 // chunks of partners, each a share of the partners left (at most 32), so
 // that the warps run out of work together.  A list longer than half the table is hashed
 // in equal segments, one after another, each probed by all partners:
@@ -499,7 +497,7 @@ struct CtaShared {
 // table (SLOTS slots) is empty on entry and on exit.
 template <bool PV, int THREADS, int SLOTS, int W>
 __device__ __forceinline__ void cta_groups(const Lists &g, const int32_t *__restrict__ list,
-                                           uint32_t n_list, uint32_t *cursor, Table tb,
+                                           int step, uint32_t n_list, uint32_t *cursor, Table tb,
                                            uint16_t *slot_of, WarpScratch *s_ws, CtaShared &sh,
                                            int64_t *t, int64_t *tg, uint64_t &found_total) {
   constexpr int WARPS = THREADS / 32;
@@ -514,7 +512,7 @@ __device__ __forceinline__ void cta_groups(const Lists &g, const int32_t *__rest
     if (gi >= n_list) break;
     // lists are filled in about ascending rank, and high ranks (high
     // degrees) carry the most work: take them first to shorten the tail
-    const int32_t h = __ldg(list + (n_list - 1 - gi));
+    const int32_t h = __ldg(list + (int64_t)gi * step);
     const int2 hld = __ldg(g.ldesc + h);
     const int32_t hd = hld.y;
     const int32_t *hl = g.col4 + 4 * (size_t)hld.x;
@@ -616,7 +614,7 @@ __global__ void __launch_bounds__(256)
 k_stream_desc(const int32_t *__restrict__ part, const int32_t *__restrict__ pskip,
               const int2 *__restrict__ ldesc, const Ctrl *ctrl, int2 *__restrict__ desc) {
   if (aborted(ctrl)) return;  // an earlier wait of this call ran out
-  const uint32_t m = ctrl->m;
+  const uint32_t m = ctrl->n_part;
   const uint32_t stride = gridDim.x * blockDim.x;
   for (uint32_t e0 = blockIdx.x * blockDim.x + threadIdx.x; e0 < m; e0 += 4 * stride) {
     int32_t l[4], skip[4];
@@ -637,17 +635,6 @@ k_stream_desc(const int32_t *__restrict__ part, const int32_t *__restrict__ pski
   }
 }
 
-// ldesc[v] = {voff[v], off[v+1] - off[v]}: each list's first col4 word and
-// length in one record (after the list sort's recount).
-__global__ void __launch_bounds__(256)
-k_list_desc(const int32_t *__restrict__ off, const int32_t *__restrict__ voff, int32_t n,
-            const Ctrl *ctrl, int2 *__restrict__ ldesc) {
-  if (aborted(ctrl)) return;
-  const uint32_t stride = gridDim.x * blockDim.x;
-  for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < (uint32_t)n; v += stride)
-    ldesc[v] = make_int2(__ldg(voff + v), __ldg(off + v + 1) - __ldg(off + v));
-}
-
 // Dynamic shared memory of the counting kernels: the hash table, the slot
 // counters (per-vertex mode) and the slot of every hashed entry.
 constexpr size_t table_smem(int slots, int max_len, bool pv) {
@@ -662,8 +649,8 @@ static_assert(kMainWarps * kWarpMaxRow <= kCtaMaxRow, "warp slot maps must fit t
 // Main counting kernel: CTA groups first (the heavy ones), then warp groups.
 template <bool PV>
 __global__ void __launch_bounds__(kMainThreads, kMainMinBlocks)
-k_count(Lists g, const int32_t *__restrict__ warp_list, const int32_t *__restrict__ cta_list,
-        int32_t n, Ctrl *ctrl, int64_t *t, int64_t *tg) {
+k_count(Lists g, const int32_t *__restrict__ groups, int32_t n, Ctrl *ctrl, int64_t *t,
+        int64_t *tg) {
   constexpr int SLOTS = main_slots<PV>();
   constexpr int WSLOTS = SLOTS / kMainWarps;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -677,12 +664,14 @@ k_count(Lists g, const int32_t *__restrict__ warp_list, const int32_t *__restric
   clear_table<PV>(s_tab, s_cnt, SLOTS, tid, kMainThreads);
   uint64_t found_total = 0;
   Table tb{s_tab, s_cnt, shared_addr(s_cnt), SLOTS};
-  cta_groups<PV, kMainThreads, SLOTS, kWindows>(g, cta_list, ctrl->n_cta_groups,
+  // the CTA groups fill `groups` from its end down, the last binned first
+  const uint32_t n_cta = ctrl->n_cta_groups;
+  cta_groups<PV, kMainThreads, SLOTS, kWindows>(g, groups + ((uint32_t)n - n_cta), 1, n_cta,
                                                 &ctrl->next_cta_group, tb, s_slot, s_ws, s_sh,
                                                 t, tg, found_total);
   Table wtb{s_tab + warp * WSLOTS, s_cnt + warp * WSLOTS, shared_addr(s_cnt + warp * WSLOTS),
             WSLOTS};
-  warp_groups<PV, WSLOTS>(g, warp_list, ctrl->n_warp_groups, &ctrl->next_warp_group, wtb,
+  warp_groups<PV, WSLOTS>(g, groups, ctrl->n_warp_groups, &ctrl->next_warp_group, wtb,
                           s_slot + warp * kWarpMaxRow, s_ws[warp], t, tg, found_total);
   found_total = warp_sum_u64(found_total);
   if (lane == 0 && found_total) atomicAdd(&ctrl->total, (unsigned long long)found_total);
@@ -691,7 +680,7 @@ k_count(Lists g, const int32_t *__restrict__ warp_list, const int32_t *__restric
 // Groups whose hashed list is longer than kCtaMaxRow (rare).
 template <bool PV>
 __global__ void __launch_bounds__(kBigThreads, kBigMinBlocks)
-k_count_big(Lists g, const int32_t *__restrict__ big_list, int32_t n, Ctrl *ctrl, int64_t *t,
+k_count_big(Lists g, const int32_t *__restrict__ big_list, Ctrl *ctrl, int64_t *t,
             int64_t *tg) {
   extern __shared__ __align__(16) unsigned char smem[];
   int32_t *tab = reinterpret_cast<int32_t *>(smem);
@@ -701,10 +690,12 @@ k_count_big(Lists g, const int32_t *__restrict__ big_list, int32_t n, Ctrl *ctrl
   __shared__ CtaShared s_sh;
   if (aborted(ctrl)) return;  // an earlier wait of this call ran out: the lists are not complete
   const int tid = threadIdx.x, lane = tid & 31;
+  const uint32_t n_big = ctrl->n_big_groups;
+  if (n_big == 0) return;  // most graphs: not even the tables are emptied
   clear_table<PV>(tab, cnt, kBigSlots, tid, kBigThreads);
   uint64_t found_total = 0;
   Table tb{tab, cnt, shared_addr(cnt), kBigSlots};
-  cta_groups<PV, kBigThreads, kBigSlots, kBigWindows>(g, big_list, ctrl->n_big_groups,
+  cta_groups<PV, kBigThreads, kBigSlots, kBigWindows>(g, big_list + (n_big - 1), -1, n_big,
                                                       &ctrl->next_big_group, tb, slot_of, s_ws,
                                                       s_sh, t, tg, found_total);
   found_total = warp_sum_u64(found_total);
@@ -834,12 +825,10 @@ cudaError_t prepare_count_kernels() {
   return e;
 }
 
-cudaError_t launch_count(const int32_t *off, const int32_t *voff, const int2 *ldesc,
-                         const int32_t *col4,
-                         const int32_t *goff, const int32_t *part, const int32_t *pskip,
-                         int2 *desc, const int32_t *warp_groups,
-                         const int32_t *cta_groups, const int32_t *big_groups, int32_t n,
-                         Ctrl *ctrl, int64_t *t, int64_t *tg, cudaStream_t st) {
+cudaError_t launch_count(const int2 *ldesc, const int32_t *col4, const int32_t *goff,
+                         const int32_t *part, const int32_t *pskip, int2 *desc,
+                         const int32_t *groups, const int32_t *big_groups, int32_t n, Ctrl *ctrl,
+                         int64_t *t, int64_t *tg, cudaStream_t st) {
   const bool pv = t != nullptr;
   CountGrid cg;
   cudaError_t e = count_grid(pv, &cg);
@@ -851,35 +840,22 @@ cudaError_t launch_count(const int32_t *off, const int32_t *voff, const int2 *ld
     k_stream_desc<<<(sms > 0 ? sms : 1) * 16, 256, 0, st>>>(part, pskip, ldesc, ctrl, desc);
     note_launch();
   }
-  const Lists g{off, voff, col4, goff, part, pskip, desc, ldesc};
+  const Lists g{col4, goff, part, pskip, desc, ldesc};
   // the long lists first, on their own wide CTAs
   if (pv) {
-    k_count_big<true><<<cg.big_blocks, kBigThreads, big_smem<true>(), st>>>(g, big_groups, n, ctrl,
-                                                                          t, nullptr);
-    k_count<true><<<cg.main_blocks, kMainThreads, main_smem<true>(), st>>>(g, warp_groups,
-                                                                         cta_groups, n, ctrl, t,
+    k_count_big<true><<<cg.big_blocks, kBigThreads, big_smem<true>(), st>>>(g, big_groups, ctrl, t,
+                                                                          nullptr);
+    k_count<true><<<cg.main_blocks, kMainThreads, main_smem<true>(), st>>>(g, groups, n, ctrl, t,
                                                                          nullptr);
   } else {
-    k_count_big<false><<<cg.big_blocks, kBigThreads, big_smem<false>(), st>>>(g, big_groups, n,
-                                                                            ctrl, nullptr, tg);
-    k_count<false><<<cg.main_blocks, kMainThreads, main_smem<false>(), st>>>(g, warp_groups,
-                                                                           cta_groups, n, ctrl,
+    k_count_big<false><<<cg.big_blocks, kBigThreads, big_smem<false>(), st>>>(g, big_groups, ctrl,
+                                                                            nullptr, tg);
+    k_count<false><<<cg.main_blocks, kMainThreads, main_smem<false>(), st>>>(g, groups, n, ctrl,
                                                                            nullptr, tg);
   }
   note_launch();
   note_launch();
   return cudaGetLastError();
-}
-
-void launch_list_desc(const int32_t *off, const int32_t *voff, int32_t n, const Ctrl *ctrl,
-                      int2 *ldesc, cudaStream_t st) {
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const uint32_t want = ((uint32_t)n + 255u) / 256u;
-  const uint32_t grid = max(1u, min(want, (uint32_t)(sms > 0 ? sms : 1) * 8u));
-  k_list_desc<<<grid, 256, 0, st>>>(off, voff, n, ctrl, ldesc);
-  note_launch();
 }
 
 void launch_clustering(const int64_t *t, const int32_t *deg, int32_t n, double *cc,

@@ -38,7 +38,11 @@ constexpr unsigned kFull = 0xffffffffu;
 constexpr int kListThreads = 256;
 constexpr int kListWarps = kListThreads / 32;
 constexpr int kLongListThreads = 512;
-constexpr int kLongListBlocks = 4;  // CTAs per SM: a CTA mostly waits at its barriers
+constexpr int kLongListBlocks = 2;  // CTAs per SM (64 registers a thread)
+// Lists of up to kWarpLaneMax entries are sorted where they are met, longer
+// ones are queued (see k_sort_lists).
+constexpr int kWarpLaneMax = 64;
+constexpr int kWarpLongMax = 2 * kWarpSortMax;
 
 __device__ __forceinline__ void cswap(int32_t &a, int32_t &b) {
   const int32_t x = min(a, b);
@@ -95,15 +99,23 @@ struct ListOut {
   int32_t *col4;   // sorted lists, padded with -1 to whole 32-byte blocks
   int32_t *dlen;   // length of a list that held repeats, after dropping them
   int32_t *dcorr;  // per rank: repeated edges dropped at that vertex
+  int2 *ldesc;     // per vertex: {first col4 word, length without repeats}
   Ctrl *ctrl;
 };
 
-// A repeat of edge (u, x) in the sorted list of u is dropped: it had added
-// one to the degree of both ends.
-__device__ __forceinline__ void drop_repeat(int32_t u, int32_t x, const ListOut &o) {
-  atomicAdd(&o.dcorr[u], 1);
-  atomicAdd(&o.dcorr[x], 1);
-  *(volatile uint32_t *)&o.ctrl->dups = 1u;
+// The list of u held `dropped` repeats and keeps len entries.  A repeat of
+// edge (u, x) had added one to the degree of both ends: u's share is taken
+// back here in one atomic for the list, x's where the repeat is met.  The
+// flag is stored only until the SM's L1 has seen it set: with every edge
+// given twice (50M pairs) a store and two atomics per repeat took 1.1 of the
+// list sort's 1.65 ms.  Called by one lane.
+__device__ __forceinline__ void note_repeats(int32_t u, int32_t dropped, int32_t len,
+                                             const ListOut &o) {
+  atomicAdd(&o.dcorr[u], dropped);
+  o.dlen[u] = len;
+  uint32_t seen;
+  asm volatile("ld.global.ca.u32 %0, [%1];" : "=r"(seen) : "l"(&o.ctrl->dups));
+  if (!seen) *(volatile uint32_t *)&o.ctrl->dups = 1u;
 }
 
 // Key e*32 + lane of a warp-striped sorted list repeats the key before it.
@@ -118,11 +130,12 @@ __device__ __forceinline__ bool warp_repeat(const int32_t (&x)[E], int e, int32_
 }
 
 // The warp sorts list v (d entries from col + b) into col4 from entry w4,
-// with E keys per lane (32 E >= d), dropping repeated entries.
+// with E keys per lane (32 E >= d), dropping repeated entries; returns the
+// entries left.
 template <int E>
-__device__ __forceinline__ void warp_sort_list(const int32_t *__restrict__ col, int32_t b,
-                                               int32_t d, long long w4, int32_t v,
-                                               const ListOut &o) {
+__device__ __forceinline__ int32_t warp_sort_list(const int32_t *__restrict__ col, int32_t b,
+                                                  int32_t d, long long w4, int32_t v,
+                                                  const ListOut &o) {
   const int lane = threadIdx.x & 31;
   int32_t x[E];
 #pragma unroll
@@ -141,7 +154,7 @@ __device__ __forceinline__ void warp_sort_list(const int32_t *__restrict__ col, 
       const int i = e * 32 + lane;
       if (i < r8) o.col4[w4 + i] = i < d ? x[e] : -1;
     }
-    return;
+    return d;
   }
   // some entry repeats (an edge given more than once): compact the rest
   const uint32_t lt = (1u << lane) - 1u;
@@ -153,11 +166,48 @@ __device__ __forceinline__ void warp_sort_list(const int32_t *__restrict__ col, 
     const bool keep = i < d && !rep;
     const uint32_t bk = __ballot_sync(kFull, keep);
     if (keep) o.col4[w4 + len + __popc(bk & lt)] = x[e];
-    if (rep) drop_repeat(v, x[e], o);
+    if (rep) atomicAdd(&o.dcorr[x[e]], 1);
     len += __popc(bk);
   }
   for (int i = len + lane; i < r8; i += 32) o.col4[w4 + i] = -1;
-  if (lane == 0) o.dlen[v] = len;
+  if (lane == 0) note_repeats(v, d - len, len, o);
+  return len;
+}
+
+// Both halves of the warp sort one list of 9 to 16 entries each, one entry
+// per lane (d = 0: that half has none); returns the entries left.  Half the
+// steps of a whole warp per list, which these lists (most of a random
+// geometric graph's) would leave half empty.
+__device__ __forceinline__ int32_t half_sort_list(const int32_t *__restrict__ col, int32_t b,
+                                                  int32_t d, long long w4, int32_t v,
+                                                  const ListOut &o) {
+  const int lane = threadIdx.x & 31, i = lane & 15;
+  int32_t x = i < d ? __ldg(col + b + i) : INT32_MAX;
+#pragma unroll
+  for (int k = 2; k <= 16; k <<= 1) {
+#pragma unroll
+    for (int j = k >> 1; j > 0; j >>= 1) {
+      const int32_t y = __shfl_xor_sync(kFull, x, j);
+      const bool up = (i & k) == 0, low = (i & j) == 0;
+      x = low == up ? min(x, y) : max(x, y);
+    }
+  }
+  const int32_t p = __shfl_up_sync(kFull, x, 1, 16);
+  const bool rep = i > 0 && i < d && x == p;
+  const uint32_t half = lane & 16 ? 0xffff0000u : 0x0000ffffu;
+  const uint32_t reps = __ballot_sync(kFull, rep) & half;
+  const uint32_t kept = __ballot_sync(kFull, i < d && !rep) & half;
+  if (d == 0) return 0;
+  const int32_t len = __popc(kept);
+  if (reps == 0) {
+    o.col4[w4 + i] = i < d ? x : -1;
+  } else {  // an edge given more than once
+    if (i < d && !rep) o.col4[w4 + __popc(kept & ((1u << lane) - 1u))] = x;
+    if (rep) atomicAdd(&o.dcorr[x], 1);
+    if (i >= len) o.col4[w4 + i] = -1;
+    if (i == 0) note_repeats(v, d - len, len, o);
+  }
+  return len;
 }
 
 // Bitonic sort of buf[0..P) (P a power of two) by a whole block of G
@@ -212,11 +262,11 @@ __device__ __forceinline__ uint32_t block_scan(uint32_t x, uint32_t *s_warp, uin
 
 // Copies the sorted list buf[0..d) of vertex v to dst without its repeated
 // entries, padded with -1 up to r8 entries, by a block of G threads (buf in
-// shared or global memory, written before the last barrier).
+// shared or global memory, written before the last barrier); returns the
+// entries left.
 template <int G>
-__device__ void cta_unique_copy(const int32_t *buf, int32_t d, int32_t *__restrict__ dst,
-                                int32_t r8, int32_t v, const ListOut &o, uint32_t *s_warp,
-                                int32_t *s_len) {
+__device__ int32_t cta_unique_copy(const int32_t *buf, int32_t d, int32_t *__restrict__ dst,
+                                   int32_t r8, int32_t v, const ListOut &o, uint32_t *s_warp) {
   constexpr int PER = 16;  // consecutive entries per thread
   const int tid = threadIdx.x;
   int32_t len = 0;  // uniform: entries written so far
@@ -230,7 +280,7 @@ __device__ void cta_unique_copy(const int32_t *buf, int32_t d, int32_t *__restri
       if (j < d) {
         const int32_t x = buf[j];
         const bool k = j == 0 || x != prev;
-        if (!k) drop_repeat(v, x, o);
+        if (!k) atomicAdd(&o.dcorr[x], 1);
         prev = x;
         keep |= (uint32_t)k << q;
         cnt += k;
@@ -244,35 +294,37 @@ __device__ void cta_unique_copy(const int32_t *buf, int32_t d, int32_t *__restri
     len += (int32_t)total;
   }
   for (int32_t j = len + tid; j < r8; j += G) dst[j] = -1;
-  if (tid == 0) {
-    if (len < d) o.dlen[v] = len;
-    *s_len = len;
-  }
+  if (tid == 0 && len < d) note_repeats(v, d - len, len, o);
+  return len;
 }
 
 // Every forward list into col4, sorted ascending, without repeated entries
 // and padded with -1 to whole 32-byte blocks.  Warps take 32 consecutive
 // vertices at a time: a list of up to 8 entries is sorted by its own lane in
-// registers (a sorting network), one of up to kWarpSortMax entries by the
-// warp in registers (bitonic, up to 16 keys per lane); longer lists go to
-// k_sort_long_lists_warp and k_sort_long_lists.
+// registers (a sorting network), one of up to 16 by half a warp, one of up
+// to kWarpLaneMax by the warp (bitonic, in registers).  Longer ones are
+// queued for k_sort_long_lists, where every warp of the GPU takes one at a
+// time: the long lists belong to neighbouring ranks, and a warp that met 32
+// of them finished long after all others (all lists of R-MAT scale 16 with
+// 2.5M edges: 168 us, with the queue 64 us).
 __global__ void __launch_bounds__(kListThreads)
 k_sort_lists(const int32_t *__restrict__ col, const int32_t *__restrict__ off,
              const int32_t *__restrict__ voff, int32_t n, ListOut o,
-             int32_t *__restrict__ long_lists) {
+             int32_t *__restrict__ queue) {
   Ctrl *ctrl = o.ctrl;
   if (aborted(ctrl)) return;  // an earlier wait of this call ran out
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t warps = gridDim.x * kListWarps;
+  const uint32_t lt = (1u << lane) - 1u;
   for (uint32_t c = blockIdx.x * kListWarps + warp; c * 32u < (uint32_t)n; c += warps) {
     const uint32_t v = c * 32u + lane;
-    int32_t b = 0, d = 0;
-    long long w4 = 0;  // first col4 entry of the list
+    int32_t b = 0, d = 0, w = 0, len = 0;
     if (v < (uint32_t)n) {
       b = __ldg(off + v);
       d = __ldg(off + v + 1) - b;
-      w4 = 4ll * __ldg(voff + v);
+      w = __ldg(voff + v);
     }
+    const long long w4 = 4ll * w;  // first col4 entry of the list
     if (d > 0 && d <= 8) {
       int32_t x[8];
 #pragma unroll
@@ -288,62 +340,56 @@ k_sort_lists(const int32_t *__restrict__ col, const int32_t *__restrict__ off,
         int4 *dst = reinterpret_cast<int4 *>(o.col4 + w4);
         dst[0] = make_int4(x[0], x[1], x[2], x[3]);
         dst[1] = make_int4(x[4], x[5], x[6], x[7]);
+        len = d;
       } else {  // an edge given more than once
-        int len = 0;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-          if (i < d && ((reps >> i) & 1u)) drop_repeat((int32_t)v, x[i], o);
+          if (i < d && ((reps >> i) & 1u)) atomicAdd(&o.dcorr[x[i]], 1);
           else if (i < d) o.col4[w4 + len++] = x[i];
         }
         for (int i = len; i < 8; ++i) o.col4[w4 + i] = -1;
-        o.dlen[v] = len;
+        note_repeats((int32_t)v, d - len, len, o);
       }
     }
-    uint32_t todo = __ballot_sync(kFull, d > 8 && d <= kWarpSortMax);
+    uint32_t todo = __ballot_sync(kFull, d > 8 && d <= 16);
+    while (todo) {  // two lists at a time
+      const int s0 = __ffs(todo) - 1;
+      todo &= todo - 1;
+      const int s1 = todo ? __ffs(todo) - 1 : s0;
+      const bool second = lane >= 16, none = second && s1 == s0;
+      todo &= todo - 1;
+      const int src = second ? s1 : s0;
+      const int32_t lb = __shfl_sync(kFull, b, src), ld = __shfl_sync(kFull, d, src);
+      const long long lw = __shfl_sync(kFull, w4, src);
+      const int32_t l = half_sort_list(col, lb, none ? 0 : ld, lw, (int32_t)(c * 32u) + src, o);
+      const int32_t l0 = __shfl_sync(kFull, l, 0), l1 = __shfl_sync(kFull, l, 16);
+      if (lane == s0) len = l0;
+      else if (lane == s1) len = l1;
+    }
+    todo = __ballot_sync(kFull, d > 16 && d <= kWarpLaneMax);
     while (todo) {
       const int src = __ffs(todo) - 1;
       todo &= todo - 1;
       const int32_t lb = __shfl_sync(kFull, b, src), ld = __shfl_sync(kFull, d, src);
       const long long lw = __shfl_sync(kFull, w4, src);
       const int32_t lv = (int32_t)(c * 32u) + src;
-      if (ld <= 32) warp_sort_list<1>(col, lb, ld, lw, lv, o);
-      else if (ld <= 64) warp_sort_list<2>(col, lb, ld, lw, lv, o);
-      else if (ld <= 128) warp_sort_list<4>(col, lb, ld, lw, lv, o);
-      else if (ld <= 256) warp_sort_list<8>(col, lb, ld, lw, lv, o);
-      else warp_sort_list<16>(col, lb, ld, lw, lv, o);
+      const int32_t l = ld <= 32 ? warp_sort_list<1>(col, lb, ld, lw, lv, o)
+                                 : warp_sort_list<2>(col, lb, ld, lw, lv, o);
+      if (lane == src) len = l;
     }
-    const bool is_long = d > kWarpSortMax;
-    const uint32_t bl = __ballot_sync(kFull, is_long);
-    if (bl) {
-      uint32_t base = 0;
-      if (lane == 0) base = atomicAdd(&ctrl->n_long_lists, (uint32_t)__popc(bl));
-      base = __shfl_sync(kFull, base, 0);
-      if (is_long) long_lists[base + __popc(bl & ((1u << lane) - 1u))] = (int32_t)v;
+    if (v < (uint32_t)n && d <= kWarpLaneMax) o.ldesc[v] = make_int2(w, len);
+    // the queues: lists for a warp from the front of the array, lists for a
+    // CTA in its second half
+    const bool is_warp = d > kWarpLaneMax && d <= kWarpLongMax, is_cta = d > kWarpLongMax;
+    const uint32_t bw = __ballot_sync(kFull, is_warp), bc = __ballot_sync(kFull, is_cta);
+    if (bw | bc) {
+      uint32_t at = 0;
+      if (lane == 0 && bw) at = atomicAdd(&ctrl->n_warp_lists, (uint32_t)__popc(bw));
+      if (lane == 1 && bc) at = atomicAdd(&ctrl->n_cta_lists, (uint32_t)__popc(bc));
+      const uint32_t aw = __shfl_sync(kFull, at, 0), ac = __shfl_sync(kFull, at, 1);
+      if (is_warp) queue[aw + __popc(bw & lt)] = (int32_t)v;
+      if (is_cta) queue[(uint32_t)n + ac + __popc(bc & lt)] = (int32_t)v;
     }
-  }
-}
-
-// Lists of kWarpSortMax + 1 to 2 kWarpSortMax entries: one warp each, 32
-// keys per lane in registers.
-constexpr int kWarpLongMax = 2 * kWarpSortMax;
-
-__global__ void __launch_bounds__(kListThreads)
-k_sort_long_lists_warp(const int32_t *__restrict__ col, const int32_t *__restrict__ off,
-                       const int32_t *__restrict__ voff, ListOut o,
-                       const int32_t *__restrict__ long_lists) {
-  Ctrl *ctrl = o.ctrl;
-  if (aborted(ctrl)) return;
-  const int lane = threadIdx.x & 31;
-  const uint32_t count = ctrl->n_long_lists;
-  for (;;) {
-    uint32_t i = 0;
-    if (lane == 0) i = atomicAdd(&ctrl->next_long_list_warp, 1u);
-    i = __shfl_sync(kFull, i, 0);
-    if (i >= count) break;
-    const int32_t v = __ldg(long_lists + i);
-    const int32_t b = __ldg(off + v), d = __ldg(off + v + 1) - b;
-    if (d > kWarpLongMax) continue;  // the CTA kernel's
-    warp_sort_list<kWarpLongMax / 32>(col, b, d, 4ll * __ldg(voff + v), v, o);
   }
 }
 
@@ -361,106 +407,112 @@ __device__ __forceinline__ int32_t count_below(const int32_t *a, int32_t len, in
   return lo;
 }
 
-// Lists longer than kWarpLongMax: one CTA each.  Up to kCtaSortMax entries
-// the list is sorted in shared memory; a longer one (only with a dense core
-// of more than kCtaSortMax vertices) is sorted in chunks of kCtaSortMax,
-// which are then merged pairwise in global memory, alternating between the
-// list's own region of the column array and its region of col4 so that the
-// last merge lands in the column array.  Then the repeats are dropped on
-// the way into col4.
+// The queued lists: first those longer than kWarpLongMax, one CTA each, then
+// the others, one warp each with up to 32 keys per lane in registers.  A CTA
+// sorts up to kCtaSortMax entries in shared memory; a longer list (only with
+// a dense core of more than kCtaSortMax vertices) is sorted in chunks of
+// kCtaSortMax, which are then merged pairwise in global memory, alternating
+// between the list's own region of the column array and its region of col4
+// so that the last merge lands in the column array.  Then the repeats are
+// dropped on the way into col4.
 __global__ void __launch_bounds__(kLongListThreads, kLongListBlocks)
 k_sort_long_lists(int32_t *col, const int32_t *__restrict__ off,
-                  const int32_t *__restrict__ voff, ListOut o,
-                  const int32_t *__restrict__ long_lists) {
+                  const int32_t *__restrict__ voff, int32_t n, ListOut o,
+                  const int32_t *__restrict__ queue) {
   constexpr int G = kLongListThreads;
   __shared__ int32_t s_buf[kCtaSortMax];
   __shared__ uint32_t s_warp[G / 32];
   __shared__ uint32_t s_i;
-  __shared__ int32_t s_len;
   Ctrl *ctrl = o.ctrl;
   if (aborted(ctrl)) return;
-  const int tid = threadIdx.x;
-  const uint32_t count = ctrl->n_long_lists;
-  for (;;) {
-    if (tid == 0) s_i = atomicAdd(&ctrl->next_long_list, 1u);
+  const int tid = threadIdx.x, lane = tid & 31;
+  const uint32_t n_cta = ctrl->n_cta_lists, n_warp = ctrl->n_warp_lists;
+  while (n_cta) {
+    if (tid == 0) s_i = atomicAdd(&ctrl->next_cta_list, 1u);
     __syncthreads();
     const uint32_t i = s_i;
-    if (i >= count) break;
-    const int32_t v = __ldg(long_lists + i);
-    const int32_t b = __ldg(off + v), d = __ldg(off + v + 1) - b;
-    if (d > kWarpLongMax) {  // shorter lists are the warp kernel's (uniform for the block)
-      int32_t *dst = o.col4 + 4ll * __ldg(voff + v);
-      const int r8 = (d + 7) & ~7;
-      if (d <= kCtaSortMax) {
-        const int P = pow2_at_least(d);
-        for (int j = tid; j < P; j += G) s_buf[j] = j < d ? col[b + j] : INT32_MAX;
+    if (i >= n_cta) break;
+    const int32_t v = __ldg(queue + n + i);
+    const int32_t b = __ldg(off + v), d = __ldg(off + v + 1) - b, w = __ldg(voff + v);
+    int32_t *dst = o.col4 + 4ll * w;
+    const int r8 = (d + 7) & ~7;
+    int32_t len;
+    if (d <= kCtaSortMax) {
+      const int P = pow2_at_least(d);
+      for (int j = tid; j < P; j += G) s_buf[j] = j < d ? col[b + j] : INT32_MAX;
+      __syncthreads();
+      bitonic_smem<G>(s_buf, P, tid);
+      len = cta_unique_copy<G>(s_buf, d, dst, r8, v, o, s_warp);
+    } else {
+      int32_t *A = col + b;  // the list's region of the column array: d entries
+      int32_t *B = dst;      // its region of col4: r8 >= d entries
+      const int32_t chunks = (d + kCtaSortMax - 1) / kCtaSortMax;
+      int levels = 0;
+      while ((1 << levels) < chunks) ++levels;
+      int32_t *src = (levels & 1) ? B : A;
+      for (int32_t c0 = 0; c0 < d; c0 += kCtaSortMax) {
+        const int32_t part = min(kCtaSortMax, d - c0);
+        for (int j = tid; j < kCtaSortMax; j += G) s_buf[j] = j < part ? A[c0 + j] : INT32_MAX;
         __syncthreads();
-        bitonic_smem<G>(s_buf, P, tid);
-        cta_unique_copy<G>(s_buf, d, dst, r8, v, o, s_warp, &s_len);
-      } else {
-        int32_t *A = col + b;  // the list's region of the column array: d entries
-        int32_t *B = dst;      // its region of col4: r8 >= d entries
-        const int32_t chunks = (d + kCtaSortMax - 1) / kCtaSortMax;
-        int levels = 0;
-        while ((1 << levels) < chunks) ++levels;
-        int32_t *src = (levels & 1) ? B : A;
-        for (int32_t c0 = 0; c0 < d; c0 += kCtaSortMax) {
-          const int32_t len = min(kCtaSortMax, d - c0);
-          for (int j = tid; j < kCtaSortMax; j += G) s_buf[j] = j < len ? A[c0 + j] : INT32_MAX;
-          __syncthreads();
-          bitonic_smem<G>(s_buf, kCtaSortMax, tid);
-          for (int j = tid; j < len; j += G) src[c0 + j] = s_buf[j];
-          __syncthreads();
-        }
-        int32_t *to = src == A ? B : A;
-        for (int32_t w = kCtaSortMax; w < d; w <<= 1) {
-          // runs [s0, s0 + w) and [s0 + w, s0 + 2w) merged into to[s0 ..):
-          // an entry's place is its place in its run plus the entries of the
-          // other run before it (ties: the first run's entries first)
-          for (int32_t j = tid; j < d; j += G) {
-            const int32_t s0 = j / (2 * w) * (2 * w);
-            const int32_t am = min(s0 + w, d), be = min(s0 + 2 * w, d);
-            const int32_t x = src[j];
-            const int32_t at = j < am ? (j - s0) + count_below(src + am, be - am, x, false)
-                                      : (j - am) + count_below(src + s0, am - s0, x, true);
-            to[s0 + at] = x;
-          }
-          __syncthreads();
-          int32_t *t = src;
-          src = to;
-          to = t;
-        }
-        cta_unique_copy<G>(A, d, B, r8, v, o, s_warp, &s_len);
+        bitonic_smem<G>(s_buf, kCtaSortMax, tid);
+        for (int j = tid; j < part; j += G) src[c0 + j] = s_buf[j];
+        __syncthreads();
       }
+      int32_t *to = src == A ? B : A;
+      for (int32_t run = kCtaSortMax; run < d; run <<= 1) {
+        // runs [s0, s0 + run) and [s0 + run, s0 + 2 run) merged into
+        // to[s0 ..): an entry's place is its place in its run plus the
+        // entries of the other run before it (ties: the first run's first)
+        for (int32_t j = tid; j < d; j += G) {
+          const int32_t s0 = j / (2 * run) * (2 * run);
+          const int32_t am = min(s0 + run, d), be = min(s0 + 2 * run, d);
+          const int32_t x = src[j];
+          const int32_t at = j < am ? (j - s0) + count_below(src + am, be - am, x, false)
+                                    : (j - am) + count_below(src + s0, am - s0, x, true);
+          to[s0 + at] = x;
+        }
+        __syncthreads();
+        int32_t *t = src;
+        src = to;
+        to = t;
+      }
+      len = cta_unique_copy<G>(A, d, B, r8, v, o, s_warp);
     }
+    if (tid == 0) o.ldesc[v] = make_int2(w, len);
     __syncthreads();  // s_buf and s_i are reused
+  }
+  while (n_warp) {
+    uint32_t i = 0;
+    if (lane == 0) i = atomicAdd(&ctrl->next_warp_list, 1u);
+    i = __shfl_sync(kFull, i, 0);
+    if (i >= n_warp) break;
+    const int32_t v = __ldg(queue + i);
+    const int32_t b = __ldg(off + v), d = __ldg(off + v + 1) - b, w = __ldg(voff + v);
+    const int32_t len = d <= 128   ? warp_sort_list<4>(col, b, d, 4ll * w, v, o)
+                        : d <= 256 ? warp_sort_list<8>(col, b, d, 4ll * w, v, o)
+                        : d <= 512 ? warp_sort_list<16>(col, b, d, 4ll * w, v, o)
+                                   : warp_sort_list<32>(col, b, d, 4ll * w, v, o);
+    if (lane == 0) o.ldesc[v] = make_int2(w, len);
   }
 }
 
-// The row array again after repeats were dropped: row[off[v] + i] = v (off:
-// the recounted node array).  One warp per vertex; only when some list held
-// a repeat.
+// After repeats were dropped: the row array again, row[off[v] + i] = v (off:
+// the recounted node array), one warp per vertex, and the degrees without
+// the repeats, deg[v] -= dcorr[rank[v]] (caller ids).  Nothing when no list
+// held a repeat.
 __global__ void __launch_bounds__(kListThreads)
-k_fix_rows(const int32_t *__restrict__ off, int32_t n, const Ctrl *ctrl,
-           int32_t *__restrict__ row) {
-  if (aborted(ctrl) || *(volatile const uint32_t *)&ctrl->dups == 0u) return;
+k_fix_repeats(const int32_t *__restrict__ off, int32_t n, const int32_t *__restrict__ dcorr,
+              const int32_t *__restrict__ rank, const Ctrl *ctrl, int32_t *__restrict__ row,
+              int32_t *__restrict__ deg) {
+  if (aborted(ctrl) || ctrl->dups == 0u) return;
   const int lane = threadIdx.x & 31;
-  const uint32_t warps = gridDim.x * kListWarps;
-  for (uint32_t v = (blockIdx.x * kListThreads + threadIdx.x) >> 5; v < (uint32_t)n; v += warps) {
+  const uint32_t first = blockIdx.x * kListThreads + threadIdx.x;
+  const uint32_t stride = gridDim.x * kListThreads;
+  for (uint32_t v = first; v < (uint32_t)n; v += stride) deg[v] -= __ldg(dcorr + __ldg(rank + v));
+  for (uint32_t v = first >> 5; v < (uint32_t)n; v += stride >> 5) {
     const int32_t b = __ldg(off + v), e = __ldg(off + v + 1);
     for (int32_t i = b + lane; i < e; i += 32) row[i] = (int32_t)v;
   }
-}
-
-// The degrees without repeats: deg[v] -= dcorr[rank[v]] (caller ids); only
-// when some list held a repeat.
-__global__ void __launch_bounds__(kListThreads)
-k_fix_degree(const int32_t *__restrict__ dcorr, const int32_t *__restrict__ rank, int32_t n,
-             const Ctrl *ctrl, int32_t *__restrict__ deg) {
-  if (aborted(ctrl) || *(volatile const uint32_t *)&ctrl->dups == 0u) return;
-  const uint32_t stride = gridDim.x * kListThreads;
-  for (uint32_t v = blockIdx.x * kListThreads + threadIdx.x; v < (uint32_t)n; v += stride)
-    deg[v] -= __ldg(dcorr + __ldg(rank + v));
 }
 
 // heavy_ratio_pct = 100: the longer list is always the one hashed; larger
@@ -616,34 +668,29 @@ uint32_t group_grid(uint32_t m_bound) {
 
 }  // namespace
 
-void launch_sort_lists(int32_t *col, const int32_t *off, const int32_t *voff, int32_t n,
-                       Ctrl *ctrl, int32_t *col4, int32_t *long_lists, int32_t *dlen,
-                       int32_t *dcorr, cudaStream_t st) {
+static uint32_t num_sms() {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  sms = sms > 0 ? sms : 1;
-  const ListOut o{col4, dlen, dcorr, ctrl};
+  return (uint32_t)(sms > 0 ? sms : 1);
+}
+
+void launch_sort_lists(int32_t *col, const int32_t *off, const int32_t *voff, int32_t n,
+                       Ctrl *ctrl, int32_t *col4, int32_t *queue, int32_t *dlen,
+                       int32_t *dcorr, int2 *ldesc, cudaStream_t st) {
+  const ListOut o{col4, dlen, dcorr, ldesc, ctrl};
   const uint32_t chunks = ((uint32_t)n + 31u) / 32u;
-  const uint32_t grid = max(1u, min((chunks + kListWarps - 1) / kListWarps, (uint32_t)sms * 8u));
-  k_sort_lists<<<grid, kListThreads, 0, st>>>(col, off, voff, n, o, long_lists);
-  k_sort_long_lists_warp<<<sms * 4, kListThreads, 0, st>>>(col, off, voff, o, long_lists);
-  k_sort_long_lists<<<sms * kLongListBlocks, kLongListThreads, 0, st>>>(col, off, voff, o,
-                                                                        long_lists);
-  note_launch();
+  const uint32_t grid = max(1u, min((chunks + kListWarps - 1) / kListWarps, num_sms() * 8u));
+  k_sort_lists<<<grid, kListThreads, 0, st>>>(col, off, voff, n, o, queue);
+  k_sort_long_lists<<<num_sms() * kLongListBlocks, kLongListThreads, 0, st>>>(col, off, voff, n,
+                                                                              o, queue);
   note_launch();
   note_launch();
 }
 
 void launch_fix_repeats(const int32_t *off, int32_t n, const int32_t *dcorr, const int32_t *rank,
                         Ctrl *ctrl, int32_t *row, int32_t *deg, cudaStream_t st) {
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const uint32_t grid = (uint32_t)(sms > 0 ? sms : 1) * 8u;
-  k_fix_rows<<<grid, kListThreads, 0, st>>>(off, n, ctrl, row);
-  k_fix_degree<<<grid, kListThreads, 0, st>>>(dcorr, rank, n, ctrl, deg);
-  note_launch();
+  k_fix_repeats<<<num_sms() * 8u, kListThreads, 0, st>>>(off, n, dcorr, rank, ctrl, row, deg);
   note_launch();
 }
 

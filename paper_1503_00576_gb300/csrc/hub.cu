@@ -287,17 +287,17 @@ k_hub_zero(uint8_t *__restrict__ A, int32_t Hmax, const Ctrl *ctrl) {
 // A(u - lo, v - lo) = A(v - lo, u - lo) = 1 for every forward edge of H
 // (the matrix was zeroed before).  One warp per vertex of H.
 __global__ void __launch_bounds__(256)
-k_hub_scatter(const int32_t *__restrict__ off, const int32_t *__restrict__ voff,
-              const int32_t *__restrict__ col4, int32_t n, int32_t pitch, const Ctrl *ctrl,
-              uint8_t *__restrict__ A) {
+k_hub_scatter(const int2 *__restrict__ ldesc, const int32_t *__restrict__ col4, int32_t n,
+              int32_t pitch, const Ctrl *ctrl, uint8_t *__restrict__ A) {
   if (aborted(ctrl) || !ctrl->hub_on) return;
   const int32_t H = (int32_t)ctrl->hub_size, lo = n - H;
   const int lane = threadIdx.x & 31;
   const uint32_t warps = gridDim.x * (blockDim.x / 32);
   for (uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < (uint32_t)H; w += warps) {
     const int32_t u = lo + (int32_t)w;
-    const int32_t d = __ldg(off + u + 1) - __ldg(off + u);
-    const int32_t *list = col4 + 4ll * __ldg(voff + u);
+    const int2 ld = __ldg(ldesc + u);  // {first col4 word, length}
+    const int32_t d = ld.y;
+    const int32_t *list = col4 + 4ll * ld.x;
     for (int32_t i = lane; i < d; i += 32) {
       const int32_t v = __ldg(list + i) - lo;  // > u - lo >= 0
       A[(size_t)w * pitch + v] = kOne;
@@ -492,9 +492,8 @@ void launch_hub_decide(const int32_t *off, const int32_t *col, int32_t n, int32_
   note_launch();
 }
 
-cudaError_t launch_hub_count(const int32_t *off, const int32_t *voff, const int32_t *col4,
-                             int32_t n, int32_t Hmax, uint8_t *region, Ctrl *ctrl, int64_t *t,
-                             cudaStream_t st) {
+cudaError_t launch_hub_count(const int2 *ldesc, const int32_t *col4, int32_t n, int32_t Hmax,
+                             uint8_t *region, Ctrl *ctrl, int64_t *t, cudaStream_t st) {
   uint8_t *A = region;
   uint32_t *r = reinterpret_cast<uint32_t *>(region + (size_t)Hmax * Hmax);
   EncodeTiled enc = encode_fn();
@@ -523,7 +522,7 @@ cudaError_t launch_hub_count(const int32_t *off, const int32_t *voff, const int3
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   k_hub_zero<<<(sms > 0 ? sms : 1) * 8, 256, 0, st>>>(A, Hmax, ctrl);
-  k_hub_scatter<<<(Hmax + 7) / 8, 256, 0, st>>>(off, voff, col4, n, Hmax, ctrl, A);
+  k_hub_scatter<<<(Hmax + 7) / 8, 256, 0, st>>>(ldesc, col4, n, Hmax, ctrl, A);
   const int T = Hmax / kHubTile;
   k_hub_gemm<<<T * (T + 1) / 2, kHubThreads, kHubSmemBytes, st>>>(map, A, Hmax, ctrl, r);
   k_hub_finish<<<1, 1024, 0, st>>>(r, ctrl, t);

@@ -213,7 +213,6 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
   auto *st_orient = reinterpret_cast<unsigned long long *>(ws + L.st_orient);
   auto *st_scan = reinterpret_cast<unsigned long long *>(ws + L.st_scan);
   auto *st_scan2 = reinterpret_cast<unsigned long long *>(ws + L.st_scan2);
-  auto *st_scan3 = reinterpret_cast<unsigned long long *>(ws + L.st_scan3);
   auto *st_scan4 = reinterpret_cast<unsigned long long *>(ws + L.st_scan4);
   uint64_t *keys_a = reinterpret_cast<uint64_t *>(ws + L.keys_a);
   uint64_t *keys_b = reinterpret_cast<uint64_t *>(ws + L.keys_b);
@@ -225,13 +224,11 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
   int32_t *voff = reinterpret_cast<int32_t *>(ws + L.voff);
   int32_t *col4 = reinterpret_cast<int32_t *>(ws + L.col4);
   int32_t *goff = reinterpret_cast<int32_t *>(ws + L.goff);
-  int32_t *warp_groups = reinterpret_cast<int32_t *>(ws + L.warp_groups);
-  int32_t *cta_groups = reinterpret_cast<int32_t *>(ws + L.cta_groups);
-  int32_t *big_groups = reinterpret_cast<int32_t *>(ws + L.big_groups);
+  int32_t *gcnt = reinterpret_cast<int32_t *>(ws + L.gcnt);
+  int32_t *groups = reinterpret_cast<int32_t *>(ws + L.groups);
+  int32_t *big_groups = voff;  // free once the lists' records are written
   int32_t *rank = reinterpret_cast<int32_t *>(ws + L.rank);
-  // per rank: repeated edges dropped by the list sort (the rank keys are
-  // free by then)
-  int32_t *dcorr = reinterpret_cast<int32_t *>(ws + L.vkeys_a);
+  int32_t *dcorr = reinterpret_cast<int32_t *>(ws + L.dcorr);  // per rank: repeats dropped
   // per vertex: its list's first col4 word and length (the second rank-key
   // buffer, free after the rank sort)
   int2 *ldesc = reinterpret_cast<int2 *>(ws + L.vkeys_b);
@@ -249,14 +246,17 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
     ++slot;
   };
 
-  // zero the control block, histograms and the look-back status words in use
-  TC_CUDA(cudaMemsetAsync(ws, 0, L.st_sort + sizeof(unsigned long long) * words *
-                                                  (size_t)radix_passes(b), st),
+  // zeroed in one piece: degrees (if they are not the caller's), control
+  // block, histograms, look-back status, counters, counts, and the radix
+  // passes' look-back status behind them
+  if (deg_out)
+    TC_CUDA(cudaMemsetAsync(deg, 0, sizeof(int32_t) * (size_t)n, st), "memset deg");
+  const size_t zero_from = deg_out ? L.ctrl : L.deg;
+  TC_CUDA(cudaMemsetAsync(ws + zero_from, 0, (t_rank ? L.st_sort : L.t_rank) - zero_from, st),
           "memset control");
-  TC_CUDA(cudaMemsetAsync(ws + L.st_orient, 0, L.keys_a - L.st_orient, st), "memset status");
-  TC_CUDA(cudaMemsetAsync(deg, 0, sizeof(int32_t) * (size_t)n, st), "memset deg");
-  TC_CUDA(cudaMemsetAsync(outdeg, 0, sizeof(int32_t) * (size_t)n, st), "memset outdeg");
-  if (t_rank) TC_CUDA(cudaMemsetAsync(t_rank, 0, sizeof(int64_t) * (size_t)n, st), "memset t");
+  TC_CUDA(cudaMemsetAsync(ws + L.st_sort, 0,
+                          sizeof(unsigned long long) * words * (size_t)radix_passes(b), st),
+          "memset status");
 
   // undirected keys and the degrees (repeated edges counted as often as
   // they are given; the list sort takes them back)
@@ -316,9 +316,7 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
   pt.stop(TC_PHASE_SORT);
 
   pt.start(TC_PHASE_OFFSETS);
-  launch_offsets(outdeg, n, off, nullptr, nullptr, nullptr, nullptr, tune, st_scan,
-                 &ctrl->tile_ticket[kTicketScan], ctrl, st);
-  launch_word_offsets(outdeg, n, voff, st_scan3, &ctrl->tile_ticket[kTicketVecScan], ctrl, st);
+  launch_offsets(outdeg, n, off, voff, st_scan, &ctrl->tile_ticket[kTicketScan], ctrl, st);
   // whether the top ranks are counted densely (their edges are then left
   // out of the partner groups)
   const bool hub = L.has_hub && tune.hub_min_edges >= 0;
@@ -326,30 +324,27 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
   if (hub) launch_hub_decide(off, col, n, H, tune.hub_min_edges, t_out != nullptr, ctrl, st);
   pt.stop(TC_PHASE_OFFSETS);
 
-  // every forward list sorted into the padded column array col4 (the
-  // warp-group list is free scratch until the binning), repeated edges
-  // dropped: their lists' new lengths overwrite the out-degrees, and only if
-  // there were any, the node array, the edge count, the row array and the
-  // degrees are made right again
+  // every forward list sorted into the padded column array col4 (the rank
+  // keys' first buffer is free scratch by now), repeated edges dropped: their
+  // lists' new lengths overwrite the out-degrees, and only if there were any,
+  // the node array, the edge count, the row array and the degrees are made
+  // right again
   pt.start(TC_PHASE_LISTS);
-  TC_CUDA(cudaMemsetAsync(dcorr, 0, sizeof(int32_t) * (size_t)n, st), "memset repeats");
-  launch_sort_lists(col, off, voff, n, ctrl, col4, warp_groups, outdeg, dcorr, st);
+  launch_sort_lists(col, off, voff, n, ctrl, col4, reinterpret_cast<int32_t *>(vkeys_a), outdeg,
+                    dcorr, ldesc, st);
   launch_recount(outdeg, n, off, st_scan4, &ctrl->tile_ticket[kTicketRecount], ctrl, st);
   launch_fix_repeats(off, n, dcorr, rank, ctrl, row, deg, st);
-  launch_list_desc(off, voff, n, ctrl, ldesc, st);
   pt.stop(TC_PHASE_LISTS);
 
   // partner groups: each forward edge goes to the endpoint with the longer
   // forward list.  Group keys, read from the sorted lists, go to `in` (the
   // owner sort's input, free now); a radix sort over the group bits then
   // gathers every group's partners, its last pass counting the group sizes
-  // into gcnt (the out-degree array's space) and writing the skipped blocks
-  // of each partner's stream beside the partner array.
+  // into gcnt and writing the skipped blocks of each partner's stream beside
+  // the partner array.
   pt.start(TC_PHASE_GROUPS);
   launch_group_keys(row, col4, off, ldesc, m, b, passes3, tune.heavy_ratio_pct, ctrl, in,
                     hist + 256 * kGroupSlot, st);
-  int32_t *gcnt = outdeg;
-  TC_CUDA(cudaMemsetAsync(gcnt, 0, sizeof(int32_t) * (size_t)n, st), "memset groups");
   const bool skip_in_key = 2 * b <= kSkipShift;
   uint64_t *gin = in, *gout = out;  // row and col are dead after the group keys
   for (int p = 0; p < passes3; ++p) {
@@ -380,8 +375,8 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
             "memset skips");
   // only this run's share of the groups is binned (all of them unless the
   // counting is split over several devices, Sec. III-E)
-  launch_offsets(gcnt, n, goff, off, warp_groups, cta_groups, big_groups, tune, st_scan2,
-                 &ctrl->tile_ticket[kTicketGroupScan], ctrl, st, shard, shards);
+  launch_group_offsets(gcnt, nullptr, n, goff, ldesc, groups, big_groups, tune, st_scan2,
+                       &ctrl->tile_ticket[kTicketGroupScan], ctrl, st, shard, shards);
   pt.stop(TC_PHASE_GROUPS);
   if (work_stats) launch_work(off, goff, part, pskip, n, ctrl, st, shard, shards);
 
@@ -389,16 +384,14 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
   // the dense block's triangles belong to the first share alone (every share
   // leaves the block's edges off its hash path)
   if (hub && shard == 0) {
-    TC_CUDA(launch_hub_count(off, voff, col4, n, H, ws + L.hub, ctrl,
+    TC_CUDA(launch_hub_count(ldesc, col4, n, H, ws + L.hub, ctrl,
                              t_out ? t_rank : nullptr, st),
             "dense hub block");
   }
   // each partner's stream goes to the group sort's other buffer (free now)
   int2 *desc = reinterpret_cast<int2 *>(gin);
-  cudaError_t e = launch_count(off, voff, ldesc, col4, goff, part, pskip, desc, warp_groups,
-                               cta_groups,
-                               big_groups, n, ctrl, t_out ? t_rank : nullptr,
-                               t_out ? nullptr : t_rank, st);
+  cudaError_t e = launch_count(ldesc, col4, goff, part, pskip, desc, groups, big_groups, n, ctrl,
+                               t_out ? t_rank : nullptr, t_out ? nullptr : t_rank, st);
   if (e == cudaSuccess && t_out) launch_gather_counts(t_rank, rank, n, t_out, ctrl, st);
   if (e == cudaSuccess && batch) {
     if (t_out) {  // per graph: (sum of t) / 3

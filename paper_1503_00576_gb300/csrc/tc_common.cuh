@@ -74,9 +74,12 @@ struct Ctrl {
   uint32_t next_big_group;
   unsigned long long total;        // triangle count T
   uint32_t m_in;                   // input pairs that are real (not batch padding)
-  uint32_t n_long_lists;           // forward lists sorted by the long-list kernels
-  uint32_t next_long_list;         // work cursor of the CTA-per-list kernel
-  uint32_t next_long_list_warp;    // work cursor of the warp-per-list kernel
+  uint32_t n_part;                 // partners of all groups (set by the group scan)
+  uint32_t n_warp_lists;           // queued forward lists: sorted by one warp each
+  uint32_t n_cta_lists;            // ... by a CTA each
+  uint32_t next_warp_list;         // work cursors of the queued lists
+  uint32_t next_cta_list;
+  uint32_t pad_[2];
   uint32_t hub_on;                 // the hub block is counted densely (hub.cu)
   uint32_t hub_lo;                 // its first rank
   uint32_t hub_size;               // its number of vertices (hub_lo + hub_size = n)
@@ -96,8 +99,7 @@ enum {
   kTicketOrient = kMaxPasses,
   kTicketScan = kMaxPasses + 1,
   kTicketGroupScan = kMaxPasses + 2,
-  kTicketVecScan = kMaxPasses + 3,
-  kTicketRecount = kMaxPasses + 4
+  kTicketRecount = kMaxPasses + 3
 };
 static_assert(kTicketRecount < 24, "ticket slots");
 
@@ -109,9 +111,12 @@ constexpr unsigned long long kValueMask = (1ull << 62) - 1;
 
 #ifdef __CUDACC__
 // True once some kernel of this call has recorded a wait that ran out: the
-// data it left behind is incomplete, so later kernels must not read it.
+// data it left behind is incomplete, so later kernels must not read it.  A
+// plain load: what an earlier kernel recorded is seen, and the threads of an
+// SM share one L1 line (a volatile load per thread, 300,000 of them on one
+// L2 word, made a kernel that had nothing to do last 6 us instead of 2).
 __device__ __forceinline__ bool aborted(const Ctrl *ctrl) {
-  return (*(const volatile uint32_t *)&ctrl->err & kErrTimeout) != 0u;
+  return (ctrl->err & kErrTimeout) != 0u;
 }
 
 #endif
@@ -150,10 +155,14 @@ struct BatchDesc {
 // Workspace layout for an input of m_in pairs and n vertices.  All offsets
 // are 256-byte aligned.
 struct Layout {
-  size_t ctrl, hist, st_sort, st_orient, st_scan, st_scan2, st_scan3, st_scan4;
-  size_t keys_a, keys_b, deg, outdeg, off, voff, goff, warp_groups, cta_groups, big_groups;
+  // zeroed by every run, in one piece: deg (unless the caller's array is
+  // used), ctrl .. dcorr, t_rank (runs that need it), st_sort (runs that sort
+  // by radix passes)
+  size_t deg, ctrl, hist, st_orient, st_scan, st_scan2, st_scan4, outdeg, gcnt, dcorr, t_rank,
+      st_sort;
+  size_t keys_a, keys_b, off, voff, goff, groups;
   size_t col4;
-  size_t rank, vkeys_a, vkeys_b, t_rank;
+  size_t rank, vkeys_a, vkeys_b;
   size_t hub;  // dense hub block (0 bytes unless the layout asked for it)
   bool has_hub;
   int32_t hub_vertices;  // size of the hub set the hub region was laid out for
@@ -207,31 +216,30 @@ inline Layout make_layout(int64_t m_in, int32_t n, bool with_hub = false,
   L.orient_tiles = (uint32_t)((m + kOrientTile - 1) / kOrientTile);
   L.scan_tiles = (uint32_t)((nv + 1 + kScanTile - 1) / kScanTile);
   L.st_sort_words_per_pass = (size_t)L.sort_tiles * 256;
+  L.deg = take(sizeof(int32_t) * nv);
   L.ctrl = take(sizeof(Ctrl));
   L.hist = take(sizeof(uint32_t) * 256 * kMaxPasses);
+  L.st_orient = take(sizeof(unsigned long long) * L.orient_tiles);
+  L.st_scan = take(sizeof(unsigned long long) * L.scan_tiles);
+  L.st_scan2 = take(sizeof(unsigned long long) * L.scan_tiles);
+  L.st_scan4 = take(sizeof(unsigned long long) * L.scan_tiles);
+  L.outdeg = take(sizeof(int32_t) * nv);
+  L.gcnt = take(sizeof(int32_t) * nv);
+  L.dcorr = take(sizeof(int32_t) * nv);
+  L.t_rank = take(sizeof(int64_t) * nv);
   // look-back status words for the passes that ids of [0, n) need (a run
   // with fewer vertices needs no more)
   L.st_sort = take(sizeof(unsigned long long) * L.st_sort_words_per_pass *
                    (size_t)radix_passes(id_bits(n > 0 ? n : 1)));
-  L.st_orient = take(sizeof(unsigned long long) * L.orient_tiles);
-  L.st_scan = take(sizeof(unsigned long long) * L.scan_tiles);
-  L.st_scan2 = take(sizeof(unsigned long long) * L.scan_tiles);
-  L.st_scan3 = take(sizeof(unsigned long long) * L.scan_tiles);
-  L.st_scan4 = take(sizeof(unsigned long long) * L.scan_tiles);
   L.keys_a = take(sizeof(uint64_t) * m);
   L.keys_b = take(sizeof(uint64_t) * m);
-  L.deg = take(sizeof(int32_t) * nv);
-  L.outdeg = take(sizeof(int32_t) * nv);
   L.off = take(sizeof(int32_t) * (nv + 1));
   L.voff = take(sizeof(int32_t) * (nv + 1));
   L.goff = take(sizeof(int32_t) * (nv + 1));
-  L.warp_groups = take(sizeof(int32_t) * nv);
-  L.cta_groups = take(sizeof(int32_t) * nv);
-  L.big_groups = take(sizeof(int32_t) * nv);
+  L.groups = take(sizeof(int32_t) * nv);
   L.rank = take(sizeof(int32_t) * nv);
   L.vkeys_a = take(sizeof(uint64_t) * nv);
   L.vkeys_b = take(sizeof(uint64_t) * nv);
-  L.t_rank = take(sizeof(int64_t) * nv);
   // forward lists padded to whole 32-byte blocks: at most m + 7 min(n, m)
   // elements, since each non-empty list adds at most 7
   L.col4 = take(sizeof(int32_t) * (m + 7 * (nv < m ? nv : m)));
@@ -289,25 +297,28 @@ void launch_rank_keys(const int32_t *deg, int32_t n, int b, int passes, uint64_t
 void launch_orient(const uint64_t *keys, uint32_t m_in, int b, const int32_t *rank,
                    uint64_t *okeys, uint32_t *hist2, int passes2, unsigned long long *status,
                    Ctrl *ctrl, cudaStream_t st);
-// Exclusive scan counts[0..n) -> off[0..n].  With row_off != nullptr the
-// entries are partner groups and are binned into warp_list / cta_list /
-// big_list by the length of their hashed list; only the groups h with
-// h mod shards = shard are binned (the share of the counting work this run
-// does; shards = 1 bins them all).
-void launch_offsets(const int32_t *counts, int32_t n, int32_t *off, const int32_t *row_off,
-                    int32_t *warp_list, int32_t *cta_list, int32_t *big_list, Tuning tune,
-                    unsigned long long *status, uint32_t *ticket, Ctrl *ctrl, cudaStream_t st,
-                    int32_t shard = 0, int32_t shards = 1);
+// The two node arrays of the forward lists from the list lengths counts[0..n):
+// off[0..n], their exclusive scan, and voff[0..n], the exclusive scan of 2
+// ceil(counts / 8): the node array of the padded column array (lists in
+// whole 32-byte blocks), in 16-byte words.  Sets ctrl->m = off[n].
+void launch_offsets(const int32_t *counts, int32_t n, int32_t *off, int32_t *voff,
+                    unsigned long long *status, uint32_t *ticket, Ctrl *ctrl, cudaStream_t st);
+// Exclusive scan of the partner-group sizes counts[h] (+ own[h], if not
+// nullptr) -> goff[0..n], ctrl->n_part = goff[n]; the groups are binned into
+// the lists by the length of their hashed list (ldesc): warp groups from
+// the front of `groups` up, CTA groups from its end down (n entries hold
+// both), big groups into big_list.  Only the groups h with h mod shards =
+// shard are binned (the share of the counting work this run does; shards = 1
+// bins them all).
+void launch_group_offsets(const int32_t *counts, const int32_t *own, int32_t n, int32_t *goff,
+                          const int2 *ldesc, int32_t *groups, int32_t *big_list, Tuning tune,
+                          unsigned long long *status, uint32_t *ticket, Ctrl *ctrl,
+                          cudaStream_t st, int32_t shard = 0, int32_t shards = 1);
 // The node array again, from the list lengths left after the list sort
 // dropped repeated edges, and ctrl->m = their sum; nothing (the kernel
 // returns at once) when no list held a repeat.
 void launch_recount(const int32_t *counts, int32_t n, int32_t *off, unsigned long long *status,
                     uint32_t *ticket, Ctrl *ctrl, cudaStream_t st);
-// Exclusive scan of 2 ceil(counts / 8) -> voff[0..n]: the node array of the
-// padded column array (lists in whole 32-byte blocks), in 16-byte words.
-void launch_word_offsets(const int32_t *counts, int32_t n, int32_t *voff,
-                         unsigned long long *status, uint32_t *ticket, Ctrl *ctrl,
-                         cudaStream_t st);
 // ---- launchers (hub.cu) ----
 // Workspace of the dense hub block of H vertices: the H x H fp8 matrix and
 // the per-vertex sums.
@@ -321,34 +332,34 @@ void launch_hub_decide(const int32_t *off, const int32_t *col, int32_t n, int32_
 // Counts the triangles inside the hub block (if ctrl->hub_on): adds them to
 // ctrl->total and, if t != nullptr, to the per-vertex counts t (rank space).
 // Needs the forward lists; region: hub_bytes(Hmax) bytes, 256-byte aligned.
-cudaError_t launch_hub_count(const int32_t *off, const int32_t *voff, const int32_t *col4,
-                             int32_t n, int32_t Hmax, uint8_t *region, Ctrl *ctrl, int64_t *t,
-                             cudaStream_t st);
+cudaError_t launch_hub_count(const int2 *ldesc, const int32_t *col4, int32_t n, int32_t Hmax,
+                             uint8_t *region, Ctrl *ctrl, int64_t *t, cudaStream_t st);
 // ---- launchers (group.cu) ----
 // Sorts every forward list (the column array col, grouped by owner, node
 // array off) into the padded column array col4 (list v from 16-byte word
-// voff[v], padded with -1 to whole 32-byte blocks).  A
+// voff[v], padded with -1 to whole 32-byte blocks) and writes ldesc[v] =
+// {voff[v], length}: each list's first word and length in one record.  A
 // repeated entry (an edge given more than once) is dropped: the list's
 // length goes to dlen[v] (written only for such lists; dlen holds the
 // lengths with repeats on entry), each dropped copy adds one to dcorr at
 // both its ends (rank space; zero on entry) and ctrl->dups is set.
-// long_lists: scratch of n entries; col is scratch for lists longer than
+// queue: scratch of 2n entries; col is scratch for lists longer than
 // kCtaSortMax.
 void launch_sort_lists(int32_t *col, const int32_t *off, const int32_t *voff, int32_t n,
-                       Ctrl *ctrl, int32_t *col4, int32_t *long_lists, int32_t *dlen,
-                       int32_t *dcorr, cudaStream_t st);
+                       Ctrl *ctrl, int32_t *col4, int32_t *queue, int32_t *dlen,
+                       int32_t *dcorr, int2 *ldesc, cudaStream_t st);
 // After the list sort, if some list held repeats: the row array again
 // (row[off[v] + i] = v, from the recounted node array) and the degrees
-// without repeats (deg[v] -= dcorr[rank[v]], caller ids).  Both return at
-// once otherwise.
+// without repeats (deg[v] -= dcorr[rank[v]], caller ids).  Returns at once
+// otherwise.
 void launch_fix_repeats(const int32_t *off, int32_t n, const int32_t *dcorr, const int32_t *rank,
                         Ctrl *ctrl, int32_t *row, int32_t *deg, cudaStream_t st);
 // Group keys s << kSkipShift | h << b | l of every forward edge (h: the
 // endpoint with the longer forward list, l: the other one, s: the leading
 // blocks of N+(l) the intersection skips, 0 when 2b > kSkipShift), with the
 // digit histograms of the h field for the group sort.  Reads the sorted
-// lists (col4; their first words and lengths from ldesc, see
-// launch_list_desc) in owner order (row, node array off).
+// lists (col4; their first words and lengths from ldesc) in owner order
+// (row, node array off).
 void launch_group_keys(const int32_t *row, const int32_t *col4, const int32_t *off,
                        const int2 *ldesc, uint32_t m_bound, int b,
                        int passes, int32_t heavy_ratio_pct, Ctrl *ctrl, uint64_t *gkeys,
@@ -364,16 +375,11 @@ void launch_work(const int32_t *off, const int32_t *goff, const int32_t *part,
 // nullptr, tg[h] += triangles found in group h (their sum per graph is the
 // graph's count).  desc: scratch of 8 bytes per partner (each partner's
 // stream, written first).
-// ldesc[v] = {voff[v], off[v+1] - off[v]} for every vertex (the lists' first
-// col4 word and length in one record), for the counting kernels.
-void launch_list_desc(const int32_t *off, const int32_t *voff, int32_t n, const Ctrl *ctrl,
-                      int2 *ldesc, cudaStream_t st);
-cudaError_t launch_count(const int32_t *off, const int32_t *voff, const int2 *ldesc,
-                         const int32_t *col4,
-                         const int32_t *goff, const int32_t *part, const int32_t *pskip,
-                         int2 *desc, const int32_t *warp_groups,
-                         const int32_t *cta_groups, const int32_t *big_groups, int32_t n,
-                         Ctrl *ctrl, int64_t *t, int64_t *tg, cudaStream_t st);
+// groups, big_groups: the binned groups (launch_group_offsets).
+cudaError_t launch_count(const int2 *ldesc, const int32_t *col4, const int32_t *goff,
+                         const int32_t *part, const int32_t *pskip, int2 *desc,
+                         const int32_t *groups, const int32_t *big_groups, int32_t n, Ctrl *ctrl,
+                         int64_t *t, int64_t *tg, cudaStream_t st);
 // Sets the counting kernels' attributes and occupancy for the current
 // device (done lazily otherwise; needed before capturing a CUDA graph).
 cudaError_t prepare_count_kernels();
