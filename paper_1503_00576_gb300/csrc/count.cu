@@ -96,9 +96,11 @@ struct Lists {
   const int32_t *__restrict__ part;   // partners
   const int32_t *__restrict__ pskip;  // per partner: leading blocks of its list skipped
   const int2 *__restrict__ desc;      // per-vertex mode, per partner: its stream
-                                      //   {first col4 word, entries} (k_stream_desc)
+                                      //   {first col4 word, entries | cut << 16}
+                                      //   (k_stream_desc)
   const int2 *__restrict__ ldesc;     // per vertex: its list {voff[v], d+(v)}, one
                                       //   8-byte gather instead of three 4-byte ones
+  const uint32_t *__restrict__ rec;   // per vertex: its bitmap's record (nullptr: none)
 };
 
 // One hash set in shared memory.
@@ -360,6 +362,8 @@ __device__ __forceinline__ void probe_windows(const Lists &g, int32_t w, int32_t
 //    positions p, p+32, ... with a cursor on the list holding its position.
 //    For chunks of a few short lists, where whole blocks would be mostly
 //    padding.
+// bits: the group's list has a bitmap, so the streams of partners that have
+// one too end where the bitmaps take over (bits.cu).
 // Matches are counted in registers; per partner they go to a shared counter
 // (per block, or when an element-mode lane leaves the partner's list), per w
 // to the counter beside w's slot.
@@ -367,7 +371,7 @@ template <bool PV, int W>
 __device__ __forceinline__ void probe_chunk(const Lists &g, const int32_t *__restrict__ part,
                                             const int32_t *__restrict__ pskip,
                                             const int2 *__restrict__ desc, int32_t np,
-                                            int32_t c0, int32_t cs, const Table &tb,
+                                            int32_t c0, int32_t cs, bool bits, const Table &tb,
                                             WarpScratch &ws, int64_t *t, uint64_t &found_total,
                                             uint64_t &found_group) {
   const int lane = threadIdx.x & 31;
@@ -382,7 +386,8 @@ __device__ __forceinline__ void probe_chunk(const Lists &g, const int32_t *__res
       // counters the separate pass costs more than it saves)
       const int2 ds = __ldg(desc + j);
       vb = ds.x;
-      dl = ds.y;
+      dl = ds.y & 0xffff;
+      if (bits) dl = min(dl, (int32_t)((uint32_t)ds.y >> 16));
     } else {
       const int32_t skip = __ldg(pskip + j);
       const int2 ld = __ldg(g.ldesc + l);
@@ -391,6 +396,10 @@ __device__ __forceinline__ void probe_chunk(const Lists &g, const int32_t *__res
       // the leading blocks of N+(l) below the hashed list's smallest id
       // cannot meet it: stream from the first block that can
       vb += 2 * skip;
+      if (bits) {
+        const uint32_t rec = __ldg(g.rec + l);
+        if (bits_used<PV>(rec, skip, dl)) dl = 8 * (int32_t)(rec & kBitTbMask);
+      }
       dl = max(dl - 8 * skip, 0);
     }
   }
@@ -520,6 +529,7 @@ __device__ __forceinline__ void cta_groups(const Lists &g, const int32_t *__rest
     const int32_t nseg = (hd + SLOTS / 2 - 1) / (SLOTS / 2);
     const int32_t seg_len = (hd + nseg - 1) / nseg;
     tb.slots = table_slots(seg_len, SLOTS);
+    const bool bits = g.rec && bits_group<PV>(__ldg(g.rec + h), np);
     uint64_t found_group = 0;
     for (int32_t s0 = 0; s0 < hd; s0 += seg_len) {
       const int32_t len = min(seg_len, hd - s0);
@@ -538,7 +548,7 @@ __device__ __forceinline__ void cta_groups(const Lists &g, const int32_t *__rest
         c = __shfl_sync(kFull, c, 0);
         cs = __shfl_sync(kFull, cs, 0);
         if ((int32_t)c >= np) break;
-        probe_chunk<PV, W>(g, g.part + pb, g.pskip + pb, g.desc + pb, np, (int32_t)c, (int32_t)cs, tb, s_ws[warp],
+        probe_chunk<PV, W>(g, g.part + pb, g.pskip + pb, g.desc + pb, np, (int32_t)c, (int32_t)cs, bits, tb, s_ws[warp],
                            t, found_total, found_group);
       }
       __syncthreads();
@@ -583,11 +593,12 @@ __device__ __forceinline__ void warp_groups(const Lists &g, const int32_t *__res
       const int32_t *hl = g.col4 + 4 * (size_t)hld.x;
       const int32_t pb = __ldg(g.goff + h), np = __ldg(g.goff + h + 1) - pb;
       tb.slots = table_slots(hd, WSLOTS);
+      const bool bits = g.rec && bits_group<PV>(__ldg(g.rec + h), np);
       fill_table(hl, hd, tb, slot_of, lane, 32);
       __syncwarp();
       uint64_t found_group = 0;
       for (int32_t c0 = 0; c0 < np; c0 += 32)
-        probe_chunk<PV, kWindows>(g, g.part + pb, g.pskip + pb, g.desc + pb, np, c0, 32, tb, ws, t, found_total,
+        probe_chunk<PV, kWindows>(g, g.part + pb, g.pskip + pb, g.desc + pb, np, c0, 32, bits, tb, ws, t, found_total,
                                   found_group);
       if (PV || tg) {
         found_group = warp_sum_u64(found_group);
@@ -609,16 +620,21 @@ __device__ __forceinline__ void warp_groups(const Lists &g, const int32_t *__res
 // one coalesced load and no gathers.  Partner l of an edge streams N+(l)
 // from its first block that can meet the hashed list (the pskip leading
 // blocks below it cannot): {col4 word voff[l] + 2 skip, d+(l) - 8 skip
-// entries, at least 0}.
+// entries, at least 0, in the low half (d+ <= sqrt(2m) < 2^16)}; the high
+// half holds the entries left to the hash path when the group's list has a
+// bitmap and l's takes over from block tb on (0xffff: it does not).
 __global__ void __launch_bounds__(256)
 k_stream_desc(const int32_t *__restrict__ part, const int32_t *__restrict__ pskip,
-              const int2 *__restrict__ ldesc, const Ctrl *ctrl, int2 *__restrict__ desc) {
+              const int2 *__restrict__ ldesc, const uint32_t *rec, const Ctrl *ctrl,
+              int2 *__restrict__ desc) {
   if (aborted(ctrl)) return;  // an earlier wait of this call ran out
   const uint32_t m = ctrl->n_part;
+  if (ctrl->n_bit_items == 0u) rec = nullptr;  // no group uses bitmaps
   const uint32_t stride = gridDim.x * blockDim.x;
   for (uint32_t e0 = blockIdx.x * blockDim.x + threadIdx.x; e0 < m; e0 += 4 * stride) {
     int32_t l[4], skip[4];
     int2 ld[4];
+    uint32_t r[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const uint32_t e = e0 + q * stride;
@@ -626,11 +642,19 @@ k_stream_desc(const int32_t *__restrict__ part, const int32_t *__restrict__ pski
       skip[q] = e < m ? __ldg(pskip + e) : 0;
     }
 #pragma unroll
-    for (int q = 0; q < 4; ++q) ld[q] = __ldg(ldesc + l[q]);
+    for (int q = 0; q < 4; ++q) {
+      ld[q] = __ldg(ldesc + l[q]);
+      r[q] = rec ? __ldg(rec + l[q]) : 0u;
+    }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const uint32_t e = e0 + q * stride;
-      if (e < m) desc[e] = make_int2(ld[q].x + 2 * skip[q], max(ld[q].y - 8 * skip[q], 0));
+      const uint32_t cut = bits_used<true>(r[q], skip[q], ld[q].y)
+                               ? 8u * (uint32_t)max((int32_t)(r[q] & kBitTbMask) - skip[q], 0)
+                               : 0xffffu;
+      if (e < m)
+        desc[e] = make_int2(ld[q].x + 2 * skip[q],
+                            (int32_t)((uint32_t)max(ld[q].y - 8 * skip[q], 0) | cut << 16));
     }
   }
 }
@@ -661,6 +685,7 @@ k_count(Lists g, const int32_t *__restrict__ groups, int32_t n, Ctrl *ctrl, int6
   __shared__ CtaShared s_sh;
   if (aborted(ctrl)) return;  // an earlier wait of this call ran out: the lists are not complete
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (ctrl->n_bit_items == 0u) g.rec = nullptr;  // no group uses bitmaps: no record is read
   clear_table<PV>(s_tab, s_cnt, SLOTS, tid, kMainThreads);
   uint64_t found_total = 0;
   Table tb{s_tab, s_cnt, shared_addr(s_cnt), SLOTS};
@@ -692,6 +717,7 @@ k_count_big(Lists g, const int32_t *__restrict__ big_list, Ctrl *ctrl, int64_t *
   const int tid = threadIdx.x, lane = tid & 31;
   const uint32_t n_big = ctrl->n_big_groups;
   if (n_big == 0) return;  // most graphs: not even the tables are emptied
+  if (ctrl->n_bit_items == 0u) g.rec = nullptr;
   clear_table<PV>(tab, cnt, kBigSlots, tid, kBigThreads);
   uint64_t found_total = 0;
   Table tb{tab, cnt, shared_addr(cnt), kBigSlots};
@@ -827,8 +853,8 @@ cudaError_t prepare_count_kernels() {
 
 cudaError_t launch_count(const int2 *ldesc, const int32_t *col4, const int32_t *goff,
                          const int32_t *part, const int32_t *pskip, int2 *desc,
-                         const int32_t *groups, const int32_t *big_groups, int32_t n, Ctrl *ctrl,
-                         int64_t *t, int64_t *tg, cudaStream_t st) {
+                         const int32_t *groups, const int32_t *big_groups, const uint32_t *rec,
+                         int32_t n, Ctrl *ctrl, int64_t *t, int64_t *tg, cudaStream_t st) {
   const bool pv = t != nullptr;
   CountGrid cg;
   cudaError_t e = count_grid(pv, &cg);
@@ -837,10 +863,10 @@ cudaError_t launch_count(const int2 *ldesc, const int32_t *col4, const int32_t *
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    k_stream_desc<<<(sms > 0 ? sms : 1) * 16, 256, 0, st>>>(part, pskip, ldesc, ctrl, desc);
+    k_stream_desc<<<(sms > 0 ? sms : 1) * 16, 256, 0, st>>>(part, pskip, ldesc, rec, ctrl, desc);
     note_launch();
   }
-  const Lists g{col4, goff, part, pskip, desc, ldesc};
+  const Lists g{col4, goff, part, pskip, desc, ldesc, rec};
   // the long lists first, on their own wide CTAs
   if (pv) {
     k_count_big<true><<<cg.big_blocks, kBigThreads, big_smem<true>(), st>>>(g, big_groups, ctrl, t,

@@ -379,7 +379,7 @@ k_sort_lists(const int32_t *__restrict__ col, const int32_t *__restrict__ off,
     }
     if (v < (uint32_t)n && d <= kWarpLaneMax) o.ldesc[v] = make_int2(w, len);
     // the queues: lists for a warp from the front of the array, lists for a
-    // CTA in its second half
+    // CTA from its end down
     const bool is_warp = d > kWarpLaneMax && d <= kWarpLongMax, is_cta = d > kWarpLongMax;
     const uint32_t bw = __ballot_sync(kFull, is_warp), bc = __ballot_sync(kFull, is_cta);
     if (bw | bc) {
@@ -388,7 +388,7 @@ k_sort_lists(const int32_t *__restrict__ col, const int32_t *__restrict__ off,
       if (lane == 1 && bc) at = atomicAdd(&ctrl->n_cta_lists, (uint32_t)__popc(bc));
       const uint32_t aw = __shfl_sync(kFull, at, 0), ac = __shfl_sync(kFull, at, 1);
       if (is_warp) queue[aw + __popc(bw & lt)] = (int32_t)v;
-      if (is_cta) queue[(uint32_t)n + ac + __popc(bc & lt)] = (int32_t)v;
+      if (is_cta) queue[(uint32_t)n - 1u - (ac + __popc(bc & lt))] = (int32_t)v;
     }
   }
 }
@@ -432,7 +432,7 @@ k_sort_long_lists(int32_t *col, const int32_t *__restrict__ off,
     __syncthreads();
     const uint32_t i = s_i;
     if (i >= n_cta) break;
-    const int32_t v = __ldg(queue + n + i);
+    const int32_t v = __ldg(queue + ((uint32_t)n - 1u - i));
     const int32_t b = __ldg(off + v), d = __ldg(off + v + 1) - b, w = __ldg(voff + v);
     int32_t *dst = o.col4 + 4ll * w;
     const int r8 = (d + 7) & ~7;

@@ -662,6 +662,7 @@ struct ScanArgs {
   const int2 *ldesc;      // kScanGroups: the lists' lengths
   int32_t *groups;        // kScanGroups: warp groups from the front, CTA groups from the end
   int32_t *big_list;
+  BitItems bits;          // kScanGroups: the bitmap path's work items
   Tuning tune;
   unsigned long long *status;
   uint32_t *ticket;
@@ -776,6 +777,32 @@ k_offsets(const ScanArgs a) {
       if ((mc >> i) & 1u) a.groups[n - 1u - c++] = v;
       if ((mb >> i) & 1u) a.big_list[g++] = v;
     }
+    if (a.bits.rec) {  // uniform
+      // the groups that intersect by bitmaps, in items of at most a range of
+      // partners each
+      uint32_t mi = 0, cnt = 0;
+#pragma unroll
+      for (int i = 0; i < IPT; ++i) {
+        const uint32_t v = first + i;
+        if (((mw | mc | mb) >> i & 1u) && d[i] >= a.bits.min_partners &&
+            __ldg(a.bits.rec + v) != 0u) {
+          mi |= 1u << i;
+          cnt += ((uint32_t)d[i] + a.bits.range - 1) / a.bits.range;
+        }
+      }
+      uint64_t total;
+      const uint64_t mine_at = block_scan_exclusive<kScanThreads>((uint64_t)cnt, s_scratch, &total);
+      if (tid == 0) s_base[0] = total ? atomicAdd(&ctrl->n_bit_items, (uint32_t)total) : 0u;
+      __syncthreads();
+      uint32_t at = s_base[0] + (uint32_t)mine_at, from = (uint32_t)(s_excl + toff);
+#pragma unroll
+      for (int i = 0; i < IPT; ++i) {
+        if ((mi >> i) & 1u)
+          for (uint32_t s = 0; s < (uint32_t)d[i]; s += a.bits.range)
+            a.bits.items[at++] = make_int2((int32_t)(first + i), (int32_t)(from + s));
+        from += (uint32_t)d[i];
+      }
+    }
   }
 }
 
@@ -871,12 +898,12 @@ void launch_offsets(const int32_t *counts, int32_t n, int32_t *off, int32_t *vof
 }
 
 void launch_group_offsets(const int32_t *counts, const int32_t *own, int32_t n, int32_t *goff,
-                          const int2 *ldesc, int32_t *groups, int32_t *big_list, Tuning tune,
-                          unsigned long long *status, uint32_t *ticket, Ctrl *ctrl,
+                          const int2 *ldesc, int32_t *groups, int32_t *big_list,
+                          const BitItems &bits, Tuning tune, unsigned long long *status, uint32_t *ticket, Ctrl *ctrl,
                           cudaStream_t st, int32_t shard, int32_t shards) {
   tune.warp_max_list = min(max(tune.warp_max_list, 0), kWarpMaxRow);  // warp table capacity
-  const ScanArgs a{counts,   own,  n,      goff,   nullptr, ldesc,           groups,
-                   big_list, tune, status, ticket, ctrl,    (uint32_t)shard, (uint32_t)shards};
+  const ScanArgs a{counts, own,  n,      goff,   nullptr, ldesc,           groups,          big_list,
+                   bits,   tune, status, ticket, ctrl,    (uint32_t)shard, (uint32_t)shards};
   k_offsets<kScanGroups><<<scan_grid(n), kScanThreads, 0, st>>>(a);
   note_launch();
 }

@@ -236,6 +236,10 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
   int64_t *t_rank = (t_out || batch) ? reinterpret_cast<int64_t *>(ws + L.t_rank) : nullptr;
   // group totals back in union ids (the rank keys are free by then)
   int64_t *tg_union = reinterpret_cast<int64_t *>(ws + L.vkeys_a);
+  // long lists also as bitmaps of the top ranks: records (zeroed with t_rank)
+  // and, once the groups are sorted, the bitmaps
+  const bool bits_on = L.has_bits && !batch;
+  uint32_t *bit_rec = reinterpret_cast<uint32_t *>(ws + L.bit_rec);
   const size_t words = L.st_sort_words_per_pass;
   // look-back status and tile tickets: one slot per radix pass, in the order
   // the passes run (rank sort, sort by owner, group sort)
@@ -252,7 +256,8 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
   if (deg_out)
     TC_CUDA(cudaMemsetAsync(deg, 0, sizeof(int32_t) * (size_t)n, st), "memset deg");
   const size_t zero_from = deg_out ? L.ctrl : L.deg;
-  TC_CUDA(cudaMemsetAsync(ws + zero_from, 0, (t_rank ? L.st_sort : L.t_rank) - zero_from, st),
+  TC_CUDA(cudaMemsetAsync(ws + zero_from, 0,
+                          (t_rank || bits_on ? L.st_sort : L.t_rank) - zero_from, st),
           "memset control");
   TC_CUDA(cudaMemsetAsync(ws + L.st_sort, 0,
                           sizeof(unsigned long long) * words * (size_t)radix_passes(b), st),
@@ -330,8 +335,8 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
   // the node array, the edge count, the row array and the degrees are made
   // right again
   pt.start(TC_PHASE_LISTS);
-  launch_sort_lists(col, off, voff, n, ctrl, col4, reinterpret_cast<int32_t *>(vkeys_a), outdeg,
-                    dcorr, ldesc, st);
+  int32_t *queue = reinterpret_cast<int32_t *>(vkeys_a);
+  launch_sort_lists(col, off, voff, n, ctrl, col4, queue, outdeg, dcorr, ldesc, st);
   launch_recount(outdeg, n, off, st_scan4, &ctrl->tile_ticket[kTicketRecount], ctrl, st);
   launch_fix_repeats(off, n, dcorr, rank, ctrl, row, deg, st);
   pt.stop(TC_PHASE_LISTS);
@@ -373,9 +378,23 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
     TC_CUDA(cudaMemsetAsync(reinterpret_cast<int32_t *>(gout) + m, 0, sizeof(int32_t) * (size_t)m,
                             st),
             "memset skips");
+  // the group sort's other buffer (free now) takes the bitmaps, or each
+  // partner's stream where there are per-vertex counts; the bitmap path's work
+  // items (less than 0.2 bytes per pair) take the radix passes' look-back
+  // status
+  uint32_t *bits = t_out ? reinterpret_cast<uint32_t *>(ws + L.bits)
+                         : reinterpret_cast<uint32_t *>(gin);
+  BitItems items{};
+  if (bits_on) {
+    items = BitItems{bit_rec, reinterpret_cast<int2 *>(ws + L.st_sort),
+                     t_out ? kBitRange<true> : kBitRange<false>,
+                     t_out ? kBitMinPartners<true> : kBitMinPartners<false>};
+    launch_bits_build(queue, n, ldesc, col4, L.bit_slots, t_out != nullptr, bits, bit_rec, ctrl,
+                      st);
+  }
   // only this run's share of the groups is binned (all of them unless the
   // counting is split over several devices, Sec. III-E)
-  launch_group_offsets(gcnt, nullptr, n, goff, ldesc, groups, big_groups, tune, st_scan2,
+  launch_group_offsets(gcnt, nullptr, n, goff, ldesc, groups, big_groups, items, tune, st_scan2,
                        &ctrl->tile_ticket[kTicketGroupScan], ctrl, st, shard, shards);
   pt.stop(TC_PHASE_GROUPS);
   if (work_stats) launch_work(off, goff, part, pskip, n, ctrl, st, shard, shards);
@@ -388,10 +407,13 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
                              t_out ? t_rank : nullptr, st),
             "dense hub block");
   }
-  // each partner's stream goes to the group sort's other buffer (free now)
+  if (bits_on)
+    launch_count_bits(ldesc, col4, goff, part, pskip, items, bits, n, ctrl,
+                      t_out ? t_rank : nullptr, st);
   int2 *desc = reinterpret_cast<int2 *>(gin);
-  cudaError_t e = launch_count(ldesc, col4, goff, part, pskip, desc, groups, big_groups, n, ctrl,
-                               t_out ? t_rank : nullptr, t_out ? nullptr : t_rank, st);
+  cudaError_t e = launch_count(ldesc, col4, goff, part, pskip, desc, groups, big_groups,
+                               bits_on ? bit_rec : nullptr, n, ctrl, t_out ? t_rank : nullptr,
+                               t_out ? nullptr : t_rank, st);
   if (e == cudaSuccess && t_out) launch_gather_counts(t_rank, rank, n, t_out, ctrl, st);
   if (e == cudaSuccess && batch) {
     if (t_out) {  // per graph: (sum of t) / 3
@@ -462,7 +484,8 @@ tc_status count_impl(const int32_t *src, const int32_t *dst, int64_t m, int32_t 
     *total = 0;
     return set_status(TC_OK);
   }
-  const Layout L = make_layout(m, n, true, current_tuning().hub_vertices);
+  const Layout L =
+      make_layout(m, n, true, current_tuning().hub_vertices, false, t_out != nullptr);
   if (ws_user) {
     if (ws_bytes < L.total)
       return set_status(TC_ERR_INVALID_ARG, "workspace has %zu bytes, needs %zu", ws_bytes,
@@ -688,7 +711,7 @@ tc_status batch_impl(const int32_t *src, const int32_t *dst, int32_t G, const in
     return set_status(TC_OK);
   }
   if (p.vertices == 0) return set_status(TC_ERR_ID_RANGE, "edges but no vertices");
-  const Layout L = make_layout(p.pairs, (int32_t)p.vertices);
+  const Layout L = make_layout(p.pairs, (int32_t)p.vertices, false, kHubSize, true);
   const BatchRegion R = batch_region(G);
   keep_pool_memory();
   unsigned char *ws = nullptr;
@@ -772,7 +795,7 @@ tc_status engine_build(tc_engine *e) {
   TC_CUDA(cudaGetDevice(&e->device), "current device");
   TC_CUDA(prepare_count_kernels(), "count kernel attributes");
   TC_CUDA(cudaStreamCreateWithFlags(&e->st, cudaStreamNonBlocking), "stream");
-  e->L = make_layout(e->max_pairs, e->max_vertices);
+  e->L = make_layout(e->max_pairs, e->max_vertices, false, kHubSize, true);
   e->R = batch_region(e->max_graphs);
   const size_t in_bytes = align256(sizeof(int32_t) * (size_t)e->max_pairs);
   TC_CUDA(dev_alloc((void **)&e->dbuf, 2 * in_bytes + e->L.total + e->R.bytes),

@@ -37,6 +37,32 @@ constexpr int kSkipShift = 48;
 // streamed list is skipped whole.
 constexpr uint32_t kSkipAll = 0xFFFFu;
 
+// Bitmaps of the top ranks (bits.cu): kBitCols columns; a list has one if at
+// least kBitMinBlocks of its 32-byte blocks lie among them, a group uses them
+// if it has at least kBitMinPartners partners.  A list's record is (slot + 1)
+// << kBitTbBits | tb, tb the first block that the bitmap stands for; 0: none.
+// Per vertex (PV) an edge costs about three times as much (counts per column
+// and partner), so the lines lie higher there.  Measured on R-MAT graphs (T
+// only / per vertex, ms; 4, 5, 6, 8 and 5, 8, 12, 16, 24 blocks tried): more
+// or fewer blocks change a call by less than 1%; 8192 columns instead of 4096
+// cost 10% more per call for 4% more of the lookups.
+constexpr int kBitCols = 4096;
+template <bool PV> constexpr int kBitMinBlocks = PV ? 12 : 6;
+template <bool PV> constexpr int kBitMinPartners = PV ? 64 : 16;
+// Partners that a warp intersects at a time.  With per-vertex counts the bit
+// planes hold 255, and emptying them costs the same for any number.
+template <bool PV> constexpr uint32_t kBitRange = PV ? 248u : 128u;
+constexpr int kBitTbBits = 11;
+constexpr uint32_t kBitTbMask = (1u << kBitTbBits) - 1;
+constexpr uint32_t kBitMaxSlots = (1u << (32 - kBitTbBits)) - 1;
+// Only for single graphs of at least this many pairs.  T only: below it few
+// lists are that long, and two launches cost more.  Per vertex, without / with
+// them: R-MAT 18 of 10.5M pairs 2.50 / 2.53 ms, 20 of 16.8M 3.30 / 3.46, 20
+// of 44.5M 11.6 / 10.3, 21 of 91M 28.5 / 21.6, 24 of 180M 41.7 / 40.2, 22 of
+// 180M 69.9 / 49.6 (T only, before / with: 16 of 2.5M 0.64 / 0.61 ms, 21 of
+// 91M 22.5 / 16.9).
+template <bool PV> constexpr int64_t kBitMinPairs = PV ? 1 << 25 : 1 << 18;
+
 // Dense hub block (hub.cu): the kHubSize vertices of highest rank, counted
 // on the tensor cores when they hold at least kHubMinEdges edges.  Only for
 // single graphs with n >= kHubMinVertices and ids of at most 24 bits (the
@@ -79,7 +105,8 @@ struct Ctrl {
   uint32_t n_cta_lists;            // ... by a CTA each
   uint32_t next_warp_list;         // work cursors of the queued lists
   uint32_t next_cta_list;
-  uint32_t pad_[2];
+  uint32_t n_bit_items;            // work items of the bitmap path
+  uint32_t pad_;
   uint32_t hub_on;                 // the hub block is counted densely (hub.cu)
   uint32_t hub_lo;                 // its first rank
   uint32_t hub_size;               // its number of vertices (hub_lo + hub_size = n)
@@ -119,6 +146,22 @@ __device__ __forceinline__ bool aborted(const Ctrl *ctrl) {
   return (ctrl->err & kErrTimeout) != 0u;
 }
 
+// Whether a group of np partners whose list has bitmap record rec (0: none)
+// intersects by bitmaps.
+template <bool PV>
+__device__ __forceinline__ bool bits_group(uint32_t rec, int32_t np) {
+  return rec != 0u && np >= kBitMinPartners<PV>;
+}
+
+// Whether a partner whose list of len entries has bitmap record rec (0: none)
+// and skips its first `skip` blocks is intersected by bitmaps from block tb
+// on (if the group's list has a bitmap too): enough blocks must be left there.
+template <bool PV>
+__device__ __forceinline__ bool bits_used(uint32_t rec, int32_t skip, int32_t len) {
+  if (rec == 0u || skip == (int32_t)kSkipAll) return false;
+  return ((len + 7) >> 3) - max(skip, (int32_t)(rec & kBitTbMask)) >= kBitMinBlocks<PV>;
+}
+
 #endif
 
 // Partner groups whose hashed forward list has at most kWarpMaxRow entries
@@ -152,6 +195,17 @@ struct BatchDesc {
   int32_t *gerr;            // [num_graphs], zero on entry; set: an id outside its graph
 };
 
+// Work items of the bitmap path (bits.cu): {group, first partner} for every
+// `range` partners of every group that intersects by bitmaps (rec[h] != 0
+// and at least min_partners partners), ctrl->n_bit_items of them in any
+// order.  rec == nullptr: no bitmaps.
+struct BitItems {
+  const uint32_t *rec;
+  int2 *items;
+  uint32_t range;
+  int32_t min_partners;
+};
+
 // Workspace layout for an input of m_in pairs and n vertices.  All offsets
 // are 256-byte aligned.
 struct Layout {
@@ -164,6 +218,12 @@ struct Layout {
   size_t col4;
   size_t rank, vkeys_a, vkeys_b;
   size_t hub;  // dense hub block (0 bytes unless the layout asked for it)
+  // bitmaps (single graphs of at least kBitMinPairs pairs): without per-vertex
+  // counts the records take the place of t_rank and the bitmaps that of the
+  // group sort's free key buffer; with them both have their own
+  bool has_bits;
+  size_t bit_rec, bits;
+  uint32_t bit_slots;
   bool has_hub;
   int32_t hub_vertices;  // size of the hub set the hub region was laid out for
   size_t total;
@@ -201,7 +261,8 @@ inline int radix_passes(int b) { return 3 * ((b + 7) / 8); }
 inline bool hub_enabled(int32_t n, int b) { return n >= kHubMinVertices && 2 * b <= kSkipShift; }
 
 inline Layout make_layout(int64_t m_in, int32_t n, bool with_hub = false,
-                          int32_t hub_vertices = kHubSize) {
+                          int32_t hub_vertices = kHubSize, bool batch = false,
+                          bool per_vertex = false) {
   Layout L{};
   size_t p = 0;
   auto take = [&](size_t bytes) {
@@ -227,6 +288,10 @@ inline Layout make_layout(int64_t m_in, int32_t n, bool with_hub = false,
   L.gcnt = take(sizeof(int32_t) * nv);
   L.dcorr = take(sizeof(int32_t) * nv);
   L.t_rank = take(sizeof(int64_t) * nv);
+  L.has_bits = !batch && m_in >= (per_vertex ? kBitMinPairs<true> : kBitMinPairs<false>);
+  const uint64_t slots = m / (kBitCols / 32);  // two bitmaps each, in 8 m bytes
+  L.bit_slots = (uint32_t)(slots < kBitMaxSlots ? slots : kBitMaxSlots);
+  L.bit_rec = per_vertex && L.has_bits ? take(sizeof(uint32_t) * nv) : L.t_rank;
   // look-back status words for the passes that ids of [0, n) need (a run
   // with fewer vertices needs no more)
   L.st_sort = take(sizeof(unsigned long long) * L.st_sort_words_per_pass *
@@ -243,6 +308,7 @@ inline Layout make_layout(int64_t m_in, int32_t n, bool with_hub = false,
   // forward lists padded to whole 32-byte blocks: at most m + 7 min(n, m)
   // elements, since each non-empty list adds at most 7
   L.col4 = take(sizeof(int32_t) * (m + 7 * (nv < m ? nv : m)));
+  L.bits = per_vertex && L.has_bits ? take((size_t)L.bit_slots * (kBitCols / 4)) : 0;
   const bool hub = with_hub && hub_enabled(n, id_bits(n > 0 ? n : 1));
   const size_t H = (size_t)hub_vertices;
   L.hub = take(hub ? H * H + 4 * H : 0);
@@ -307,12 +373,13 @@ void launch_offsets(const int32_t *counts, int32_t n, int32_t *off, int32_t *vof
 // nullptr) -> goff[0..n], ctrl->n_part = goff[n]; the groups are binned into
 // the lists by the length of their hashed list (ldesc): warp groups from
 // the front of `groups` up, CTA groups from its end down (n entries hold
-// both), big groups into big_list.  Only the groups h with h mod shards =
+// both), big groups into big_list; bits: the bitmap path's work items are
+// written too (BitItems).  Only the groups h with h mod shards =
 // shard are binned (the share of the counting work this run does; shards = 1
 // bins them all).
 void launch_group_offsets(const int32_t *counts, const int32_t *own, int32_t n, int32_t *goff,
-                          const int2 *ldesc, int32_t *groups, int32_t *big_list, Tuning tune,
-                          unsigned long long *status, uint32_t *ticket, Ctrl *ctrl,
+                          const int2 *ldesc, int32_t *groups, int32_t *big_list,
+                          const BitItems &bits, Tuning tune, unsigned long long *status, uint32_t *ticket, Ctrl *ctrl,
                           cudaStream_t st, int32_t shard = 0, int32_t shards = 1);
 // The node array again, from the list lengths left after the list sort
 // dropped repeated edges, and ctrl->m = their sum; nothing (the kernel
@@ -343,7 +410,9 @@ cudaError_t launch_hub_count(const int2 *ldesc, const int32_t *col4, int32_t n, 
 // length goes to dlen[v] (written only for such lists; dlen holds the
 // lengths with repeats on entry), each dropped copy adds one to dcorr at
 // both its ends (rank space; zero on entry) and ctrl->dups is set.
-// queue: scratch of 2n entries; col is scratch for lists longer than
+// queue: n entries; the lists of more than 64 entries, ctrl->n_warp_lists
+// of them from its front and ctrl->n_cta_lists (the longest) from its end
+// down; col is scratch for lists longer than
 // kCtaSortMax.
 void launch_sort_lists(int32_t *col, const int32_t *off, const int32_t *voff, int32_t n,
                        Ctrl *ctrl, int32_t *col4, int32_t *queue, int32_t *dlen,
@@ -370,16 +439,30 @@ void launch_group_keys(const int32_t *row, const int32_t *col4, const int32_t *o
 void launch_work(const int32_t *off, const int32_t *goff, const int32_t *part,
                  const int32_t *pskip, int32_t n, Ctrl *ctrl, cudaStream_t st,
                  int32_t shard = 0, int32_t shards = 1);
+// ---- launchers (bits.cu) ----
+// Bitmaps of the queued lists (launch_sort_lists) that have enough entries
+// among the top ranks, at most `slots` - 1 of them: 2 kBitCols bits each into
+// bits, their records into rec[v] (zero on entry).
+void launch_bits_build(const int32_t *queue, int32_t n, const int2 *ldesc, const int32_t *col4,
+                       uint32_t slots, bool per_vertex, uint32_t *bits, uint32_t *rec, Ctrl *ctrl,
+                       cudaStream_t st);
+// Intersections by bitmaps: adds what they find to ctrl->total and, if t !=
+// nullptr, to the per-vertex counts t (rank space).  launch_count leaves
+// exactly this part out when it is given the records.
+void launch_count_bits(const int2 *ldesc, const int32_t *col4, const int32_t *goff,
+                       const int32_t *part, const int32_t *pskip, const BitItems &items,
+                       const uint32_t *bits, int32_t n, Ctrl *ctrl, int64_t *t, cudaStream_t st);
 // ---- launchers (count.cu) ----
 // t != nullptr: per-vertex counts (rank space).  Otherwise, if tg is not
 // nullptr, tg[h] += triangles found in group h (their sum per graph is the
 // graph's count).  desc: scratch of 8 bytes per partner (each partner's
 // stream, written first).
-// groups, big_groups: the binned groups (launch_group_offsets).
+// groups, big_groups: the binned groups (launch_group_offsets).  rec: the
+// bitmap records (nullptr: no bitmaps).
 cudaError_t launch_count(const int2 *ldesc, const int32_t *col4, const int32_t *goff,
                          const int32_t *part, const int32_t *pskip, int2 *desc,
-                         const int32_t *groups, const int32_t *big_groups, int32_t n, Ctrl *ctrl,
-                         int64_t *t, int64_t *tg, cudaStream_t st);
+                         const int32_t *groups, const int32_t *big_groups, const uint32_t *rec,
+                         int32_t n, Ctrl *ctrl, int64_t *t, int64_t *tg, cudaStream_t st);
 // Sets the counting kernels' attributes and occupancy for the current
 // device (done lazily otherwise; needed before capturing a CUDA graph).
 cudaError_t prepare_count_kernels();
