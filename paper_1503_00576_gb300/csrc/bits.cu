@@ -45,8 +45,9 @@ __device__ __forceinline__ int32_t bits_base(int32_t n) { return max(n - kBitCol
 template <bool PV>
 __global__ void __launch_bounds__(kThreads)
 k_bits_build(const int32_t *__restrict__ queue, int32_t n, const int2 *__restrict__ ldesc,
-             const int32_t *__restrict__ col4, uint32_t slots, uint32_t *__restrict__ bits,
-             uint32_t *__restrict__ rec, const Ctrl *ctrl) {
+             const int32_t *__restrict__ col4, const int32_t *__restrict__ goff, uint32_t slots,
+             uint32_t *__restrict__ bits, uint32_t *__restrict__ rec, int2 *__restrict__ items,
+             Ctrl *ctrl, uint32_t shard, uint32_t shards) {
   __shared__ uint32_t s_bits[kWarps][kWords];
   if (aborted(ctrl)) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -56,6 +57,25 @@ k_bits_build(const int32_t *__restrict__ queue, int32_t n, const int2 *__restric
   uint32_t *sb = s_bits[warp];
   uint4 *rows = reinterpret_cast<uint4 *>(bits);  // 32 per bitmap, two bitmaps per slot
   if (blockIdx.x == 0 && warp == 0) rows[lane] = make_uint4(0, 0, 0, 0);
+  // the groups of up to 32 lists (one per lane) before their items are placed
+  int pending = 0;
+  int32_t group = 0;
+  uint32_t from = 0, to = 0;
+  auto place_items = [&] {
+    const uint32_t mine = lane < pending ? (to - from + kBitRange<PV> - 1) / kBitRange<PV> : 0u;
+    uint32_t incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(kFull, incl, o);
+      if (lane >= o) incl += y;
+    }
+    uint32_t at = 0;
+    if (lane == 31) at = atomicAdd(&ctrl->n_bit_items, incl);
+    at = __shfl_sync(kFull, at, 31) + incl - mine;
+    for (uint32_t k = 0; k < mine; ++k)
+      items[at + k] = make_int2(group, (int32_t)(from + k * kBitRange<PV>));
+    pending = 0;
+  };
   for (uint32_t i = blockIdx.x * kWarps + warp; i < count; i += gridDim.x * kWarps) {
     const int32_t v = __ldg(queue + (i < n_warp ? i : (uint32_t)n - 1u - (i - n_warp)));
     const int2 ld = __ldg(ldesc + v);
@@ -89,10 +109,21 @@ k_bits_build(const int32_t *__restrict__ queue, int32_t n, const int2 *__restric
       }
       __syncwarp();
       dst[0] = reinterpret_cast<const uint4 *>(sb)[lane];  // B
-      if (lane == 0) rec[v] = ((i + 1u) << kBitTbBits) | (uint32_t)tb;
+      const uint32_t r = ((i + 1u) << kBitTbBits) | (uint32_t)tb;
+      if (lane == 0) rec[v] = r;
+      const int32_t gs = __ldg(goff + v), ge = __ldg(goff + v + 1);
+      if (bits_group<PV>(r, ge - gs) && (uint32_t)v % shards == shard) {
+        if (lane == pending) {
+          group = v;
+          from = (uint32_t)gs;
+          to = (uint32_t)ge;
+        }
+        if (++pending == 32) place_items();
+      }
     }
     __syncwarp();
   }
+  if (pending) place_items();
 }
 
 // Carry-save adder: a + b + c = sum + 2 carry, bit by bit.
@@ -398,10 +429,13 @@ uint32_t sm_count() {
 }  // namespace
 
 void launch_bits_build(const int32_t *queue, int32_t n, const int2 *ldesc, const int32_t *col4,
-                       uint32_t slots, bool per_vertex, uint32_t *bits, uint32_t *rec, Ctrl *ctrl,
-                       cudaStream_t st) {
+                       const int32_t *goff, uint32_t slots, bool per_vertex, uint32_t *bits,
+                       const BitItems &items, Ctrl *ctrl, cudaStream_t st, int32_t shard,
+                       int32_t shards) {
   const auto kernel = per_vertex ? k_bits_build<true> : k_bits_build<false>;
-  kernel<<<sm_count() * 8u, kThreads, 0, st>>>(queue, n, ldesc, col4, slots, bits, rec, ctrl);
+  kernel<<<sm_count() * 8u, kThreads, 0, st>>>(queue, n, ldesc, col4, goff, slots, bits, items.rec,
+                                               items.items, ctrl, (uint32_t)shard,
+                                               (uint32_t)shards);
   note_launch();
 }
 

@@ -4,18 +4,20 @@
 // (Sec. II-B).  The intersection is symmetric in u and v, and the counting
 // kernel computes it by hashing one list and streaming the other through
 // the hash set, which costs one probe per element of the streamed list.
-// Streaming the shorter list is cheapest, so every forward edge is assigned
-// to the endpoint whose forward list is longer:
+// Streaming the shorter list is cheapest.  When the hashed list is N+(v)'s,
+// only the entries of N+(u) after v can match, so every forward edge is
+// assigned to
 //
-//   h = v if |N+(v)| > |N+(u)| else u,     l = the other endpoint,
+//   h = v if what follows v in N+(u) is shorter (in 32-byte blocks) than
+//   N+(v), else h = u;     l = the other endpoint,
 //
-// and the edges are grouped by h: k_group_keys writes the key h << b | l of
-// every edge, and a stable LSD radix sort over the h bits (the passes of
-// preprocess.cu) leaves the partners l of each group together, its last
-// pass counting the group sizes.  A group then hashes N+(h) once and
-// streams N+(l) for each of its partners l.  On the R-MAT graphs of the
-// benchmarks this cuts the probes by a factor of 2.7 against always
-// streaming N+(v).
+// and the edges are grouped by h, either by a counting sort (the list sort
+// emits every edge, direct.cu scatters it) or by k_group_keys and radix passes
+// over the h bits (preprocess.cu), whose last pass counts the group sizes.
+// (Shares of a run and the work counters weigh the whole lists instead, see
+// k_group_keys.)  A group then hashes N+(h) once and streams N+(l) for each of
+// its partners l.  On the R-MAT graphs of the benchmarks this cuts the probes
+// by a factor of 3 against always streaming N+(v).
 //
 // The lists themselves are sorted here (Sec. II-B sorts every forward list;
 // the paper merges them, this path hashes, and uses the order only to skip
@@ -103,6 +105,67 @@ struct ListOut {
   Ctrl *ctrl;
 };
 
+// What the list sort needs to emit edges (GroupOut) beside the lists.
+struct Emit {
+  GroupOut g;
+  const int32_t *len;  // list lengths (with repeats, or without once dropped)
+  int32_t hub_lo;      // lists of vertices from this rank on are counted densely
+  int32_t *hot;        // shared counters of the edges emitted to the ranks from
+  int32_t hot_lo;      //   hot_lo on (nullptr: none)
+};
+
+__device__ __forceinline__ void count_edge(const Emit &o, int32_t h) {
+  if (o.hot && h >= o.hot_lo) atomicAdd(&o.hot[h - o.hot_lo], 1);
+  else atomicAdd(&o.g.gcnt[h], 1);
+}
+
+// The key of edge (u, v), v entry i of the du entries of the sorted N+(u);
+// kHole if it needs no intersection.  The longer side is hashed, and what
+// could be streamed of N+(u) is only its entries after v (those before it are
+// below everything in N+(v)): so N+(u) from entry i + 1 on is weighed against
+// N+(v), in whole 32-byte blocks.  (Weighing the whole lists, as
+// k_group_keys does, streams 10% to 25% more blocks.)  A heavy ratio other
+// than 100 weighs the whole lists by it.
+__device__ __forceinline__ uint64_t edge_key(const Emit &o, int32_t u, int32_t du, int32_t i,
+                                             int32_t v, bool &own) {
+  const int32_t dv = o.len[v];
+  bool at_v;
+  int32_t skip;
+  if (o.g.heavy_ratio_pct == 100) {
+    skip = (i + 1) >> 3;
+    if (i + 1 == du || dv == 0) return kHole;
+    at_v = ((du + 7) >> 3) - skip < (dv + 7) >> 3;
+  } else {
+    skip = i >> 3;
+    at_v = (int64_t)dv * 100 > (int64_t)du * o.g.heavy_ratio_pct;
+  }
+  own = !at_v;
+  const uint64_t hu = (uint64_t)(uint32_t)u, hv = (uint64_t)(uint32_t)v;
+  return at_v ? ((uint64_t)skip << kSkipShift) | (hv << o.g.b) | hu : (hu << o.g.b) | hv;
+}
+
+// Emits entry i (value x; valid: it exists) of the du entries of list u to
+// slot `slot`; called by all lanes of `members` (a power-of-two part of the
+// warp that works on list u) together.  own: u's own edges so far.
+__device__ __forceinline__ void emit_entry(const Emit &o, int32_t u, int32_t du, int32_t i,
+                                           int32_t x, bool valid, int64_t slot, uint32_t members,
+                                           int32_t &own) {
+  uint64_t key = kHole;
+  bool mine = false;
+  if (valid && u < o.hub_lo) key = edge_key(o, u, du, i, x, mine);
+  mine = mine && key != kHole;
+  const uint32_t bits = __ballot_sync(kFull, mine) & members;
+  if (mine) {
+    const int32_t k = own + __popc(bits & ((1u << (threadIdx.x & 31)) - 1u));
+    key |= kOwnEdge | ((uint64_t)k << kSkipShift);
+  }
+  own += __popc(bits);
+  if (valid) {
+    o.g.gkeys[slot] = key;
+    if (key != kHole && !mine) count_edge(o, x);
+  }
+}
+
 // The list of u held `dropped` repeats and keeps len entries.  A repeat of
 // edge (u, x) had added one to the degree of both ends: u's share is taken
 // back here in one atomic for the list, x's where the repeat is met.  The
@@ -129,13 +192,29 @@ __device__ __forceinline__ bool warp_repeat(const int32_t (&x)[E], int e, int32_
   return i > 0 && i < d && x[e] == p;
 }
 
+// The warp emits the len entries of the finished list u (slots from b on, d of
+// them); returns its own edges.
+__device__ __forceinline__ int32_t emit_list(const Emit &em, int32_t u, int32_t b, int32_t d,
+                                             int32_t len, const int32_t *list) {
+  const int lane = threadIdx.x & 31;
+  int32_t own = 0;
+#pragma unroll 2
+  for (int32_t i0 = 0; i0 < d; i0 += 32) {
+    const int32_t i = i0 + lane;
+    const int32_t x = i < len ? list[i] : 0;
+    emit_entry(em, u, len, i, x, i < len, (int64_t)b + i, kFull, own);
+    if (i >= len && i < d) em.g.gkeys[(int64_t)b + i] = kHole;
+  }
+  return own;
+}
+
 // The warp sorts list v (d entries from col + b) into col4 from entry w4,
 // with E keys per lane (32 E >= d), dropping repeated entries; returns the
 // entries left.
-template <int E>
+template <int E, bool EMIT>
 __device__ __forceinline__ int32_t warp_sort_list(const int32_t *__restrict__ col, int32_t b,
                                                   int32_t d, long long w4, int32_t v,
-                                                  const ListOut &o) {
+                                                  const ListOut &o, const Emit &em) {
   const int lane = threadIdx.x & 31;
   int32_t x[E];
 #pragma unroll
@@ -154,6 +233,20 @@ __device__ __forceinline__ int32_t warp_sort_list(const int32_t *__restrict__ co
       const int i = e * 32 + lane;
       if (i < r8) o.col4[w4 + i] = i < d ? x[e] : -1;
     }
+    if (EMIT) {
+      int32_t own = 0;
+      if constexpr (E <= 2) {
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          const int i = e * 32 + lane;
+          emit_entry(em, v, d, i, x[e], i < d, (int64_t)b + i, kFull, own);
+        }
+      } else {  // from memory: the keys' registers are needed
+        __syncwarp();
+        own = emit_list(em, v, b, d, d, o.col4 + w4);
+      }
+      if (lane == 0) em.g.own[v] = own;
+    }
     return d;
   }
   // some entry repeats (an edge given more than once): compact the rest
@@ -171,6 +264,11 @@ __device__ __forceinline__ int32_t warp_sort_list(const int32_t *__restrict__ co
   }
   for (int i = len + lane; i < r8; i += 32) o.col4[w4 + i] = -1;
   if (lane == 0) note_repeats(v, d - len, len, o);
+  if (EMIT) {
+    __syncwarp();
+    const int32_t own = emit_list(em, v, b, d, len, o.col4 + w4);
+    if (lane == 0) em.g.own[v] = own;
+  }
   return len;
 }
 
@@ -178,9 +276,10 @@ __device__ __forceinline__ int32_t warp_sort_list(const int32_t *__restrict__ co
 // per lane (d = 0: that half has none); returns the entries left.  Half the
 // steps of a whole warp per list, which these lists (most of a random
 // geometric graph's) would leave half empty.
+template <bool EMIT>
 __device__ __forceinline__ int32_t half_sort_list(const int32_t *__restrict__ col, int32_t b,
                                                   int32_t d, long long w4, int32_t v,
-                                                  const ListOut &o) {
+                                                  const ListOut &o, const Emit &em) {
   const int lane = threadIdx.x & 31, i = lane & 15;
   int32_t x = i < d ? __ldg(col + b + i) : INT32_MAX;
 #pragma unroll
@@ -197,15 +296,24 @@ __device__ __forceinline__ int32_t half_sort_list(const int32_t *__restrict__ co
   const uint32_t half = lane & 16 ? 0xffff0000u : 0x0000ffffu;
   const uint32_t reps = __ballot_sync(kFull, rep) & half;
   const uint32_t kept = __ballot_sync(kFull, i < d && !rep) & half;
-  if (d == 0) return 0;
   const int32_t len = __popc(kept);
-  if (reps == 0) {
+  if (d == 0) {
+    // this half has no list
+  } else if (reps == 0) {
     o.col4[w4 + i] = i < d ? x : -1;
   } else {  // an edge given more than once
     if (i < d && !rep) o.col4[w4 + __popc(kept & ((1u << lane) - 1u))] = x;
     if (rep) atomicAdd(&o.dcorr[x], 1);
     if (i >= len) o.col4[w4 + i] = -1;
     if (i == 0) note_repeats(v, d - len, len, o);
+  }
+  if (EMIT) {
+    __syncwarp();
+    if (reps != 0) x = i < len ? o.col4[w4 + i] : 0;
+    int32_t own = 0;
+    emit_entry(em, v, len, i, x, i < len, (int64_t)b + i, half, own);
+    if (i >= len && i < d) em.g.gkeys[(int64_t)b + i] = kHole;
+    if (i == 0 && d > 0) em.g.own[v] = own;
   }
   return len;
 }
@@ -307,12 +415,14 @@ __device__ int32_t cta_unique_copy(const int32_t *buf, int32_t d, int32_t *__res
 // time: the long lists belong to neighbouring ranks, and a warp that met 32
 // of them finished long after all others (all lists of R-MAT scale 16 with
 // 2.5M edges: 168 us, with the queue 64 us).
+template <bool EMIT>
 __global__ void __launch_bounds__(kListThreads)
 k_sort_lists(const int32_t *__restrict__ col, const int32_t *__restrict__ off,
-             const int32_t *__restrict__ voff, int32_t n, ListOut o,
+             const int32_t *__restrict__ voff, int32_t n, ListOut o, GroupOut g,
              int32_t *__restrict__ queue) {
   Ctrl *ctrl = o.ctrl;
   if (aborted(ctrl)) return;  // an earlier wait of this call ran out
+  const Emit em{g, o.dlen, ctrl->hub_on ? (int32_t)ctrl->hub_lo : n, nullptr, n};
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t warps = gridDim.x * kListWarps;
   const uint32_t lt = (1u << lane) - 1u;
@@ -350,7 +460,25 @@ k_sort_lists(const int32_t *__restrict__ col, const int32_t *__restrict__ off,
         for (int i = len; i < 8; ++i) o.col4[w4 + i] = -1;
         note_repeats((int32_t)v, d - len, len, o);
       }
+      if (EMIT) {
+        int32_t own = 0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          if (i >= d) break;
+          uint64_t key = kHole;
+          if (i < len && (int32_t)v < em.hub_lo) {
+            const int32_t y = reps == 0 ? x[i] : o.col4[w4 + i];
+            bool mine = false;
+            key = edge_key(em, (int32_t)v, len, i, y, mine);
+            if (key != kHole && mine) key |= kOwnEdge | ((uint64_t)own++ << kSkipShift);
+            else if (key != kHole) count_edge(em, y);
+          }
+          em.g.gkeys[(int64_t)b + i] = key;
+        }
+        em.g.own[v] = own;
+      }
     }
+    if (EMIT && d == 0 && v < (uint32_t)n) em.g.own[v] = 0;
     uint32_t todo = __ballot_sync(kFull, d > 8 && d <= 16);
     while (todo) {  // two lists at a time
       const int s0 = __ffs(todo) - 1;
@@ -361,7 +489,8 @@ k_sort_lists(const int32_t *__restrict__ col, const int32_t *__restrict__ off,
       const int src = second ? s1 : s0;
       const int32_t lb = __shfl_sync(kFull, b, src), ld = __shfl_sync(kFull, d, src);
       const long long lw = __shfl_sync(kFull, w4, src);
-      const int32_t l = half_sort_list(col, lb, none ? 0 : ld, lw, (int32_t)(c * 32u) + src, o);
+      const int32_t l = half_sort_list<EMIT>(col, lb, none ? 0 : ld, lw,
+                                             (int32_t)(c * 32u) + src, o, em);
       const int32_t l0 = __shfl_sync(kFull, l, 0), l1 = __shfl_sync(kFull, l, 16);
       if (lane == s0) len = l0;
       else if (lane == s1) len = l1;
@@ -373,8 +502,8 @@ k_sort_lists(const int32_t *__restrict__ col, const int32_t *__restrict__ off,
       const int32_t lb = __shfl_sync(kFull, b, src), ld = __shfl_sync(kFull, d, src);
       const long long lw = __shfl_sync(kFull, w4, src);
       const int32_t lv = (int32_t)(c * 32u) + src;
-      const int32_t l = ld <= 32 ? warp_sort_list<1>(col, lb, ld, lw, lv, o)
-                                 : warp_sort_list<2>(col, lb, ld, lw, lv, o);
+      const int32_t l = ld <= 32 ? warp_sort_list<1, EMIT>(col, lb, ld, lw, lv, o, em)
+                                 : warp_sort_list<2, EMIT>(col, lb, ld, lw, lv, o, em);
       if (lane == src) len = l;
     }
     if (v < (uint32_t)n && d <= kWarpLaneMax) o.ldesc[v] = make_int2(w, len);
@@ -415,9 +544,10 @@ __device__ __forceinline__ int32_t count_below(const int32_t *a, int32_t len, in
 // between the list's own region of the column array and its region of col4
 // so that the last merge lands in the column array.  Then the repeats are
 // dropped on the way into col4.
+template <bool EMIT>
 __global__ void __launch_bounds__(kLongListThreads, kLongListBlocks)
 k_sort_long_lists(int32_t *col, const int32_t *__restrict__ off,
-                  const int32_t *__restrict__ voff, int32_t n, ListOut o,
+                  const int32_t *__restrict__ voff, int32_t n, ListOut o, GroupOut g,
                   const int32_t *__restrict__ queue) {
   constexpr int G = kLongListThreads;
   __shared__ int32_t s_buf[kCtaSortMax];
@@ -425,8 +555,10 @@ k_sort_long_lists(int32_t *col, const int32_t *__restrict__ off,
   __shared__ uint32_t s_i;
   Ctrl *ctrl = o.ctrl;
   if (aborted(ctrl)) return;
+  __shared__ int32_t s_own;
   const int tid = threadIdx.x, lane = tid & 31;
   const uint32_t n_cta = ctrl->n_cta_lists, n_warp = ctrl->n_warp_lists;
+  Emit em{g, o.dlen, ctrl->hub_on ? (int32_t)ctrl->hub_lo : n, nullptr, n};
   while (n_cta) {
     if (tid == 0) s_i = atomicAdd(&ctrl->next_cta_list, 1u);
     __syncthreads();
@@ -479,20 +611,61 @@ k_sort_long_lists(int32_t *col, const int32_t *__restrict__ off,
       len = cta_unique_copy<G>(A, d, B, r8, v, o, s_warp);
     }
     if (tid == 0) o.ldesc[v] = make_int2(w, len);
-    __syncthreads();  // s_buf and s_i are reused
+    if (EMIT) {
+      // the warps' own edges take numbers from a shared counter, a chunk at
+      // a time
+      if (tid == 0) s_own = 0;
+      __syncthreads();  // also: the list is written
+      for (int32_t i0 = 32 * (tid >> 5); i0 < d; i0 += G) {
+        const int32_t i = i0 + lane;
+        const int32_t x = i < len ? dst[i] : 0;
+        bool mine = false;
+        uint64_t key = kHole;
+        if (i < len && v < em.hub_lo) key = edge_key(em, v, len, i, x, mine);
+        mine = mine && key != kHole;
+        const uint32_t bal = __ballot_sync(kFull, mine);
+        int32_t first = 0;
+        if (lane == 0 && bal) first = atomicAdd(&s_own, __popc(bal));
+        first = __shfl_sync(kFull, first, 0);
+        if (mine)
+          key |= kOwnEdge |
+                 ((uint64_t)(first + __popc(bal & ((1u << lane) - 1u))) << kSkipShift);
+        if (i < d) em.g.gkeys[(int64_t)b + i] = key;
+        if (key != kHole && !mine) count_edge(em, x);
+      }
+      __syncthreads();
+      if (tid == 0) em.g.own[v] = s_own;
+    }
+    __syncthreads();  // s_buf, s_i and s_own are reused
   }
-  while (n_warp) {
+  if (n_warp == 0) return;
+  if (EMIT) {
+    // most edges of these lists go to the groups of the highest ranks: counted
+    // in shared memory first (one counter in L2 took 30,000 additions of a
+    // graph of 2.5M edges, and the kernel 90 us instead of 30)
+    __syncthreads();
+    for (int j = tid; j < kCtaSortMax; j += G) s_buf[j] = 0;
+    __syncthreads();
+    em.hot = s_buf;
+    em.hot_lo = max(n - kCtaSortMax, 0);
+  }
+  for (;;) {
     uint32_t i = 0;
     if (lane == 0) i = atomicAdd(&ctrl->next_warp_list, 1u);
     i = __shfl_sync(kFull, i, 0);
     if (i >= n_warp) break;
     const int32_t v = __ldg(queue + i);
     const int32_t b = __ldg(off + v), d = __ldg(off + v + 1) - b, w = __ldg(voff + v);
-    const int32_t len = d <= 128   ? warp_sort_list<4>(col, b, d, 4ll * w, v, o)
-                        : d <= 256 ? warp_sort_list<8>(col, b, d, 4ll * w, v, o)
-                        : d <= 512 ? warp_sort_list<16>(col, b, d, 4ll * w, v, o)
-                                   : warp_sort_list<32>(col, b, d, 4ll * w, v, o);
+    const int32_t len = d <= 128   ? warp_sort_list<4, EMIT>(col, b, d, 4ll * w, v, o, em)
+                        : d <= 256 ? warp_sort_list<8, EMIT>(col, b, d, 4ll * w, v, o, em)
+                        : d <= 512 ? warp_sort_list<16, EMIT>(col, b, d, 4ll * w, v, o, em)
+                                   : warp_sort_list<32, EMIT>(col, b, d, 4ll * w, v, o, em);
     if (lane == 0) o.ldesc[v] = make_int2(w, len);
+  }
+  if (EMIT) {
+    __syncthreads();
+    for (int j = tid; j < kCtaSortMax; j += G)
+      if (s_buf[j]) atomicAdd(&g.gcnt[em.hot_lo + j], s_buf[j]);
   }
 }
 
@@ -509,6 +682,7 @@ k_fix_repeats(const int32_t *__restrict__ off, int32_t n, const int32_t *__restr
   const uint32_t first = blockIdx.x * kListThreads + threadIdx.x;
   const uint32_t stride = gridDim.x * kListThreads;
   for (uint32_t v = first; v < (uint32_t)n; v += stride) deg[v] -= __ldg(dcorr + __ldg(rank + v));
+  if (!row) return;
   for (uint32_t v = first >> 5; v < (uint32_t)n; v += stride >> 5) {
     const int32_t b = __ldg(off + v), e = __ldg(off + v + 1);
     for (int32_t i = b + lane; i < e; i += 32) row[i] = (int32_t)v;
@@ -531,19 +705,31 @@ __device__ __forceinline__ void split_edge(int32_t u, int32_t v, int64_t du, int
 // One pass over the forward edges in owner order (row[e] = u; the sorted
 // list N+(u) of col4 holds v at position i = e - off[u]; row and off are
 // those left after the list sort dropped repeated edges): the group key of
-// every edge with the digit histograms of its h field.  When the longer
-// list is v's (h = v), the intersection streams N+(u), whose entries before
-// position i are all below v; N+(h) holds only ids above h = v, so those
-// entries cannot match and the whole blocks among them, i >> 3, are
-// skipped.  Their count rides in the key's top bits to the partner array.
-// (When h = u, N+(v) is streamed and all its entries lie above v, itself
-// in N+(u): nothing to skip.)
+// every edge with the digit histograms of its h field.
+//
+// WHOLE: the whole lists are weighed against each other, every edge has a
+// key.  When the longer list is v's (h = v), the intersection streams N+(u),
+// whose entries before position i are all below v; N+(h) holds only ids above
+// h = v, so those entries cannot match and the whole blocks among them,
+// i >> 3, are skipped.  Their count rides in the key's top bits to the partner
+// array.  (When h = u, N+(v) is streamed and all its entries lie above v,
+// itself in N+(u): nothing to skip.)  This is the split whose work
+// tc_count_work reports and whose shares tc_count_part deals out.
+//
+// Otherwise edge_key() decides, and the edges that need no intersection (the
+// last entry of a list, an empty N+(v), an edge inside the dense hub block) are
+// left out: a warp takes the places of its round's keys with one atomic (the
+// first pass of the sort orders equal digits freely, so their order does not
+// matter).  R-MAT scale 21 (91M edges): a quarter of the keys and an eighth
+// of the streamed blocks less.
+template <bool WHOLE>
 __global__ void __launch_bounds__(kGroupThreads)
 k_group_keys(const int32_t *__restrict__ row, const int32_t *__restrict__ col4,
              const int32_t *__restrict__ off, const int2 *__restrict__ ldesc,
-             int b, int passes, int32_t heavy_ratio_pct,
-             const Ctrl *__restrict__ ctrl, uint64_t *__restrict__ gkeys,
+             const int32_t *__restrict__ len, int b, int passes, int32_t heavy_ratio_pct,
+             Ctrl *__restrict__ ctrl, uint64_t *__restrict__ gkeys,
              uint32_t *__restrict__ hist) {
+  constexpr int UNROLL = WHOLE ? kGroupUnroll : 2 * kGroupUnroll;
   __shared__ uint32_t s_hist[kMaxGroupPasses * 256];
   if (aborted(ctrl)) return;  // an earlier wait of this call ran out
   for (int i = threadIdx.x; i < passes * 256; i += kGroupThreads) s_hist[i] = 0;
@@ -552,44 +738,86 @@ k_group_keys(const int32_t *__restrict__ row, const int32_t *__restrict__ col4,
   const bool carry_skip = 2 * b <= kSkipShift;
   const bool hub_on = carry_skip && ctrl->hub_on != 0u;
   const int32_t hub_lo = (int32_t)ctrl->hub_lo;
+  const Emit em{GroupOut{nullptr, nullptr, nullptr, b, heavy_ratio_pct}, len, 0, nullptr, 0};
   const uint32_t stride = gridDim.x * kGroupThreads;
-  // kGroupUnroll edges per thread per round, each step's loads issued for
+  // UNROLL edges per thread per round, each step's loads issued for
   // all of them together: the offsets are gathers that depend on the edge
-  for (uint32_t e0 = blockIdx.x * kGroupThreads + threadIdx.x; e0 < m;
-       e0 += kGroupUnroll * stride) {
-    int32_t u[kGroupUnroll], ub[kGroupUnroll], ue[kGroupUnroll], uw[kGroupUnroll];
+  const int lane = threadIdx.x & 31;
+  for (uint32_t e0 = blockIdx.x * kGroupThreads + threadIdx.x; e0 - lane < m;
+       e0 += UNROLL * stride) {
+    int32_t u[UNROLL], ub[UNROLL], ue[UNROLL], uw[UNROLL];
 #pragma unroll
-    for (int q = 0; q < kGroupUnroll; ++q) {
+    for (int q = 0; q < UNROLL; ++q) {
       const uint32_t e = e0 + q * stride;
       u[q] = e < m ? __ldg(row + e) : 0;
     }
 #pragma unroll
-    for (int q = 0; q < kGroupUnroll; ++q) {
+    for (int q = 0; q < UNROLL; ++q) {
       ub[q] = __ldg(off + u[q]);
       const int2 ld = __ldg(ldesc + u[q]);  // {first col4 word, length}
       ue[q] = ub[q] + ld.y;
       uw[q] = ld.x;
     }
-    int32_t v[kGroupUnroll], vd[kGroupUnroll];
+    int32_t v[UNROLL];
 #pragma unroll
-    for (int q = 0; q < kGroupUnroll; ++q) {
+    for (int q = 0; q < UNROLL; ++q) {
       const uint32_t e = e0 + q * stride;
       v[q] = e < m ? __ldg(col4 + 4ll * uw[q] + ((int32_t)e - ub[q])) : 0;
     }
+    uint64_t key[UNROLL];
+    uint32_t kept = 0;
+    if (WHOLE) {
+      int32_t vd[UNROLL];
 #pragma unroll
-    for (int q = 0; q < kGroupUnroll; ++q) vd[q] = __ldg(ldesc + v[q]).y;
+      for (int q = 0; q < UNROLL; ++q) vd[q] = __ldg(ldesc + v[q]).y;
 #pragma unroll
-    for (int q = 0; q < kGroupUnroll; ++q) {
-      const uint32_t e = e0 + q * stride;
-      if (e >= m) break;
-      int32_t h, l;
-      split_edge(u[q], v[q], ue[q] - ub[q], vd[q], heavy_ratio_pct, h, l);
-      // an edge inside the dense hub block (owner u, hence v, of rank >=
-      // hub_lo) is left to it: its stream is skipped whole
-      uint64_t skip = (carry_skip && h == v[q]) ? (uint64_t)(((int32_t)e - ub[q]) >> 3) : 0ull;
-      if (hub_on && u[q] >= hub_lo) skip = kSkipAll;
-      gkeys[e] = (skip << kSkipShift) | ((uint64_t)(uint32_t)h << b) | (uint32_t)l;
-      for (int p = 0; p < passes; ++p) atomicAdd(&s_hist[p * 256 + ((h >> (8 * p)) & 255)], 1u);
+      for (int q = 0; q < UNROLL; ++q) {
+        const uint32_t e = e0 + q * stride;
+        int32_t h, l;
+        split_edge(u[q], v[q], ue[q] - ub[q], vd[q], heavy_ratio_pct, h, l);
+        // an edge inside the dense hub block (owner u, hence v, of rank >=
+        // hub_lo) is left to it: its stream is skipped whole
+        uint64_t skip =
+            (carry_skip && h == v[q]) ? (uint64_t)(((int32_t)e - ub[q]) >> 3) : 0ull;
+        if (hub_on && u[q] >= hub_lo) skip = kSkipAll;
+        key[q] = (skip << kSkipShift) | ((uint64_t)(uint32_t)h << b) | (uint32_t)l;
+        kept |= (uint32_t)(e < m) << q;
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < UNROLL; ++q) {
+        const uint32_t e = e0 + q * stride;
+        bool own;
+        key[q] = kHole;
+        if (e < m && !(hub_on && u[q] >= hub_lo))
+          key[q] = edge_key(em, u[q], ue[q] - ub[q], (int32_t)e - ub[q], v[q], own);
+        kept |= (uint32_t)(key[q] != kHole) << q;
+      }
+    }
+    uint32_t at[UNROLL];
+    if (WHOLE) {
+#pragma unroll
+      for (int q = 0; q < UNROLL; ++q) at[q] = e0 + q * stride;
+    } else {  // the warp takes the places of its round's keys
+      uint32_t total = 0;
+#pragma unroll
+      for (int q = 0; q < UNROLL; ++q) {
+        const uint32_t bits = __ballot_sync(kFull, (kept >> q) & 1u);
+        at[q] = total + __popc(bits & ((1u << lane) - 1u));
+        total += __popc(bits);
+      }
+      uint32_t base = 0;
+      if (lane == 0 && total) base = atomicAdd(&ctrl->n_part, total);
+      base = __shfl_sync(kFull, base, 0);
+#pragma unroll
+      for (int q = 0; q < UNROLL; ++q) at[q] += base;
+    }
+#pragma unroll
+    for (int q = 0; q < UNROLL; ++q) {
+      if (!((kept >> q) & 1u)) continue;
+      gkeys[at[q]] = key[q];
+      const uint32_t h = (uint32_t)(key[q] >> b) & (uint32_t)((1ull << b) - 1);
+      for (int p = 0; p < passes; ++p) atomicAdd(&s_hist[p * 256 + ((h >> (8 * p)) & 255u)], 1u);
     }
   }
   __syncthreads();
@@ -677,13 +905,16 @@ static uint32_t num_sms() {
 
 void launch_sort_lists(int32_t *col, const int32_t *off, const int32_t *voff, int32_t n,
                        Ctrl *ctrl, int32_t *col4, int32_t *queue, int32_t *dlen,
-                       int32_t *dcorr, int2 *ldesc, cudaStream_t st) {
+                       int32_t *dcorr, int2 *ldesc, const GroupOut *emit, cudaStream_t st) {
   const ListOut o{col4, dlen, dcorr, ldesc, ctrl};
   const uint32_t chunks = ((uint32_t)n + 31u) / 32u;
   const uint32_t grid = max(1u, min((chunks + kListWarps - 1) / kListWarps, num_sms() * 8u));
-  k_sort_lists<<<grid, kListThreads, 0, st>>>(col, off, voff, n, o, queue);
-  k_sort_long_lists<<<num_sms() * kLongListBlocks, kLongListThreads, 0, st>>>(col, off, voff, n,
-                                                                              o, queue);
+  const GroupOut g = emit ? *emit : GroupOut{};
+  const auto lists = emit ? k_sort_lists<true> : k_sort_lists<false>;
+  const auto long_lists = emit ? k_sort_long_lists<true> : k_sort_long_lists<false>;
+  lists<<<grid, kListThreads, 0, st>>>(col, off, voff, n, o, g, queue);
+  long_lists<<<num_sms() * kLongListBlocks, kLongListThreads, 0, st>>>(col, off, voff, n, o, g,
+                                                                       queue);
   note_launch();
   note_launch();
 }
@@ -695,12 +926,12 @@ void launch_fix_repeats(const int32_t *off, int32_t n, const int32_t *dcorr, con
 }
 
 void launch_group_keys(const int32_t *row, const int32_t *col4, const int32_t *off,
-                       const int2 *ldesc, uint32_t m_bound, int b,
-                       int passes, int32_t heavy_ratio_pct, Ctrl *ctrl, uint64_t *gkeys,
+                       const int2 *ldesc, const int32_t *len, uint32_t m_bound, int b, int passes,
+                       int32_t heavy_ratio_pct, bool whole, Ctrl *ctrl, uint64_t *gkeys,
                        uint32_t *hist, cudaStream_t st) {
-  k_group_keys<<<group_grid(m_bound), kGroupThreads, 0, st>>>(row, col4, off, ldesc, b,
-                                                              passes, heavy_ratio_pct, ctrl,
-                                                              gkeys, hist);
+  const auto kernel = whole ? k_group_keys<true> : k_group_keys<false>;
+  kernel<<<group_grid(m_bound), kGroupThreads, 0, st>>>(row, col4, off, ldesc, len, b, passes,
+                                                        heavy_ratio_pct, ctrl, gkeys, hist);
   note_launch();
 }
 

@@ -1,4 +1,6 @@
 // preprocess.cu -- preprocessing of the forward algorithm on sm_103a.
+// (Calls of up to kDirectMaxPairs pairs replace the rank sort, the orient and
+// sort steps and the group sort by the counting sorts of direct.cu.)
 //
 // Sec. III-B of the paper builds, from an edge array, the sorted forward
 // adjacency lists: sort the edges (as 64-bit integers, Sec. III-D), build the
@@ -640,9 +642,8 @@ k_orient(const uint64_t *__restrict__ keys, int b,
 //                 <= m < 2^31 and the padded lists stay below 2^31 16-byte
 //                 words, which the entry points check.
 //   kScanGroups   the partner-group offsets; also bins the groups that can
-//                 hold a triangle (>= 1 partner, >= 2 entries in the hashed
-//                 list) by the length of the hashed list: one warp, a
-//                 256-thread CTA or a 512-thread CTA.
+//                 hold a triangle by the length of the hashed list: one warp,
+//                 a 256-thread CTA or a 512-thread CTA.
 //   kScanRecount  off again after repeated edges were dropped.
 // One scan for both node arrays halves the reads of the counts and saves a
 // launch (R-MAT scale 24: 204 -> 106 us).  The bins take one atomic per tile
@@ -662,7 +663,6 @@ struct ScanArgs {
   const int2 *ldesc;      // kScanGroups: the lists' lengths
   int32_t *groups;        // kScanGroups: warp groups from the front, CTA groups from the end
   int32_t *big_list;
-  BitItems bits;          // kScanGroups: the bitmap path's work items
   Tuning tune;
   unsigned long long *status;
   uint32_t *ticket;
@@ -741,6 +741,9 @@ k_offsets(const ScanArgs a) {
     // bins: per thread the vertices of each kind as a bit mask, their counts
     // scanned over the block in 21-bit fields
     uint32_t mw = 0, mc = 0, mb = 0;
+    // a group by whole list lengths finds nothing in a list of one entry; one
+    // that the list sort emitted may (it weighed the lists with repeats)
+    const int32_t least = a.own ? 1 : 2;
 #pragma unroll
     for (int i = 0; i < IPT; ++i) {
       const uint32_t v = first + i;
@@ -749,9 +752,9 @@ k_offsets(const ScanArgs a) {
       // a warp takes a group only if both its list and its partner count are
       // short: one warp streaming thousands of partners would finish last
       const bool is_warp =
-          dh >= 2 && dh <= a.tune.warp_max_list && d[i] <= a.tune.warp_max_partners;
+          dh >= least && dh <= a.tune.warp_max_list && d[i] <= a.tune.warp_max_partners;
       mw |= (uint32_t)is_warp << i;
-      mc |= (uint32_t)(dh >= 2 && dh <= kCtaMaxRow && !is_warp) << i;
+      mc |= (uint32_t)(dh >= least && dh <= kCtaMaxRow && !is_warp) << i;
       mb |= (uint32_t)(dh > kCtaMaxRow) << i;
     }
     const uint64_t mine = (uint64_t)__popc(mw) | ((uint64_t)__popc(mc) << 21) |
@@ -776,32 +779,6 @@ k_offsets(const ScanArgs a) {
       if ((mw >> i) & 1u) a.groups[w++] = v;
       if ((mc >> i) & 1u) a.groups[n - 1u - c++] = v;
       if ((mb >> i) & 1u) a.big_list[g++] = v;
-    }
-    if (a.bits.rec) {  // uniform
-      // the groups that intersect by bitmaps, in items of at most a range of
-      // partners each
-      uint32_t mi = 0, cnt = 0;
-#pragma unroll
-      for (int i = 0; i < IPT; ++i) {
-        const uint32_t v = first + i;
-        if (((mw | mc | mb) >> i & 1u) && d[i] >= a.bits.min_partners &&
-            __ldg(a.bits.rec + v) != 0u) {
-          mi |= 1u << i;
-          cnt += ((uint32_t)d[i] + a.bits.range - 1) / a.bits.range;
-        }
-      }
-      uint64_t total;
-      const uint64_t mine_at = block_scan_exclusive<kScanThreads>((uint64_t)cnt, s_scratch, &total);
-      if (tid == 0) s_base[0] = total ? atomicAdd(&ctrl->n_bit_items, (uint32_t)total) : 0u;
-      __syncthreads();
-      uint32_t at = s_base[0] + (uint32_t)mine_at, from = (uint32_t)(s_excl + toff);
-#pragma unroll
-      for (int i = 0; i < IPT; ++i) {
-        if ((mi >> i) & 1u)
-          for (uint32_t s = 0; s < (uint32_t)d[i]; s += a.bits.range)
-            a.bits.items[at++] = make_int2((int32_t)(first + i), (int32_t)(from + s));
-        from += (uint32_t)d[i];
-      }
     }
   }
 }
@@ -899,11 +876,11 @@ void launch_offsets(const int32_t *counts, int32_t n, int32_t *off, int32_t *vof
 
 void launch_group_offsets(const int32_t *counts, const int32_t *own, int32_t n, int32_t *goff,
                           const int2 *ldesc, int32_t *groups, int32_t *big_list,
-                          const BitItems &bits, Tuning tune, unsigned long long *status, uint32_t *ticket, Ctrl *ctrl,
+                          Tuning tune, unsigned long long *status, uint32_t *ticket, Ctrl *ctrl,
                           cudaStream_t st, int32_t shard, int32_t shards) {
   tune.warp_max_list = min(max(tune.warp_max_list, 0), kWarpMaxRow);  // warp table capacity
   const ScanArgs a{counts, own,  n,      goff,   nullptr, ldesc,           groups,          big_list,
-                   bits,   tune, status, ticket, ctrl,    (uint32_t)shard, (uint32_t)shards};
+                   tune,   status, ticket, ctrl, (uint32_t)shard, (uint32_t)shards};
   k_offsets<kScanGroups><<<scan_grid(n), kScanThreads, 0, st>>>(a);
   note_launch();
 }

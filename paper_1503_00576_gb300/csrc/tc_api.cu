@@ -192,6 +192,10 @@ struct BatchRun {
   unsigned long long *totals;   // device: triangles per graph
 };
 
+// Set while a failure-path test limits the device's waits: the waits it aims at
+// are those of the radix passes, so every run sorts by them.
+std::atomic<bool> g_wait_hooks{false};
+
 // Enqueues every phase on `st` using workspace `ws` laid out by L, ending
 // with a copy of the control block into `staging` (host).  Nothing here
 // synchronises or allocates, so the whole sequence can be captured in a
@@ -259,9 +263,13 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
   TC_CUDA(cudaMemsetAsync(ws + zero_from, 0,
                           (t_rank || bits_on ? L.st_sort : L.t_rank) - zero_from, st),
           "memset control");
-  TC_CUDA(cudaMemsetAsync(ws + L.st_sort, 0,
-                          sizeof(unsigned long long) * words * (size_t)radix_passes(b), st),
-          "memset status");
+  // counting sorts by atomics, or radix passes (see kDirectMaxPairs)
+  const bool direct = m_in <= kDirectMaxPairs && 2 * b <= kSkipShift && shards == 1 &&
+                      !work_stats && !g_wait_hooks.load();
+  if (!direct)
+    TC_CUDA(cudaMemsetAsync(ws + L.st_sort, 0,
+                            sizeof(unsigned long long) * words * (size_t)radix_passes(b), st),
+            "memset status");
 
   // undirected keys and the degrees (repeated edges counted as often as
   // they are given; the list sort takes them back)
@@ -272,27 +280,36 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
   // rank of every vertex in the (degree, id) order
   pt.start(TC_PHASE_RANK);
   const uint32_t id_mask = (uint32_t)((1ull << b) - 1);
-  launch_rank_keys(deg, n, b, passes_r, vkeys_a, hist + 256 * kRankSlot, st);
-  {
-    uint64_t *vin = vkeys_a, *vout = vkeys_b;
-    for (int p = 0; p < passes_r; ++p) {
-      unsigned long long *status;
-      uint32_t *ticket;
-      next_pass(&status, &ticket);
-      const bool last = p == passes_r - 1;
-      launch_radix_pass(vin, last ? (void *)rank : (void *)vout, last ? kOutRank : kOutKeys,
-                        nullptr, nullptr, (uint32_t)n, nullptr, b + 8 * p, id_mask, 0,
-                        hist + 256 * (kRankSlot + p), status, ticket, ctrl, st);
-      uint64_t *x = vin;
-      vin = vout;
-      vout = x;
+  if (direct) {
+    launch_rank_classes(deg, n, hist, rank, st);
+  } else {
+    launch_rank_keys(deg, n, b, passes_r, vkeys_a, hist + 256 * kRankSlot, st);
+    {
+      uint64_t *vin = vkeys_a, *vout = vkeys_b;
+      for (int p = 0; p < passes_r; ++p) {
+        unsigned long long *status;
+        uint32_t *ticket;
+        next_pass(&status, &ticket);
+        const bool last = p == passes_r - 1;
+        launch_radix_pass(vin, last ? (void *)rank : (void *)vout, last ? kOutRank : kOutKeys,
+                          nullptr, nullptr, (uint32_t)n, nullptr, b + 8 * p, id_mask, 0,
+                          hist + 256 * (kRankSlot + p), status, ticket, ctrl, st);
+        uint64_t *x = vin;
+        vin = vout;
+        vout = x;
+      }
     }
   }
   pt.stop(TC_PHASE_RANK);
 
   pt.start(TC_PHASE_ORIENT);
-  launch_orient(keys_a, m, b, rank, keys_b, hist + 256 * kSort2Slot, passes2, st_orient, ctrl,
-                st);
+  // each entry's place in its list goes to col4's space, free until the lists
+  int32_t *place = col4;
+  if (direct)
+    launch_direct_orient(keys_a, m, b, rank, keys_b, place, outdeg, ctrl, st);
+  else
+    launch_orient(keys_a, m, b, rank, keys_b, hist + 256 * kSort2Slot, passes2, st_orient, ctrl,
+                  st);
   pt.stop(TC_PHASE_ORIENT);
 
   pt.start(TC_PHASE_SORT);
@@ -301,7 +318,7 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
   // row array to the second half of the same buffer.  The order within a
   // list does not matter (each list is sorted on its own later), so the
   // first pass ranks equal digits in any order.
-  for (int p = 0; p < passes2; ++p) {
+  for (int p = 0; p < passes2 && !direct; ++p) {
     unsigned long long *status;
     uint32_t *ticket;
     next_pass(&status, &ticket);
@@ -322,6 +339,7 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
 
   pt.start(TC_PHASE_OFFSETS);
   launch_offsets(outdeg, n, off, voff, st_scan, &ctrl->tile_ticket[kTicketScan], ctrl, st);
+  if (direct) launch_direct_lists(keys_b, place, m, b, off, col, ctrl, st);
   // whether the top ranks are counted densely (their edges are then left
   // out of the partner groups)
   const bool hub = L.has_hub && tune.hub_min_edges >= 0;
@@ -336,9 +354,13 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
   // right again
   pt.start(TC_PHASE_LISTS);
   int32_t *queue = reinterpret_cast<int32_t *>(vkeys_a);
-  launch_sort_lists(col, off, voff, n, ctrl, col4, queue, outdeg, dcorr, ldesc, st);
-  launch_recount(outdeg, n, off, st_scan4, &ctrl->tile_ticket[kTicketRecount], ctrl, st);
-  launch_fix_repeats(off, n, dcorr, rank, ctrl, row, deg, st);
+  int32_t *own = queue + n;  // the rank keys' first buffer holds both
+  const GroupOut emit{in, gcnt, own, b, tune.heavy_ratio_pct};
+  launch_sort_lists(col, off, voff, n, ctrl, col4, queue, outdeg, dcorr, ldesc,
+                    direct ? &emit : nullptr, st);
+  if (!direct)
+    launch_recount(outdeg, n, off, st_scan4, &ctrl->tile_ticket[kTicketRecount], ctrl, st);
+  launch_fix_repeats(off, n, dcorr, rank, ctrl, direct ? nullptr : row, deg, st);
   pt.stop(TC_PHASE_LISTS);
 
   // partner groups: each forward edge goes to the endpoint with the longer
@@ -348,11 +370,15 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
   // into gcnt and writing the skipped blocks of each partner's stream beside
   // the partner array.
   pt.start(TC_PHASE_GROUPS);
-  launch_group_keys(row, col4, off, ldesc, m, b, passes3, tune.heavy_ratio_pct, ctrl, in,
-                    hist + 256 * kGroupSlot, st);
+  // shares and the work counters go by the whole lists' lengths
+  const bool whole = shards > 1 || work_stats || tune.heavy_ratio_pct != 100 ||
+                     2 * b > kSkipShift;
+  if (!direct)
+    launch_group_keys(row, col4, off, ldesc, outdeg, m, b, passes3, tune.heavy_ratio_pct, whole,
+                      ctrl, in, hist + 256 * kGroupSlot, st);
   const bool skip_in_key = 2 * b <= kSkipShift;
   uint64_t *gin = in, *gout = out;  // row and col are dead after the group keys
-  for (int p = 0; p < passes3; ++p) {
+  for (int p = 0; p < passes3 && !direct; ++p) {
     unsigned long long *status;
     uint32_t *ticket;
     next_pass(&status, &ticket);
@@ -363,7 +389,8 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
     // any order
     const RadixOut mode = !last ? kOutKeys : skip_in_key ? kOutPartSkip : kOutColRow;
     uint32_t *skip_target = last && skip_in_key ? reinterpret_cast<uint32_t *>(gout) + m : nullptr;
-    launch_radix_pass(gin, gout, mode, skip_target, last ? gcnt : nullptr, m, &ctrl->m, b + 8 * p,
+    launch_radix_pass(gin, gout, mode, skip_target, last ? gcnt : nullptr, m,
+                      whole ? &ctrl->m : &ctrl->n_part, b + 8 * p,
                       id_mask, b, hist + 256 * (kGroupSlot + p), status, ticket, ctrl, st,
                       /*unstable=*/p == 0);
     if (!last) {
@@ -372,30 +399,25 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
       gout = x;
     }
   }
-  const int32_t *part = reinterpret_cast<const int32_t *>(gout);
-  const int32_t *pskip = reinterpret_cast<const int32_t *>(gout) + m;
+  int32_t *part = reinterpret_cast<int32_t *>(gout);
+  int32_t *pskip = reinterpret_cast<int32_t *>(gout) + m;
   if (!skip_in_key)  // ids of more than 24 bits leave no room for the skip: stream lists whole
-    TC_CUDA(cudaMemsetAsync(reinterpret_cast<int32_t *>(gout) + m, 0, sizeof(int32_t) * (size_t)m,
-                            st),
-            "memset skips");
+    TC_CUDA(cudaMemsetAsync(pskip, 0, sizeof(int32_t) * (size_t)m, st), "memset skips");
   // the group sort's other buffer (free now) takes the bitmaps, or each
   // partner's stream where there are per-vertex counts; the bitmap path's work
   // items (less than 0.2 bytes per pair) take the radix passes' look-back
   // status
   uint32_t *bits = t_out ? reinterpret_cast<uint32_t *>(ws + L.bits)
                          : reinterpret_cast<uint32_t *>(gin);
-  BitItems items{};
-  if (bits_on) {
-    items = BitItems{bit_rec, reinterpret_cast<int2 *>(ws + L.st_sort),
-                     t_out ? kBitRange<true> : kBitRange<false>,
-                     t_out ? kBitMinPartners<true> : kBitMinPartners<false>};
-    launch_bits_build(queue, n, ldesc, col4, L.bit_slots, t_out != nullptr, bits, bit_rec, ctrl,
-                      st);
-  }
+  const BitItems items{bit_rec, reinterpret_cast<int2 *>(ws + L.st_sort)};
   // only this run's share of the groups is binned (all of them unless the
   // counting is split over several devices, Sec. III-E)
-  launch_group_offsets(gcnt, nullptr, n, goff, ldesc, groups, big_groups, items, tune, st_scan2,
-                       &ctrl->tile_ticket[kTicketGroupScan], ctrl, st, shard, shards);
+  launch_group_offsets(gcnt, direct ? own : nullptr, n, goff, ldesc, groups, big_groups, tune,
+                       st_scan2, &ctrl->tile_ticket[kTicketGroupScan], ctrl, st, shard, shards);
+  if (direct) launch_direct_groups(gin, m, b, n, goff, gcnt, part, pskip, ctrl, st);
+  if (bits_on)
+    launch_bits_build(queue, n, ldesc, col4, goff, L.bit_slots, t_out != nullptr, bits, items,
+                      ctrl, st, shard, shards);
   pt.stop(TC_PHASE_GROUPS);
   if (work_stats) launch_work(off, goff, part, pskip, n, ctrl, st, shard, shards);
 
@@ -1175,6 +1197,7 @@ tc_status tc_get_tuning(tc_tuning *out) {
 
 tc_status tc_debug_set_wait_limit(uint32_t spin_limit, int32_t unpublished_tile) {
   TC_CUDA(cudaDeviceSynchronize(), "synchronize");
+  g_wait_hooks.store(spin_limit != kSpinLimit || unpublished_tile >= 0);
   TC_CUDA(set_wait_hooks(spin_limit, unpublished_tile < 0 ? 0xffffffffu : (uint32_t)unpublished_tile),
           "wait hooks");
   return set_status(TC_OK);

@@ -63,6 +63,19 @@ constexpr uint32_t kBitMaxSlots = (1u << (32 - kBitTbBits)) - 1;
 // 91M 22.5 / 16.9).
 template <bool PV> constexpr int64_t kBitMinPairs = PV ? 1 << 25 : 1 << 18;
 
+// Counting sorts by atomics (direct.cu) instead of radix passes: runs of at
+// most this many pairs with ids of at most 24 bits, but for shares of a run
+// (their dealing needs the exact vertex order).  Whole calls, radix passes /
+// counting sorts: 8,191 pairs 196 / 134 us, R-MAT 16 of 2.5M 604 / 539 us, a
+// union of 300 small graphs (3.1M) 745 / 581 us, Barabasi-Albert of 10M 1.88 /
+// 1.69 ms, R-MAT 20 of 16.8M 3.37 / 3.15 ms, 64 graphs of 33M 5.31 / 4.93 ms;
+// ring lattice of 50M 4.91 / 5.05 ms, geometric of 67M 9.4 / 10.6 ms, R-MAT 24
+// of 180M 39 / 45 ms (the scattered writes leave L2).
+constexpr int64_t kDirectMaxPairs = 1ll << 25;
+constexpr int kRankClasses = 1024;
+constexpr uint64_t kHole = ~0ull;            // no edge (dropped pair or edge)
+constexpr uint64_t kOwnEdge = 1ull << 63;    // emitted edge of its owner's group
+
 // Dense hub block (hub.cu): the kHubSize vertices of highest rank, counted
 // on the tensor cores when they hold at least kHubMinEdges edges.  Only for
 // single graphs with n >= kHubMinVertices and ids of at most 24 bits (the
@@ -195,15 +208,26 @@ struct BatchDesc {
   int32_t *gerr;            // [num_graphs], zero on entry; set: an id outside its graph
 };
 
-// Work items of the bitmap path (bits.cu): {group, first partner} for every
-// `range` partners of every group that intersects by bitmaps (rec[h] != 0
-// and at least min_partners partners), ctrl->n_bit_items of them in any
-// order.  rec == nullptr: no bitmaps.
+// Edges emitted to their partner groups by the list sort (direct.cu scatters
+// them).  Slot off[u] + i holds the i-th entry of the sorted N+(u) as
+//   skip << kSkipShift | h << b | l, h the endpoint whose list is hashed, l
+//   the other, skip the leading blocks of N+(l) that cannot match; with
+//   kOwnEdge when h = u, the skip field (0 then) being the edge's number among
+//   u's own edges;
+// or kHole: the entry was a repeat, or no triangle can be found there.
+// gcnt[h] counts the edges emitted to h by others, own[u] gets u's own.
+struct GroupOut {
+  uint64_t *gkeys;
+  int32_t *gcnt, *own;
+  int32_t b, heavy_ratio_pct;
+};
+
+// The bitmaps' records and the work items of the bitmap path (bits.cu):
+// {group, first partner} for every kBitRange partners of every group that
+// intersects by bitmaps, ctrl->n_bit_items of them in any order.
 struct BitItems {
-  const uint32_t *rec;
+  uint32_t *rec;
   int2 *items;
-  uint32_t range;
-  int32_t min_partners;
 };
 
 // Workspace layout for an input of m_in pairs and n vertices.  All offsets
@@ -373,13 +397,12 @@ void launch_offsets(const int32_t *counts, int32_t n, int32_t *off, int32_t *vof
 // nullptr) -> goff[0..n], ctrl->n_part = goff[n]; the groups are binned into
 // the lists by the length of their hashed list (ldesc): warp groups from
 // the front of `groups` up, CTA groups from its end down (n entries hold
-// both), big groups into big_list; bits: the bitmap path's work items are
-// written too (BitItems).  Only the groups h with h mod shards =
+// both), big groups into big_list.  Only the groups h with h mod shards =
 // shard are binned (the share of the counting work this run does; shards = 1
 // bins them all).
 void launch_group_offsets(const int32_t *counts, const int32_t *own, int32_t n, int32_t *goff,
                           const int2 *ldesc, int32_t *groups, int32_t *big_list,
-                          const BitItems &bits, Tuning tune, unsigned long long *status, uint32_t *ticket, Ctrl *ctrl,
+                          Tuning tune, unsigned long long *status, uint32_t *ticket, Ctrl *ctrl,
                           cudaStream_t st, int32_t shard = 0, int32_t shards = 1);
 // The node array again, from the list lengths left after the list sort
 // dropped repeated edges, and ctrl->m = their sum; nothing (the kernel
@@ -410,28 +433,33 @@ cudaError_t launch_hub_count(const int2 *ldesc, const int32_t *col4, int32_t n, 
 // length goes to dlen[v] (written only for such lists; dlen holds the
 // lengths with repeats on entry), each dropped copy adds one to dcorr at
 // both its ends (rank space; zero on entry) and ctrl->dups is set.
+// emit (may be nullptr): the list sort also emits every edge to its partner
+// group (see GroupOut).
 // queue: n entries; the lists of more than 64 entries, ctrl->n_warp_lists
 // of them from its front and ctrl->n_cta_lists (the longest) from its end
 // down; col is scratch for lists longer than
 // kCtaSortMax.
 void launch_sort_lists(int32_t *col, const int32_t *off, const int32_t *voff, int32_t n,
                        Ctrl *ctrl, int32_t *col4, int32_t *queue, int32_t *dlen,
-                       int32_t *dcorr, int2 *ldesc, cudaStream_t st);
+                       int32_t *dcorr, int2 *ldesc, const GroupOut *emit, cudaStream_t st);
 // After the list sort, if some list held repeats: the row array again
 // (row[off[v] + i] = v, from the recounted node array) and the degrees
 // without repeats (deg[v] -= dcorr[rank[v]], caller ids).  Returns at once
-// otherwise.
+// otherwise.  row == nullptr: the degrees alone.
 void launch_fix_repeats(const int32_t *off, int32_t n, const int32_t *dcorr, const int32_t *rank,
                         Ctrl *ctrl, int32_t *row, int32_t *deg, cudaStream_t st);
-// Group keys s << kSkipShift | h << b | l of every forward edge (h: the
-// endpoint with the longer forward list, l: the other one, s: the leading
-// blocks of N+(l) the intersection skips, 0 when 2b > kSkipShift), with the
-// digit histograms of the h field for the group sort.  Reads the sorted
-// lists (col4; their first words and lengths from ldesc) in owner order
-// (row, node array off).
+// Group keys s << kSkipShift | h << b | l of the forward edges (h: the
+// endpoint whose list is hashed, l: the other one, s: the leading blocks of
+// N+(l) the intersection skips, 0 when 2b > kSkipShift), with the digit
+// histograms of the h field for the group sort.  Reads the sorted lists (col4;
+// their first words and lengths from ldesc, the lengths alone from len) in
+// owner order (row, node array off).  whole: every edge, h the endpoint with
+// the longer list; otherwise (2b <= kSkipShift) only the edges that need an
+// intersection, by what is streamed, and ctrl->n_part (zero on entry) is
+// their number.
 void launch_group_keys(const int32_t *row, const int32_t *col4, const int32_t *off,
-                       const int2 *ldesc, uint32_t m_bound, int b,
-                       int passes, int32_t heavy_ratio_pct, Ctrl *ctrl, uint64_t *gkeys,
+                       const int2 *ldesc, const int32_t *len, uint32_t m_bound, int b, int passes,
+                       int32_t heavy_ratio_pct, bool whole, Ctrl *ctrl, uint64_t *gkeys,
                        uint32_t *hist, cudaStream_t st);
 // Instrumentation: adds the counting phase's work into ctrl->work (from the
 // partner groups, the node array and the skipped blocks), over the groups h
@@ -439,13 +467,33 @@ void launch_group_keys(const int32_t *row, const int32_t *col4, const int32_t *o
 void launch_work(const int32_t *off, const int32_t *goff, const int32_t *part,
                  const int32_t *pskip, int32_t n, Ctrl *ctrl, cudaStream_t st,
                  int32_t shard = 0, int32_t shards = 1);
+// ---- launchers (direct.cu) ----
+// rank[v] in an order by degree classes (ties in any order).  counters: 2
+// kRankClasses words, zero on entry.
+void launch_rank_classes(const int32_t *deg, int32_t n, uint32_t *counters, int32_t *rank,
+                         cudaStream_t st);
+// Every key as (lower rank) << b | (higher rank) with its place in the owner's
+// list, the out-degrees counted (zero on entry); dropped pairs as kHole.
+void launch_direct_orient(const uint64_t *keys, uint32_t m_in, int b, const int32_t *rank,
+                          uint64_t *okeys, int32_t *place, int32_t *outdeg, Ctrl *ctrl,
+                          cudaStream_t st);
+// The column array from the oriented keys, their places and the node array.
+void launch_direct_lists(const uint64_t *okeys, const int32_t *place, uint32_t m_in, int b,
+                         const int32_t *off, int32_t *col, Ctrl *ctrl, cudaStream_t st);
+// The partner and skip arrays from the emitted edges and the group offsets;
+// gcnt counts down to zero.
+void launch_direct_groups(const uint64_t *gkeys, uint32_t m_bound, int b, int32_t n,
+                          const int32_t *goff, int32_t *gcnt, int32_t *part, int32_t *pskip,
+                          Ctrl *ctrl, cudaStream_t st);
 // ---- launchers (bits.cu) ----
 // Bitmaps of the queued lists (launch_sort_lists) that have enough entries
 // among the top ranks, at most `slots` - 1 of them: 2 kBitCols bits each into
-// bits, their records into rec[v] (zero on entry).
+// bits, their records into items.rec (zero on entry), and the work items of
+// the groups h with h mod shards = shard (group offsets goff).
 void launch_bits_build(const int32_t *queue, int32_t n, const int2 *ldesc, const int32_t *col4,
-                       uint32_t slots, bool per_vertex, uint32_t *bits, uint32_t *rec, Ctrl *ctrl,
-                       cudaStream_t st);
+                       const int32_t *goff, uint32_t slots, bool per_vertex, uint32_t *bits,
+                       const BitItems &items, Ctrl *ctrl, cudaStream_t st, int32_t shard,
+                       int32_t shards);
 // Intersections by bitmaps: adds what they find to ctrl->total and, if t !=
 // nullptr, to the per-vertex counts t (rank space).  launch_count leaves
 // exactly this part out when it is given the records.
