@@ -199,16 +199,19 @@ __device__ __forceinline__ int32_t column_sums32(int32_t (&v)[32]) {
 // Which hub set, if any, is worth its cost.  The candidates are the top
 // Hmax/4, Hmax/2, 3Hmax/4 and Hmax ranks (multiples of 128).  For every
 // edge inside the largest one, the hash lookups it would cost
-// (min(d+(u), d+(v)), before skipping) are added to the smallest candidate
-// that holds it: one warp per owner u.
+// (min(d+(u), d+(v)), before skipping; at most `cap`, what an intersection by
+// bitmaps costs) are added to the smallest candidate that holds it: one warp
+// per owner u.  Nothing is added up when the largest candidate holds fewer
+// than min_edges edges.
 __device__ __forceinline__ int32_t hub_candidate(int32_t Hmax, int k) {
   return ((Hmax * (k + 1) / 4) / 128) * 128;
 }
 
 __global__ void __launch_bounds__(256)
 k_hub_estimate(const int32_t *__restrict__ off, const int32_t *__restrict__ col, int32_t n,
-               int32_t Hmax, Ctrl *ctrl) {
+               int32_t Hmax, int64_t min_edges, int32_t cap, Ctrl *ctrl) {
   if (aborted(ctrl)) return;
+  if ((int64_t)ctrl->m - (int64_t)__ldg(off + (n - Hmax)) < min_edges) return;
   const int lane = threadIdx.x & 31;
   const uint32_t warps = gridDim.x * (blockDim.x / 32);
   unsigned long long acc[4] = {0, 0, 0, 0};
@@ -223,7 +226,7 @@ k_hub_estimate(const int32_t *__restrict__ off, const int32_t *__restrict__ col,
     for (int32_t i = lane; i < du; i += 32) {
       const int32_t v = __ldg(col + __ldg(off + u) + i);
       const int32_t dv = __ldg(off + v + 1) - __ldg(off + v);
-      sum += (unsigned long long)min(du, dv);
+      sum += (unsigned long long)min(min(du, dv), cap);
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) acc[q] += q == k ? sum : 0ull;
@@ -236,20 +239,23 @@ k_hub_estimate(const int32_t *__restrict__ off, const int32_t *__restrict__ col,
   }
 }
 
-// Cost model (GB300, measured on R-MAT scale 20 and 24 over hub sizes of
-// 8192 to 24576): a lookup taken off the hash path saves about 0.63 ps of
-// the whole GPU's time when only T is counted and 1.03 ps with per-vertex
-// counts (whose match counters go too); one figure between the two, 0.85
-// ps, serves both, so that a graph gets the same hub set in either mode
-// (and tc_count_work reports the work of the run it describes).  The dense
-// block costs about 0.15 ms plus 1.55 ms (H / 16384)^3.
-// The candidate with the largest saving is used if it saves anything.
-// force (hub_min_edges == 0): the largest candidate, whatever the model.
+// Cost model.  A lookup taken off the hash path saves ps_per_lookup
+// picoseconds of the whole GPU's time; the dense block costs about 0.15 ms plus
+// 1.55 ms (H / 16384)^3.  The candidate with the largest saving is used if it
+// saves anything.  force (hub_min_edges == 0): the largest candidate, whatever
+// the model.
+//
+// Where long lists also intersect as bitmaps, an edge saves no more than that
+// would cost: 64 lookups of 0.6 ps when only T is counted, 128 of 0.85 ps with
+// per-vertex counts; without bitmaps 0.85 ps each, however many.  Measured
+// (R-MAT, T only / per vertex, ms; none, 8192, 16384 vertices): scale 18 of
+// 10.5M edges 1.69 1.82 3.15 / 2.67 2.15 3.27, scale 20 of 16.8M 2.57 2.71 4.05
+// / 3.38 2.98 4.20, scale 21 of 91M 15.8 15.4 16.3 / 21.4 20.4 20.9, scale 24
+// of 180M 30.9 30.9 31.7 / 38.6 38.3 38.6.
 __global__ void k_hub_decide(const int32_t *__restrict__ off, int32_t n, int32_t Hmax,
-                             int64_t min_edges, int per_vertex, Ctrl *ctrl) {
+                             int64_t min_edges, double ps_per_lookup, Ctrl *ctrl) {
   if (aborted(ctrl)) return;
-  (void)per_vertex;
-  const double ms_per_lookup = 0.85e-9;
+  const double ms_per_lookup = 1e-9 * ps_per_lookup;
   double best = 0.0;
   int32_t H = 0;
   unsigned long long inside = 0;
@@ -306,8 +312,9 @@ k_hub_scatter(const int2 *__restrict__ ldesc, const int32_t *__restrict__ col4, 
   }
 }
 
-// C tiles of the upper triangle, one per CTA; r(i) += masked row (and
-// column) sums.  Warp 0 lane 0 issues the TMA loads, warp 1 lane 0 the
+// C tiles of the upper triangle, every gridDim.x-th by the same CTA (one CTA per
+// tile of the largest set made the kernel last 32 us where no hub set is
+// used); r(i) += masked row (and column) sums.  Warp 0 lane 0 issues the TMA loads, warp 1 lane 0 the
 // MMAs; all four warps read the accumulator back.
 __global__ void __launch_bounds__(kHubThreads, 2)
 k_hub_gemm(const __grid_constant__ CUtensorMap amap, const uint8_t *__restrict__ A,
@@ -315,17 +322,12 @@ k_hub_gemm(const __grid_constant__ CUtensorMap amap, const uint8_t *__restrict__
   extern __shared__ uint8_t smem_raw[];
   if (!ctrl->hub_on || aborted(ctrl)) return;  // uniform for the block
   const int32_t H = (int32_t)ctrl->hub_size;
-  {
-    const uint32_t T = (uint32_t)H / kHubTile;
-    if (blockIdx.x >= T * (T + 1) / 2) return;  // a tile of a larger hub set
-  }
+  const int T = H / kHubTile, KT = H / kHubKStep;
+  const uint32_t tiles = (uint32_t)T * (uint32_t)(T + 1) / 2;
+  if (blockIdx.x >= tiles) return;
   HubSmem &S = *reinterpret_cast<HubSmem *>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int T = H / kHubTile, KT = H / kHubKStep;
-  int I, J;
-  tile_of(blockIdx.x, T, &I, &J);
-
   if (tid == 0) {
     for (int s = 0; s < kHubStages; ++s) {
       mbar_init(&S.full[s], 1);
@@ -346,82 +348,91 @@ k_hub_gemm(const __grid_constant__ CUtensorMap amap, const uint8_t *__restrict__
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = S.tmem;
 
-  if (warp == 0 && lane == 0) {  // producer
-    int issued = 0;
-    for (int k = 0; k < KT; ++k) {
-      const int s = k % kHubStages;
-      if (k >= kHubStages && !mbar_wait(&S.empty[s], ((k / kHubStages) & 1) ^ 1)) {
-        S.abort = 1;
-        break;
+  // a stage's barriers alternate phases over all K slices that the CTA meets
+  // (g0: those of its earlier tiles), the accumulator's over its tiles
+  uint32_t g0 = 0, parity = 0;
+  for (uint32_t tile = blockIdx.x; tile < tiles; tile += gridDim.x, g0 += KT, parity ^= 1) {
+    int I, J;
+    tile_of(tile, T, &I, &J);
+    if (warp == 0 && lane == 0) {  // producer
+      uint32_t issued = g0;
+      for (int k = 0; k < KT; ++k) {
+        const uint32_t g = g0 + k, s = g % kHubStages;
+        if (g >= kHubStages && !mbar_wait(&S.empty[s], ((g / kHubStages) & 1) ^ 1)) {
+          S.abort = 1;
+          break;
+        }
+        mbar_expect_tx(&S.full[s], 2 * kStageBytes);
+        tma_load(S.a[s], &amap, k * kHubKStep, I * kHubTile, &S.full[s]);
+        tma_load(S.b[s], &amap, k * kHubKStep, J * kHubTile, &S.full[s]);
+        issued = g + 1;
       }
-      mbar_expect_tx(&S.full[s], 2 * kStageBytes);
-      tma_load(S.a[s], &amap, k * kHubKStep, I * kHubTile, &S.full[s]);
-      tma_load(S.b[s], &amap, k * kHubKStep, J * kHubTile, &S.full[s]);
-      issued = k + 1;
-    }
-    // the loads still in flight land before the block may exit
-    for (int k = max(issued - kHubStages, 0); k < issued; ++k)
-      mbar_wait(&S.full[k % kHubStages], (k / kHubStages) & 1);
-  } else if (warp == 1 && lane == 0) {  // MMA issuer
-    for (int k = 0; k < KT; ++k) {
-      const int s = k % kHubStages;
-      if (!mbar_wait(&S.full[s], (k / kHubStages) & 1)) {
-        S.abort = 1;
-        break;
-      }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint64_t ad = smem_desc(S.a[s]), bd = smem_desc(S.b[s]);
+      // the loads still in flight land before the block may exit
+      for (uint32_t g = max(issued, g0 + kHubStages) - kHubStages; g < issued; ++g)
+        mbar_wait(&S.full[g % kHubStages], (g / kHubStages) & 1);
+    } else if (warp == 1 && lane == 0) {  // MMA issuer
+      for (int k = 0; k < KT; ++k) {
+        const uint32_t g = g0 + k, s = g % kHubStages;
+        if (!mbar_wait(&S.full[s], (g / kHubStages) & 1)) {
+          S.abort = 1;
+          break;
+        }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint64_t ad = smem_desc(S.a[s]), bd = smem_desc(S.b[s]);
 #pragma unroll
-      for (int kk = 0; kk < kHubKStep / 32; ++kk)  // K = 32 bytes per instruction
-        mma_f8(tmem, ad + 2 * kk, bd + 2 * kk, (k > 0 || kk > 0) ? 1u : 0u);
-      mma_commit(&S.empty[s]);  // the stage is free once these MMAs have read it
+        for (int kk = 0; kk < kHubKStep / 32; ++kk)  // K = 32 bytes per instruction
+          mma_f8(tmem, ad + 2 * kk, bd + 2 * kk, (k > 0 || kk > 0) ? 1u : 0u);
+        mma_commit(&S.empty[s]);  // the stage is free once these MMAs have read it
+      }
+      mma_commit(&S.done);  // arrives when every MMA issued above is complete
     }
-    mma_commit(&S.done);  // arrives when every MMA issued above is complete
-  }
-  __syncwarp();
+    __syncwarp();
 
-  // epilogue: thread tid owns row i = tid of the tile (tensor-memory lane tid)
-  const bool ok = mbar_wait(&S.done, 0) && !S.abort;
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const int i = tid;
-  const uint8_t *arow = A + (size_t)(I * kHubTile + i) * pitch + (size_t)J * kHubTile;
-  int32_t rowsum = 0;
+    // epilogue: thread tid owns row i = tid of the tile (tensor-memory lane tid)
+    const bool ok = mbar_wait(&S.done, parity) && !S.abort;
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const int i = tid;
+    const uint8_t *arow = A + (size_t)(I * kHubTile + i) * pitch + (size_t)J * kHubTile;
+    int32_t rowsum = 0;
 #pragma unroll 1
-  for (int c = 0; c < kHubTile / 32; ++c) {
-    uint32_t x[32];
-    const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(c * 32);
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
-        "%11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, "
-        "%28, %29, %30, %31}, [%32];"
-        : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]), "=r"(x[4]), "=r"(x[5]), "=r"(x[6]),
-          "=r"(x[7]), "=r"(x[8]), "=r"(x[9]), "=r"(x[10]), "=r"(x[11]), "=r"(x[12]),
-          "=r"(x[13]), "=r"(x[14]), "=r"(x[15]), "=r"(x[16]), "=r"(x[17]), "=r"(x[18]),
-          "=r"(x[19]), "=r"(x[20]), "=r"(x[21]), "=r"(x[22]), "=r"(x[23]), "=r"(x[24]),
-          "=r"(x[25]), "=r"(x[26]), "=r"(x[27]), "=r"(x[28]), "=r"(x[29]), "=r"(x[30]),
-          "=r"(x[31])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-    const uint4 m0 = *reinterpret_cast<const uint4 *>(arow + 32 * c);
-    const uint4 m1 = *reinterpret_cast<const uint4 *>(arow + 32 * c + 16);
-    const uint32_t mw[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
-    int32_t v[32];
+    for (int c = 0; c < kHubTile / 32; ++c) {
+      uint32_t x[32];
+      const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(c * 32);
+      asm volatile(
+          "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
+          "%11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, "
+          "%28, %29, %30, %31}, [%32];"
+          : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]), "=r"(x[4]), "=r"(x[5]), "=r"(x[6]),
+            "=r"(x[7]), "=r"(x[8]), "=r"(x[9]), "=r"(x[10]), "=r"(x[11]), "=r"(x[12]),
+            "=r"(x[13]), "=r"(x[14]), "=r"(x[15]), "=r"(x[16]), "=r"(x[17]), "=r"(x[18]),
+            "=r"(x[19]), "=r"(x[20]), "=r"(x[21]), "=r"(x[22]), "=r"(x[23]), "=r"(x[24]),
+            "=r"(x[25]), "=r"(x[26]), "=r"(x[27]), "=r"(x[28]), "=r"(x[29]), "=r"(x[30]),
+            "=r"(x[31])
+          : "r"(taddr));
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      const uint4 m0 = *reinterpret_cast<const uint4 *>(arow + 32 * c);
+      const uint4 m1 = *reinterpret_cast<const uint4 *>(arow + 32 * c + 16);
+      const uint32_t mw[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
+      int32_t v[32];
 #pragma unroll
-    for (int j = 0; j < 32; ++j) {
-      const bool edge = ((mw[j >> 2] >> (8 * (j & 3))) & 0xffu) != 0u;
-      v[j] = (ok && edge) ? (int32_t)__float2int_rn(__uint_as_float(x[j])) : 0;
-      rowsum += v[j];
+      for (int j = 0; j < 32; ++j) {
+        const bool edge = ((mw[j >> 2] >> (8 * (j & 3))) & 0xffu) != 0u;
+        v[j] = (ok && edge) ? (int32_t)__float2int_rn(__uint_as_float(x[j])) : 0;
+        rowsum += v[j];
+      }
+      if (I != J) S.col[warp][32 * c + lane] = column_sums32(v);
     }
-    if (I != J) S.col[warp][32 * c + lane] = column_sums32(v);
+    if (rowsum) atomicAdd(r + I * kHubTile + i, (uint32_t)rowsum);
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (I != J) {
+      const int32_t cs = S.col[0][tid] + S.col[1][tid] + S.col[2][tid] + S.col[3][tid];
+      if (cs) atomicAdd(r + J * kHubTile + tid, (uint32_t)cs);
+    }
+    if (!ok && tid == 0) atomicOr(&ctrl->err, kErrTimeout);
+    __syncthreads();  // S.col and the accumulator are written again
+    if (S.abort) break;  // uniform: nothing writes it between the barriers
   }
-  if (rowsum) atomicAdd(r + I * kHubTile + i, (uint32_t)rowsum);
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  if (I != J) {
-    const int32_t cs = S.col[0][tid] + S.col[1][tid] + S.col[2][tid] + S.col[3][tid];
-    if (cs) atomicAdd(r + J * kHubTile + tid, (uint32_t)cs);
-  }
-  if (!ok && tid == 0) atomicOr(&ctrl->err, kErrTimeout);
   if (warp == 1) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
@@ -485,9 +496,10 @@ EncodeTiled encode_fn() {
 size_t hub_bytes(int32_t H) { return (size_t)H * (size_t)H + 4 * (size_t)H; }
 
 void launch_hub_decide(const int32_t *off, const int32_t *col, int32_t n, int32_t Hmax,
-                       int64_t min_edges, bool per_vertex, Ctrl *ctrl, cudaStream_t st) {
-  k_hub_estimate<<<(Hmax + 7) / 8, 256, 0, st>>>(off, col, n, Hmax, ctrl);
-  k_hub_decide<<<1, 1, 0, st>>>(off, n, Hmax, min_edges, per_vertex ? 1 : 0, ctrl);
+                       int64_t min_edges, int32_t cap, double ps_per_lookup, Ctrl *ctrl,
+                       cudaStream_t st) {
+  k_hub_estimate<<<(Hmax + 7) / 8, 256, 0, st>>>(off, col, n, Hmax, min_edges, cap, ctrl);
+  k_hub_decide<<<1, 1, 0, st>>>(off, n, Hmax, min_edges, ps_per_lookup, ctrl);
   note_launch();
   note_launch();
 }
@@ -524,7 +536,9 @@ cudaError_t launch_hub_count(const int2 *ldesc, const int32_t *col4, int32_t n, 
   k_hub_zero<<<(sms > 0 ? sms : 1) * 8, 256, 0, st>>>(A, Hmax, ctrl);
   k_hub_scatter<<<(Hmax + 7) / 8, 256, 0, st>>>(ldesc, col4, n, Hmax, ctrl, A);
   const int T = Hmax / kHubTile;
-  k_hub_gemm<<<T * (T + 1) / 2, kHubThreads, kHubSmemBytes, st>>>(map, A, Hmax, ctrl, r);
+  const int tiles = T * (T + 1) / 2;
+  k_hub_gemm<<<min(tiles, 2 * (sms > 0 ? sms : 1)), kHubThreads, kHubSmemBytes, st>>>(
+      map, A, Hmax, ctrl, r);
   k_hub_finish<<<1, 1024, 0, st>>>(r, ctrl, t);
   for (int i = 0; i < 4; ++i) note_launch();
   return cudaGetLastError();

@@ -263,6 +263,9 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
   TC_CUDA(cudaMemsetAsync(ws + zero_from, 0,
                           (t_rank || bits_on ? L.st_sort : L.t_rank) - zero_from, st),
           "memset control");
+  // shares and the work counters go by the whole lists' lengths
+  const bool whole = shards > 1 || work_stats || tune.heavy_ratio_pct != 100 ||
+                     2 * b > kSkipShift;
   // counting sorts by atomics, or radix passes (see kDirectMaxPairs)
   const bool direct = m_in <= kDirectMaxPairs && 2 * b <= kSkipShift && shards == 1 &&
                       !work_stats && !g_wait_hooks.load();
@@ -344,7 +347,13 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
   // out of the partner groups)
   const bool hub = L.has_hub && tune.hub_min_edges >= 0;
   const int32_t H = L.hub_vertices;  // the size the workspace was laid out for
-  if (hub) launch_hub_decide(off, col, n, H, tune.hub_min_edges, t_out != nullptr, ctrl, st);
+  // what an edge inside the block saves (shares and the work counters go by
+  // the model without bitmaps, so that their split does not depend on them)
+  const bool by_bits = bits_on && !whole;
+  if (hub)
+    launch_hub_decide(off, col, n, H, tune.hub_min_edges,
+                      !by_bits ? INT32_MAX : t_out ? 128 : 64, by_bits && !t_out ? 0.6 : 0.85,
+                      ctrl, st);
   pt.stop(TC_PHASE_OFFSETS);
 
   // every forward list sorted into the padded column array col4 (the rank
@@ -370,9 +379,6 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
   // into gcnt and writing the skipped blocks of each partner's stream beside
   // the partner array.
   pt.start(TC_PHASE_GROUPS);
-  // shares and the work counters go by the whole lists' lengths
-  const bool whole = shards > 1 || work_stats || tune.heavy_ratio_pct != 100 ||
-                     2 * b > kSkipShift;
   if (!direct)
     launch_group_keys(row, col4, off, ldesc, outdeg, m, b, passes3, tune.heavy_ratio_pct, whole,
                       ctrl, in, hist + 256 * kGroupSlot, st);

@@ -416,9 +416,11 @@ size_t hub_bytes(int32_t H);
 // Decides on the device (into ctrl->hub_on, hub_size, hub_lo) whether, and
 // with how many of the top ranks (a candidate up to Hmax), the hub block is
 // counted densely; needs the node array and the column array (any order
-// within a list).
+// within a list).  An edge is taken to save at most `cap` lookups of
+// ps_per_lookup picoseconds each.
 void launch_hub_decide(const int32_t *off, const int32_t *col, int32_t n, int32_t Hmax,
-                       int64_t min_edges, bool per_vertex, Ctrl *ctrl, cudaStream_t st);
+                       int64_t min_edges, int32_t cap, double ps_per_lookup, Ctrl *ctrl,
+                       cudaStream_t st);
 // Counts the triangles inside the hub block (if ctrl->hub_on): adds them to
 // ctrl->total and, if t != nullptr, to the per-vertex counts t (rank space).
 // Needs the forward lists; region: hub_bytes(Hmax) bytes, 256-byte aligned.
