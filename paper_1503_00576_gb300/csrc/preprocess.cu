@@ -189,73 +189,111 @@ __device__ __forceinline__ void publish_aggregate(unsigned long long *status, ui
 constexpr int kCanonThreads = 256;
 constexpr int kCanonUnroll = 8;
 
+// The key of pair (u, v) of a graph with ids in [0, lim), shifted by its first
+// union id; counts the degrees.  bad: an id is out of range.
+__device__ __forceinline__ uint64_t pair_key(int32_t u, int32_t v, int32_t lim, int32_t shift,
+                                             int b, uint64_t sentinel, int32_t *deg, bool &bad) {
+  if ((uint32_t)u >= (uint32_t)lim || (uint32_t)v >= (uint32_t)lim) {
+    bad = true;
+    return sentinel;
+  }
+  if (u == v) return sentinel;  // self-loop: dropped with the sentinels
+  const uint32_t lo = (uint32_t)(min(u, v) + shift), hi = (uint32_t)(max(u, v) + shift);
+  atomicAdd(&deg[lo], 1);
+  atomicAdd(&deg[hi], 1);
+  return ((uint64_t)lo << b) | hi;
+}
+
+// The pairs of kCanonUnroll rounds are loaded before any is keyed: the inputs
+// may be host memory read in place, where each load waits a long time.  Pairs
+// and keys pass through L2 marked to be evicted first (they are read or
+// written once here), so that the degree array stays in L2 for the atomics
+// (-0.27 ms of 2.55 at R-MAT scale 24).
 __global__ void __launch_bounds__(kCanonThreads)
 k_canon(const int32_t *__restrict__ src, const int32_t *__restrict__ dst, uint32_t m_in,
-        int32_t n, int b, const BatchDesc *__restrict__ batch, uint64_t *__restrict__ keys,
-        int32_t *__restrict__ deg, Ctrl *ctrl) {
+        int32_t n, int b, uint64_t *__restrict__ keys, int32_t *__restrict__ deg, Ctrl *ctrl) {
   const uint64_t sentinel = (1ull << (2 * b)) - 1;  // > every valid key; 2b <= 62
-  // batch: graph g owns pairs [eo[g], eo[g+1]) and union ids from vo[g]
-  int32_t ng = 0;
-  const int32_t *eo = nullptr, *vo = nullptr;
-  uint32_t m_real = m_in;
-  if (batch) {
-    ng = batch->num_graphs;
-    eo = batch->edge_off;
-    vo = batch->voff;
-    m_real = min((uint32_t)__ldg(eo + ng), m_in);
-  }
-  if (blockIdx.x == 0 && threadIdx.x == 0) ctrl->m_in = m_real;
+  if (blockIdx.x == 0 && threadIdx.x == 0) ctrl->m_in = m_in;
   bool bad = false;
   const uint32_t stride = gridDim.x * kCanonThreads;
-  // pairs past m_real are batch padding: not keyed, not sorted.  The pairs
-  // of kCanonUnroll rounds are loaded before any is keyed: the inputs may be
-  // host memory read in place, where each load waits a long time.  Pairs and
-  // keys pass through L2 marked to be evicted first (they are read or
-  // written once here), so that the degree array stays in L2 for the atomics
-  // (-0.27 ms of 2.55 at R-MAT scale 24).
-  for (uint32_t i0 = blockIdx.x * kCanonThreads + threadIdx.x; i0 < m_real;
+  for (uint32_t i0 = blockIdx.x * kCanonThreads + threadIdx.x; i0 < m_in;
        i0 += kCanonUnroll * stride) {
     int32_t us[kCanonUnroll], vs[kCanonUnroll];
 #pragma unroll
     for (int q = 0; q < kCanonUnroll; ++q) {
       const uint32_t i = i0 + q * stride;
-      us[q] = i < m_real ? __ldcs(src + i) : 0;
-      vs[q] = i < m_real ? __ldcs(dst + i) : 0;
+      us[q] = i < m_in ? __ldcs(src + i) : 0;
+      vs[q] = i < m_in ? __ldcs(dst + i) : 0;
     }
 #pragma unroll
     for (int q = 0; q < kCanonUnroll; ++q) {
       const uint32_t i = i0 + q * stride;
-      if (i >= m_real) break;
-      const int32_t u = us[q], v = vs[q];
-      int32_t lim = n, shift = 0, lo_graph = 0;
-      if (batch) {
-        int32_t lo = 0, hi = ng;  // the last graph g with eo[g] <= i
-        while (hi - lo > 1) {
-          const int32_t mid = (lo + hi) >> 1;
-          if ((uint32_t)__ldg(eo + mid) <= i) lo = mid; else hi = mid;
-        }
-        lo_graph = lo;
-        shift = __ldg(vo + lo);
-        lim = __ldg(vo + lo + 1) - shift;
-      }
-      uint64_t key;
-      if ((uint32_t)u >= (uint32_t)lim || (uint32_t)v >= (uint32_t)lim) {
-        // a batch fails only the graph that holds the pair; the pair is dropped
-        // so the other graphs of the union are counted exactly
-        if (batch) batch->gerr[lo_graph] = 1; else bad = true;
-        key = sentinel;
-      } else if (u == v) {
-        key = sentinel;  // self-loop: sorts last, dropped with the sentinels
-      } else {
-        const uint32_t lo = (uint32_t)(min(u, v) + shift), hi = (uint32_t)(max(u, v) + shift);
-        key = ((uint64_t)lo << b) | hi;
-        atomicAdd(&deg[lo], 1);
-        atomicAdd(&deg[hi], 1);
-      }
-      __stcs(reinterpret_cast<unsigned long long *>(keys) + i, (unsigned long long)key);
+      if (i >= m_in) break;
+      __stcs(reinterpret_cast<unsigned long long *>(keys) + i,
+             (unsigned long long)pair_key(us[q], vs[q], n, 0, b, sentinel, deg, bad));
     }
   }
   if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(&ctrl->err, kErrIdRange);
+}
+
+// A batch: graph g owns pairs [eo[g], eo[g+1]) and union ids from vo[g]; pairs
+// past the last graph's are padding: not keyed, not sorted.  A warp takes 256
+// consecutive pairs, searches the graph of the first and steps on from there.
+// Consecutive warps work in kSpread different parts of the batch: all on one
+// graph, they queue at the counters of its few hubs (64 graphs, 33M pairs: 638
+// us, spread 459).  A pair
+// with an id out of range fails only the graph that holds it; the pair is
+// dropped so the other graphs of the union are counted exactly.  Also zeroes
+// the totals that k_batch_totals adds to.
+__global__ void __launch_bounds__(kCanonThreads)
+k_canon_batch(const int32_t *__restrict__ src, const int32_t *__restrict__ dst, uint32_t m_in,
+              int b, const BatchDesc *__restrict__ batch, int32_t num_graphs_bound,
+              unsigned long long *__restrict__ totals, uint64_t *__restrict__ keys,
+              int32_t *__restrict__ deg, Ctrl *ctrl) {
+  constexpr uint32_t CHUNK = 32 * kCanonUnroll, kSpread = 256;
+  const uint64_t sentinel = (1ull << (2 * b)) - 1;
+  const int32_t ng = batch->num_graphs;
+  const int32_t *eo = batch->edge_off, *vo = batch->voff;
+  const uint32_t m = min((uint32_t)__ldg(eo + ng), m_in);
+  const int lane = threadIdx.x & 31;
+  const uint32_t first = blockIdx.x * kCanonThreads + threadIdx.x;
+  if (first == 0) ctrl->m_in = m;
+  for (uint32_t g = first; g < (uint32_t)num_graphs_bound; g += gridDim.x * kCanonThreads)
+    totals[g] = 0ull;
+  const uint32_t rows = ((m + CHUNK - 1) / CHUNK + kSpread - 1) / kSpread;  // chunks per part
+  for (uint32_t c = first >> 5; c < rows * kSpread; c += gridDim.x * kCanonThreads >> 5) {
+    const uint32_t chunk = c % kSpread * rows + c / kSpread;
+    if (chunk * CHUNK >= m) continue;
+    const uint32_t i0 = chunk * CHUNK;
+    int32_t us[kCanonUnroll], vs[kCanonUnroll];
+#pragma unroll
+    for (int q = 0; q < kCanonUnroll; ++q) {
+      const uint32_t i = i0 + 32 * q + lane;
+      us[q] = i < m ? __ldcs(src + i) : 0;
+      vs[q] = i < m ? __ldcs(dst + i) : 0;
+    }
+    int32_t g = 0, hi = ng;  // the last graph with eo[g] <= i0
+    while (hi - g > 1) {
+      const int32_t mid = (g + hi) >> 1;
+      if ((uint32_t)__ldg(eo + mid) <= i0) g = mid; else hi = mid;
+    }
+    uint32_t end = (uint32_t)__ldg(eo + g + 1);
+    int32_t shift = __ldg(vo + g), lim = __ldg(vo + g + 1) - shift;
+#pragma unroll
+    for (int q = 0; q < kCanonUnroll; ++q) {
+      const uint32_t i = i0 + 32 * q + lane;
+      if (i >= m) break;
+      if (i >= end) {
+        do end = (uint32_t)__ldg(eo + ++g + 1); while (i >= end);
+        shift = __ldg(vo + g);
+        lim = __ldg(vo + g + 1) - shift;
+      }
+      bool bad = false;
+      __stcs(reinterpret_cast<unsigned long long *>(keys) + i,
+             (unsigned long long)pair_key(us[q], vs[q], lim, shift, b, sentinel, deg, bad));
+      if (bad) batch->gerr[g] = 1;
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -803,14 +841,26 @@ cudaError_t set_wait_hooks(uint32_t spin_limit, uint32_t unpublished_tile) {
   return e;
 }
 
-void launch_canon(const int32_t *src, const int32_t *dst, uint32_t m_in, int32_t n, int b,
-                  const BatchDesc *batch, uint64_t *keys, int32_t *deg, Ctrl *ctrl,
-                  cudaStream_t st) {
+static uint32_t canon_grid(uint32_t m_in) {
   // many pairs in flight: the degree atomics wait on L2
   const uint32_t want = (m_in + kCanonThreads * 8 - 1) / (kCanonThreads * 8);
   const uint32_t cap = (uint32_t)num_sms() * 32;
-  const uint32_t grid = max(1u, min(want, cap));
-  k_canon<<<grid, kCanonThreads, 0, st>>>(src, dst, m_in, n, b, batch, keys, deg, ctrl);
+  return max(1u, min(want, cap));
+}
+
+void launch_canon(const int32_t *src, const int32_t *dst, uint32_t m_in, int32_t n, int b,
+                  uint64_t *keys, int32_t *deg, Ctrl *ctrl, cudaStream_t st) {
+  k_canon<<<canon_grid(m_in), kCanonThreads, 0, st>>>(src, dst, m_in, n, b, keys, deg, ctrl);
+  note_launch();
+}
+
+void launch_canon_batch(const int32_t *src, const int32_t *dst, uint32_t m_in, int b,
+                        const BatchDesc *batch, int32_t num_graphs_bound,
+                        unsigned long long *totals, uint64_t *keys, int32_t *deg, Ctrl *ctrl,
+                        cudaStream_t st) {
+  k_canon_batch<<<canon_grid(m_in), kCanonThreads, 0, st>>>(src, dst, m_in, b, batch,
+                                                            num_graphs_bound, totals, keys, deg,
+                                                            ctrl);
   note_launch();
 }
 

@@ -188,7 +188,7 @@ tc_status check_args(const int32_t *src, const int32_t *dst, int64_t m, int32_t 
 // disjoint union).
 struct BatchRun {
   const BatchDesc *desc;        // device descriptor of the graphs
-  int32_t num_graphs_bound;     // grid bound of the per-graph sums
+  int32_t num_graphs_bound;     // at least the batch's graphs
   unsigned long long *totals;   // device: triangles per graph
 };
 
@@ -238,8 +238,6 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
   int2 *ldesc = reinterpret_cast<int2 *>(ws + L.vkeys_b);
   // per-vertex counts, or per-group totals of a batch, in rank space
   int64_t *t_rank = (t_out || batch) ? reinterpret_cast<int64_t *>(ws + L.t_rank) : nullptr;
-  // group totals back in union ids (the rank keys are free by then)
-  int64_t *tg_union = reinterpret_cast<int64_t *>(ws + L.vkeys_a);
   // long lists also as bitmaps of the top ranks: records (zeroed with t_rank)
   // and, once the groups are sorted, the bitmaps
   const bool bits_on = L.has_bits && !batch;
@@ -277,7 +275,11 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
   // undirected keys and the degrees (repeated edges counted as often as
   // they are given; the list sort takes them back)
   pt.start(TC_PHASE_CANON);
-  launch_canon(src, dst, m, n, b, batch ? batch->desc : nullptr, keys_a, deg, ctrl, st);
+  if (batch)
+    launch_canon_batch(src, dst, m, b, batch->desc, batch->num_graphs_bound, batch->totals, keys_a,
+                       deg, ctrl, st);
+  else
+    launch_canon(src, dst, m, n, b, keys_a, deg, ctrl, st);
   pt.stop(TC_PHASE_CANON);
 
   // rank of every vertex in the (degree, id) order
@@ -443,14 +445,8 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
                                bits_on ? bit_rec : nullptr, n, ctrl, t_out ? t_rank : nullptr,
                                t_out ? nullptr : t_rank, st);
   if (e == cudaSuccess && t_out) launch_gather_counts(t_rank, rank, n, t_out, ctrl, st);
-  if (e == cudaSuccess && batch) {
-    if (t_out) {  // per graph: (sum of t) / 3
-      launch_segment_sums(t_out, batch->desc, batch->num_graphs_bound, 3, batch->totals, st);
-    } else {      // per graph: sum of the group totals
-      launch_gather_counts(t_rank, rank, n, tg_union, ctrl, st);
-      launch_segment_sums(tg_union, batch->desc, batch->num_graphs_bound, 1, batch->totals, st);
-    }
-  }
+  if (e == cudaSuccess && batch)  // per graph: the sum of the group totals
+    launch_batch_totals(t_rank, rank, batch->desc, n, ctrl, batch->totals, st);
   pt.stop(TC_PHASE_COUNT);
   if (e != cudaSuccess) return cuda_fail(e, "count kernel");
   TC_CUDA(cudaGetLastError(), "kernel launch");

@@ -356,12 +356,15 @@ cudaError_t set_wait_hooks(uint32_t spin_limit, uint32_t unpublished_tile);
 // Undirected keys min << b | max of the pairs (self-loops and pairs with an
 // id out of range: the sentinel 2^(2b) - 1) and deg[v] += 1 at both ends of
 // every other pair (the degree with repeats; deg must be zero on entry).
-// batch == nullptr: one graph on ids [0, n).  Otherwise ids of pair i are
-// local to its graph, checked against that graph's vertex count, and
-// shifted by the graph's first union id.
 void launch_canon(const int32_t *src, const int32_t *dst, uint32_t m_in, int32_t n, int b,
-                  const BatchDesc *batch, uint64_t *keys, int32_t *deg, Ctrl *ctrl,
-                  cudaStream_t st);
+                  uint64_t *keys, int32_t *deg, Ctrl *ctrl, cudaStream_t st);
+// The same for a batch: ids of pair i are local to its graph, checked against
+// that graph's vertex count, and shifted by the graph's first union id.
+// Zeroes totals[0 .. num_graphs_bound).
+void launch_canon_batch(const int32_t *src, const int32_t *dst, uint32_t m_in, int b,
+                        const BatchDesc *batch, int32_t num_graphs_bound,
+                        unsigned long long *totals, uint64_t *keys, int32_t *deg, Ctrl *ctrl,
+                        cudaStream_t st);
 // Output of a radix pass: the keys themselves; the column array (low bits,
 // to `out`) plus the row array (key >> owner_shift, to `row_out`) with the
 // out-degrees added to `outdeg`; or the rank scatter rank[low bits] =
@@ -516,9 +519,12 @@ cudaError_t launch_count(const int2 *ldesc, const int32_t *col4, const int32_t *
 // Sets the counting kernels' attributes and occupancy for the current
 // device (done lazily otherwise; needed before capturing a CUDA graph).
 cudaError_t prepare_count_kernels();
-// out[g] = (sum of vals over graph g's union ids) / divisor.
-void launch_segment_sums(const int64_t *vals, const BatchDesc *batch, int32_t num_graphs,
-                         int32_t divisor, unsigned long long *out, cudaStream_t st);
+// Adds every graph's group totals (tg, rank space) to totals[g] (zero on
+// entry); ~0 (TC_COUNT_ERROR) for a graph that had an id out of range.  n:
+// bound of the union's vertices.
+void launch_batch_totals(const int64_t *tg, const int32_t *rank, const BatchDesc *batch,
+                         int32_t n, const Ctrl *ctrl, unsigned long long *totals,
+                         cudaStream_t st);
 // ---- clustering (count.cu) ----
 void launch_clustering(const int64_t *t, const int32_t *deg, int32_t n, double *cc,
                        unsigned long long *sums /* [2]: sum t, sum C(deg,2) */, cudaStream_t st);
