@@ -48,6 +48,7 @@ k_bits_build(const int32_t *__restrict__ queue, int32_t n, const int2 *__restric
              const int32_t *__restrict__ col4, const int32_t *__restrict__ goff, uint32_t slots,
              uint32_t *__restrict__ bits, uint32_t *__restrict__ rec, int2 *__restrict__ items,
              Ctrl *ctrl, uint32_t shard, uint32_t shards) {
+  grid_begin();
   __shared__ uint32_t s_bits[kWarps][kWords];
   if (aborted(ctrl)) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -82,7 +83,8 @@ k_bits_build(const int32_t *__restrict__ queue, int32_t n, const int2 *__restric
     const int32_t len = ld.y, blocks = (len + 7) >> 3;
     const int32_t *list = col4 + 4ll * ld.x;
     // enough top ranks at all?
-    if (blocks < kBitMinBlocks<PV> || __ldg(list + len - 8 * (kBitMinBlocks<PV> - 1) - 1) < base) continue;
+    constexpr int32_t kLeast = 8 * (kBitMinBlocks<PV> - 1) + 1;
+    if (blocks < kBitMinBlocks<PV> || __ldg(list + len - kLeast) < base) continue;
     for (int w = lane; w < kWords; w += 32) sb[w] = 0u;
     __syncwarp();
     int32_t top = 0;  // entries before the first top rank
@@ -382,6 +384,7 @@ __device__ __forceinline__ void bits_vertex(const BitArgs &a, int32_t h, uint32_
 template <bool PV>
 __global__ void __launch_bounds__(kThreads, PV ? 4 : 8)
 k_count_bits(const BitArgs a) {
+  grid_begin();
   __shared__ Queue<PV> s_queue[kWarps];
   __shared__ __align__(16) uint32_t s_planes[PV ? kWarps : 1][PV ? kPlanes * kWords : 4];
   __shared__ uint32_t s_t[PV ? kBitCols : 1];
@@ -433,10 +436,8 @@ void launch_bits_build(const int32_t *queue, int32_t n, const int2 *ldesc, const
                        const BitItems &items, Ctrl *ctrl, cudaStream_t st, int32_t shard,
                        int32_t shards) {
   const auto kernel = per_vertex ? k_bits_build<true> : k_bits_build<false>;
-  kernel<<<sm_count() * 8u, kThreads, 0, st>>>(queue, n, ldesc, col4, goff, slots, bits, items.rec,
-                                               items.items, ctrl, (uint32_t)shard,
-                                               (uint32_t)shards);
-  note_launch();
+  launch(kernel, sm_count() * 8u, kThreads, 0, st, queue, n, ldesc, col4, goff, slots, bits,
+         items.rec, items.items, ctrl, (uint32_t)shard, (uint32_t)shards);
 }
 
 void launch_count_bits(const int2 *ldesc, const int32_t *col4, const int32_t *goff,
@@ -444,10 +445,9 @@ void launch_count_bits(const int2 *ldesc, const int32_t *col4, const int32_t *go
                        const uint32_t *bits, int32_t n, Ctrl *ctrl, int64_t *t, cudaStream_t st) {
   const BitArgs a{goff, part, pskip, ldesc, col4, items.rec, bits, items.items, n, ctrl, t};
   if (t)
-    k_count_bits<true><<<sm_count() * 4u, kThreads, 0, st>>>(a);
+    launch(k_count_bits<true>, sm_count() * 4u, kThreads, 0, st, a);
   else
-    k_count_bits<false><<<sm_count() * 8u, kThreads, 0, st>>>(a);
-  note_launch();
+    launch(k_count_bits<false>, sm_count() * 8u, kThreads, 0, st, a);
 }
 
 }  // namespace tc

@@ -36,7 +36,7 @@ namespace tc {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kGroupChunk = 8;  // warp groups per atomic
+constexpr int kGroupChunk = 8;  // warp groups per atomic (at most)
 constexpr int kMinChunk = 8;    // fewest partners a warp of a CTA group claims
 constexpr int kWindows = 4;     // 16-byte words per lane loaded before probing (two blocks)
 constexpr int kBigWindows = 4;  // ... in the long-list kernel
@@ -91,7 +91,7 @@ __device__ __forceinline__ uint32_t table_slots(int32_t len, uint32_t capacity) 
 
 // Read-only view of the forward lists and partner groups.
 struct Lists {
-  const int32_t *__restrict__ col4;  // forward lists, sorted, each padded with -1 to whole 32-byte blocks
+  const int32_t *__restrict__ col4;  // forward lists, sorted, in whole 32-byte blocks (-1 pads)
   const int32_t *__restrict__ goff;  // partner-group offsets
   const int32_t *__restrict__ part;   // partners
   const int32_t *__restrict__ pskip;  // per partner: leading blocks of its list skipped
@@ -548,8 +548,8 @@ __device__ __forceinline__ void cta_groups(const Lists &g, const int32_t *__rest
         c = __shfl_sync(kFull, c, 0);
         cs = __shfl_sync(kFull, cs, 0);
         if ((int32_t)c >= np) break;
-        probe_chunk<PV, W>(g, g.part + pb, g.pskip + pb, g.desc + pb, np, (int32_t)c, (int32_t)cs, bits, tb, s_ws[warp],
-                           t, found_total, found_group);
+        probe_chunk<PV, W>(g, g.part + pb, g.pskip + pb, g.desc + pb, np, (int32_t)c, (int32_t)cs,
+                           bits, tb, s_ws[warp], t, found_total, found_group);
       }
       __syncthreads();
       if (PV) {
@@ -573,19 +573,21 @@ __device__ __forceinline__ void cta_groups(const Lists &g, const int32_t *__rest
 }
 
 // Groups of `list` counted by one warp each with a private table of
-// WSLOTS slots (empty on entry and on exit).
+// WSLOTS slots (empty on entry and on exit).  claim: groups taken at a time (in
+// shared memory: a register for it cost 7% on random geometric graphs).
 template <bool PV, int WSLOTS>
 __device__ __forceinline__ void warp_groups(const Lists &g, const int32_t *__restrict__ list,
-                                            uint32_t n_list, uint32_t *cursor, Table tb,
+                                            uint32_t n_list, uint32_t *cursor,
+                                            const uint32_t *claim, Table tb,
                                             uint16_t *slot_of, WarpScratch &ws, int64_t *t,
                                             int64_t *tg, uint64_t &found_total) {
   const int lane = threadIdx.x & 31;
   for (;;) {
     uint32_t g0 = 0;
-    if (lane == 0) g0 = atomicAdd(cursor, (uint32_t)kGroupChunk);
+    if (lane == 0) g0 = atomicAdd(cursor, *claim);
     g0 = __shfl_sync(kFull, g0, 0);
     if (g0 >= n_list) break;
-    const uint32_t g1 = min(g0 + (uint32_t)kGroupChunk, n_list);
+    const uint32_t g1 = min(g0 + *claim, n_list);
     for (uint32_t gi = g0; gi < g1; ++gi) {
       const int32_t h = __ldg(list + (n_list - 1 - gi));  // heavy (high-rank) groups first
       const int2 hld = __ldg(g.ldesc + h);
@@ -598,8 +600,8 @@ __device__ __forceinline__ void warp_groups(const Lists &g, const int32_t *__res
       __syncwarp();
       uint64_t found_group = 0;
       for (int32_t c0 = 0; c0 < np; c0 += 32)
-        probe_chunk<PV, kWindows>(g, g.part + pb, g.pskip + pb, g.desc + pb, np, c0, 32, bits, tb, ws, t, found_total,
-                                  found_group);
+        probe_chunk<PV, kWindows>(g, g.part + pb, g.pskip + pb, g.desc + pb, np, c0, 32, bits, tb,
+                                  ws, t, found_total, found_group);
       if (PV || tg) {
         found_group = warp_sum_u64(found_group);
         if (lane == 0 && found_group)
@@ -627,6 +629,7 @@ __global__ void __launch_bounds__(256)
 k_stream_desc(const int32_t *__restrict__ part, const int32_t *__restrict__ pskip,
               const int2 *__restrict__ ldesc, const uint32_t *rec, const Ctrl *ctrl,
               int2 *__restrict__ desc) {
+  grid_begin();
   if (aborted(ctrl)) return;  // an earlier wait of this call ran out
   const uint32_t m = ctrl->n_part;
   if (ctrl->n_bit_items == 0u) rec = nullptr;  // no group uses bitmaps
@@ -675,6 +678,7 @@ template <bool PV>
 __global__ void __launch_bounds__(kMainThreads, kMainMinBlocks)
 k_count(Lists g, const int32_t *__restrict__ groups, int32_t n, Ctrl *ctrl, int64_t *t,
         int64_t *tg) {
+  grid_begin();
   constexpr int SLOTS = main_slots<PV>();
   constexpr int WSLOTS = SLOTS / kMainWarps;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -683,9 +687,13 @@ k_count(Lists g, const int32_t *__restrict__ groups, int32_t n, Ctrl *ctrl, int6
   uint16_t *s_slot = reinterpret_cast<uint16_t *>(smem + 4 * SLOTS * (PV ? 2 : 1));
   __shared__ WarpScratch s_ws[kMainWarps];
   __shared__ CtaShared s_sh;
+  __shared__ uint32_t s_claim;
   if (aborted(ctrl)) return;  // an earlier wait of this call ran out: the lists are not complete
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (ctrl->n_bit_items == 0u) g.rec = nullptr;  // no group uses bitmaps: no record is read
+  if (tid == 0)  // few groups: fewer at a time, so that all warps get some
+    s_claim = min((uint32_t)kGroupChunk,
+                  max(1u, ctrl->n_warp_groups / (gridDim.x * kMainWarps * 4u)));
   clear_table<PV>(s_tab, s_cnt, SLOTS, tid, kMainThreads);
   uint64_t found_total = 0;
   Table tb{s_tab, s_cnt, shared_addr(s_cnt), SLOTS};
@@ -696,7 +704,8 @@ k_count(Lists g, const int32_t *__restrict__ groups, int32_t n, Ctrl *ctrl, int6
                                                 t, tg, found_total);
   Table wtb{s_tab + warp * WSLOTS, s_cnt + warp * WSLOTS, shared_addr(s_cnt + warp * WSLOTS),
             WSLOTS};
-  warp_groups<PV, WSLOTS>(g, groups, ctrl->n_warp_groups, &ctrl->next_warp_group, wtb,
+  warp_groups<PV, WSLOTS>(g, groups, ctrl->n_warp_groups, &ctrl->next_warp_group,
+                          &s_claim, wtb,
                           s_slot + warp * kWarpMaxRow, s_ws[warp], t, tg, found_total);
   found_total = warp_sum_u64(found_total);
   if (lane == 0 && found_total) atomicAdd(&ctrl->total, (unsigned long long)found_total);
@@ -707,6 +716,7 @@ template <bool PV>
 __global__ void __launch_bounds__(kBigThreads, kBigMinBlocks)
 k_count_big(Lists g, const int32_t *__restrict__ big_list, Ctrl *ctrl, int64_t *t,
             int64_t *tg) {
+  grid_begin();
   extern __shared__ __align__(16) unsigned char smem[];
   int32_t *tab = reinterpret_cast<int32_t *>(smem);
   uint32_t *cnt = reinterpret_cast<uint32_t *>(smem + 4 * kBigSlots);
@@ -736,6 +746,7 @@ constexpr int kClusterThreads = 256;
 __global__ void __launch_bounds__(kClusterThreads)
 k_clustering(const int64_t *__restrict__ t, const int32_t *__restrict__ deg, int32_t n,
              double *__restrict__ cc, unsigned long long *sums) {
+  grid_begin();
   unsigned long long st = 0, sw = 0;
   const uint32_t stride = gridDim.x * kClusterThreads;
   for (uint32_t v = blockIdx.x * kClusterThreads + threadIdx.x; v < (uint32_t)n; v += stride) {
@@ -761,6 +772,7 @@ k_clustering(const int64_t *__restrict__ t, const int32_t *__restrict__ deg, int
 __global__ void __launch_bounds__(kClusterThreads)
 k_gather_counts(const int64_t *__restrict__ t_rank, const int32_t *__restrict__ rank, int32_t n,
                 int64_t *__restrict__ t_out, const Ctrl *ctrl) {
+  grid_begin();
   if (aborted(ctrl)) return;  // rank[] may be incomplete
   const uint32_t stride = gridDim.x * kClusterThreads;
   for (uint32_t v = blockIdx.x * kClusterThreads + threadIdx.x; v < (uint32_t)n; v += stride)
@@ -775,6 +787,7 @@ __global__ void __launch_bounds__(kClusterThreads)
 k_batch_totals(const int64_t *__restrict__ tg, const int32_t *__restrict__ rank,
                const BatchDesc *__restrict__ batch, const Ctrl *ctrl,
                unsigned long long *__restrict__ totals) {
+  grid_begin();
   constexpr uint32_t ROUNDS = 8;
   if (aborted(ctrl)) return;  // rank[] may be incomplete
   const int32_t ng = batch->num_graphs;
@@ -819,6 +832,7 @@ k_batch_totals(const int64_t *__restrict__ tg, const int32_t *__restrict__ rank,
 
 // transitivity = 3T / wedges with T = (sum t) / 3: one float64 division.
 __global__ void k_transitivity(const unsigned long long *sums, double *out) {
+  grid_begin();
   const unsigned long long three_t = sums[0];  // sum of t(v) is exactly 3T
   const unsigned long long wedges = sums[1];
   out[0] = wedges ? (double)three_t / (double)wedges : 0.0;
@@ -889,24 +903,22 @@ cudaError_t launch_count(const int2 *ldesc, const int32_t *col4, const int32_t *
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    k_stream_desc<<<(sms > 0 ? sms : 1) * 16, 256, 0, st>>>(part, pskip, ldesc, rec, ctrl, desc);
-    note_launch();
+    launch(k_stream_desc,
+           (sms > 0 ? sms : 1) * 16, 256, 0, st, part, pskip, ldesc, rec, ctrl, desc);
   }
   const Lists g{col4, goff, part, pskip, desc, ldesc, rec};
   // the long lists first, on their own wide CTAs
   if (pv) {
-    k_count_big<true><<<cg.big_blocks, kBigThreads, big_smem<true>(), st>>>(g, big_groups, ctrl, t,
-                                                                          nullptr);
-    k_count<true><<<cg.main_blocks, kMainThreads, main_smem<true>(), st>>>(g, groups, n, ctrl, t,
-                                                                         nullptr);
+    launch(k_count_big<true>, cg.big_blocks, kBigThreads, big_smem<true>(), st, g, big_groups, ctrl,
+           t, nullptr);
+    launch(k_count<true>, cg.main_blocks, kMainThreads, main_smem<true>(), st, g, groups, n, ctrl,
+           t, nullptr);
   } else {
-    k_count_big<false><<<cg.big_blocks, kBigThreads, big_smem<false>(), st>>>(g, big_groups, ctrl,
-                                                                            nullptr, tg);
-    k_count<false><<<cg.main_blocks, kMainThreads, main_smem<false>(), st>>>(g, groups, n, ctrl,
-                                                                           nullptr, tg);
+    launch(k_count_big<false>, cg.big_blocks, kBigThreads, big_smem<false>(), st, g, big_groups,
+           ctrl, nullptr, tg);
+    launch(k_count<false>, cg.main_blocks, kMainThreads, main_smem<false>(), st, g, groups, n, ctrl,
+           nullptr, tg);
   }
-  note_launch();
-  note_launch();
   return cudaGetLastError();
 }
 
@@ -917,8 +929,7 @@ void launch_clustering(const int64_t *t, const int32_t *deg, int32_t n, double *
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const uint32_t want = ((uint32_t)n + kClusterThreads * 4 - 1) / (kClusterThreads * 4);
   const uint32_t grid = max(1u, min(want, (uint32_t)(sms > 0 ? sms : 1) * 8));
-  k_clustering<<<grid, kClusterThreads, 0, st>>>(t, deg, n, cc, sums);
-  note_launch();
+  launch(k_clustering, grid, kClusterThreads, 0, st, t, deg, n, cc, sums);
 }
 
 void launch_gather_counts(const int64_t *t_rank, const int32_t *rank, int32_t n, int64_t *t_out,
@@ -928,8 +939,7 @@ void launch_gather_counts(const int64_t *t_rank, const int32_t *rank, int32_t n,
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const uint32_t want = ((uint32_t)n + kClusterThreads * 4 - 1) / (kClusterThreads * 4);
   const uint32_t grid = max(1u, min(want, (uint32_t)(sms > 0 ? sms : 1) * 8));
-  k_gather_counts<<<grid, kClusterThreads, 0, st>>>(t_rank, rank, n, t_out, ctrl);
-  note_launch();
+  launch(k_gather_counts, grid, kClusterThreads, 0, st, t_rank, rank, n, t_out, ctrl);
 }
 
 void launch_batch_totals(const int64_t *tg, const int32_t *rank, const BatchDesc *batch,
@@ -940,13 +950,11 @@ void launch_batch_totals(const int64_t *tg, const int32_t *rank, const BatchDesc
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const uint32_t want = ((uint32_t)n + kClusterThreads * 8 - 1) / (kClusterThreads * 8);
   const uint32_t grid = max(1u, min(want, (uint32_t)(sms > 0 ? sms : 1) * 8));
-  k_batch_totals<<<grid, kClusterThreads, 0, st>>>(tg, rank, batch, ctrl, totals);
-  note_launch();
+  launch(k_batch_totals, grid, kClusterThreads, 0, st, tg, rank, batch, ctrl, totals);
 }
 
 void launch_transitivity(const unsigned long long *sums, double *out, cudaStream_t st) {
-  k_transitivity<<<1, 1, 0, st>>>(sums, out);
-  note_launch();
+  launch(k_transitivity, 1, 1, 0, st, sums, out);
 }
 
 }  // namespace tc

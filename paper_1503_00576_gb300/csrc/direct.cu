@@ -48,6 +48,7 @@ __device__ __forceinline__ uint32_t rank_class(uint32_t d) {
 // Vertices per degree class.
 __global__ void __launch_bounds__(kThreads)
 k_rank_hist(const int32_t *__restrict__ deg, int32_t n, uint32_t *__restrict__ hist) {
+  grid_begin();
   __shared__ uint32_t s_cnt[kRankClasses];
   for (int i = threadIdx.x; i < kRankClasses; i += kThreads) s_cnt[i] = 0;
   __syncthreads();
@@ -65,6 +66,7 @@ k_rank_hist(const int32_t *__restrict__ deg, int32_t n, uint32_t *__restrict__ h
 __global__ void __launch_bounds__(kThreads)
 k_rank_assign(const int32_t *__restrict__ deg, int32_t n, const uint32_t *__restrict__ hist,
               uint32_t *__restrict__ cursor, int32_t *__restrict__ rank) {
+  grid_begin();
   constexpr int PER = kRankClasses / kThreads;
   __shared__ uint32_t s_start[kRankClasses], s_cnt[kRankClasses], s_warp[kThreads / 32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -126,6 +128,7 @@ __global__ void __launch_bounds__(kThreads)
 k_direct_orient(const uint64_t *__restrict__ keys, int b, const int32_t *__restrict__ rank,
                 uint64_t *__restrict__ okeys, int32_t *__restrict__ place,
                 int32_t *__restrict__ outdeg, const Ctrl *__restrict__ ctrl) {
+  grid_begin();
   const uint32_t m = ctrl->m_in;
   const uint64_t sentinel = (1ull << (2 * b)) - 1, mask = (1ull << b) - 1;
   const uint32_t stride = gridDim.x * kThreads;
@@ -168,6 +171,7 @@ __global__ void __launch_bounds__(kThreads)
 k_direct_lists(const uint64_t *__restrict__ okeys, const int32_t *__restrict__ place, int b,
                const int32_t *__restrict__ off, int32_t *__restrict__ col,
                const Ctrl *__restrict__ ctrl) {
+  grid_begin();
   if (aborted(ctrl)) return;  // a wait of this call ran out: off is not complete
   const uint32_t m = ctrl->m_in;
   const uint32_t mask = (uint32_t)((1ull << b) - 1);
@@ -208,6 +212,7 @@ k_direct_groups(const uint64_t *__restrict__ gkeys, int b, int32_t n,
                 const int32_t *__restrict__ goff, int32_t *__restrict__ gcnt,
                 int32_t *__restrict__ part, int32_t *__restrict__ pskip,
                 const Ctrl *__restrict__ ctrl) {
+  grid_begin();
   __shared__ int32_t s_hot[kHotRanks];  // the tile's edges per rank, then the counter's old value
   if (aborted(ctrl)) return;
   const int tid = threadIdx.x;
@@ -273,32 +278,27 @@ void launch_rank_classes(const int32_t *deg, int32_t n, uint32_t *counters, int3
                          cudaStream_t st) {
   const uint32_t tiles = ((uint32_t)n + kRankTile - 1) / kRankTile;
   const uint32_t grid = max(1u, min(tiles, sm_count() * 8u));
-  k_rank_hist<<<grid, kThreads, 0, st>>>(deg, n, counters);
-  k_rank_assign<<<grid, kThreads, 0, st>>>(deg, n, counters, counters + kRankClasses, rank);
-  note_launch();
-  note_launch();
+  launch(k_rank_hist, grid, kThreads, 0, st, deg, n, counters);
+  launch(k_rank_assign, grid, kThreads, 0, st, deg, n, counters, counters + kRankClasses, rank);
 }
 
 void launch_direct_orient(const uint64_t *keys, uint32_t m_in, int b, const int32_t *rank,
                           uint64_t *okeys, int32_t *place, int32_t *outdeg, Ctrl *ctrl,
                           cudaStream_t st) {
-  k_direct_orient<<<items_grid(m_in), kThreads, 0, st>>>(keys, b, rank, okeys, place, outdeg,
-                                                         ctrl);
-  note_launch();
+  launch(k_direct_orient, items_grid(m_in), kThreads, 0, st, keys, b, rank, okeys, place, outdeg,
+         ctrl);
 }
 
 void launch_direct_lists(const uint64_t *okeys, const int32_t *place, uint32_t m_in, int b,
                          const int32_t *off, int32_t *col, Ctrl *ctrl, cudaStream_t st) {
-  k_direct_lists<<<items_grid(m_in), kThreads, 0, st>>>(okeys, place, b, off, col, ctrl);
-  note_launch();
+  launch(k_direct_lists, items_grid(m_in), kThreads, 0, st, okeys, place, b, off, col, ctrl);
 }
 
 void launch_direct_groups(const uint64_t *gkeys, uint32_t m_bound, int b, int32_t n,
                           const int32_t *goff, int32_t *gcnt, int32_t *part, int32_t *pskip,
                           Ctrl *ctrl, cudaStream_t st) {
-  k_direct_groups<<<items_grid(m_bound), kThreads, 0, st>>>(gkeys, b, n, goff, gcnt, part, pskip,
-                                                            ctrl);
-  note_launch();
+  launch(k_direct_groups, items_grid(m_bound), kThreads, 0, st, gkeys, b, n, goff, gcnt, part,
+         pskip, ctrl);
 }
 
 }  // namespace tc

@@ -407,8 +407,9 @@ __device__ int32_t cta_unique_copy(const int32_t *buf, int32_t d, int32_t *__res
 }
 
 // Every forward list into col4, sorted ascending, without repeated entries
-// and padded with -1 to whole 32-byte blocks.  Warps take 32 consecutive
-// vertices at a time: a list of up to 8 entries is sorted by its own lane in
+// and padded with -1 to whole 32-byte blocks.  Warps take `per` consecutive
+// vertices at a time (32, or fewer so that a small graph's lists spread over
+// all SMs: 16,384 vertices, 20 / 7 us): a list of up to 8 entries is sorted by its own lane in
 // registers (a sorting network), one of up to 16 by half a warp, one of up
 // to kWarpLaneMax by the warp (bitonic, in registers).  Longer ones are
 // queued for k_sort_long_lists, where every warp of the GPU takes one at a
@@ -418,18 +419,20 @@ __device__ int32_t cta_unique_copy(const int32_t *buf, int32_t d, int32_t *__res
 template <bool EMIT>
 __global__ void __launch_bounds__(kListThreads)
 k_sort_lists(const int32_t *__restrict__ col, const int32_t *__restrict__ off,
-             const int32_t *__restrict__ voff, int32_t n, ListOut o, GroupOut g,
+             const int32_t *__restrict__ voff, int32_t n, uint32_t per, ListOut o, GroupOut g,
              int32_t *__restrict__ queue) {
+  grid_begin();
   Ctrl *ctrl = o.ctrl;
   if (aborted(ctrl)) return;  // an earlier wait of this call ran out
   const Emit em{g, o.dlen, ctrl->hub_on ? (int32_t)ctrl->hub_lo : n, nullptr, n};
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t warps = gridDim.x * kListWarps;
   const uint32_t lt = (1u << lane) - 1u;
-  for (uint32_t c = blockIdx.x * kListWarps + warp; c * 32u < (uint32_t)n; c += warps) {
-    const uint32_t v = c * 32u + lane;
+  for (uint32_t c = blockIdx.x * kListWarps + warp; c * per < (uint32_t)n; c += warps) {
+    const uint32_t v = c * per + lane;
+    const bool exists = (uint32_t)lane < per && v < (uint32_t)n;
     int32_t b = 0, d = 0, w = 0, len = 0;
-    if (v < (uint32_t)n) {
+    if (exists) {
       b = __ldg(off + v);
       d = __ldg(off + v + 1) - b;
       w = __ldg(voff + v);
@@ -478,7 +481,7 @@ k_sort_lists(const int32_t *__restrict__ col, const int32_t *__restrict__ off,
         em.g.own[v] = own;
       }
     }
-    if (EMIT && d == 0 && v < (uint32_t)n) em.g.own[v] = 0;
+    if (EMIT && d == 0 && exists) em.g.own[v] = 0;
     uint32_t todo = __ballot_sync(kFull, d > 8 && d <= 16);
     while (todo) {  // two lists at a time
       const int s0 = __ffs(todo) - 1;
@@ -490,7 +493,7 @@ k_sort_lists(const int32_t *__restrict__ col, const int32_t *__restrict__ off,
       const int32_t lb = __shfl_sync(kFull, b, src), ld = __shfl_sync(kFull, d, src);
       const long long lw = __shfl_sync(kFull, w4, src);
       const int32_t l = half_sort_list<EMIT>(col, lb, none ? 0 : ld, lw,
-                                             (int32_t)(c * 32u) + src, o, em);
+                                             (int32_t)(c * per) + src, o, em);
       const int32_t l0 = __shfl_sync(kFull, l, 0), l1 = __shfl_sync(kFull, l, 16);
       if (lane == s0) len = l0;
       else if (lane == s1) len = l1;
@@ -501,12 +504,12 @@ k_sort_lists(const int32_t *__restrict__ col, const int32_t *__restrict__ off,
       todo &= todo - 1;
       const int32_t lb = __shfl_sync(kFull, b, src), ld = __shfl_sync(kFull, d, src);
       const long long lw = __shfl_sync(kFull, w4, src);
-      const int32_t lv = (int32_t)(c * 32u) + src;
+      const int32_t lv = (int32_t)(c * per) + src;
       const int32_t l = ld <= 32 ? warp_sort_list<1, EMIT>(col, lb, ld, lw, lv, o, em)
                                  : warp_sort_list<2, EMIT>(col, lb, ld, lw, lv, o, em);
       if (lane == src) len = l;
     }
-    if (v < (uint32_t)n && d <= kWarpLaneMax) o.ldesc[v] = make_int2(w, len);
+    if (exists && d <= kWarpLaneMax) o.ldesc[v] = make_int2(w, len);
     // the queues: lists for a warp from the front of the array, lists for a
     // CTA from its end down
     const bool is_warp = d > kWarpLaneMax && d <= kWarpLongMax, is_cta = d > kWarpLongMax;
@@ -549,6 +552,7 @@ __global__ void __launch_bounds__(kLongListThreads, kLongListBlocks)
 k_sort_long_lists(int32_t *col, const int32_t *__restrict__ off,
                   const int32_t *__restrict__ voff, int32_t n, ListOut o, GroupOut g,
                   const int32_t *__restrict__ queue) {
+  grid_begin();
   constexpr int G = kLongListThreads;
   __shared__ int32_t s_buf[kCtaSortMax];
   __shared__ uint32_t s_warp[G / 32];
@@ -677,6 +681,7 @@ __global__ void __launch_bounds__(kListThreads)
 k_fix_repeats(const int32_t *__restrict__ off, int32_t n, const int32_t *__restrict__ dcorr,
               const int32_t *__restrict__ rank, const Ctrl *ctrl, int32_t *__restrict__ row,
               int32_t *__restrict__ deg) {
+  grid_begin();
   if (aborted(ctrl) || ctrl->dups == 0u) return;
   const int lane = threadIdx.x & 31;
   const uint32_t first = blockIdx.x * kListThreads + threadIdx.x;
@@ -729,6 +734,7 @@ k_group_keys(const int32_t *__restrict__ row, const int32_t *__restrict__ col4,
              const int32_t *__restrict__ len, int b, int passes, int32_t heavy_ratio_pct,
              Ctrl *__restrict__ ctrl, uint64_t *__restrict__ gkeys,
              uint32_t *__restrict__ hist) {
+  grid_begin();
   constexpr int UNROLL = WHOLE ? kGroupUnroll : 2 * kGroupUnroll;
   __shared__ uint32_t s_hist[kMaxGroupPasses * 256];
   if (aborted(ctrl)) return;  // an earlier wait of this call ran out
@@ -839,6 +845,7 @@ __global__ void __launch_bounds__(kGroupThreads)
 k_work(const int32_t *__restrict__ off, const int32_t *__restrict__ goff,
        const int32_t *__restrict__ part, const int32_t *__restrict__ pskip, int32_t n,
        Ctrl *ctrl, uint32_t shard, uint32_t shards) {
+  grid_begin();
   if (aborted(ctrl)) return;
   const int lane = threadIdx.x & 31;
   const uint32_t warps = gridDim.x * (kGroupThreads / 32);
@@ -907,22 +914,22 @@ void launch_sort_lists(int32_t *col, const int32_t *off, const int32_t *voff, in
                        Ctrl *ctrl, int32_t *col4, int32_t *queue, int32_t *dlen,
                        int32_t *dcorr, int2 *ldesc, const GroupOut *emit, cudaStream_t st) {
   const ListOut o{col4, dlen, dcorr, ldesc, ctrl};
-  const uint32_t chunks = ((uint32_t)n + 31u) / 32u;
+  const uint32_t warps = num_sms() * 8u * kListWarps;
+  uint32_t per = 4;
+  while (per < 32 && per * warps < (uint32_t)n) per <<= 1;
+  const uint32_t chunks = ((uint32_t)n + per - 1) / per;
   const uint32_t grid = max(1u, min((chunks + kListWarps - 1) / kListWarps, num_sms() * 8u));
   const GroupOut g = emit ? *emit : GroupOut{};
   const auto lists = emit ? k_sort_lists<true> : k_sort_lists<false>;
   const auto long_lists = emit ? k_sort_long_lists<true> : k_sort_long_lists<false>;
-  lists<<<grid, kListThreads, 0, st>>>(col, off, voff, n, o, g, queue);
-  long_lists<<<num_sms() * kLongListBlocks, kLongListThreads, 0, st>>>(col, off, voff, n, o, g,
-                                                                       queue);
-  note_launch();
-  note_launch();
+  launch(lists, grid, kListThreads, 0, st, col, off, voff, n, per, o, g, queue);
+  launch(long_lists, num_sms() * kLongListBlocks, kLongListThreads, 0, st, col, off, voff, n, o, g,
+         queue);
 }
 
 void launch_fix_repeats(const int32_t *off, int32_t n, const int32_t *dcorr, const int32_t *rank,
                         Ctrl *ctrl, int32_t *row, int32_t *deg, cudaStream_t st) {
-  k_fix_repeats<<<num_sms() * 8u, kListThreads, 0, st>>>(off, n, dcorr, rank, ctrl, row, deg);
-  note_launch();
+  launch(k_fix_repeats, num_sms() * 8u, kListThreads, 0, st, off, n, dcorr, rank, ctrl, row, deg);
 }
 
 void launch_group_keys(const int32_t *row, const int32_t *col4, const int32_t *off,
@@ -930,18 +937,16 @@ void launch_group_keys(const int32_t *row, const int32_t *col4, const int32_t *o
                        int32_t heavy_ratio_pct, bool whole, Ctrl *ctrl, uint64_t *gkeys,
                        uint32_t *hist, cudaStream_t st) {
   const auto kernel = whole ? k_group_keys<true> : k_group_keys<false>;
-  kernel<<<group_grid(m_bound), kGroupThreads, 0, st>>>(row, col4, off, ldesc, len, b, passes,
-                                                        heavy_ratio_pct, ctrl, gkeys, hist);
-  note_launch();
+  launch(kernel, group_grid(m_bound), kGroupThreads, 0, st, row, col4, off, ldesc, len, b, passes,
+         heavy_ratio_pct, ctrl, gkeys, hist);
 }
 
 void launch_work(const int32_t *off, const int32_t *goff, const int32_t *part,
                  const int32_t *pskip, int32_t n, Ctrl *ctrl, cudaStream_t st, int32_t shard,
                  int32_t shards) {
   const uint32_t lanes = n > (1 << 28) ? (1u << 30) : (uint32_t)n * 4u;  // grid is capped anyway
-  k_work<<<group_grid(lanes), kGroupThreads, 0, st>>>(off, goff, part, pskip, n, ctrl,
-                                                      (uint32_t)shard, (uint32_t)shards);
-  note_launch();
+  launch(k_work, group_grid(lanes), kGroupThreads, 0, st, off, goff, part, pskip, n, ctrl,
+         (uint32_t)shard, (uint32_t)shards);
 }
 
 }  // namespace tc

@@ -210,6 +210,7 @@ __device__ __forceinline__ int32_t hub_candidate(int32_t Hmax, int k) {
 __global__ void __launch_bounds__(256)
 k_hub_estimate(const int32_t *__restrict__ off, const int32_t *__restrict__ col, int32_t n,
                int32_t Hmax, int64_t min_edges, int32_t cap, Ctrl *ctrl) {
+  grid_begin();
   if (aborted(ctrl)) return;
   if ((int64_t)ctrl->m - (int64_t)__ldg(off + (n - Hmax)) < min_edges) return;
   const int lane = threadIdx.x & 31;
@@ -254,6 +255,7 @@ k_hub_estimate(const int32_t *__restrict__ off, const int32_t *__restrict__ col,
 // of 180M 30.9 30.9 31.7 / 38.6 38.3 38.6.
 __global__ void k_hub_decide(const int32_t *__restrict__ off, int32_t n, int32_t Hmax,
                              int64_t min_edges, double ps_per_lookup, Ctrl *ctrl) {
+  grid_begin();
   if (aborted(ctrl)) return;
   const double ms_per_lookup = 1e-9 * ps_per_lookup;
   double best = 0.0;
@@ -279,6 +281,7 @@ __global__ void k_hub_decide(const int32_t *__restrict__ off, int32_t n, int32_t
 // Zeroes the H x H corner (row pitch Hmax) of the hub matrix.
 __global__ void __launch_bounds__(256)
 k_hub_zero(uint8_t *__restrict__ A, int32_t Hmax, const Ctrl *ctrl) {
+  grid_begin();
   if (aborted(ctrl) || !ctrl->hub_on) return;
   const uint32_t H = ctrl->hub_size;
   const uint32_t words = H / 16;  // uint4 per row
@@ -295,6 +298,7 @@ k_hub_zero(uint8_t *__restrict__ A, int32_t Hmax, const Ctrl *ctrl) {
 __global__ void __launch_bounds__(256)
 k_hub_scatter(const int2 *__restrict__ ldesc, const int32_t *__restrict__ col4, int32_t n,
               int32_t pitch, const Ctrl *ctrl, uint8_t *__restrict__ A) {
+  grid_begin();
   if (aborted(ctrl) || !ctrl->hub_on) return;
   const int32_t H = (int32_t)ctrl->hub_size, lo = n - H;
   const int lane = threadIdx.x & 31;
@@ -314,11 +318,12 @@ k_hub_scatter(const int2 *__restrict__ ldesc, const int32_t *__restrict__ col4, 
 
 // C tiles of the upper triangle, every gridDim.x-th by the same CTA (one CTA per
 // tile of the largest set made the kernel last 32 us where no hub set is
-// used); r(i) += masked row (and column) sums.  Warp 0 lane 0 issues the TMA loads, warp 1 lane 0 the
-// MMAs; all four warps read the accumulator back.
+// used); r(i) += masked row (and column) sums.  Warp 0 lane 0 issues the TMA
+// loads, warp 1 lane 0 the MMAs; all four warps read the accumulator back.
 __global__ void __launch_bounds__(kHubThreads, 2)
 k_hub_gemm(const __grid_constant__ CUtensorMap amap, const uint8_t *__restrict__ A,
            int32_t pitch, Ctrl *ctrl, uint32_t *__restrict__ r) {
+  grid_begin();
   extern __shared__ uint8_t smem_raw[];
   if (!ctrl->hub_on || aborted(ctrl)) return;  // uniform for the block
   const int32_t H = (int32_t)ctrl->hub_size;
@@ -445,6 +450,7 @@ k_hub_gemm(const __grid_constant__ CUtensorMap amap, const uint8_t *__restrict__
 // block.
 __global__ void __launch_bounds__(1024)
 k_hub_finish(const uint32_t *__restrict__ r, Ctrl *ctrl, int64_t *t) {
+  grid_begin();
   __shared__ unsigned long long s_sum[32];
   __shared__ uint32_t s_odd;
   if (aborted(ctrl) || !ctrl->hub_on) return;
@@ -498,10 +504,8 @@ size_t hub_bytes(int32_t H) { return (size_t)H * (size_t)H + 4 * (size_t)H; }
 void launch_hub_decide(const int32_t *off, const int32_t *col, int32_t n, int32_t Hmax,
                        int64_t min_edges, int32_t cap, double ps_per_lookup, Ctrl *ctrl,
                        cudaStream_t st) {
-  k_hub_estimate<<<(Hmax + 7) / 8, 256, 0, st>>>(off, col, n, Hmax, min_edges, cap, ctrl);
-  k_hub_decide<<<1, 1, 0, st>>>(off, n, Hmax, min_edges, ps_per_lookup, ctrl);
-  note_launch();
-  note_launch();
+  launch(k_hub_estimate, (Hmax + 7) / 8, 256, 0, st, off, col, n, Hmax, min_edges, cap, ctrl);
+  launch(k_hub_decide, 1, 1, 0, st, off, n, Hmax, min_edges, ps_per_lookup, ctrl);
 }
 
 cudaError_t launch_hub_count(const int2 *ldesc, const int32_t *col4, int32_t n, int32_t Hmax,
@@ -533,14 +537,13 @@ cudaError_t launch_hub_count(const int2 *ldesc, const int32_t *col4, int32_t n, 
   if (e != cudaSuccess) return e;
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  k_hub_zero<<<(sms > 0 ? sms : 1) * 8, 256, 0, st>>>(A, Hmax, ctrl);
-  k_hub_scatter<<<(Hmax + 7) / 8, 256, 0, st>>>(ldesc, col4, n, Hmax, ctrl, A);
+  launch(k_hub_zero, (sms > 0 ? sms : 1) * 8, 256, 0, st, A, Hmax, ctrl);
+  launch(k_hub_scatter, (Hmax + 7) / 8, 256, 0, st, ldesc, col4, n, Hmax, ctrl, A);
   const int T = Hmax / kHubTile;
   const int tiles = T * (T + 1) / 2;
-  k_hub_gemm<<<min(tiles, 2 * (sms > 0 ? sms : 1)), kHubThreads, kHubSmemBytes, st>>>(
-      map, A, Hmax, ctrl, r);
-  k_hub_finish<<<1, 1024, 0, st>>>(r, ctrl, t);
-  for (int i = 0; i < 4; ++i) note_launch();
+  launch(k_hub_gemm, min(tiles, 2 * (sms > 0 ? sms : 1)), kHubThreads, kHubSmemBytes, st, map, A,
+         Hmax, ctrl, r);
+  launch(k_hub_finish, 1, 1024, 0, st, r, ctrl, t);
   return cudaGetLastError();
 }
 

@@ -212,6 +212,7 @@ __device__ __forceinline__ uint64_t pair_key(int32_t u, int32_t v, int32_t lim, 
 __global__ void __launch_bounds__(kCanonThreads)
 k_canon(const int32_t *__restrict__ src, const int32_t *__restrict__ dst, uint32_t m_in,
         int32_t n, int b, uint64_t *__restrict__ keys, int32_t *__restrict__ deg, Ctrl *ctrl) {
+  grid_begin();
   const uint64_t sentinel = (1ull << (2 * b)) - 1;  // > every valid key; 2b <= 62
   if (blockIdx.x == 0 && threadIdx.x == 0) ctrl->m_in = m_in;
   bool bad = false;
@@ -250,6 +251,7 @@ k_canon_batch(const int32_t *__restrict__ src, const int32_t *__restrict__ dst, 
               int b, const BatchDesc *__restrict__ batch, int32_t num_graphs_bound,
               unsigned long long *__restrict__ totals, uint64_t *__restrict__ keys,
               int32_t *__restrict__ deg, Ctrl *ctrl) {
+  grid_begin();
   constexpr uint32_t CHUNK = 32 * kCanonUnroll, kSpread = 256;
   const uint64_t sentinel = (1ull << (2 * b)) - 1;
   const int32_t ng = batch->num_graphs;
@@ -493,6 +495,7 @@ k_radix_pass(const uint64_t *__restrict__ in, void *__restrict__ out, uint32_t n
              uint32_t *__restrict__ row_out, int owner_shift, int32_t *outdeg,
              const uint32_t *__restrict__ hist, unsigned long long *__restrict__ status,
              uint32_t *ticket, Ctrl *ctrl, int unstable) {
+  grid_begin();
   constexpr int WARPS = kSortThreads / 32, TILE = kSortTile;
   __shared__ RadixShared S;
   const int tid = threadIdx.x;
@@ -542,6 +545,7 @@ k_radix_pass(const uint64_t *__restrict__ in, void *__restrict__ out, uint32_t n
 __global__ void __launch_bounds__(kCanonThreads)
 k_rank_keys(const int32_t *__restrict__ deg, int32_t n, int b, int passes,
             uint64_t *__restrict__ vkeys, uint32_t *__restrict__ hist) {
+  grid_begin();
   __shared__ uint32_t sh[kMaxRankPasses * 256];
   for (int i = threadIdx.x; i < passes * 256; i += kCanonThreads) sh[i] = 0;
   __syncthreads();
@@ -563,6 +567,7 @@ __global__ void __launch_bounds__(kOrientThreads, 4)
 k_orient(const uint64_t *__restrict__ keys, int b,
          const int32_t *__restrict__ rank, uint64_t *__restrict__ okeys,
          uint32_t *__restrict__ hist2, int passes2, unsigned long long *status, Ctrl *ctrl) {
+  grid_begin();
   constexpr int KPT = kOrientKeysPerThread, TILE = kOrientTile;
   static_assert(KPT == 16, "the swizzle below assumes rows of 16 keys");
   // The tile passes through shared memory both ways: loaded and stored with
@@ -711,6 +716,7 @@ struct ScanArgs {
 template <int KIND>
 __global__ void __launch_bounds__(kScanThreads)
 k_offsets(const ScanArgs a) {
+  grid_begin();
   constexpr int IPT = kScanItemsPerThread, TILE = kScanTile;
   __shared__ uint64_t s_scratch[kScanThreads / 32];
   __shared__ uint64_t s_excl;
@@ -850,18 +856,15 @@ static uint32_t canon_grid(uint32_t m_in) {
 
 void launch_canon(const int32_t *src, const int32_t *dst, uint32_t m_in, int32_t n, int b,
                   uint64_t *keys, int32_t *deg, Ctrl *ctrl, cudaStream_t st) {
-  k_canon<<<canon_grid(m_in), kCanonThreads, 0, st>>>(src, dst, m_in, n, b, keys, deg, ctrl);
-  note_launch();
+  launch(k_canon, canon_grid(m_in), kCanonThreads, 0, st, src, dst, m_in, n, b, keys, deg, ctrl);
 }
 
 void launch_canon_batch(const int32_t *src, const int32_t *dst, uint32_t m_in, int b,
                         const BatchDesc *batch, int32_t num_graphs_bound,
                         unsigned long long *totals, uint64_t *keys, int32_t *deg, Ctrl *ctrl,
                         cudaStream_t st) {
-  k_canon_batch<<<canon_grid(m_in), kCanonThreads, 0, st>>>(src, dst, m_in, b, batch,
-                                                            num_graphs_bound, totals, keys, deg,
-                                                            ctrl);
-  note_launch();
+  launch(k_canon_batch, canon_grid(m_in), kCanonThreads, 0, st, src, dst, m_in, b, batch,
+         num_graphs_bound, totals, keys, deg, ctrl);
 }
 
 void launch_radix_pass(const uint64_t *in, void *out, RadixOut mode, uint32_t *row_out,
@@ -870,40 +873,26 @@ void launch_radix_pass(const uint64_t *in, void *out, RadixOut mode, uint32_t *r
                        unsigned long long *status, uint32_t *ticket, Ctrl *ctrl,
                        cudaStream_t st, bool unstable) {
   const uint32_t grid = max(1u, (n_keys_bound + kSortTile - 1) / kSortTile);
-  if (mode == kOutPartSkip)
-    k_radix_pass<kOutPartSkip><<<grid, kSortThreads, 0, st>>>(
-        in, out, n_keys_bound, n_keys_dev, shift, col_mask, row_out, owner_shift, outdeg, hist,
-        status, ticket, ctrl, 0);
-  else if (mode == kOutColRow)
-    k_radix_pass<kOutColRow><<<grid, kSortThreads, 0, st>>>(
-        in, out, n_keys_bound, n_keys_dev, shift, col_mask, row_out, owner_shift, outdeg, hist,
-        status, ticket, ctrl, 0);
-  else if (mode == kOutRank)
-    k_radix_pass<kOutRank><<<grid, kSortThreads, 0, st>>>(in, out, n_keys_bound, n_keys_dev,
-                                                          shift, col_mask, nullptr, 0, nullptr,
-                                                          hist, status, ticket, ctrl, 0);
-  else
-    k_radix_pass<kOutKeys><<<grid, kSortThreads, 0, st>>>(in, out, n_keys_bound, n_keys_dev,
-                                                          shift, col_mask, nullptr, 0, nullptr,
-                                                          hist, status, ticket, ctrl,
-                                                          unstable ? 1 : 0);
-  note_launch();
+  const auto kernel = mode == kOutPartSkip ? k_radix_pass<kOutPartSkip>
+                      : mode == kOutColRow ? k_radix_pass<kOutColRow>
+                      : mode == kOutRank   ? k_radix_pass<kOutRank>
+                                           : k_radix_pass<kOutKeys>;
+  launch(kernel, grid, kSortThreads, 0, st, in, out, n_keys_bound, n_keys_dev, shift, col_mask,
+         row_out, owner_shift, outdeg, hist, status, ticket, ctrl, unstable ? 1 : 0);
 }
 
 void launch_rank_keys(const int32_t *deg, int32_t n, int b, int passes, uint64_t *vkeys,
                       uint32_t *hist, cudaStream_t st) {
   const uint32_t want = ((uint32_t)n + kCanonThreads * 8 - 1) / (kCanonThreads * 8);
   const uint32_t grid = max(1u, min(want, (uint32_t)num_sms() * 8));
-  k_rank_keys<<<grid, kCanonThreads, 0, st>>>(deg, n, b, passes, vkeys, hist);
-  note_launch();
+  launch(k_rank_keys, grid, kCanonThreads, 0, st, deg, n, b, passes, vkeys, hist);
 }
 
 void launch_orient(const uint64_t *keys, uint32_t m_in, int b, const int32_t *rank,
                    uint64_t *okeys, uint32_t *hist2, int passes2, unsigned long long *status,
                    Ctrl *ctrl, cudaStream_t st) {
   const uint32_t grid = max(1u, (m_in + kOrientTile - 1) / kOrientTile);
-  k_orient<<<grid, kOrientThreads, 0, st>>>(keys, b, rank, okeys, hist2, passes2, status, ctrl);
-  note_launch();
+  launch(k_orient, grid, kOrientThreads, 0, st, keys, b, rank, okeys, hist2, passes2, status, ctrl);
 }
 
 static uint32_t scan_grid(int32_t n) {
@@ -920,8 +909,7 @@ void launch_offsets(const int32_t *counts, int32_t n, int32_t *off, int32_t *vof
   a.status = status;
   a.ticket = ticket;
   a.ctrl = ctrl;
-  k_offsets<kScanLists><<<scan_grid(n), kScanThreads, 0, st>>>(a);
-  note_launch();
+  launch(k_offsets<kScanLists>, scan_grid(n), kScanThreads, 0, st, a);
 }
 
 void launch_group_offsets(const int32_t *counts, const int32_t *own, int32_t n, int32_t *goff,
@@ -929,10 +917,9 @@ void launch_group_offsets(const int32_t *counts, const int32_t *own, int32_t n, 
                           Tuning tune, unsigned long long *status, uint32_t *ticket, Ctrl *ctrl,
                           cudaStream_t st, int32_t shard, int32_t shards) {
   tune.warp_max_list = min(max(tune.warp_max_list, 0), kWarpMaxRow);  // warp table capacity
-  const ScanArgs a{counts, own,  n,      goff,   nullptr, ldesc,           groups,          big_list,
+  const ScanArgs a{counts, own,    n,      goff, nullptr,         ldesc,          groups, big_list,
                    tune,   status, ticket, ctrl, (uint32_t)shard, (uint32_t)shards};
-  k_offsets<kScanGroups><<<scan_grid(n), kScanThreads, 0, st>>>(a);
-  note_launch();
+  launch(k_offsets<kScanGroups>, scan_grid(n), kScanThreads, 0, st, a);
 }
 
 void launch_recount(const int32_t *counts, int32_t n, int32_t *off, unsigned long long *status,
@@ -944,8 +931,7 @@ void launch_recount(const int32_t *counts, int32_t n, int32_t *off, unsigned lon
   a.status = status;
   a.ticket = ticket;
   a.ctrl = ctrl;
-  k_offsets<kScanRecount><<<scan_grid(n), kScanThreads, 0, st>>>(a);
-  note_launch();
+  launch(k_offsets<kScanRecount>, scan_grid(n), kScanThreads, 0, st, a);
 }
 
 }  // namespace tc

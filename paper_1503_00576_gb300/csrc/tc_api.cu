@@ -16,6 +16,11 @@ namespace tc {
 static std::atomic<uint64_t> g_launches{0};
 void note_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 
+static thread_local bool t_early = false;
+EarlyLaunches::EarlyLaunches(int64_t pairs) { t_early = pairs <= kEarlyMaxPairs; }
+EarlyLaunches::~EarlyLaunches() { t_early = false; }
+bool EarlyLaunches::allowed() { return t_early; }
+
 }  // namespace tc
 
 using namespace tc;
@@ -206,6 +211,7 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
                        int32_t *deg_out, const BatchRun *batch, const Tuning &tune,
                        PhaseTimer &pt, Ctrl *staging, bool work_stats = false,
                        int32_t shard = 0, int32_t shards = 1) {
+  const EarlyLaunches early(m_in);
   const uint32_t m = (uint32_t)m_in;
   const int b = id_bits(n);
   // radix passes: rank keys (degree bits < 2^b), oriented keys (owner bits)

@@ -73,6 +73,11 @@ template <bool PV> constexpr int64_t kBitMinPairs = PV ? 1 << 25 : 1 << 18;
 // of 180M 39 / 45 ms (the scattered writes leave L2).
 constexpr int64_t kDirectMaxPairs = 1ll << 25;
 constexpr int kRankClasses = 1024;
+// Runs whose kernels are launched early (see launch()).  Whole calls, in turn /
+// early: 8,191 pairs 135 / 85 us, 131,072 with clustering 259 / 198 us, R-MAT
+// 16 of 2.5M 541 / 469 us, R-MAT 18 of 10.5M 2.03 / 1.96 ms; R-MAT 20 of 16.8M
+// 3.13 / 3.22 ms, 21 of 91M 15.5 / 18.6 ms, 24 of 180M 38.2 / 43.4 ms.
+constexpr int64_t kEarlyMaxPairs = 12ll << 20;
 constexpr uint64_t kHole = ~0ull;            // no edge (dropped pair or edge)
 constexpr uint64_t kOwnEdge = 1ull << 63;    // emitted edge of its owner's group
 
@@ -345,6 +350,47 @@ inline Layout make_layout(int64_t m_in, int32_t n, bool with_hub = false,
 
 // Kernel-launch bookkeeping (defined in tc_api.cu).
 void note_launch();
+
+#ifdef __CUDACC__
+// Every kernel of the library begins with grid_begin(), before any access to
+// memory that another kernel of the stream may write or read: it lets the next
+// kernel's blocks be launched as this one's have started, and waits until the
+// kernels before this one have completed.  launch() marks a launch as allowed
+// to begin that early while an EarlyLaunches of a small run is alive on the
+// calling thread, so the kernels of the run follow each other without the gap
+// of a launch (about 1 us each, of 4 to 20 us of kernel).  Blocks that wait
+// take shared memory, and with it L1, from the kernel that runs, so larger
+// runs launch in turn (kEarlyMaxPairs).
+__device__ __forceinline__ void grid_begin() {
+  asm volatile("griddepcontrol.launch_dependents;");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+struct EarlyLaunches {
+  explicit EarlyLaunches(int64_t pairs);
+  ~EarlyLaunches();
+  EarlyLaunches(const EarlyLaunches &) = delete;
+  EarlyLaunches &operator=(const EarlyLaunches &) = delete;
+  static bool allowed();
+};
+
+template <typename... Params, typename... Args>
+void launch(void (*kernel)(Params...), uint32_t grid, uint32_t block, size_t smem,
+            cudaStream_t st, Args &&...args) {
+  cudaLaunchAttribute early{};
+  early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  early.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &early;
+  cfg.numAttrs = EarlyLaunches::allowed() ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+  note_launch();
+}
+#endif
 
 // Test hooks of the wait paths (preprocess.cu), on the current device:
 // spin_limit bounds every spin-wait (kSpinLimit by default); the radix-pass
