@@ -640,13 +640,8 @@ __device__ __forceinline__ void warp_groups(const Lists &g, const int32_t *__res
   }
 }
 
-// Per-vertex mode: the stream of every partner, so that a chunk's set-up is
-// one coalesced load and no gathers.  Partner l of an edge streams N+(l)
-// from its first block that can meet the hashed list (the pskip leading
-// blocks below it cannot): {col4 word voff[l] + 2 skip, d+(l) - 8 skip
-// entries, at least 0, in the low half (d+ <= sqrt(2m) < 2^16)}; the high
-// half holds the entries left to the hash path when the group's list has a
-// bitmap and l's takes over from block tb on (0xffff: it does not).
+// Per-vertex mode: the stream of every partner (stream_desc), so that a
+// chunk's set-up is one coalesced load and no gathers.
 __global__ void __launch_bounds__(256)
 k_stream_desc(const int32_t *__restrict__ part, const int32_t *__restrict__ pskip,
               const int2 *__restrict__ ldesc, const uint32_t *rec, const Ctrl *ctrl,
@@ -677,9 +672,7 @@ k_stream_desc(const int32_t *__restrict__ part, const int32_t *__restrict__ pski
       const uint32_t cut = bits_used<true>(r[q], skip[q], ld[q].y)
                                ? 8u * (uint32_t)max((int32_t)(r[q] & kBitTbMask) - skip[q], 0)
                                : 0xffffu;
-      if (e < m)
-        desc[e] = make_int2(ld[q].x + 2 * skip[q],
-                            (int32_t)((uint32_t)max(ld[q].y - 8 * skip[q], 0) | cut << 16));
+      if (e < m) desc[e] = stream_desc(ld[q], skip[q], cut);
     }
   }
 }
@@ -913,13 +906,14 @@ cudaError_t prepare_count_kernels() {
 
 cudaError_t launch_count(const int2 *ldesc, const int32_t *col4, const int32_t *goff,
                          const int32_t *part, const int32_t *pskip, int2 *desc,
-                         const int32_t *groups, const int32_t *big_groups, const uint32_t *rec,
-                         int32_t n, Ctrl *ctrl, int64_t *t, int64_t *tg, cudaStream_t st) {
+                         bool desc_ready, const int32_t *groups, const int32_t *big_groups,
+                         const uint32_t *rec, int32_t n, Ctrl *ctrl, int64_t *t, int64_t *tg,
+                         cudaStream_t st) {
   const bool pv = t != nullptr;
   CountGrid cg;
   cudaError_t e = count_grid(pv, &cg);
   if (e != cudaSuccess) return e;
-  if (pv) {
+  if (pv && !desc_ready) {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -947,7 +941,7 @@ void launch_clustering(const int64_t *t, const int32_t *deg, int32_t n, double *
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const uint32_t want = ((uint32_t)n + kClusterThreads * 4 - 1) / (kClusterThreads * 4);
+  const uint32_t want = ((uint32_t)n + kClusterThreads - 1) / kClusterThreads;
   const uint32_t grid = max(1u, min(want, (uint32_t)(sms > 0 ? sms : 1) * 8));
   launch(k_clustering, grid, kClusterThreads, 0, st, t, deg, n, cc, sums);
 }
@@ -957,7 +951,7 @@ void launch_gather_counts(const int64_t *t_rank, const int32_t *rank, int32_t n,
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const uint32_t want = ((uint32_t)n + kClusterThreads * 4 - 1) / (kClusterThreads * 4);
+  const uint32_t want = ((uint32_t)n + kClusterThreads - 1) / kClusterThreads;
   const uint32_t grid = max(1u, min(want, (uint32_t)(sms > 0 ? sms : 1) * 8));
   launch(k_gather_counts, grid, kClusterThreads, 0, st, t_rank, rank, n, t_out, ctrl);
 }

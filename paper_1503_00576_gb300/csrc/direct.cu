@@ -211,6 +211,7 @@ __global__ void __launch_bounds__(kThreads)
 k_direct_groups(const uint64_t *__restrict__ gkeys, int b, int32_t n,
                 const int32_t *__restrict__ goff, int32_t *__restrict__ gcnt,
                 int32_t *__restrict__ part, int32_t *__restrict__ pskip,
+                const int2 *__restrict__ ldesc, int2 *__restrict__ desc,
                 const Ctrl *__restrict__ ctrl) {
   grid_begin();
   __shared__ int32_t s_hot[kHotRanks];  // the tile's edges per rank, then the counter's old value
@@ -253,8 +254,11 @@ k_direct_groups(const uint64_t *__restrict__ gkeys, int b, int32_t n,
       if (k[q] == kHole) continue;
       const uint32_t h = (uint32_t)(k[q] >> b) & mask;
       if (!(k[q] & kOwnEdge) && h >= hot) at[q] += __ldg(goff + h + 1) - s_hot[h - hot];
-      part[at[q]] = (int32_t)((uint32_t)k[q] & mask);
-      pskip[at[q]] = k[q] & kOwnEdge ? 0 : (int32_t)(k[q] >> kSkipShift);
+      const uint32_t l = (uint32_t)k[q] & mask;
+      const int32_t skip = k[q] & kOwnEdge ? 0 : (int32_t)(k[q] >> kSkipShift);
+      part[at[q]] = (int32_t)l;
+      if (desc) desc[at[q]] = stream_desc(__ldg(ldesc + l), skip, 0xffffu);
+      else pskip[at[q]] = skip;
     }
     __syncthreads();  // s_hot is emptied again
   }
@@ -296,9 +300,9 @@ void launch_direct_lists(const uint64_t *okeys, const int32_t *place, uint32_t m
 
 void launch_direct_groups(const uint64_t *gkeys, uint32_t m_bound, int b, int32_t n,
                           const int32_t *goff, int32_t *gcnt, int32_t *part, int32_t *pskip,
-                          Ctrl *ctrl, cudaStream_t st) {
+                          const int2 *ldesc, int2 *desc, Ctrl *ctrl, cudaStream_t st) {
   launch(k_direct_groups, items_grid(m_bound), kThreads, 0, st, gkeys, b, n, goff, gcnt, part,
-         pskip, ctrl);
+         pskip, ldesc, desc, ctrl);
 }
 
 }  // namespace tc

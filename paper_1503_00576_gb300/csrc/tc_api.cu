@@ -428,7 +428,13 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
   // counting is split over several devices, Sec. III-E)
   launch_group_offsets(gcnt, direct ? own : nullptr, n, goff, ldesc, groups, big_groups, tune,
                        st_scan2, &ctrl->tile_ticket[kTicketGroupScan], ctrl, st, shard, shards);
-  if (direct) launch_direct_groups(gin, m, b, n, goff, gcnt, part, pskip, ctrl, st);
+  // per vertex, each partner's stream: written with the partners, or from them
+  // into the group sort's other buffer
+  const bool desc_ready = direct && t_out && !bits_on;
+  int2 *desc = reinterpret_cast<int2 *>(desc_ready ? ws + L.desc : (unsigned char *)gin);
+  if (direct)
+    launch_direct_groups(gin, m, b, n, goff, gcnt, part, pskip, ldesc, desc_ready ? desc : nullptr,
+                         ctrl, st);
   if (bits_on)
     launch_bits_build(queue, n, ldesc, col4, goff, L.bit_slots, t_out != nullptr, bits, items,
                       ctrl, st, shard, shards);
@@ -446,8 +452,7 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
   if (bits_on)
     launch_count_bits(ldesc, col4, goff, part, pskip, items, bits, n, ctrl,
                       t_out ? t_rank : nullptr, st);
-  int2 *desc = reinterpret_cast<int2 *>(gin);
-  cudaError_t e = launch_count(ldesc, col4, goff, part, pskip, desc, groups, big_groups,
+  cudaError_t e = launch_count(ldesc, col4, goff, part, pskip, desc, desc_ready, groups, big_groups,
                                bits_on ? bit_rec : nullptr, n, ctrl, t_out ? t_rank : nullptr,
                                t_out ? nullptr : t_rank, st);
   if (e == cudaSuccess && t_out) launch_gather_counts(t_rank, rank, n, t_out, ctrl, st);

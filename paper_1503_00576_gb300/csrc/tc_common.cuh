@@ -164,6 +164,15 @@ __device__ __forceinline__ bool aborted(const Ctrl *ctrl) {
   return (ctrl->err & kErrTimeout) != 0u;
 }
 
+// The stream of a partner whose list has record ld, from its first block that
+// can meet the hashed list on (the `skip` leading blocks cannot): {first col4
+// word, entries (d+ <= sqrt(2m) < 2^16) in the low half; in the high half the
+// entries left to the hash path when the group's list has a bitmap and this
+// one's takes over (0xffff: it does not)}.
+__device__ __forceinline__ int2 stream_desc(int2 ld, int32_t skip, uint32_t cut) {
+  return make_int2(ld.x + 2 * skip, (int32_t)((uint32_t)max(ld.y - 8 * skip, 0) | cut << 16));
+}
+
 // Whether a group of np partners whose list has bitmap record rec (0: none)
 // intersects by bitmaps.
 template <bool PV>
@@ -250,6 +259,9 @@ struct Layout {
   // bitmaps (single graphs of at least kBitMinPairs pairs): without per-vertex
   // counts the records take the place of t_rank and the bitmaps that of the
   // group sort's free key buffer; with them both have their own
+  // per-vertex runs that sort by counting have each partner's stream in `desc`
+  // (others in the group sort's free key buffer)
+  size_t desc;
   bool has_bits;
   size_t bit_rec, bits;
   uint32_t bit_slots;
@@ -338,6 +350,7 @@ inline Layout make_layout(int64_t m_in, int32_t n, bool with_hub = false,
   // elements, since each non-empty list adds at most 7
   L.col4 = take(sizeof(int32_t) * (m + 7 * (nv < m ? nv : m)));
   L.bits = per_vertex && L.has_bits ? take((size_t)L.bit_slots * (kBitCols / 4)) : 0;
+  L.desc = per_vertex && m_in <= kDirectMaxPairs ? take(sizeof(uint64_t) * m) : 0;
   const bool hub = with_hub && hub_enabled(n, id_bits(n > 0 ? n : 1));
   const size_t H = (size_t)hub_vertices;
   L.hub = take(hub ? H * H + 4 * H : 0);
@@ -532,10 +545,11 @@ void launch_direct_orient(const uint64_t *keys, uint32_t m_in, int b, const int3
 void launch_direct_lists(const uint64_t *okeys, const int32_t *place, uint32_t m_in, int b,
                          const int32_t *off, int32_t *col, Ctrl *ctrl, cudaStream_t st);
 // The partner and skip arrays from the emitted edges and the group offsets;
-// gcnt counts down to zero.
+// gcnt counts down to zero.  desc != nullptr (no bitmaps): each partner's stream
+// (see stream_desc) instead of its skip.
 void launch_direct_groups(const uint64_t *gkeys, uint32_t m_bound, int b, int32_t n,
                           const int32_t *goff, int32_t *gcnt, int32_t *part, int32_t *pskip,
-                          Ctrl *ctrl, cudaStream_t st);
+                          const int2 *ldesc, int2 *desc, Ctrl *ctrl, cudaStream_t st);
 // ---- launchers (bits.cu) ----
 // Bitmaps of the queued lists (launch_sort_lists) that have enough entries
 // among the top ranks, at most `slots` - 1 of them: 2 kBitCols bits each into
@@ -555,13 +569,14 @@ void launch_count_bits(const int2 *ldesc, const int32_t *col4, const int32_t *go
 // t != nullptr: per-vertex counts (rank space).  Otherwise, if tg is not
 // nullptr, tg[h] += triangles found in group h (their sum per graph is the
 // graph's count).  desc: scratch of 8 bytes per partner (each partner's
-// stream, written first).
+// stream, written first unless desc_ready; with t only).
 // groups, big_groups: the binned groups (launch_group_offsets).  rec: the
 // bitmap records (nullptr: no bitmaps).
 cudaError_t launch_count(const int2 *ldesc, const int32_t *col4, const int32_t *goff,
                          const int32_t *part, const int32_t *pskip, int2 *desc,
-                         const int32_t *groups, const int32_t *big_groups, const uint32_t *rec,
-                         int32_t n, Ctrl *ctrl, int64_t *t, int64_t *tg, cudaStream_t st);
+                         bool desc_ready, const int32_t *groups, const int32_t *big_groups,
+                         const uint32_t *rec, int32_t n, Ctrl *ctrl, int64_t *t, int64_t *tg,
+                         cudaStream_t st);
 // Sets the counting kernels' attributes and occupancy for the current
 // device (done lazily otherwise; needed before capturing a CUDA graph).
 cudaError_t prepare_count_kernels();
