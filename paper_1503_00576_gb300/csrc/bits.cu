@@ -33,6 +33,11 @@ constexpr unsigned kFull = 0xffffffffu;
 constexpr int kWords = kBitCols / 32;
 constexpr int kThreads = 128;
 constexpr int kWarps = kThreads / 32;
+// The per-vertex kernel's CTAs: eight warps share one set of hub counters, and a
+// warp's queue and planes one buffer, so that 110 KB of an SM stay L1, where the
+// loads in flight are held (four CTAs of four warps with both: 3.8 ms at R-MAT
+// scale 24, five 5.2 ms, these 3.3 ms).
+constexpr int kVertexThreads = 256;
 static_assert(kWords == 4 * 32, "a lane holds four words of a bitmap");
 
 // First of the top ranks: column 0 of the bitmaps.
@@ -368,6 +373,7 @@ __device__ __forceinline__ void bits_vertex(const BitArgs &a, int32_t h, uint32_
       const uint32_t ci = qu.cnt[i];
       if (ci) atomicAdd((unsigned long long *)&a.t[qu.l[i]], (unsigned long long)ci);
     }
+    __syncwarp();  // the planes take the queue's place
     if (sum) {
       empty_planes(a, pl, h, 8 * max((int32_t)(rh & kBitTbMask) - 1, 0), count, sb, s_t);
       if (lane == 0) atomicAdd((unsigned long long *)&a.t[h], (unsigned long long)sum);
@@ -377,41 +383,56 @@ __device__ __forceinline__ void bits_vertex(const BitArgs &a, int32_t h, uint32_
   __syncwarp();  // the queue is filled again
 }
 
+// Shared memory of a warp: its queue, and in the queue's place the planes that
+// it empties.
+template <bool PV>
+constexpr __host__ __device__ size_t warp_bytes() {
+  return PV && sizeof(uint32_t) * kPlanes * kWords > sizeof(Queue<PV>)
+             ? sizeof(uint32_t) * kPlanes * kWords
+             : sizeof(Queue<PV>);
+}
+constexpr size_t kVertexSmem =
+    warp_bytes<true>() * (kVertexThreads / 32) + sizeof(uint32_t) * kBitCols;
+static_assert(kVertexSmem <= 48 * 1024, "no attribute needed");
+
 // One work item per warp in turn: at most kBitRange partners of one group,
 // however large the group is.  (Ranges of the whole partner array, with a
 // walk over the groups in them, spent half of the kernel on groups without
 // bitmaps.)
 template <bool PV>
-__global__ void __launch_bounds__(kThreads, PV ? 4 : 8)
+__global__ void __launch_bounds__(PV ? kVertexThreads : kThreads, PV ? 2 : 8)
 k_count_bits(const BitArgs a) {
   grid_begin();
-  __shared__ Queue<PV> s_queue[kWarps];
-  __shared__ __align__(16) uint32_t s_planes[PV ? kWarps : 1][PV ? kPlanes * kWords : 4];
-  __shared__ uint32_t s_t[PV ? kBitCols : 1];
+  constexpr int THREADS = PV ? kVertexThreads : kThreads, WARPS = THREADS / 32;
+  extern __shared__ __align__(16) unsigned char smem[];
+  unsigned char *s_mine = smem + warp_bytes<PV>() * (threadIdx.x >> 5);
+  Queue<PV> &s_queue = *reinterpret_cast<Queue<PV> *>(s_mine);
+  uint32_t *s_planes = reinterpret_cast<uint32_t *>(s_mine);  // once the queue is done with
+  uint32_t *s_t = reinterpret_cast<uint32_t *>(smem + warp_bytes<PV>() * WARPS);  // PV only
   Ctrl *ctrl = a.ctrl;
   if (aborted(ctrl) || ctrl->n_bit_items == 0u) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t items = ctrl->n_bit_items;
   if (PV) {
-    for (int c = threadIdx.x; c < kBitCols; c += kThreads) s_t[c] = 0u;
+    for (int c = threadIdx.x; c < kBitCols; c += THREADS) s_t[c] = 0u;
     __syncthreads();
   }
   unsigned long long total = 0;
   Sums sums{0u, 0u, 0u, 0ull};
-  for (uint32_t i = blockIdx.x * kWarps + warp; i < items; i += gridDim.x * kWarps) {
+  for (uint32_t i = blockIdx.x * WARPS + warp; i < items; i += gridDim.x * WARPS) {
     const int2 item = __ldg(a.items + i);
     const uint32_t s = (uint32_t)item.y;
     const uint32_t t = min(s + kBitRange<PV>, (uint32_t)__ldg(a.goff + item.x + 1));
     const uint32_t rh = __ldg(a.rec + item.x);
     if constexpr (PV)
-      bits_vertex(a, item.x, rh, s, t, s_queue[warp], s_planes[warp], s_t, total);
+      bits_vertex(a, item.x, rh, s, t, s_queue, s_planes, s_t, total);
     else
-      bits_total(a, rh, s, t, s_queue[warp], sums);
+      bits_total(a, rh, s, t, s_queue, sums);
   }
   if (PV) {
     __syncthreads();
     const int32_t base = bits_base(a.n);
-    for (int c = threadIdx.x; c < kBitCols; c += kThreads)
+    for (int c = threadIdx.x; c < kBitCols; c += THREADS)
       if (s_t[c]) atomicAdd((unsigned long long *)&a.t[base + c], (unsigned long long)s_t[c]);
   } else {
     total = 8ull * sums.eights + 4u * (unsigned)__popc(sums.fours) +
@@ -445,9 +466,9 @@ void launch_count_bits(const int2 *ldesc, const int32_t *col4, const int32_t *go
                        const uint32_t *bits, int32_t n, Ctrl *ctrl, int64_t *t, cudaStream_t st) {
   const BitArgs a{goff, part, pskip, ldesc, col4, items.rec, bits, items.items, n, ctrl, t};
   if (t)
-    launch(k_count_bits<true>, sm_count() * 4u, kThreads, 0, st, a);
+    launch(k_count_bits<true>, sm_count() * 2u, kVertexThreads, kVertexSmem, st, a);
   else
-    launch(k_count_bits<false>, sm_count() * 8u, kThreads, 0, st, a);
+    launch(k_count_bits<false>, sm_count() * 8u, kThreads, warp_bytes<false>() * kWarps, st, a);
 }
 
 }  // namespace tc
