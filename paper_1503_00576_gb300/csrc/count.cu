@@ -4,8 +4,9 @@
 // each running a two-pointer merge of N+(u) and N+(v) from global memory,
 // and then sums the per-thread counts (thrust::reduce).  The result is the
 // sum over forward edges of |N+(u) & N+(v)|.  Here the same sum is computed
-// over the partner groups built in group.cu (group h: the edges whose
-// longer forward list is N+(h); partners l: their other endpoints):
+// over the partner groups built in group.cu (group h: the edges for which
+// N+(h) is hashed; partners l: their other endpoints; what the bitmaps of
+// bits.cu or the dense block of hub.cu take over is not streamed here):
 //
 //  * N+(h) is staged once in shared memory as an open-addressing hash set
 //    (multiplicative hashing, linear probing, load <= 1/32 where it fits),

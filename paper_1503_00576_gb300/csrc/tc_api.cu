@@ -271,8 +271,8 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
   const bool whole = shards > 1 || work_stats || tune.heavy_ratio_pct != 100 ||
                      2 * b > kSkipShift;
   // counting sorts by atomics, or radix passes (see kDirectMaxPairs)
-  const bool direct = m_in <= kDirectMaxPairs && 2 * b <= kSkipShift && shards == 1 &&
-                      !work_stats && !g_wait_hooks.load();
+  const bool direct = m_in <= (batch ? kDirectMaxBatchPairs : kDirectMaxPairs) &&
+                      2 * b <= kSkipShift && shards == 1 && !work_stats && !g_wait_hooks.load();
   if (!direct)
     TC_CUDA(cudaMemsetAsync(ws + L.st_sort, 0,
                             sizeof(unsigned long long) * words * (size_t)radix_passes(b), st),

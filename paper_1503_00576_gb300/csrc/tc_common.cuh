@@ -64,14 +64,17 @@ constexpr uint32_t kBitMaxSlots = (1u << (32 - kBitTbBits)) - 1;
 template <bool PV> constexpr int64_t kBitMinPairs = PV ? 1 << 25 : 1 << 18;
 
 // Counting sorts by atomics (direct.cu) instead of radix passes: runs of at
-// most this many pairs with ids of at most 24 bits, but for shares of a run
-// (their dealing needs the exact vertex order).  Whole calls, radix passes /
-// counting sorts: 8,191 pairs 196 / 134 us, R-MAT 16 of 2.5M 604 / 539 us, a
-// union of 300 small graphs (3.1M) 745 / 581 us, Barabasi-Albert of 10M 1.88 /
-// 1.69 ms, R-MAT 20 of 16.8M 3.37 / 3.15 ms, 64 graphs of 33M 5.31 / 4.93 ms;
-// ring lattice of 50M 4.91 / 5.05 ms, geometric of 67M 9.4 / 10.6 ms, R-MAT 24
-// of 180M 39 / 45 ms (the scattered writes leave L2).
-constexpr int64_t kDirectMaxPairs = 1ll << 25;
+// most this many pairs (a single graph; a batch) with ids of at most 24 bits,
+// but for shares of a run (their dealing needs the exact vertex order).  Whole
+// calls, radix passes / counting sorts: 8,191 pairs 196 / 134 us, R-MAT 16 of
+// 2.5M 604 / 539 us, a union of 300 small graphs (3.1M) 745 / 581 us, R-MAT 20
+// of 16.8M 3.37 / 3.15 ms, uniform of 16M 2.49 / 2.13 and of 32M 4.82 / 4.55 ms,
+// Barabasi-Albert of 12M 1.85 / 1.59, of 20M 2.85 / 2.68, of 24M 3.35 / 3.32 and
+// of 32M 4.42 / 4.72 ms; 64 graphs of 33M 5.31 / 4.93 ms; ring lattice of 50M
+// 4.91 / 5.05 ms, geometric of 67M 9.4 / 10.6 ms, R-MAT 24 of 180M 39 / 45 ms
+// (the scattered writes leave L2).
+constexpr int64_t kDirectMaxPairs = 20ll << 20;
+constexpr int64_t kDirectMaxBatchPairs = 1ll << 25;
 constexpr int kRankClasses = 1024;
 // Runs whose kernels are launched early (see launch()).  Whole calls, in turn /
 // early: 8,191 pairs 135 / 85 us, 131,072 with clustering 259 / 198 us, R-MAT

@@ -1,6 +1,6 @@
 """The two ways to sort forward lists and partner groups against each other and
-the oracle: counting sorts by atomics (csrc/direct.cu; calls of up to 2^25
-pairs) and radix passes (larger calls; shares, which also weigh whole lists).
+the oracle: counting sorts by atomics (csrc/direct.cu; calls of up to
+20 * 2^20 pairs) and radix passes (larger calls; shares, which also weigh whole lists).
 
 Graphs at the sizes where the first can go wrong: vertex counts around a tile of
 the rank classes, degrees around 256 and far above (the classes coarsen there),
