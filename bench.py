@@ -221,7 +221,8 @@ def measured_peaks() -> dict:
 
 def kernel_source_hash() -> str:
     h = hashlib.sha256()
-    for name in ("preprocess.cu", "group.cu", "count.cu", "hub.cu", "tc_common.cuh"):
+    for name in ("preprocess.cu", "direct.cu", "group.cu", "bits.cu", "count.cu", "hub.cu",
+                 "tc_common.cuh"):
         with open(os.path.join(ROOT, "paper_1503_00576_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]
@@ -252,7 +253,9 @@ def roofline(prof: dict, steps: int, m_in: int, m: int, n: int, workload: str,
     gather of t[] to vertex ids.  Its algorithmic bytes are the forward-list
     elements the hash intersections read -- each partner group's hashed list
     once (inserts) and, per forward edge, the list streamed through it
-    (lookups), 4 bytes each, counted exactly by tc_count_work -- plus the
+    (lookups), 4 bytes each, counted exactly by tc_count_work for the split of
+    the edges by whole lists (the kernels weigh what is streamed and leave the
+    top ranks of long lists to bitmaps, so they read less) -- plus the
     partner ids (4m), both offset arrays (8(n+1)) and, per vertex, t[] in
     rank space written, gathered and written again (28n)."""
     b = max(1, (max(n, 2) - 1).bit_length())

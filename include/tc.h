@@ -7,9 +7,10 @@
  * its lower endpoint, sort every forward list, and add |N+(u) & N+(v)| for
  * every forward edge (u, v).  Preprocessing reaches the sorted forward lists
  * of Sec. III-B by its own steps (degrees by atomics, backward edges dropped
- * while orienting, one sort of the oriented 64-bit keys by owner whose last
- * pass unzips, node arrays by scans, every list then sorted on its own);
- * counting computes the sum of Sec. III-C by hashing.  The order uses the
+ * while orienting, one sort of the oriented keys by owner -- radix passes or
+ * a counting sort -- node arrays by scans, every list then sorted on its own);
+ * counting computes the sum of Sec. III-C by hashing, by bitmaps of the highest
+ * ranks, and by a dense block.  The order uses the
  * degree with repeated pairs counted as given (any order counts every
  * triangle once; without repeats it is the paper's).  All arithmetic is
  * exact integer.
@@ -261,9 +262,12 @@ tc_status tc_engine_destroy(tc_engine *engine);
 
 /*
  * Work of the counting phase (instrumentation; the paper reports running
- * times only).  Runs the same pipeline as tc_count with the current tuning,
- * plus one reduction kernel over the forward edges, and reports what the
- * counting phase does for this graph:
+ * times only).  Counts the graph with the current tuning, with every edge
+ * grouped by the lengths of its whole lists (as tc_count_part deals them),
+ * plus one reduction kernel over the forward edges, and reports the work of
+ * that split by hashing.  (tc_count itself weighs what would be streamed,
+ * leaves out edges that need no intersection and intersects long lists by
+ * bitmaps, so it reads less.)
  *   edges          m, distinct undirected edges = forward edges (Sec. II-B)
  *   lookups        sum over forward edges {u, v} of the forward-list length
  *                  streamed through the hash set (the shorter of N+(u),
