@@ -49,8 +49,8 @@ __device__ __forceinline__ int32_t bits_base(int32_t n) { return max(n - kBitCol
 // slot does not fit the region has none.  Slot 0 is the empty bitmap.
 template <bool PV>
 __global__ void __launch_bounds__(kThreads)
-k_bits_build(const int32_t *__restrict__ queue, int32_t n, const int2 *__restrict__ ldesc,
-             const int32_t *__restrict__ col4, const int32_t *__restrict__ goff, uint32_t slots,
+k_bits_build(const int32_t *queue, int32_t n, const int2 *ldesc,
+             const int32_t *col4, const int32_t *goff, uint32_t slots,
              uint32_t *__restrict__ bits, uint32_t *__restrict__ rec, int2 *__restrict__ items,
              Ctrl *ctrl, uint32_t shard, uint32_t shards) {
   grid_begin();
@@ -83,19 +83,19 @@ k_bits_build(const int32_t *__restrict__ queue, int32_t n, const int2 *__restric
     pending = 0;
   };
   for (uint32_t i = blockIdx.x * kWarps + warp; i < count; i += gridDim.x * kWarps) {
-    const int32_t v = __ldg(queue + (i < n_warp ? i : (uint32_t)n - 1u - (i - n_warp)));
-    const int2 ld = __ldg(ldesc + v);
+    const int32_t v = load(queue + (i < n_warp ? i : (uint32_t)n - 1u - (i - n_warp)));
+    const int2 ld = load(ldesc + v);
     const int32_t len = ld.y, blocks = (len + 7) >> 3;
     const int32_t *list = col4 + 4ll * ld.x;
     // enough top ranks at all?
     constexpr int32_t kLeast = 8 * (kBitMinBlocks<PV> - 1) + 1;
-    if (blocks < kBitMinBlocks<PV> || __ldg(list + len - kLeast) < base) continue;
+    if (blocks < kBitMinBlocks<PV> || load(list + len - kLeast) < base) continue;
     for (int w = lane; w < kWords; w += 32) sb[w] = 0u;
     __syncwarp();
     int32_t top = 0;  // entries before the first top rank
     for (int32_t e1 = len; e1 > 0; e1 -= 32) {
       const int32_t e = e1 - 1 - lane;
-      const int32_t x = e >= 0 ? __ldg(list + e) : -1;
+      const int32_t x = e >= 0 ? load(list + e) : -1;
       const bool in = x >= base;  // lanes 0 .. k-1: the list is sorted
       if (in) atomicOr(&sb[(uint32_t)(x - base) >> 5], 1u << ((x - base) & 31));
       const int k = __popc(__ballot_sync(kFull, in));
@@ -111,14 +111,14 @@ k_bits_build(const int32_t *__restrict__ queue, int32_t n, const int2 *__restric
       dst[32] = reinterpret_cast<const uint4 *>(sb)[lane];  // F
       __syncwarp();
       if (lane < 8 * tb - top) {  // top ranks of the block before tb: streamed
-        const int32_t c = __ldg(list + top + lane) - base;
+        const int32_t c = load(list + top + lane) - base;
         atomicAnd(&sb[c >> 5], ~(1u << (c & 31)));
       }
       __syncwarp();
       dst[0] = reinterpret_cast<const uint4 *>(sb)[lane];  // B
       const uint32_t r = ((i + 1u) << kBitTbBits) | (uint32_t)tb;
       if (lane == 0) rec[v] = r;
-      const int32_t gs = __ldg(goff + v), ge = __ldg(goff + v + 1);
+      const int32_t gs = load(goff + v), ge = load(goff + v + 1);
       if (bits_group<PV>(r, ge - gs) && (uint32_t)v % shards == shard) {
         if (lane == pending) {
           group = v;
@@ -176,13 +176,13 @@ __device__ __forceinline__ int fill_queue(const BitArgs &a, uint32_t s, uint32_t
 #pragma unroll
   for (int i = 0; i < N; ++i) {
     const uint32_t e = s + 32 * i + lane;
-    l[i] = e < t ? __ldg(a.part + e) : -1;
-    skip[i] = e < t ? __ldg(a.pskip + e) : 0;
+    l[i] = e < t ? load(a.part + e) : -1;
+    skip[i] = e < t ? load(a.pskip + e) : 0;
   }
 #pragma unroll
   for (int i = 0; i < N; ++i) {
-    r[i] = l[i] >= 0 ? __ldg(a.rec + l[i]) : 0u;
-    len[i] = l[i] >= 0 ? __ldg(a.ldesc + l[i]).y : 0;
+    r[i] = l[i] >= 0 ? load(a.rec + l[i]) : 0u;
+    len[i] = l[i] >= 0 ? load(a.ldesc + l[i]).y : 0;
   }
   int count = 0;
 #pragma unroll
@@ -206,10 +206,10 @@ __device__ __forceinline__ int fill_queue(const BitArgs &a, uint32_t s, uint32_t
 __device__ __forceinline__ void load_four(const uint4 *lane_bits, const uint32_t *slot,
                                           uint4 *x) {
   const uint4 sl = *reinterpret_cast<const uint4 *>(slot);
-  x[0] = __ldg(lane_bits + (size_t)sl.x * 64);
-  x[1] = __ldg(lane_bits + (size_t)sl.y * 64);
-  x[2] = __ldg(lane_bits + (size_t)sl.z * 64);
-  x[3] = __ldg(lane_bits + (size_t)sl.w * 64);
+  x[0] = load(lane_bits + (size_t)sl.x * 64);
+  x[1] = load(lane_bits + (size_t)sl.y * 64);
+  x[2] = load(lane_bits + (size_t)sl.z * 64);
+  x[3] = load(lane_bits + (size_t)sl.w * 64);
 }
 
 // T only: Harley-Seal over the words of all partners a lane meets, whatever
@@ -232,7 +232,7 @@ __device__ __forceinline__ uint32_t add_words(Sums &s, const uint4 &x, const uin
 __device__ __forceinline__ void bits_total(const BitArgs &a, uint32_t rh, uint32_t s,
                                            uint32_t t, Queue<false> &qu, Sums &sums) {
   const uint4 *lane_bits = reinterpret_cast<const uint4 *>(a.bits) + (threadIdx.x & 31);
-  const uint4 f = __ldg(lane_bits + (size_t)(rh >> kBitTbBits) * 64 + 32);
+  const uint4 f = load(lane_bits + (size_t)(rh >> kBitTbBits) * 64 + 32);
   const uint32_t hw[4] = {f.x, f.y, f.z, f.w};
   const int count = fill_queue<false>(a, s, t, qu);
   if (count) {
@@ -282,11 +282,11 @@ __device__ __forceinline__ void empty_planes(const BitArgs &a, const Planes &pl,
       reinterpret_cast<uint4 *>(sb)[k * 32 + lane] =
           make_uint4(pl.p[0][k], pl.p[1][k], pl.p[2][k], pl.p[3][k]);
   __syncwarp();
-  const int2 ld = __ldg(a.ldesc + h);
+  const int2 ld = load(a.ldesc + h);
   const int32_t *list = a.col4 + 4ll * ld.x;
   const int32_t base = bits_base(a.n);
   for (int32_t e = from + lane; e < ld.y; e += 32) {
-    const int32_t x = __ldg(list + e), c = x - base;
+    const int32_t x = load(list + e), c = x - base;
     if (c >= 0) {
       uint32_t cnt = 0;
 #pragma unroll
@@ -336,7 +336,7 @@ __device__ __forceinline__ void bits_vertex(const BitArgs &a, int32_t h, uint32_
                                             uint32_t *s_t, unsigned long long &total) {
   const int lane = threadIdx.x & 31;
   const uint4 *lane_bits = reinterpret_cast<const uint4 *>(a.bits) + lane;
-  const uint4 fh = __ldg(lane_bits + (size_t)(rh >> kBitTbBits) * 64 + 32);
+  const uint4 fh = load(lane_bits + (size_t)(rh >> kBitTbBits) * 64 + 32);
   const uint32_t hw[4] = {fh.x, fh.y, fh.z, fh.w};
   const int count = fill_queue<true>(a, s, t, qu);
   uint32_t sum = 0;  // matches of the segment (uniform; at most kBitRange kBitCols)
@@ -420,10 +420,10 @@ k_count_bits(const BitArgs a) {
   unsigned long long total = 0;
   Sums sums{0u, 0u, 0u, 0ull};
   for (uint32_t i = blockIdx.x * WARPS + warp; i < items; i += gridDim.x * WARPS) {
-    const int2 item = __ldg(a.items + i);
+    const int2 item = load(a.items + i);
     const uint32_t s = (uint32_t)item.y;
-    const uint32_t t = min(s + kBitRange<PV>, (uint32_t)__ldg(a.goff + item.x + 1));
-    const uint32_t rh = __ldg(a.rec + item.x);
+    const uint32_t t = min(s + kBitRange<PV>, (uint32_t)load(a.goff + item.x + 1));
+    const uint32_t rh = load(a.rec + item.x);
     if constexpr (PV)
       bits_vertex(a, item.x, rh, s, t, s_queue, s_planes, s_t, total);
     else

@@ -92,16 +92,16 @@ __device__ __forceinline__ uint32_t table_slots(int32_t len, uint32_t capacity) 
 
 // Read-only view of the forward lists and partner groups.
 struct Lists {
-  const int32_t *__restrict__ col4;  // forward lists, sorted, in whole 32-byte blocks (-1 pads)
-  const int32_t *__restrict__ goff;  // partner-group offsets
-  const int32_t *__restrict__ part;   // partners
-  const int32_t *__restrict__ pskip;  // per partner: leading blocks of its list skipped
-  const int2 *__restrict__ desc;      // per-vertex mode, per partner: its stream
+  const int32_t *col4;  // forward lists, sorted, in whole 32-byte blocks (-1 pads)
+  const int32_t *goff;  // partner-group offsets
+  const int32_t *part;   // partners
+  const int32_t *pskip;  // per partner: leading blocks of its list skipped
+  const int2 *desc;      // per-vertex mode, per partner: its stream
                                       //   {first col4 word, entries | cut << 16}
                                       //   (k_stream_desc)
-  const int2 *__restrict__ ldesc;     // per vertex: its list {voff[v], d+(v)}, one
+  const int2 *ldesc;     // per vertex: its list {voff[v], d+(v)}, one
                                       //   8-byte gather instead of three 4-byte ones
-  const uint32_t *__restrict__ rec;   // per vertex: its bitmap's record (nullptr: none)
+  const uint32_t *rec;   // per vertex: its bitmap's record (nullptr: none)
 };
 
 // One hash set in shared memory.
@@ -157,12 +157,12 @@ __device__ __forceinline__ void clear_table(int32_t *tab, uint32_t *cnt, int slo
 // Inserts list[0..len) (distinct ids) into the empty hash set; the slot of
 // list[i] goes to slot_of[i].  Returns whether this thread met a taken slot:
 // if none did, every key sits at its home and a lookup is one comparison.
-__device__ __forceinline__ bool fill_table(const int32_t *__restrict__ list, int32_t len,
+__device__ __forceinline__ bool fill_table(const int32_t *list, int32_t len,
                                            const Table &tb, uint16_t *slot_of, int rank,
                                            int group) {
   bool displaced = false;
   for (int32_t i = rank; i < len; i += group) {
-    const int32_t x = __ldg(list + i);
+    const int32_t x = load(list + i);
     const uint32_t home = hash_slot((uint32_t)x, tb.slots);
     uint32_t h = home;
     for (;;) {
@@ -319,12 +319,13 @@ __device__ __forceinline__ int32_t warp_incl_scan(int32_t x) {
   return x;
 }
 
-// One 32-byte block (two words) of col4 at 16-byte word a (even).
+// One 32-byte block (two words) of col4 at 16-byte word a (even): an ordinary
+// load like load() (tc_common.cuh).
 __device__ __forceinline__ void ld_block(const int32_t *col4, int32_t a, int32_t (&x)[8]) {
-  asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-      : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]), "=r"(x[4]), "=r"(x[5]), "=r"(x[6]),
-        "=r"(x[7])
-      : "l"(col4 + 4 * (size_t)a));
+  asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]), "=r"(x[4]), "=r"(x[5]),
+                 "=r"(x[6]), "=r"(x[7])
+               : "l"(col4 + 4 * (size_t)a));
 }
 
 // Block mode of probe_chunk: windows w .. w+NQ-1 of 32 blocks (64 words) of
@@ -386,9 +387,9 @@ __device__ __forceinline__ void probe_windows(const Lists &g, int32_t w, int32_t
 // (per block, or when an element-mode lane leaves the partner's list), per w
 // to the counter beside w's slot.
 template <bool PV, int W>
-__device__ __forceinline__ void probe_chunk(const Lists &g, const int32_t *__restrict__ part,
-                                            const int32_t *__restrict__ pskip,
-                                            const int2 *__restrict__ desc, int32_t np,
+__device__ __forceinline__ void probe_chunk(const Lists &g, const int32_t *part,
+                                            const int32_t *pskip,
+                                            const int2 *desc, int32_t np,
                                             int32_t c0, int32_t cs, bool bits, const Table &tb,
                                             WarpScratch &ws, int64_t *t,
                                             uint64_t &found_group) {
@@ -396,26 +397,26 @@ __device__ __forceinline__ void probe_chunk(const Lists &g, const int32_t *__res
   const int32_t j = c0 + lane;
   int32_t l = 0, dl = 0, vb = 0;
   if (lane < cs && j < np) {
-    l = __ldg(part + j);
+    l = load(part + j);
     if (PV) {
       // the partner's stream, written before the counting (k_stream_desc):
       // no gathers in the chunk's set-up, whose registers the per-vertex
       // counters need (measured: 1.6 ms of 31 at R-MAT scale 24; without
       // counters the separate pass costs more than it saves)
-      const int2 ds = __ldg(desc + j);
+      const int2 ds = load(desc + j);
       vb = ds.x;
       dl = ds.y & 0xffff;
       if (bits) dl = min(dl, (int32_t)((uint32_t)ds.y >> 16));
     } else {
-      const int32_t skip = __ldg(pskip + j);
-      const int2 ld = __ldg(g.ldesc + l);
+      const int32_t skip = load(pskip + j);
+      const int2 ld = load(g.ldesc + l);
       dl = ld.y;
       vb = ld.x;
       // the leading blocks of N+(l) below the hashed list's smallest id
       // cannot meet it: stream from the first block that can
       vb += 2 * skip;
       if (bits) {
-        const uint32_t rec = __ldg(g.rec + l);
+        const uint32_t rec = load(g.rec + l);
         if (bits_used<PV>(rec, skip, dl)) dl = 8 * (int32_t)(rec & kBitTbMask);
       }
       dl = max(dl - 8 * skip, 0);
@@ -488,7 +489,7 @@ __device__ __forceinline__ void probe_chunk(const Lists &g, const int32_t *__res
             eb = ws.eb[r];
             next = ws.enext[r];
           }
-          x[q] = __ldg(g.col4 + (eb + p));
+          x[q] = load(g.col4 + (eb + p));
         }
         rq[q] = r;
       }
@@ -532,7 +533,7 @@ struct CtaShared {
 // N+(h) & N+(l) is the disjoint union of the segments' intersections.  The
 // table (SLOTS slots) is empty on entry and on exit.
 template <bool PV, int THREADS, int SLOTS, int W>
-__device__ __forceinline__ void cta_groups(const Lists &g, const int32_t *__restrict__ list,
+__device__ __forceinline__ void cta_groups(const Lists &g, const int32_t *list,
                                            int step, uint32_t n_list, uint32_t *cursor, Table tb,
                                            uint16_t *slot_of, WarpScratch *s_ws, CtaShared &sh,
                                            int64_t *t, int64_t *tg, uint64_t &found_total) {
@@ -548,15 +549,15 @@ __device__ __forceinline__ void cta_groups(const Lists &g, const int32_t *__rest
     if (gi >= n_list) break;
     // lists are filled in about ascending rank, and high ranks (high
     // degrees) carry the most work: take them first to shorten the tail
-    const int32_t h = __ldg(list + (int64_t)gi * step);
-    const int2 hld = __ldg(g.ldesc + h);
+    const int32_t h = load(list + (int64_t)gi * step);
+    const int2 hld = load(g.ldesc + h);
     const int32_t hd = hld.y;
     const int32_t *hl = g.col4 + 4 * (size_t)hld.x;
-    const int32_t pb = __ldg(g.goff + h), np = __ldg(g.goff + h + 1) - pb;
+    const int32_t pb = load(g.goff + h), np = load(g.goff + h + 1) - pb;
     const int32_t nseg = (hd + SLOTS / 2 - 1) / (SLOTS / 2);
     const int32_t seg_len = (hd + nseg - 1) / nseg;
     tb.slots = table_slots(seg_len, SLOTS);
-    const bool bits = g.rec && bits_group<PV>(__ldg(g.rec + h), np);
+    const bool bits = g.rec && bits_group<PV>(load(g.rec + h), np);
     uint64_t found_group = 0;  // of this warp (uniform)
     for (int32_t s0 = 0; s0 < hd; s0 += seg_len) {
       const int32_t len = min(seg_len, hd - s0);
@@ -601,7 +602,7 @@ __device__ __forceinline__ void cta_groups(const Lists &g, const int32_t *__rest
 // WSLOTS slots (empty on entry and on exit).  claim: groups taken at a time (in
 // shared memory: a register for it cost 7% on random geometric graphs).
 template <bool PV, int WSLOTS>
-__device__ __forceinline__ void warp_groups(const Lists &g, const int32_t *__restrict__ list,
+__device__ __forceinline__ void warp_groups(const Lists &g, const int32_t *list,
                                             uint32_t n_list, uint32_t *cursor,
                                             const uint32_t *claim, Table tb,
                                             uint16_t *slot_of, WarpScratch &ws, int64_t *t,
@@ -614,13 +615,13 @@ __device__ __forceinline__ void warp_groups(const Lists &g, const int32_t *__res
     if (g0 >= n_list) break;
     const uint32_t g1 = min(g0 + *claim, n_list);
     for (uint32_t gi = g0; gi < g1; ++gi) {
-      const int32_t h = __ldg(list + (n_list - 1 - gi));  // heavy (high-rank) groups first
-      const int2 hld = __ldg(g.ldesc + h);
+      const int32_t h = load(list + (n_list - 1 - gi));  // heavy (high-rank) groups first
+      const int2 hld = load(g.ldesc + h);
       const int32_t hd = hld.y;
       const int32_t *hl = g.col4 + 4 * (size_t)hld.x;
-      const int32_t pb = __ldg(g.goff + h), np = __ldg(g.goff + h + 1) - pb;
+      const int32_t pb = load(g.goff + h), np = load(g.goff + h + 1) - pb;
       tb.slots = table_slots(hd, WSLOTS);
-      const bool bits = g.rec && bits_group<PV>(__ldg(g.rec + h), np);
+      const bool bits = g.rec && bits_group<PV>(load(g.rec + h), np);
       tb.home = !__any_sync(kFull, fill_table(hl, hd, tb, slot_of, lane, 32));
       __syncwarp();
       uint64_t found_group = 0;  // uniform
@@ -644,8 +645,8 @@ __device__ __forceinline__ void warp_groups(const Lists &g, const int32_t *__res
 // Per-vertex mode: the stream of every partner (stream_desc), so that a
 // chunk's set-up is one coalesced load and no gathers.
 __global__ void __launch_bounds__(256)
-k_stream_desc(const int32_t *__restrict__ part, const int32_t *__restrict__ pskip,
-              const int2 *__restrict__ ldesc, const uint32_t *rec, const Ctrl *ctrl,
+k_stream_desc(const int32_t *part, const int32_t *pskip,
+              const int2 *ldesc, const uint32_t *rec, const Ctrl *ctrl,
               int2 *__restrict__ desc) {
   grid_begin();
   if (aborted(ctrl)) return;  // an earlier wait of this call ran out
@@ -659,13 +660,13 @@ k_stream_desc(const int32_t *__restrict__ part, const int32_t *__restrict__ pski
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const uint32_t e = e0 + q * stride;
-      l[q] = e < m ? __ldg(part + e) : 0;
-      skip[q] = e < m ? __ldg(pskip + e) : 0;
+      l[q] = e < m ? load(part + e) : 0;
+      skip[q] = e < m ? load(pskip + e) : 0;
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      ld[q] = __ldg(ldesc + l[q]);
-      r[q] = rec ? __ldg(rec + l[q]) : 0u;
+      ld[q] = load(ldesc + l[q]);
+      r[q] = rec ? load(rec + l[q]) : 0u;
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -692,7 +693,7 @@ static_assert(kMainWarps * kWarpMaxRow <= kCtaMaxRow, "warp slot maps must fit t
 // Main counting kernel: CTA groups first (the heavy ones), then warp groups.
 template <bool PV>
 __global__ void __launch_bounds__(kMainThreads, kMainMinBlocks)
-k_count(Lists g, const int32_t *__restrict__ groups, int32_t n, Ctrl *ctrl, int64_t *t,
+k_count(Lists g, const int32_t *groups, int32_t n, Ctrl *ctrl, int64_t *t,
         int64_t *tg) {
   grid_begin();
   constexpr int SLOTS = main_slots<PV>();
@@ -729,7 +730,7 @@ k_count(Lists g, const int32_t *__restrict__ groups, int32_t n, Ctrl *ctrl, int6
 // Groups whose hashed list is longer than kCtaMaxRow (rare).
 template <bool PV>
 __global__ void __launch_bounds__(kBigThreads, kBigMinBlocks)
-k_count_big(Lists g, const int32_t *__restrict__ big_list, Ctrl *ctrl, int64_t *t,
+k_count_big(Lists g, const int32_t *big_list, Ctrl *ctrl, int64_t *t,
             int64_t *tg) {
   grid_begin();
   extern __shared__ __align__(16) unsigned char smem[];
@@ -758,14 +759,14 @@ k_count_big(Lists g, const int32_t *__restrict__ big_list, Ctrl *ctrl, int64_t *
 constexpr int kClusterThreads = 256;
 
 __global__ void __launch_bounds__(kClusterThreads)
-k_clustering(const int64_t *__restrict__ t, const int32_t *__restrict__ deg, int32_t n,
+k_clustering(const int64_t *t, const int32_t *deg, int32_t n,
              double *__restrict__ cc, unsigned long long *sums) {
   grid_begin();
   unsigned long long st = 0, sw = 0;
   const uint32_t stride = gridDim.x * kClusterThreads;
   for (uint32_t v = blockIdx.x * kClusterThreads + threadIdx.x; v < (uint32_t)n; v += stride) {
-    const int64_t tv = __ldg(t + v);
-    const int64_t d = __ldg(deg + v);
+    const int64_t tv = load(t + v);
+    const int64_t d = load(deg + v);
     if (cc) {
       double c = 0.0;
       if (d >= 2) c = (2.0 * (double)tv) / ((double)d * (double)(d - 1));
@@ -784,13 +785,13 @@ k_clustering(const int64_t *__restrict__ t, const int32_t *__restrict__ deg, int
 
 // Per-vertex counts from rank space back to the caller's vertex ids.
 __global__ void __launch_bounds__(kClusterThreads)
-k_gather_counts(const int64_t *__restrict__ t_rank, const int32_t *__restrict__ rank, int32_t n,
+k_gather_counts(const int64_t *t_rank, const int32_t *rank, int32_t n,
                 int64_t *__restrict__ t_out, const Ctrl *ctrl) {
   grid_begin();
   if (aborted(ctrl)) return;  // rank[] may be incomplete
   const uint32_t stride = gridDim.x * kClusterThreads;
   for (uint32_t v = blockIdx.x * kClusterThreads + threadIdx.x; v < (uint32_t)n; v += stride)
-    t_out[v] = __ldg(t_rank + __ldg(rank + v));
+    t_out[v] = load(t_rank + load(rank + v));
 }
 
 // Per-graph sums of the group totals tg (rank space) over the graphs' union
@@ -798,15 +799,15 @@ k_gather_counts(const int64_t *__restrict__ t_rank, const int32_t *__restrict__ 
 // summed by as many warps as it fills (one warp per graph took 453 us for 64
 // graphs of up to 2^18 vertices; this and the gather it replaces take 15).
 __global__ void __launch_bounds__(kClusterThreads)
-k_batch_totals(const int64_t *__restrict__ tg, const int32_t *__restrict__ rank,
-               const BatchDesc *__restrict__ batch, const Ctrl *ctrl,
+k_batch_totals(const int64_t *tg, const int32_t *rank,
+               const BatchDesc *batch, const Ctrl *ctrl,
                unsigned long long *__restrict__ totals) {
   grid_begin();
   constexpr uint32_t ROUNDS = 8;
   if (aborted(ctrl)) return;  // rank[] may be incomplete
   const int32_t ng = batch->num_graphs;
   const int32_t *vo = batch->voff;
-  const uint32_t n = (uint32_t)__ldg(vo + ng);
+  const uint32_t n = (uint32_t)load(vo + ng);
   const int lane = threadIdx.x & 31;
   const uint32_t first = blockIdx.x * kClusterThreads + threadIdx.x;
   for (uint32_t g = first; g < (uint32_t)ng; g += gridDim.x * kClusterThreads)
@@ -817,14 +818,14 @@ k_batch_totals(const int64_t *__restrict__ tg, const int32_t *__restrict__ rank,
 #pragma unroll
     for (int q = 0; q < (int)ROUNDS; ++q) {
       const uint32_t v = v0 + 32 * q + lane;
-      x[q] = v < n ? (unsigned long long)__ldg(tg + __ldg(rank + v)) : 0ull;
+      x[q] = v < n ? (unsigned long long)load(tg + load(rank + v)) : 0ull;
     }
     int32_t g = 0, hi = ng;  // the last graph with vo[g] <= v0
     while (hi - g > 1) {
       const int32_t mid = (g + hi) >> 1;
-      if ((uint32_t)__ldg(vo + mid) <= v0) g = mid; else hi = mid;
+      if ((uint32_t)load(vo + mid) <= v0) g = mid; else hi = mid;
     }
-    uint32_t end = (uint32_t)__ldg(vo + g + 1);
+    uint32_t end = (uint32_t)load(vo + g + 1);
     unsigned long long sum = 0;
 #pragma unroll
     for (int q = 0; q < (int)ROUNDS; ++q) {
@@ -832,7 +833,7 @@ k_batch_totals(const int64_t *__restrict__ tg, const int32_t *__restrict__ rank,
       if (v < n && v >= end) {  // on to a later graph
         if (sum && !batch->gerr[g]) atomicAdd(&totals[g], sum);
         sum = 0;
-        do end = (uint32_t)__ldg(vo + ++g + 1); while (v >= end);
+        do end = (uint32_t)load(vo + ++g + 1); while (v >= end);
       }
       sum += x[q];
     }

@@ -47,14 +47,14 @@ __device__ __forceinline__ uint32_t rank_class(uint32_t d) {
 
 // Vertices per degree class.
 __global__ void __launch_bounds__(kThreads)
-k_rank_hist(const int32_t *__restrict__ deg, int32_t n, uint32_t *__restrict__ hist) {
+k_rank_hist(const int32_t *deg, int32_t n, uint32_t *__restrict__ hist) {
   grid_begin();
   __shared__ uint32_t s_cnt[kRankClasses];
   for (int i = threadIdx.x; i < kRankClasses; i += kThreads) s_cnt[i] = 0;
   __syncthreads();
   const uint32_t stride = gridDim.x * kThreads;
   for (uint32_t v = blockIdx.x * kThreads + threadIdx.x; v < (uint32_t)n; v += stride)
-    atomicAdd(&s_cnt[rank_class((uint32_t)__ldg(deg + v))], 1u);
+    atomicAdd(&s_cnt[rank_class((uint32_t)load(deg + v))], 1u);
   __syncthreads();
   for (int i = threadIdx.x; i < kRankClasses; i += kThreads)
     if (s_cnt[i]) atomicAdd(&hist[i], s_cnt[i]);
@@ -64,7 +64,7 @@ k_rank_hist(const int32_t *__restrict__ deg, int32_t n, uint32_t *__restrict__ h
 // itself), plus the places its tile reserved in the class, plus v's place
 // within the tile.
 __global__ void __launch_bounds__(kThreads)
-k_rank_assign(const int32_t *__restrict__ deg, int32_t n, const uint32_t *__restrict__ hist,
+k_rank_assign(const int32_t *deg, int32_t n, const uint32_t *hist,
               uint32_t *__restrict__ cursor, int32_t *__restrict__ rank) {
   grid_begin();
   constexpr int PER = kRankClasses / kThreads;
@@ -73,7 +73,7 @@ k_rank_assign(const int32_t *__restrict__ deg, int32_t n, const uint32_t *__rest
   uint32_t h[PER], sum = 0;
 #pragma unroll
   for (int i = 0; i < PER; ++i) {
-    h[i] = __ldg(hist + tid * PER + i);
+    h[i] = load(hist + tid * PER + i);
     sum += h[i];
   }
   uint32_t incl = sum;
@@ -100,7 +100,7 @@ k_rank_assign(const int32_t *__restrict__ deg, int32_t n, const uint32_t *__rest
     for (int i = 0; i < kRankPer; ++i) {
       const uint32_t v = tile * kRankTile + i * kThreads + tid;
       if (v < (uint32_t)n) {
-        c[i] = rank_class((uint32_t)__ldg(deg + v));
+        c[i] = rank_class((uint32_t)load(deg + v));
         at[i] = atomicAdd(&s_cnt[c[i]], 1u);
       }
     }
@@ -125,9 +125,9 @@ k_rank_assign(const int32_t *__restrict__ deg, int32_t n, const uint32_t *__rest
 // Each key as (lower rank) << b | (higher rank), with its place in the
 // owner's list; self-loops and dropped pairs (the sentinel) stay as holes.
 __global__ void __launch_bounds__(kThreads)
-k_direct_orient(const uint64_t *__restrict__ keys, int b, const int32_t *__restrict__ rank,
+k_direct_orient(const uint64_t *keys, int b, const int32_t *rank,
                 uint64_t *__restrict__ okeys, int32_t *__restrict__ place,
-                int32_t *__restrict__ outdeg, const Ctrl *__restrict__ ctrl) {
+                int32_t *__restrict__ outdeg, const Ctrl *ctrl) {
   grid_begin();
   const uint32_t m = ctrl->m_in;
   const uint64_t sentinel = (1ull << (2 * b)) - 1, mask = (1ull << b) - 1;
@@ -145,8 +145,8 @@ k_direct_orient(const uint64_t *__restrict__ keys, int b, const int32_t *__restr
     for (int q = 0; q < kUnroll; ++q) {
       ra[q] = rc[q] = 0;
       if (k[q] != sentinel) {
-        ra[q] = (uint32_t)__ldg(rank + (uint32_t)(k[q] >> b));
-        rc[q] = (uint32_t)__ldg(rank + (uint32_t)(k[q] & mask));
+        ra[q] = (uint32_t)load(rank + (uint32_t)(k[q] >> b));
+        rc[q] = (uint32_t)load(rank + (uint32_t)(k[q] & mask));
       }
     }
     int32_t at[kUnroll];
@@ -168,9 +168,9 @@ k_direct_orient(const uint64_t *__restrict__ keys, int b, const int32_t *__restr
 
 // The column array: each entry to its place in its owner's list.
 __global__ void __launch_bounds__(kThreads)
-k_direct_lists(const uint64_t *__restrict__ okeys, const int32_t *__restrict__ place, int b,
-               const int32_t *__restrict__ off, int32_t *__restrict__ col,
-               const Ctrl *__restrict__ ctrl) {
+k_direct_lists(const uint64_t *okeys, const int32_t *place, int b,
+               const int32_t *off, int32_t *__restrict__ col,
+               const Ctrl *ctrl) {
   grid_begin();
   if (aborted(ctrl)) return;  // a wait of this call ran out: off is not complete
   const uint32_t m = ctrl->m_in;
@@ -188,7 +188,7 @@ k_direct_lists(const uint64_t *__restrict__ okeys, const int32_t *__restrict__ p
     }
 #pragma unroll
     for (int q = 0; q < kUnroll; ++q)
-      if (k[q] != kHole) at[q] += __ldg(off + (uint32_t)(k[q] >> b));
+      if (k[q] != kHole) at[q] += load(off + (uint32_t)(k[q] >> b));
 #pragma unroll
     for (int q = 0; q < kUnroll; ++q)
       if (k[q] != kHole) col[at[q]] = (int32_t)((uint32_t)k[q] & mask);
@@ -208,11 +208,11 @@ constexpr int kHotRanks = 4096;
 constexpr int kGroupTile = kThreads * kUnroll;
 
 __global__ void __launch_bounds__(kThreads)
-k_direct_groups(const uint64_t *__restrict__ gkeys, int b, int32_t n,
-                const int32_t *__restrict__ goff, int32_t *__restrict__ gcnt,
+k_direct_groups(const uint64_t *gkeys, int b, int32_t n,
+                const int32_t *goff, int32_t *__restrict__ gcnt,
                 int32_t *__restrict__ part, int32_t *__restrict__ pskip,
-                const int2 *__restrict__ ldesc, int2 *__restrict__ desc,
-                const Ctrl *__restrict__ ctrl) {
+                const int2 *ldesc, int2 *__restrict__ desc,
+                const Ctrl *ctrl) {
   grid_begin();
   __shared__ int32_t s_hot[kHotRanks];  // the tile's edges per rank, then the counter's old value
   if (aborted(ctrl)) return;
@@ -237,11 +237,11 @@ k_direct_groups(const uint64_t *__restrict__ gkeys, int b, int32_t n,
       if (k[q] == kHole) continue;
       const uint32_t h = (uint32_t)(k[q] >> b) & mask;
       if (k[q] & kOwnEdge)
-        at[q] = __ldg(goff + h) + (int32_t)((k[q] & ~kOwnEdge) >> kSkipShift);
+        at[q] = load(goff + h) + (int32_t)((k[q] & ~kOwnEdge) >> kSkipShift);
       else if (h >= hot)
         at[q] = atomicAdd(&s_hot[h - hot], 1);
       else
-        at[q] = __ldg(goff + h + 1) - atomicSub(&gcnt[h], 1);
+        at[q] = load(goff + h + 1) - atomicSub(&gcnt[h], 1);
     }
     __syncthreads();
     for (int i = tid; i < kHotRanks; i += kThreads) {
@@ -253,11 +253,11 @@ k_direct_groups(const uint64_t *__restrict__ gkeys, int b, int32_t n,
     for (int q = 0; q < kUnroll; ++q) {
       if (k[q] == kHole) continue;
       const uint32_t h = (uint32_t)(k[q] >> b) & mask;
-      if (!(k[q] & kOwnEdge) && h >= hot) at[q] += __ldg(goff + h + 1) - s_hot[h - hot];
+      if (!(k[q] & kOwnEdge) && h >= hot) at[q] += load(goff + h + 1) - s_hot[h - hot];
       const uint32_t l = (uint32_t)k[q] & mask;
       const int32_t skip = k[q] & kOwnEdge ? 0 : (int32_t)(k[q] >> kSkipShift);
       part[at[q]] = (int32_t)l;
-      if (desc) desc[at[q]] = stream_desc(__ldg(ldesc + l), skip, 0xffffu);
+      if (desc) desc[at[q]] = stream_desc(load(ldesc + l), skip, 0xffffu);
       else pskip[at[q]] = skip;
     }
     __syncthreads();  // s_hot is emptied again

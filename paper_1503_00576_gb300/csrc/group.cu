@@ -216,7 +216,7 @@ __device__ __forceinline__ int32_t emit_list(const Emit &em, int32_t u, int32_t 
 // with E keys per lane (32 E >= d), dropping repeated entries; returns the
 // entries left.
 template <int E, bool EMIT>
-__device__ __forceinline__ int32_t warp_sort_list(const int32_t *__restrict__ col, int32_t b,
+__device__ __forceinline__ int32_t warp_sort_list(const int32_t *col, int32_t b,
                                                   int32_t d, long long w4, int32_t v,
                                                   const ListOut &o, const Emit &em) {
   const int lane = threadIdx.x & 31;
@@ -224,7 +224,7 @@ __device__ __forceinline__ int32_t warp_sort_list(const int32_t *__restrict__ co
 #pragma unroll
   for (int e = 0; e < E; ++e) {
     const int i = e * 32 + lane;
-    x[e] = i < d ? __ldg(col + b + i) : INT32_MAX;
+    x[e] = i < d ? load(col + b + i) : INT32_MAX;
   }
   warp_sort_regs<E>(x);
   const int r8 = (d + 7) & ~7;
@@ -281,11 +281,11 @@ __device__ __forceinline__ int32_t warp_sort_list(const int32_t *__restrict__ co
 // steps of a whole warp per list, which these lists (most of a random
 // geometric graph's) would leave half empty.
 template <bool EMIT>
-__device__ __forceinline__ int32_t half_sort_list(const int32_t *__restrict__ col, int32_t b,
+__device__ __forceinline__ int32_t half_sort_list(const int32_t *col, int32_t b,
                                                   int32_t d, long long w4, int32_t v,
                                                   const ListOut &o, const Emit &em) {
   const int lane = threadIdx.x & 31, i = lane & 15;
-  int32_t x = i < d ? __ldg(col + b + i) : INT32_MAX;
+  int32_t x = i < d ? load(col + b + i) : INT32_MAX;
 #pragma unroll
   for (int k = 2; k <= 16; k <<= 1) {
 #pragma unroll
@@ -422,8 +422,8 @@ __device__ int32_t cta_unique_copy(const int32_t *buf, int32_t d, int32_t *__res
 // 2.5M edges: 168 us, with the queue 64 us).
 template <bool EMIT>
 __global__ void __launch_bounds__(kListThreads)
-k_sort_lists(const int32_t *__restrict__ col, const int32_t *__restrict__ off,
-             const int32_t *__restrict__ voff, int32_t n, uint32_t per, ListOut o, GroupOut g,
+k_sort_lists(const int32_t *col, const int32_t *off,
+             const int32_t *voff, int32_t n, uint32_t per, ListOut o, GroupOut g,
              int32_t *__restrict__ queue) {
   grid_begin();
   Ctrl *ctrl = o.ctrl;
@@ -437,15 +437,15 @@ k_sort_lists(const int32_t *__restrict__ col, const int32_t *__restrict__ off,
     const bool exists = (uint32_t)lane < per && v < (uint32_t)n;
     int32_t b = 0, d = 0, w = 0, len = 0;
     if (exists) {
-      b = __ldg(off + v);
-      d = __ldg(off + v + 1) - b;
-      w = __ldg(voff + v);
+      b = load(off + v);
+      d = load(off + v + 1) - b;
+      w = load(voff + v);
     }
     const long long w4 = 4ll * w;  // first col4 entry of the list
     if (d > 0 && d <= 8) {
       int32_t x[8];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) x[i] = i < d ? __ldg(col + b + i) : INT32_MAX;
+      for (int i = 0; i < 8; ++i) x[i] = i < d ? load(col + b + i) : INT32_MAX;
       sort8(x);
       uint32_t reps = 0;  // bit i: entry i repeats entry i - 1
 #pragma unroll
@@ -553,9 +553,9 @@ __device__ __forceinline__ int32_t count_below(const int32_t *a, int32_t len, in
 // dropped on the way into col4.
 template <bool EMIT>
 __global__ void __launch_bounds__(kLongListThreads, kLongListBlocks)
-k_sort_long_lists(int32_t *col, const int32_t *__restrict__ off,
-                  const int32_t *__restrict__ voff, int32_t n, ListOut o, GroupOut g,
-                  const int32_t *__restrict__ queue) {
+k_sort_long_lists(int32_t *col, const int32_t *off,
+                  const int32_t *voff, int32_t n, ListOut o, GroupOut g,
+                  const int32_t *queue) {
   grid_begin();
   constexpr int G = kLongListThreads;
   __shared__ int32_t s_buf[kCtaSortMax];
@@ -572,8 +572,8 @@ k_sort_long_lists(int32_t *col, const int32_t *__restrict__ off,
     __syncthreads();
     const uint32_t i = s_i;
     if (i >= n_cta) break;
-    const int32_t v = __ldg(queue + ((uint32_t)n - 1u - i));
-    const int32_t b = __ldg(off + v), d = __ldg(off + v + 1) - b, w = __ldg(voff + v);
+    const int32_t v = load(queue + ((uint32_t)n - 1u - i));
+    const int32_t b = load(off + v), d = load(off + v + 1) - b, w = load(voff + v);
     int32_t *dst = o.col4 + 4ll * w;
     const int r8 = (d + 7) & ~7;
     int32_t len;
@@ -662,8 +662,8 @@ k_sort_long_lists(int32_t *col, const int32_t *__restrict__ off,
     if (lane == 0) i = atomicAdd(&ctrl->next_warp_list, 1u);
     i = __shfl_sync(kFull, i, 0);
     if (i >= n_warp) break;
-    const int32_t v = __ldg(queue + i);
-    const int32_t b = __ldg(off + v), d = __ldg(off + v + 1) - b, w = __ldg(voff + v);
+    const int32_t v = load(queue + i);
+    const int32_t b = load(off + v), d = load(off + v + 1) - b, w = load(voff + v);
     const int32_t len = d <= 128   ? warp_sort_list<4, EMIT>(col, b, d, 4ll * w, v, o, em)
                         : d <= 256 ? warp_sort_list<8, EMIT>(col, b, d, 4ll * w, v, o, em)
                         : d <= 512 ? warp_sort_list<16, EMIT>(col, b, d, 4ll * w, v, o, em)
@@ -682,18 +682,18 @@ k_sort_long_lists(int32_t *col, const int32_t *__restrict__ off,
 // the repeats, deg[v] -= dcorr[rank[v]] (caller ids).  Nothing when no list
 // held a repeat.
 __global__ void __launch_bounds__(kListThreads)
-k_fix_repeats(const int32_t *__restrict__ off, int32_t n, const int32_t *__restrict__ dcorr,
-              const int32_t *__restrict__ rank, const Ctrl *ctrl, int32_t *__restrict__ row,
+k_fix_repeats(const int32_t *off, int32_t n, const int32_t *dcorr,
+              const int32_t *rank, const Ctrl *ctrl, int32_t *__restrict__ row,
               int32_t *__restrict__ deg) {
   grid_begin();
   if (aborted(ctrl) || ctrl->dups == 0u) return;
   const int lane = threadIdx.x & 31;
   const uint32_t first = blockIdx.x * kListThreads + threadIdx.x;
   const uint32_t stride = gridDim.x * kListThreads;
-  for (uint32_t v = first; v < (uint32_t)n; v += stride) deg[v] -= __ldg(dcorr + __ldg(rank + v));
+  for (uint32_t v = first; v < (uint32_t)n; v += stride) deg[v] -= load(dcorr + load(rank + v));
   if (!row) return;
   for (uint32_t v = first >> 5; v < (uint32_t)n; v += stride >> 5) {
-    const int32_t b = __ldg(off + v), e = __ldg(off + v + 1);
+    const int32_t b = load(off + v), e = load(off + v + 1);
     for (int32_t i = b + lane; i < e; i += 32) row[i] = (int32_t)v;
   }
 }
@@ -733,10 +733,10 @@ __device__ __forceinline__ void split_edge(int32_t u, int32_t v, int64_t du, int
 // of the streamed blocks less.
 template <bool WHOLE>
 __global__ void __launch_bounds__(kGroupThreads)
-k_group_keys(const int32_t *__restrict__ row, const int32_t *__restrict__ col4,
-             const int32_t *__restrict__ off, const int2 *__restrict__ ldesc,
-             const int32_t *__restrict__ len, int b, int passes, int32_t heavy_ratio_pct,
-             Ctrl *__restrict__ ctrl, uint64_t *__restrict__ gkeys,
+k_group_keys(const int32_t *row, const int32_t *col4,
+             const int32_t *off, const int2 *ldesc,
+             const int32_t *len, int b, int passes, int32_t heavy_ratio_pct,
+             Ctrl *ctrl, uint64_t *__restrict__ gkeys,
              uint32_t *__restrict__ hist) {
   grid_begin();
   constexpr int UNROLL = WHOLE ? kGroupUnroll : 2 * kGroupUnroll;
@@ -759,12 +759,12 @@ k_group_keys(const int32_t *__restrict__ row, const int32_t *__restrict__ col4,
 #pragma unroll
     for (int q = 0; q < UNROLL; ++q) {
       const uint32_t e = e0 + q * stride;
-      u[q] = e < m ? __ldg(row + e) : 0;
+      u[q] = e < m ? load(row + e) : 0;
     }
 #pragma unroll
     for (int q = 0; q < UNROLL; ++q) {
-      ub[q] = __ldg(off + u[q]);
-      const int2 ld = __ldg(ldesc + u[q]);  // {first col4 word, length}
+      ub[q] = load(off + u[q]);
+      const int2 ld = load(ldesc + u[q]);  // {first col4 word, length}
       ue[q] = ub[q] + ld.y;
       uw[q] = ld.x;
     }
@@ -772,14 +772,14 @@ k_group_keys(const int32_t *__restrict__ row, const int32_t *__restrict__ col4,
 #pragma unroll
     for (int q = 0; q < UNROLL; ++q) {
       const uint32_t e = e0 + q * stride;
-      v[q] = e < m ? __ldg(col4 + 4ll * uw[q] + ((int32_t)e - ub[q])) : 0;
+      v[q] = e < m ? load(col4 + 4ll * uw[q] + ((int32_t)e - ub[q])) : 0;
     }
     uint64_t key[UNROLL];
     uint32_t kept = 0;
     if (WHOLE) {
       int32_t vd[UNROLL];
 #pragma unroll
-      for (int q = 0; q < UNROLL; ++q) vd[q] = __ldg(ldesc + v[q]).y;
+      for (int q = 0; q < UNROLL; ++q) vd[q] = load(ldesc + v[q]).y;
 #pragma unroll
       for (int q = 0; q < UNROLL; ++q) {
         const uint32_t e = e0 + q * stride;
@@ -846,8 +846,8 @@ k_group_keys(const int32_t *__restrict__ row, const int32_t *__restrict__ col4,
 // intersections lie wholly inside H (what a dense count of the hub block
 // A_HH would take over, Sec. VI).  One warp per vertex h.
 __global__ void __launch_bounds__(kGroupThreads)
-k_work(const int32_t *__restrict__ off, const int32_t *__restrict__ goff,
-       const int32_t *__restrict__ part, const int32_t *__restrict__ pskip, int32_t n,
+k_work(const int32_t *off, const int32_t *goff,
+       const int32_t *part, const int32_t *pskip, int32_t n,
        Ctrl *ctrl, uint32_t shard, uint32_t shards) {
   grid_begin();
   if (aborted(ctrl)) return;
@@ -857,16 +857,16 @@ k_work(const int32_t *__restrict__ off, const int32_t *__restrict__ goff,
   for (uint32_t h = (blockIdx.x * kGroupThreads + threadIdx.x) >> 5; h < (uint32_t)n;
        h += warps) {
     if (h % shards != shard) continue;  // another part's group (uniform per warp)
-    const unsigned long long dh = (unsigned long long)(__ldg(off + h + 1) - __ldg(off + h));
-    const int32_t pb = __ldg(goff + h), pe = __ldg(goff + h + 1);
+    const unsigned long long dh = (unsigned long long)(load(off + h + 1) - load(off + h));
+    const int32_t pb = load(goff + h), pe = load(goff + h + 1);
     if (lane == 0) {
       if (pe > pb) inserts += dh;
       dmax = dh > dmax ? dh : dmax;
     }
     for (int32_t i = pb + lane; i < pe; i += 32) {
-      const int32_t l = __ldg(part + i);
-      const int32_t dfull = __ldg(off + l + 1) - __ldg(off + l);
-      const int32_t ds = max(dfull - 8 * __ldg(pskip + i), 0);  // entries streamed
+      const int32_t l = load(part + i);
+      const int32_t dfull = load(off + l + 1) - load(off + l);
+      const int32_t ds = max(dfull - 8 * load(pskip + i), 0);  // entries streamed
       const unsigned long long dl = (unsigned long long)ds;
       lookups += dl;
       merge += dh + (unsigned long long)dfull;

@@ -208,25 +208,25 @@ __device__ __forceinline__ int32_t hub_candidate(int32_t Hmax, int k) {
 }
 
 __global__ void __launch_bounds__(256)
-k_hub_estimate(const int32_t *__restrict__ off, const int32_t *__restrict__ col, int32_t n,
+k_hub_estimate(const int32_t *off, const int32_t *col, int32_t n,
                int32_t Hmax, int64_t min_edges, int32_t cap, Ctrl *ctrl) {
   grid_begin();
   if (aborted(ctrl)) return;
-  if ((int64_t)ctrl->m - (int64_t)__ldg(off + (n - Hmax)) < min_edges) return;
+  if ((int64_t)ctrl->m - (int64_t)load(off + (n - Hmax)) < min_edges) return;
   const int lane = threadIdx.x & 31;
   const uint32_t warps = gridDim.x * (blockDim.x / 32);
   unsigned long long acc[4] = {0, 0, 0, 0};
   for (uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < (uint32_t)Hmax;
        w += warps) {
     const int32_t u = n - Hmax + (int32_t)w;
-    const int32_t du = __ldg(off + u + 1) - __ldg(off + u);
+    const int32_t du = load(off + u + 1) - load(off + u);
     // the smallest candidate holding u (and so every forward neighbour)
     int k = 3;
     while (k > 0 && n - hub_candidate(Hmax, k - 1) <= u) --k;
     unsigned long long sum = 0;
     for (int32_t i = lane; i < du; i += 32) {
-      const int32_t v = __ldg(col + __ldg(off + u) + i);
-      const int32_t dv = __ldg(off + v + 1) - __ldg(off + v);
+      const int32_t v = load(col + load(off + u) + i);
+      const int32_t dv = load(off + v + 1) - load(off + v);
       sum += (unsigned long long)min(min(du, dv), cap);
     }
 #pragma unroll
@@ -253,7 +253,7 @@ k_hub_estimate(const int32_t *__restrict__ off, const int32_t *__restrict__ col,
 // 10.5M edges 1.69 1.82 3.15 / 2.67 2.15 3.27, scale 20 of 16.8M 2.57 2.71 4.05
 // / 3.38 2.98 4.20, scale 21 of 91M 15.8 15.4 16.3 / 21.4 20.4 20.9, scale 24
 // of 180M 30.9 30.9 31.7 / 38.6 38.3 38.6.
-__global__ void k_hub_decide(const int32_t *__restrict__ off, int32_t n, int32_t Hmax,
+__global__ void k_hub_decide(const int32_t *off, int32_t n, int32_t Hmax,
                              int64_t min_edges, double ps_per_lookup, Ctrl *ctrl) {
   grid_begin();
   if (aborted(ctrl)) return;
@@ -266,7 +266,7 @@ __global__ void k_hub_decide(const int32_t *__restrict__ off, int32_t n, int32_t
     const int32_t h = hub_candidate(Hmax, k);
     const double x = (double)h / 16384.0;
     const double gain = (double)inside * ms_per_lookup - (0.15 + 1.55 * x * x * x);
-    const int64_t edges = (int64_t)ctrl->m - (int64_t)__ldg(off + (n - h));
+    const int64_t edges = (int64_t)ctrl->m - (int64_t)load(off + (n - h));
     if (h > 0 && edges >= min_edges && gain > best) {
       best = gain;
       H = h;
@@ -296,7 +296,7 @@ k_hub_zero(uint8_t *__restrict__ A, int32_t Hmax, const Ctrl *ctrl) {
 // A(u - lo, v - lo) = A(v - lo, u - lo) = 1 for every forward edge of H
 // (the matrix was zeroed before).  One warp per vertex of H.
 __global__ void __launch_bounds__(256)
-k_hub_scatter(const int2 *__restrict__ ldesc, const int32_t *__restrict__ col4, int32_t n,
+k_hub_scatter(const int2 *ldesc, const int32_t *col4, int32_t n,
               int32_t pitch, const Ctrl *ctrl, uint8_t *__restrict__ A) {
   grid_begin();
   if (aborted(ctrl) || !ctrl->hub_on) return;
@@ -305,11 +305,11 @@ k_hub_scatter(const int2 *__restrict__ ldesc, const int32_t *__restrict__ col4, 
   const uint32_t warps = gridDim.x * (blockDim.x / 32);
   for (uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < (uint32_t)H; w += warps) {
     const int32_t u = lo + (int32_t)w;
-    const int2 ld = __ldg(ldesc + u);  // {first col4 word, length}
+    const int2 ld = load(ldesc + u);  // {first col4 word, length}
     const int32_t d = ld.y;
     const int32_t *list = col4 + 4ll * ld.x;
     for (int32_t i = lane; i < d; i += 32) {
-      const int32_t v = __ldg(list + i) - lo;  // > u - lo >= 0
+      const int32_t v = load(list + i) - lo;  // > u - lo >= 0
       A[(size_t)w * pitch + v] = kOne;
       A[(size_t)v * pitch + w] = kOne;
     }
@@ -321,7 +321,7 @@ k_hub_scatter(const int2 *__restrict__ ldesc, const int32_t *__restrict__ col4, 
 // used); r(i) += masked row (and column) sums.  Warp 0 lane 0 issues the TMA
 // loads, warp 1 lane 0 the MMAs; all four warps read the accumulator back.
 __global__ void __launch_bounds__(kHubThreads, 2)
-k_hub_gemm(const __grid_constant__ CUtensorMap amap, const uint8_t *__restrict__ A,
+k_hub_gemm(const __grid_constant__ CUtensorMap amap, const uint8_t *A,
            int32_t pitch, Ctrl *ctrl, uint32_t *__restrict__ r) {
   grid_begin();
   extern __shared__ uint8_t smem_raw[];
@@ -449,7 +449,7 @@ k_hub_gemm(const __grid_constant__ CUtensorMap amap, const uint8_t *__restrict__
 // T += (sum of r) / 6; r must be even and its sum a multiple of 6.  One
 // block.
 __global__ void __launch_bounds__(1024)
-k_hub_finish(const uint32_t *__restrict__ r, Ctrl *ctrl, int64_t *t) {
+k_hub_finish(const uint32_t *r, Ctrl *ctrl, int64_t *t) {
   grid_begin();
   __shared__ unsigned long long s_sum[32];
   __shared__ uint32_t s_odd;
@@ -460,7 +460,7 @@ k_hub_finish(const uint32_t *__restrict__ r, Ctrl *ctrl, int64_t *t) {
   unsigned long long sum = 0;
   uint32_t odd = 0;
   for (int32_t v = threadIdx.x; v < H; v += blockDim.x) {
-    const uint32_t x = __ldg(r + v);
+    const uint32_t x = load(r + v);
     sum += x;
     odd |= x & 1u;
     if (t && x) t[lo + v] += (int64_t)(x >> 1);

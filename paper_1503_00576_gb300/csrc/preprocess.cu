@@ -210,7 +210,7 @@ __device__ __forceinline__ uint64_t pair_key(int32_t u, int32_t v, int32_t lim, 
 // written once here), so that the degree array stays in L2 for the atomics
 // (-0.27 ms of 2.55 at R-MAT scale 24).
 __global__ void __launch_bounds__(kCanonThreads)
-k_canon(const int32_t *__restrict__ src, const int32_t *__restrict__ dst, uint32_t m_in,
+k_canon(const int32_t *src, const int32_t *dst, uint32_t m_in,
         int32_t n, int b, uint64_t *__restrict__ keys, int32_t *__restrict__ deg, Ctrl *ctrl) {
   grid_begin();
   const uint64_t sentinel = (1ull << (2 * b)) - 1;  // > every valid key; 2b <= 62
@@ -247,8 +247,8 @@ k_canon(const int32_t *__restrict__ src, const int32_t *__restrict__ dst, uint32
 // dropped so the other graphs of the union are counted exactly.  Also zeroes
 // the totals that k_batch_totals adds to.
 __global__ void __launch_bounds__(kCanonThreads)
-k_canon_batch(const int32_t *__restrict__ src, const int32_t *__restrict__ dst, uint32_t m_in,
-              int b, const BatchDesc *__restrict__ batch, int32_t num_graphs_bound,
+k_canon_batch(const int32_t *src, const int32_t *dst, uint32_t m_in,
+              int b, const BatchDesc *batch, int32_t num_graphs_bound,
               unsigned long long *__restrict__ totals, uint64_t *__restrict__ keys,
               int32_t *__restrict__ deg, Ctrl *ctrl) {
   grid_begin();
@@ -256,7 +256,7 @@ k_canon_batch(const int32_t *__restrict__ src, const int32_t *__restrict__ dst, 
   const uint64_t sentinel = (1ull << (2 * b)) - 1;
   const int32_t ng = batch->num_graphs;
   const int32_t *eo = batch->edge_off, *vo = batch->voff;
-  const uint32_t m = min((uint32_t)__ldg(eo + ng), m_in);
+  const uint32_t m = min((uint32_t)load(eo + ng), m_in);
   const int lane = threadIdx.x & 31;
   const uint32_t first = blockIdx.x * kCanonThreads + threadIdx.x;
   if (first == 0) ctrl->m_in = m;
@@ -277,18 +277,18 @@ k_canon_batch(const int32_t *__restrict__ src, const int32_t *__restrict__ dst, 
     int32_t g = 0, hi = ng;  // the last graph with eo[g] <= i0
     while (hi - g > 1) {
       const int32_t mid = (g + hi) >> 1;
-      if ((uint32_t)__ldg(eo + mid) <= i0) g = mid; else hi = mid;
+      if ((uint32_t)load(eo + mid) <= i0) g = mid; else hi = mid;
     }
-    uint32_t end = (uint32_t)__ldg(eo + g + 1);
-    int32_t shift = __ldg(vo + g), lim = __ldg(vo + g + 1) - shift;
+    uint32_t end = (uint32_t)load(eo + g + 1);
+    int32_t shift = load(vo + g), lim = load(vo + g + 1) - shift;
 #pragma unroll
     for (int q = 0; q < kCanonUnroll; ++q) {
       const uint32_t i = i0 + 32 * q + lane;
       if (i >= m) break;
       if (i >= end) {
-        do end = (uint32_t)__ldg(eo + ++g + 1); while (i >= end);
-        shift = __ldg(vo + g);
-        lim = __ldg(vo + g + 1) - shift;
+        do end = (uint32_t)load(eo + ++g + 1); while (i >= end);
+        shift = load(vo + g);
+        lim = load(vo + g + 1) - shift;
       }
       bool bad = false;
       __stcs(reinterpret_cast<unsigned long long *>(keys) + i,
@@ -339,7 +339,7 @@ __device__ __forceinline__ void radix_out(uint64_t key, uint32_t pos, void *__re
 // ballots): only for the first pass of a sort whose input order does not
 // matter.
 template <int MODE, bool FULL, bool UNSTABLE>
-__device__ __forceinline__ void radix_tile(RadixShared &S, const uint64_t *__restrict__ in,
+__device__ __forceinline__ void radix_tile(RadixShared &S, const uint64_t *in,
                                            void *__restrict__ out, uint32_t n_keys,
                                            uint32_t tile, uint32_t gofs, int shift,
                                            uint32_t col_mask, uint32_t *__restrict__ row_out,
@@ -490,10 +490,10 @@ __device__ __forceinline__ void radix_tile(RadixShared &S, const uint64_t *__res
 
 template <int MODE>
 __global__ void __launch_bounds__(kSortThreads, 4)
-k_radix_pass(const uint64_t *__restrict__ in, void *__restrict__ out, uint32_t n_keys_bound,
-             const uint32_t *__restrict__ n_keys_dev, int shift, uint32_t col_mask,
+k_radix_pass(const uint64_t *in, void *__restrict__ out, uint32_t n_keys_bound,
+             const uint32_t *n_keys_dev, int shift, uint32_t col_mask,
              uint32_t *__restrict__ row_out, int owner_shift, int32_t *outdeg,
-             const uint32_t *__restrict__ hist, unsigned long long *__restrict__ status,
+             const uint32_t *hist, unsigned long long *__restrict__ status,
              uint32_t *ticket, Ctrl *ctrl, int unstable) {
   grid_begin();
   constexpr int WARPS = kSortThreads / 32, TILE = kSortTile;
@@ -543,7 +543,7 @@ k_radix_pass(const uint64_t *__restrict__ in, void *__restrict__ out, uint32_t n
 // the highest, adjacent ids.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kCanonThreads)
-k_rank_keys(const int32_t *__restrict__ deg, int32_t n, int b, int passes,
+k_rank_keys(const int32_t *deg, int32_t n, int b, int passes,
             uint64_t *__restrict__ vkeys, uint32_t *__restrict__ hist) {
   grid_begin();
   __shared__ uint32_t sh[kMaxRankPasses * 256];
@@ -551,7 +551,7 @@ k_rank_keys(const int32_t *__restrict__ deg, int32_t n, int b, int passes,
   __syncthreads();
   const uint32_t stride = gridDim.x * kCanonThreads;
   for (uint32_t v = blockIdx.x * kCanonThreads + threadIdx.x; v < (uint32_t)n; v += stride) {
-    const uint32_t d = (uint32_t)__ldg(deg + v);
+    const uint32_t d = (uint32_t)load(deg + v);
     vkeys[v] = ((uint64_t)d << b) | v;
     for (int p = 0; p < passes; ++p) atomicAdd(&sh[p * 256 + ((d >> (8 * p)) & 255u)], 1u);
   }
@@ -564,8 +564,8 @@ k_rank_keys(const int32_t *__restrict__ deg, int32_t n, int b, int passes,
 // orient: compact the keys, orient by rank (= (degree, id) order)
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kOrientThreads, 4)
-k_orient(const uint64_t *__restrict__ keys, int b,
-         const int32_t *__restrict__ rank, uint64_t *__restrict__ okeys,
+k_orient(const uint64_t *keys, int b,
+         const int32_t *rank, uint64_t *__restrict__ okeys,
          uint32_t *__restrict__ hist2, int passes2, unsigned long long *status, Ctrl *ctrl) {
   grid_begin();
   constexpr int KPT = kOrientKeysPerThread, TILE = kOrientTile;
@@ -636,8 +636,8 @@ k_orient(const uint64_t *__restrict__ keys, int b,
 #pragma unroll
     for (int i = 0; i < HALF; ++i) {
       const bool keep = (flags >> (h0 + i)) & 1u;
-      ra[i] = keep ? (uint32_t)__ldg(rank + (uint32_t)(k[h0 + i] >> b)) : 0u;
-      rc[i] = keep ? (uint32_t)__ldg(rank + (uint32_t)(k[h0 + i] & mask)) : 0u;
+      ra[i] = keep ? (uint32_t)load(rank + (uint32_t)(k[h0 + i] >> b)) : 0u;
+      rc[i] = keep ? (uint32_t)load(rank + (uint32_t)(k[h0 + i] & mask)) : 0u;
     }
 #pragma unroll
     for (int i = 0; i < HALF; ++i) {
@@ -745,7 +745,7 @@ k_offsets(const ScanArgs a) {
   if (whole) {
 #pragma unroll
     for (int i = 0; i < IPT; i += 4) {
-      const int4 c = __ldg(reinterpret_cast<const int4 *>(a.counts + first + i));
+      const int4 c = load(reinterpret_cast<const int4 *>(a.counts + first + i));
       d[i] = c.x;
       d[i + 1] = c.y;
       d[i + 2] = c.z;
@@ -753,13 +753,13 @@ k_offsets(const ScanArgs a) {
     }
   } else {
 #pragma unroll
-    for (int i = 0; i < IPT; ++i) d[i] = first + i < n ? __ldg(a.counts + first + i) : 0;
+    for (int i = 0; i < IPT; ++i) d[i] = first + i < n ? load(a.counts + first + i) : 0;
   }
   uint64_t sum = 0;
 #pragma unroll
   for (int i = 0; i < IPT; ++i) {
     const uint32_t v = first + i;
-    if (KIND == kScanGroups && a.own && v < n) d[i] += __ldg(a.own + v);
+    if (KIND == kScanGroups && a.own && v < n) d[i] += load(a.own + v);
     sum += KIND == kScanLists
                ? ((uint64_t)(uint32_t)d[i] << kBlockBits) + ((uint32_t)(d[i] + 7) >> 3)
                : (uint64_t)(uint32_t)d[i];
@@ -820,7 +820,7 @@ k_offsets(const ScanArgs a) {
     for (int i = 0; i < IPT; ++i) {
       const uint32_t v = first + i;
       int32_t dh = 0;
-      if (v < n && d[i] > 0 && v % a.shards == a.shard) dh = __ldg(a.ldesc + v).y;
+      if (v < n && d[i] > 0 && v % a.shards == a.shard) dh = load(a.ldesc + v).y;
       // a warp takes a group only if both its list and its partner count are
       // short: one warp streaming thousands of partners would finish last
       const bool is_warp =
