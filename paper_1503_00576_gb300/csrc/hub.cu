@@ -434,9 +434,13 @@ k_hub_gemm(const __grid_constant__ CUtensorMap amap, const uint8_t *A,
       const int32_t cs = S.col[0][tid] + S.col[1][tid] + S.col[2][tid] + S.col[3][tid];
       if (cs) atomicAdd(r + J * kHubTile + tid, (uint32_t)cs);
     }
-    if (!ok && tid == 0) atomicOr(&ctrl->err, kErrTimeout);
-    __syncthreads();  // S.col and the accumulator are written again
-    if (S.abort) break;  // uniform: nothing writes it between the barriers
+    // a vote, so that the block goes on or leaves as one: the next tile's loads
+    // and products may set S.abort while a slower thread still stands here.
+    // Also the barrier before S.col and the accumulator are written again.
+    if (__syncthreads_or(!ok || S.abort)) {
+      if (tid == 0) atomicOr(&ctrl->err, kErrTimeout);
+      break;
+    }
   }
   if (warp == 1) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");

@@ -36,3 +36,16 @@ def test_every_kernel_waits_first(path):
     assert len(kernels) == len(re.findall(r"__global__", text))
     for name, first in kernels:
         assert first.strip() == "grid_begin();", name
+
+
+def test_hub_product_leaves_its_tile_loop_by_a_vote():
+    """S.abort is set by the thread that loads and the one that multiplies, in
+    the next tile as soon as they have passed a tile's last barrier: a thread
+    that tested it behind that barrier could leave a block that goes on."""
+    text = code(os.path.join(CSRC, "hub.cu"))
+    body = text[text.index("k_hub_gemm("):text.index("k_hub_finish(")]
+    loop = body[body.index("for (uint32_t tile"):body.index("tcgen05.dealloc")]
+    reads = re.findall(r"[^\n]*S\.abort(?!\s*=)[^\n]*", loop)
+    assert [r.strip() for r in reads] == [
+        "const bool ok = mbar_wait(&S.done, parity) && !S.abort;",  # before the tile's barriers
+        "if (__syncthreads_or(!ok || S.abort)) {"]
