@@ -430,7 +430,7 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
                        st_scan2, &ctrl->tile_ticket[kTicketGroupScan], ctrl, st, shard, shards);
   // per vertex, each partner's stream: written with the partners, or from them
   // into the group sort's other buffer
-  const bool desc_ready = direct && t_out && !bits_on;
+  const bool desc_ready = direct && t_out && !bits_on && L.has_desc;
   int2 *desc = reinterpret_cast<int2 *>(desc_ready ? ws + L.desc : (unsigned char *)gin);
   if (direct)
     launch_direct_groups(gin, m, b, n, goff, gcnt, part, pskip, ldesc, desc_ready ? desc : nullptr,
@@ -519,8 +519,8 @@ tc_status count_impl(const int32_t *src, const int32_t *dst, int64_t m, int32_t 
     *total = 0;
     return set_status(TC_OK);
   }
-  const Layout L =
-      make_layout(m, n, true, current_tuning().hub_vertices, false, t_out != nullptr);
+  const int32_t hub_vertices = current_tuning().hub_vertices;
+  Layout L = make_layout(m, n, true, hub_vertices, false, t_out != nullptr);
   if (ws_user) {
     if (ws_bytes < L.total)
       return set_status(TC_ERR_INVALID_ARG, "workspace has %zu bytes, needs %zu", ws_bytes,
@@ -532,13 +532,20 @@ tc_status count_impl(const int32_t *src, const int32_t *dst, int64_t m, int32_t 
   }
   keep_pool_memory();
   void *ws = nullptr;
-  TC_CUDA(dev_alloc_async(&ws, L.total, st), "workspace allocation");
+  cudaError_t e = dev_alloc_async(&ws, L.total, st);
+  if (e == cudaErrorMemoryAllocation && t_out && (L.has_bits || L.has_desc)) {
+    // what makes per-vertex counts faster is not worth refusing them
+    cudaGetLastError();
+    L = make_layout(m, n, true, hub_vertices, false, true, /*lean=*/true);
+    e = dev_alloc_async(&ws, L.total, st);
+  }
+  if (e != cudaSuccess) return cuda_fail(e, "workspace allocation");
   s = run_core(src, dst, m, n, st, (unsigned char *)ws, L, t_out, deg_out, total, nullptr, true,
                shard, shards);
   const tc_status keep = s;
   char detail[256];
   memcpy(detail, t_detail, sizeof(detail));
-  cudaError_t e = cudaFreeAsync(ws, st);
+  e = cudaFreeAsync(ws, st);
   if (keep != TC_OK) {
     t_last = keep;
     memcpy(t_detail, detail, sizeof(detail));

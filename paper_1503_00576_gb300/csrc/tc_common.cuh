@@ -261,10 +261,13 @@ struct Layout {
   size_t hub;  // dense hub block (0 bytes unless the layout asked for it)
   // bitmaps (single graphs of at least kBitMinPairs pairs): without per-vertex
   // counts the records take the place of t_rank and the bitmaps that of the
-  // group sort's free key buffer; with them both have their own
-  // per-vertex runs that sort by counting have each partner's stream in `desc`
-  // (others in the group sort's free key buffer)
+  // group sort's free key buffer; with them both have their own.  Per-vertex
+  // runs that sort by counting have each partner's stream in `desc` (others in
+  // the group sort's free key buffer).  That is up to 8 bytes per pair more than
+  // without per-vertex counts; a lean layout has neither, and takes as much as
+  // one without.
   size_t desc;
+  bool has_desc;
   bool has_bits;
   size_t bit_rec, bits;
   uint32_t bit_slots;
@@ -306,7 +309,7 @@ inline bool hub_enabled(int32_t n, int b) { return n >= kHubMinVertices && 2 * b
 
 inline Layout make_layout(int64_t m_in, int32_t n, bool with_hub = false,
                           int32_t hub_vertices = kHubSize, bool batch = false,
-                          bool per_vertex = false) {
+                          bool per_vertex = false, bool lean = false) {
   Layout L{};
   size_t p = 0;
   auto take = [&](size_t bytes) {
@@ -332,7 +335,8 @@ inline Layout make_layout(int64_t m_in, int32_t n, bool with_hub = false,
   L.gcnt = take(sizeof(int32_t) * nv);
   L.dcorr = take(sizeof(int32_t) * nv);
   L.t_rank = take(sizeof(int64_t) * nv);
-  L.has_bits = !batch && m_in >= (per_vertex ? kBitMinPairs<true> : kBitMinPairs<false>);
+  L.has_bits =
+      !batch && !lean && m_in >= (per_vertex ? kBitMinPairs<true> : kBitMinPairs<false>);
   const uint64_t slots = m / (kBitCols / 32);  // two bitmaps each, in 8 m bytes
   L.bit_slots = (uint32_t)(slots < kBitMaxSlots ? slots : kBitMaxSlots);
   L.bit_rec = per_vertex && L.has_bits ? take(sizeof(uint32_t) * nv) : L.t_rank;
@@ -353,7 +357,8 @@ inline Layout make_layout(int64_t m_in, int32_t n, bool with_hub = false,
   // elements, since each non-empty list adds at most 7
   L.col4 = take(sizeof(int32_t) * (m + 7 * (nv < m ? nv : m)));
   L.bits = per_vertex && L.has_bits ? take((size_t)L.bit_slots * (kBitCols / 4)) : 0;
-  L.desc = per_vertex && m_in <= kDirectMaxPairs ? take(sizeof(uint64_t) * m) : 0;
+  L.has_desc = per_vertex && !lean && m_in <= kDirectMaxPairs;
+  L.desc = L.has_desc ? take(sizeof(uint64_t) * m) : 0;
   const bool hub = with_hub && hub_enabled(n, id_bits(n > 0 ? n : 1));
   const size_t H = (size_t)hub_vertices;
   L.hub = take(hub ? H * H + 4 * H : 0);
