@@ -28,10 +28,20 @@ extern "C" {
  *   unpublished_tile  >= 0: the radix-sort tile with this number never
  *                     publishes its status, so the tiles after it wait on a
  *                     word that nothing sets and give up after spin_limit
- *                     iterations; < 0: every tile publishes (default)
+ *                     iterations (meanwhile every call sorts by radix passes,
+ *                     the small ones too that otherwise sort by counting);
+ *                     < 0: every tile publishes (default)
  * Synchronises the device.  Returns TC_ERR_CUDA if the device rejects it.
  */
 tc_status tc_debug_set_wait_limit(uint32_t spin_limit, int32_t unpublished_tile);
+
+/*
+ * The same for the offset scans, the waits that every call has: tile `tile`
+ * (4096 vertices each) of the scan of the forward lists (scan 0) or of the
+ * partner groups (scan 1) never publishes its status; tile < 0: all of both
+ * do (default).  Synchronises the device.
+ */
+tc_status tc_debug_set_unpublished_scan(int32_t scan, int32_t tile);
 
 /*
  * Allocation failures, injected on the host: of the library's next device
@@ -42,7 +52,7 @@ tc_status tc_debug_set_wait_limit(uint32_t spin_limit, int32_t unpublished_tile)
  */
 tc_status tc_debug_fail_allocations(int32_t skip, int32_t count);
 
-/* Default wait limit and no unpublished tile on the current device, and no
+/* Default wait limit and no unpublished tiles on the current device, and no
  * injected allocation failures. */
 tc_status tc_debug_reset(void);
 

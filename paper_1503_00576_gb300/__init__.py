@@ -59,7 +59,8 @@ EXPORTS = ("tc_count", "tc_count_per_vertex", "tc_count_part", "tc_count_per_ver
            "tc_engine_destroy", "tc_count_work", "tc_count_work_part", "tc_count_noalloc",
            "tc_last_error", "tc_status_string", "tc_last_error_detail", "tc_launch_count",
            "tc_profile_enable", "tc_profile_read", "tc_phase_name",
-           "tc_debug_set_wait_limit", "tc_debug_fail_allocations", "tc_debug_reset")
+           "tc_debug_set_wait_limit", "tc_debug_set_unpublished_scan",
+           "tc_debug_fail_allocations", "tc_debug_reset")
 
 
 class Work(ctypes.Structure):
@@ -135,6 +136,7 @@ def _bind(lib):
         "tc_profile_read": ([c.POINTER(c.c_double), c.POINTER(u64), c.c_int], None),
         "tc_phase_name": ([c.c_int], c.c_char_p),
         "tc_debug_set_wait_limit": ([c.c_uint32, i32], c.c_int),
+        "tc_debug_set_unpublished_scan": ([i32, i32], c.c_int),
         "tc_debug_fail_allocations": ([i32, i32], c.c_int),
         "tc_debug_reset": ([], c.c_int),
     }
@@ -592,6 +594,15 @@ def tc_debug_set_wait_limit(spin_limit: int, unpublished_tile: int = -1, device=
         _check(load_library().tc_debug_set_wait_limit(spin_limit, unpublished_tile))
 
 
+def tc_debug_set_unpublished_scan(scan: int, tile: int, device=None) -> None:
+    """Failure-path test hook (include/tc_debug.h): tile `tile` of the offset
+    scan of the forward lists (scan 0) or of the partner groups (scan 1) never
+    publishes (tile < 0: every tile of both does)."""
+    torch = _torch()
+    with torch.cuda.device(device if device is not None else torch.cuda.current_device()):
+        _check(load_library().tc_debug_set_unpublished_scan(scan, tile))
+
+
 def tc_debug_fail_allocations(skip: int, count: int) -> None:
     """Failure-path test hook: of the library's next device allocations the
     first `skip` succeed and the `count` after them fail (TC_ERR_OOM)."""
@@ -599,7 +610,7 @@ def tc_debug_fail_allocations(skip: int, count: int) -> None:
 
 
 def tc_debug_reset(device=None) -> None:
-    """Undo both failure-path hooks (wait limit on `device`)."""
+    """Undo the failure-path hooks (those of the waits on `device`)."""
     torch = _torch()
     with torch.cuda.device(device if device is not None else torch.cuda.current_device()):
         _check(load_library().tc_debug_reset())

@@ -48,10 +48,12 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 
-// Bound of every spin-wait of this file, and the radix-pass tile that never
-// publishes (none by default).  Only the failure-path tests change them.
+// Bound of every spin-wait of this file, and the tiles that never publish
+// (none by default): of the radix passes, and of the offset scans of the lists
+// and of the groups.  Only the failure-path tests change them.
 __device__ uint32_t g_spin_limit = kSpinLimit;
-__device__ uint32_t g_unpublished_tile = 0xffffffffu;
+__device__ uint32_t g_unpublished_tile = kNoTile;
+__device__ uint32_t g_unpublished_scan[2] = {kNoTile, kNoTile};
 
 __device__ __forceinline__ unsigned long long ld_volatile_u64(const unsigned long long *p) {
   return *(const volatile unsigned long long *)p;
@@ -123,11 +125,13 @@ __device__ __forceinline__ U block_scan_exclusive(U x, U *scratch, U *total) {
 // every lane).  If a wait runs out, or a predecessor is poisoned, the tile's
 // prefix is unknown: it publishes a poisoned status, sets *bad (in every
 // lane) and the caller must write nothing.  All 32 lanes of the warp must
-// call it.
+// call it.  silent: publishes nothing (a failure-path test).
 __device__ uint64_t lookback_warp(unsigned long long *status, uint32_t tile, uint64_t agg,
-                                  Ctrl *ctrl, bool *bad, bool published = false) {
+                                  Ctrl *ctrl, bool *bad, bool published = false,
+                                  bool silent = false) {
   const int lane = threadIdx.x & 31;
   *bad = false;
+  published = published || silent;
   if (tile == 0) {
     if (lane == 0 && !published) st_volatile_u64(&status[0], kFlagInclusive | agg);
     return 0;
@@ -164,7 +168,8 @@ __device__ uint64_t lookback_warp(unsigned long long *status, uint32_t tile, uin
     if (inc) break;
     j -= 32;
   }
-  if (lane == 0) st_volatile_u64(&status[tile], *bad ? kFlagPoison : kFlagInclusive | (excl + agg));
+  if (lane == 0 && !silent)
+    st_volatile_u64(&status[tile], *bad ? kFlagPoison : kFlagInclusive | (excl + agg));
   return excl;
 }
 
@@ -693,7 +698,7 @@ k_orient(const uint64_t *keys, int b,
 // and list; one per warp and round of 32 vertices, sixteen rounds after one
 // another, made the scan of a small graph last 14 us instead of 5.
 // ---------------------------------------------------------------------------
-enum { kScanLists = 0, kScanGroups = 1, kScanRecount = 2 };
+enum { kScanLists = 0, kScanGroups = 1, kScanRecount = 2 };  // index g_unpublished_scan
 constexpr int kBlockBits = 31;  // kScanLists: entries above, 32-byte blocks below
 constexpr uint64_t kBlockMask = (1ull << kBlockBits) - 1;
 
@@ -768,7 +773,8 @@ k_offsets(const ScanArgs a) {
   const uint64_t toff = block_scan_exclusive<kScanThreads>(sum, s_scratch, &tile_sum);
   if (tid < 32) {
     bool bad;
-    const uint64_t excl = lookback_warp(a.status, tile, tile_sum, ctrl, &bad);
+    const bool silent = KIND != kScanRecount && tile == g_unpublished_scan[KIND & 1];
+    const uint64_t excl = lookback_warp(a.status, tile, tile_sum, ctrl, &bad, false, silent);
     if (tid == 0) {
       s_excl = excl;
       s_abort = bad ? 1u : 0u;
@@ -873,6 +879,10 @@ cudaError_t set_wait_hooks(uint32_t spin_limit, uint32_t unpublished_tile) {
   if (e == cudaSuccess)
     e = cudaMemcpyToSymbol(g_unpublished_tile, &unpublished_tile, sizeof(unpublished_tile));
   return e;
+}
+
+cudaError_t set_unpublished_scan(const uint32_t (&tiles)[2]) {
+  return cudaMemcpyToSymbol(g_unpublished_scan, tiles, sizeof(tiles));
 }
 
 static uint32_t canon_grid(uint32_t m_in) {

@@ -197,9 +197,9 @@ struct BatchRun {
   unsigned long long *totals;   // device: triangles per graph
 };
 
-// Set while a failure-path test limits the device's waits: the waits it aims at
-// are those of the radix passes, so every run sorts by them.
-std::atomic<bool> g_wait_hooks{false};
+// Set while a failure-path test withholds a radix-pass tile's status: every run
+// sorts by radix passes then, so that there is such a tile.
+std::atomic<bool> g_radix_only{false};
 
 // Enqueues every phase on `st` using workspace `ws` laid out by L, ending
 // with a copy of the control block into `staging` (host).  Nothing here
@@ -272,7 +272,7 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
                      2 * b > kSkipShift;
   // counting sorts by atomics, or radix passes (see kDirectMaxPairs)
   const bool direct = m_in <= (batch ? kDirectMaxBatchPairs : kDirectMaxPairs) &&
-                      2 * b <= kSkipShift && shards == 1 && !work_stats && !g_wait_hooks.load();
+                      2 * b <= kSkipShift && shards == 1 && !work_stats && !g_radix_only.load();
   if (!direct)
     TC_CUDA(cudaMemsetAsync(ws + L.st_sort, 0,
                             sizeof(unsigned long long) * words * (size_t)radix_passes(b), st),
@@ -1217,9 +1217,18 @@ tc_status tc_get_tuning(tc_tuning *out) {
 
 tc_status tc_debug_set_wait_limit(uint32_t spin_limit, int32_t unpublished_tile) {
   TC_CUDA(cudaDeviceSynchronize(), "synchronize");
-  g_wait_hooks.store(spin_limit != kSpinLimit || unpublished_tile >= 0);
-  TC_CUDA(set_wait_hooks(spin_limit, unpublished_tile < 0 ? 0xffffffffu : (uint32_t)unpublished_tile),
+  g_radix_only.store(unpublished_tile >= 0);
+  TC_CUDA(set_wait_hooks(spin_limit, unpublished_tile < 0 ? kNoTile : (uint32_t)unpublished_tile),
           "wait hooks");
+  return set_status(TC_OK);
+}
+
+tc_status tc_debug_set_unpublished_scan(int32_t scan, int32_t tile) {
+  if (scan < 0 || scan > 1) return set_status(TC_ERR_INVALID_ARG, "scan %d", scan);
+  TC_CUDA(cudaDeviceSynchronize(), "synchronize");
+  uint32_t tiles[2] = {kNoTile, kNoTile};
+  if (tile >= 0) tiles[scan] = (uint32_t)tile;
+  TC_CUDA(set_unpublished_scan(tiles), "scan hook");
   return set_status(TC_OK);
 }
 
@@ -1233,7 +1242,9 @@ tc_status tc_debug_fail_allocations(int32_t skip, int32_t count) {
 
 tc_status tc_debug_reset(void) {
   tc_debug_fail_allocations(0, 0);
-  return tc_debug_set_wait_limit(kSpinLimit, -1);
+  const tc_status s = tc_debug_set_unpublished_scan(0, -1);
+  const tc_status w = tc_debug_set_wait_limit(kSpinLimit, -1);
+  return s != TC_OK ? set_status(s) : w;
 }
 
 tc_status tc_last_error(void) { return t_last; }

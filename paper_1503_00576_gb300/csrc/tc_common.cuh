@@ -20,6 +20,7 @@ enum : uint32_t { kErrIdRange = 1u, kErrTimeout = 2u, kErrInternal = 4u };
 // same, and every later kernel of the call returns at entry once kErrTimeout
 // is set (see aborted()), so no kernel runs on incomplete data.
 constexpr uint32_t kSpinLimit = 1u << 24;
+constexpr uint32_t kNoTile = 0xffffffffu;  // no tile withholds its status (see set_wait_hooks)
 
 // Sorted forward lists (the padded column array col4).  Lists of up to
 // kWarpSortMax entries are sorted by one warp, up to kCtaSortMax by a CTA in
@@ -460,9 +461,11 @@ void launch(void (*kernel)(Params...), uint32_t grid, uint32_t block, size_t sme
 
 // Test hooks of the wait paths (preprocess.cu), on the current device:
 // spin_limit bounds every spin-wait (kSpinLimit by default); the radix-pass
-// tile numbered unpublished_tile (UINT32_MAX: none) never publishes its
+// tile numbered unpublished_tile (kNoTile: none) never publishes its
 // status, so the tiles after it wait on a word that nothing sets.
 cudaError_t set_wait_hooks(uint32_t spin_limit, uint32_t unpublished_tile);
+// The same for a tile of the offset scan of the lists (0) and of the groups (1).
+cudaError_t set_unpublished_scan(const uint32_t (&tiles)[2]);
 
 // ---- launchers (preprocess.cu) ----
 // Undirected keys min << b | max of the pairs (self-loops and pairs with an
