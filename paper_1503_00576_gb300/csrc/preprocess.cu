@@ -542,7 +542,11 @@ k_radix_pass(const uint64_t *in, void *__restrict__ out, uint32_t n_keys_bound,
 // ---------------------------------------------------------------------------
 // rank keys: the order of Sec. II-B as a permutation.  Vertex v gets the key
 // deg(v) << b | v; a stable LSD sort over the degree bits leaves the keys in
-// (degree, id) order, and its last pass scatters rank[v] = position.  From
+// (degree, id) order, and its last pass scatters rank[v] = position.  A degree
+// that repeated pairs raise past the sort's digits stays at their largest value:
+// at most 2m / 2^24 vertices (with three digits) are tied there, and the others'
+// forward lists are no longer than sqrt(2m) as before (a degree cut to its low
+// bits would put a hub first, with all its neighbours in its list).  From
 // here on the pipeline works on ranks: an edge is oriented from its lower
 // rank, and the high-degree vertices, which fill most forward lists, get
 // the highest, adjacent ids.
@@ -556,7 +560,7 @@ k_rank_keys(const int32_t *deg, int32_t n, int b, int passes,
   __syncthreads();
   const uint32_t stride = gridDim.x * kCanonThreads;
   for (uint32_t v = blockIdx.x * kCanonThreads + threadIdx.x; v < (uint32_t)n; v += stride) {
-    const uint32_t d = (uint32_t)load(deg + v);
+    const uint32_t d = min((uint32_t)load(deg + v), 0xffffffffu >> (32 - 8 * passes));
     vkeys[v] = ((uint64_t)d << b) | v;
     for (int p = 0; p < passes; ++p) atomicAdd(&sh[p * 256 + ((d >> (8 * p)) & 255u)], 1u);
   }
