@@ -285,9 +285,13 @@ tc_status tc_engine_destroy(tc_engine *engine);
  *                  dense count of the block A_{H_i H_i} (the matrix methods
  *                  of Sec. VI) could replace exactly this share of lookups
  *   dense_vertices the size of the hub set this run counted on the tensor
- *                  cores (its highest-ranked vertices; 0: none, see tc_tuning)
+ *                  cores (its highest-ranked vertices; 0: none, see tc_tuning).
+ *                  The choice goes by the lookups of this split: tc_count and
+ *                  tc_count_per_vertex, where an edge inside the set saves no
+ *                  more than its bitmaps would cost, may choose a smaller set
+ *                  or none (tc_debug_run_work, tc_debug.h, reports theirs)
  *   dense_triangles the triangles counted there (all three vertices in it);
- *                  the hash intersections counted triangles - dense_triangles
+ *                  the intersections counted triangles - dense_triangles
  * Same arguments and errors as tc_count; synchronises `stream`.
  */
 typedef struct tc_work {

@@ -1,10 +1,11 @@
 /*
- * tc_debug.h -- failure-path test hooks of libtc (see tc.h).
+ * tc_debug.h -- test hooks of libtc (see tc.h): failure paths, work counters.
  *
  * The paper has no counterpart: these calls exist so that tests can drive
- * the library's error paths without faulting or hanging a GPU.  They change
- * process-wide (allocation failures) or per-device (waits) state and are not
- * meant for production use; tc_debug_reset() undoes all of them.
+ * the library's error paths without faulting or hanging a GPU, and see what a
+ * call's kernels do.  The hooks change process-wide (allocation failures) or
+ * per-device (waits) state and are not meant for production use;
+ * tc_debug_reset() undoes all of them.
  */
 #ifndef TC_DEBUG_H
 #define TC_DEBUG_H
@@ -51,6 +52,35 @@ tc_status tc_debug_set_unpublished_scan(int32_t scan, int32_t tile);
  * count <= 0 turns injection off.  Process-wide.
  */
 tc_status tc_debug_fail_allocations(int32_t skip, int32_t count);
+
+/*
+ * What the counting kernels of one tc_count (per_vertex == 0) or
+ * tc_count_per_vertex call do for this graph, counted over the very groups and
+ * streams of that call by one more kernel (tc_count_work reports a split of its
+ * own, see tc.h).  Vertices of equal degree class may come in any order, so the
+ * counters of calls that sort by counting can differ a little from call to call.
+ *   partners         edges left to an intersection, over all groups
+ *   lookups          list entries streamed through hash tables
+ *   inserts          list entries hashed
+ *   bitmap_pairs     partners of `partners` that are intersected by bitmaps of
+ *                    the top ranks too (512 bytes each)
+ *   triangles        T
+ *   dense_vertices   size of the hub set counted on the tensor cores (0: none)
+ *   dense_triangles  triangles counted there
+ * Same arguments and errors as those calls; synchronises `stream`.
+ */
+typedef struct tc_run_work {
+  int64_t partners;
+  int64_t lookups;
+  int64_t inserts;
+  int64_t bitmap_pairs;
+  uint64_t triangles;
+  uint64_t dense_triangles;
+  int32_t dense_vertices;
+  int32_t pad_;
+} tc_run_work;
+tc_status tc_debug_run_work(const int32_t *src, const int32_t *dst, int64_t m, int32_t n,
+                            int32_t per_vertex, tc_stream_t stream, tc_run_work *out);
 
 /* Default wait limit and no unpublished tiles on the current device, and no
  * injected allocation failures. */

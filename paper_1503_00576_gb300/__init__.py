@@ -60,7 +60,7 @@ EXPORTS = ("tc_count", "tc_count_per_vertex", "tc_count_part", "tc_count_per_ver
            "tc_last_error", "tc_status_string", "tc_last_error_detail", "tc_launch_count",
            "tc_profile_enable", "tc_profile_read", "tc_phase_name",
            "tc_debug_set_wait_limit", "tc_debug_set_unpublished_scan",
-           "tc_debug_fail_allocations", "tc_debug_reset")
+           "tc_debug_fail_allocations", "tc_debug_run_work", "tc_debug_reset")
 
 
 class Work(ctypes.Structure):
@@ -71,6 +71,14 @@ class Work(ctypes.Structure):
                 ("vertices", ctypes.c_int32), ("hub_lookups", ctypes.c_int64 * 4),
                 ("dense_triangles", ctypes.c_uint64), ("dense_vertices", ctypes.c_int32),
                 ("pad_", ctypes.c_int32)]
+
+
+class RunWork(ctypes.Structure):
+    """tc_run_work: what the counting kernels of one call do."""
+    _fields_ = [("partners", ctypes.c_int64), ("lookups", ctypes.c_int64),
+                ("inserts", ctypes.c_int64), ("bitmap_pairs", ctypes.c_int64),
+                ("triangles", ctypes.c_uint64), ("dense_triangles", ctypes.c_uint64),
+                ("dense_vertices", ctypes.c_int32), ("pad_", ctypes.c_int32)]
 
 
 class Tuning(ctypes.Structure):
@@ -138,6 +146,7 @@ def _bind(lib):
         "tc_debug_set_wait_limit": ([c.c_uint32, i32], c.c_int),
         "tc_debug_set_unpublished_scan": ([i32, i32], c.c_int),
         "tc_debug_fail_allocations": ([i32, i32], c.c_int),
+        "tc_debug_run_work": ([vp, vp, i64, i32, i32, vp, vp], c.c_int),
         "tc_debug_reset": ([], c.c_int),
     }
     for name, (args, res) in sig.items():
@@ -607,6 +616,19 @@ def tc_debug_fail_allocations(skip: int, count: int) -> None:
     """Failure-path test hook: of the library's next device allocations the
     first `skip` succeed and the `count` after them fail (TC_ERR_OOM)."""
     _check(load_library().tc_debug_fail_allocations(skip, count))
+
+
+def tc_debug_run_work(src, dst, n: int, per_vertex: bool = False, stream=None) -> dict:
+    """Work counters of one tc_count or tc_count_per_vertex call as it runs
+    (include/tc_debug.h)."""
+    torch = _torch()
+    dev = _edges(src, dst)
+    w = RunWork()
+    with torch.cuda.device(dev):
+        _check(load_library().tc_debug_run_work(src.data_ptr(), dst.data_ptr(), src.numel(), n,
+                                                1 if per_vertex else 0, _stream_of(stream, dev),
+                                                ctypes.byref(w)))
+    return {f: getattr(w, f) for f, _ in RunWork._fields_ if f != "pad_"}
 
 
 def tc_debug_reset(device=None) -> None:

@@ -897,6 +897,56 @@ k_work(const int32_t *off, const int32_t *goff,
   }
 }
 
+// What a run's counting kernels read (instrumentation): work[0] += entries
+// streamed through hash tables, work[1] += entries hashed, work[2] += partners
+// intersected by bitmaps too.  The groups and the streams are told apart by the
+// rules of the counting kernels (count.cu, bits.cu): a group of a list shorter
+// than `least` is not binned.  pskip or, where it is not nullptr, desc holds
+// what is streamed.  One warp per vertex h.
+template <bool PV>
+__global__ void __launch_bounds__(kGroupThreads)
+k_run_work(const int32_t *goff, const int32_t *part, const int32_t *pskip, const int2 *desc,
+           const int2 *ldesc, const uint32_t *rec, int32_t n, int32_t least, Ctrl *ctrl) {
+  grid_begin();
+  if (aborted(ctrl)) return;
+  const int lane = threadIdx.x & 31;
+  const uint32_t warps = gridDim.x * (kGroupThreads / 32);
+  unsigned long long lookups = 0, inserts = 0, pairs = 0;
+  for (uint32_t h = (blockIdx.x * kGroupThreads + threadIdx.x) >> 5; h < (uint32_t)n;
+       h += warps) {
+    const int32_t pb = load(goff + h), pe = load(goff + h + 1), dh = load(ldesc + h).y;
+    if (pe == pb || dh < least) continue;  // uniform
+    const bool bits = rec && bits_group<PV>(load(rec + h), pe - pb);
+    if (lane == 0) inserts += (unsigned)dh;
+    for (int32_t i = pb + lane; i < pe; i += 32) {
+      int32_t ds;
+      if (desc) {
+        ds = load(desc + i).y & 0xffff;
+      } else {
+        const int32_t l = load(part + i), skip = load(pskip + i);
+        const uint32_t rl = bits ? load(rec + l) : 0u;
+        ds = load(ldesc + l).y;
+        if (bits_used<PV>(rl, skip, ds)) {
+          ds = 8 * (int32_t)(rl & kBitTbMask);
+          ++pairs;
+        }
+        ds = max(ds - 8 * skip, 0);
+      }
+      lookups += (unsigned)ds;
+    }
+  }
+  for (int o = 16; o; o >>= 1) {
+    lookups += __shfl_xor_sync(0xffffffffu, lookups, o);
+    inserts += __shfl_xor_sync(0xffffffffu, inserts, o);
+    pairs += __shfl_xor_sync(0xffffffffu, pairs, o);
+  }
+  if (lane == 0) {
+    atomicAdd(&ctrl->work[0], lookups);
+    atomicAdd(&ctrl->work[1], inserts);
+    atomicAdd(&ctrl->work[2], pairs);
+  }
+}
+
 uint32_t group_grid(uint32_t m_bound) {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
@@ -951,6 +1001,15 @@ void launch_work(const int32_t *off, const int32_t *goff, const int32_t *part,
   const uint32_t lanes = n > (1 << 28) ? (1u << 30) : (uint32_t)n * 4u;  // grid is capped anyway
   launch(k_work, group_grid(lanes), kGroupThreads, 0, st, off, goff, part, pskip, n, ctrl,
          (uint32_t)shard, (uint32_t)shards);
+}
+
+void launch_run_work(const int32_t *goff, const int32_t *part, const int32_t *pskip,
+                     const int2 *desc, const int2 *ldesc, const uint32_t *rec, int32_t n,
+                     int32_t least, bool per_vertex, Ctrl *ctrl, cudaStream_t st) {
+  const auto kernel = per_vertex ? k_run_work<true> : k_run_work<false>;
+  const uint32_t lanes = n > (1 << 28) ? (1u << 30) : (uint32_t)n * 4u;  // grid is capped anyway
+  launch(kernel, group_grid(lanes), kGroupThreads, 0, st, goff, part, pskip, desc, ldesc, rec, n,
+         least, ctrl);
 }
 
 }  // namespace tc

@@ -205,11 +205,14 @@ std::atomic<bool> g_radix_only{false};
 // with a copy of the control block into `staging` (host).  Nothing here
 // synchronises or allocates, so the whole sequence can be captured in a
 // CUDA graph.  t_out == nullptr counts the total only (per graph with a
-// batch: group totals, summed per graph).
+// batch: group totals, summed per graph).  stats: counters that a run fills
+// beside its counts (kWholeWork: of the split by whole lists, which is then the
+// run's; kRunWork: of the run as it is).
+enum Stats { kNoStats, kWholeWork, kRunWork };
 tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int32_t n,
                        cudaStream_t st, unsigned char *ws, const Layout &L, int64_t *t_out,
                        int32_t *deg_out, const BatchRun *batch, const Tuning &tune,
-                       PhaseTimer &pt, Ctrl *staging, bool work_stats = false,
+                       PhaseTimer &pt, Ctrl *staging, Stats stats = kNoStats,
                        int32_t shard = 0, int32_t shards = 1) {
   const EarlyLaunches early(m_in);
   const uint32_t m = (uint32_t)m_in;
@@ -268,11 +271,11 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
                           (t_rank || bits_on ? L.st_sort : L.t_rank) - zero_from, st),
           "memset control");
   // shares and the work counters go by the whole lists' lengths
-  const bool whole = shards > 1 || work_stats || tune.heavy_ratio_pct != 100 ||
+  const bool whole = shards > 1 || stats == kWholeWork || tune.heavy_ratio_pct != 100 ||
                      2 * b > kSkipShift;
   // counting sorts by atomics, or radix passes (see kDirectMaxPairs)
   const bool direct = m_in <= (batch ? kDirectMaxBatchPairs : kDirectMaxPairs) &&
-                      2 * b <= kSkipShift && shards == 1 && !work_stats && !g_radix_only.load();
+                      2 * b <= kSkipShift && shards == 1 && stats != kWholeWork && !g_radix_only.load();
   if (!direct)
     TC_CUDA(cudaMemsetAsync(ws + L.st_sort, 0,
                             sizeof(unsigned long long) * words * (size_t)radix_passes(b), st),
@@ -439,7 +442,10 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
     launch_bits_build(queue, n, ldesc, col4, goff, L.bit_slots, t_out != nullptr, bits, items,
                       ctrl, st, shard, shards);
   pt.stop(TC_PHASE_GROUPS);
-  if (work_stats) launch_work(off, goff, part, pskip, n, ctrl, st, shard, shards);
+  if (stats == kWholeWork) launch_work(off, goff, part, pskip, n, ctrl, st, shard, shards);
+  if (stats == kRunWork)
+    launch_run_work(goff, part, pskip, desc_ready ? desc : nullptr, ldesc,
+                    bits_on ? bit_rec : nullptr, n, direct ? 1 : 2, t_out != nullptr, ctrl, st);
 
   pt.start(TC_PHASE_COUNT);
   // the dense block's triangles belong to the first share alone (every share
@@ -494,7 +500,7 @@ tc_status run_core(const int32_t *src, const int32_t *dst, int64_t m_in, int32_t
   Ctrl *h = staging ? staging : host_ctrl();
   if (!h) return set_status(TC_ERR_OOM, "pinned staging buffer");
   tc_status s = enqueue_core(src, dst, m_in, n, st, ws, L, t_out, deg_out, nullptr,
-                             current_tuning(), pt, h, false, shard, shards);
+                             current_tuning(), pt, h, kNoStats, shard, shards);
   if (s != TC_OK) return s;
   TC_CUDA(cudaStreamSynchronize(st), "synchronize");
   pt.fold();
@@ -1163,7 +1169,7 @@ tc_status tc_count_work_part(const int32_t *src, const int32_t *dst, int64_t m, 
   PhaseTimer pt(st, false);
   if (!h) s = set_status(TC_ERR_OOM, "pinned staging buffer");
   else s = enqueue_core(src, dst, m, n, st, ws, L, nullptr, nullptr, nullptr, current_tuning(), pt,
-                        h, true, part, parts);
+                        h, kWholeWork, part, parts);
   cudaFreeAsync(ws, st);
   const cudaError_t e = cudaStreamSynchronize(st);
   if (s != TC_OK) return s;
@@ -1237,6 +1243,42 @@ tc_status tc_debug_fail_allocations(int32_t skip, int32_t count) {
   g_inject_skip = skip > 0 ? skip : 0;
   g_inject_fail = count > 0 ? count : 0;
   g_inject_on.store(g_inject_fail > 0);
+  return set_status(TC_OK);
+}
+
+tc_status tc_debug_run_work(const int32_t *src, const int32_t *dst, int64_t m, int32_t n,
+                            int32_t per_vertex, tc_stream_t stream, tc_run_work *out) {
+  if (!out) return set_status(TC_ERR_INVALID_ARG, "out is NULL");
+  memset(out, 0, sizeof(*out));
+  tc_status s = check_args(src, dst, m, n);
+  if (s != TC_OK) return s;
+  if (m > 0 && n == 0) return set_status(TC_ERR_ID_RANGE, "n = 0 but m > 0");
+  if (m == 0) return set_status(TC_OK);
+  cudaStream_t st = (cudaStream_t)stream;
+  const Layout L =
+      make_layout(m, n, true, current_tuning().hub_vertices, false, per_vertex != 0);
+  keep_pool_memory();
+  const size_t t_bytes = per_vertex ? align256(sizeof(int64_t) * (size_t)n) : 0;
+  unsigned char *ws = nullptr;
+  TC_CUDA(dev_alloc_async((void **)&ws, t_bytes + L.total, st), "workspace allocation");
+  int64_t *t = per_vertex ? reinterpret_cast<int64_t *>(ws) : nullptr;
+  Ctrl *h = host_ctrl();
+  PhaseTimer pt(st, false);
+  if (!h) s = set_status(TC_ERR_OOM, "pinned staging buffer");
+  else s = enqueue_core(src, dst, m, n, st, ws + t_bytes, L, t, nullptr, nullptr,
+                        current_tuning(), pt, h, kRunWork);
+  cudaFreeAsync(ws, st);
+  const cudaError_t e = cudaStreamSynchronize(st);
+  if (s != TC_OK) return s;
+  if (e != cudaSuccess) return cuda_fail(e, "synchronize");
+  s = finish_core(h, n, &out->triangles);
+  if (s != TC_OK) return s;
+  out->partners = h->n_part;
+  out->lookups = (int64_t)h->work[0];
+  out->inserts = (int64_t)h->work[1];
+  out->bitmap_pairs = (int64_t)h->work[2];
+  out->dense_triangles = h->hub_triangles;
+  out->dense_vertices = h->hub_on ? (int32_t)h->hub_size : 0;
   return set_status(TC_OK);
 }
 

@@ -135,7 +135,8 @@ struct Ctrl {
   uint32_t dups;                   // some forward list held a repeated edge (set by the list sort)
   unsigned long long hub_triangles;  // triangles the dense block counted
   unsigned long long hub_est[4];   // hash lookups inside each candidate hub set (hub.cu)
-  // work of the counting phase (filled only when asked for; see launch_work):
+  // work of the counting phase (filled only when asked for; see launch_work and
+  // launch_run_work):
   // hash lookups, hash inserts, merge work W, max out-degree, then the
   // lookups of edges with both endpoints among the 2^12 .. 2^15 top ranks
   unsigned long long work[4 + kHubSizes];
@@ -587,6 +588,11 @@ void launch_group_keys(const int32_t *row, const int32_t *col4, const int32_t *o
 void launch_work(const int32_t *off, const int32_t *goff, const int32_t *part,
                  const int32_t *pskip, int32_t n, Ctrl *ctrl, cudaStream_t st,
                  int32_t shard = 0, int32_t shards = 1);
+// Instrumentation: what the counting kernels of this run read, into ctrl->work
+// (see k_run_work).  desc != nullptr: each partner's stream instead of pskip.
+void launch_run_work(const int32_t *goff, const int32_t *part, const int32_t *pskip,
+                     const int2 *desc, const int2 *ldesc, const uint32_t *rec, int32_t n,
+                     int32_t least, bool per_vertex, Ctrl *ctrl, cudaStream_t st);
 // ---- launchers (direct.cu) ----
 // rank[v] in an order by degree classes (ties in any order).  counters: 2
 // kRankClasses words, zero on entry.
