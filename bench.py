@@ -247,17 +247,18 @@ def roofline(prof: dict, steps: int, m_in: int, m: int, n: int, workload: str,
     """Dominant kernel by device time; achieved = algorithmic bytes per
     launch / average launch duration (CUDA events on the launch stream).
 
-    The counting phase is one unit: its two kernels (k_count_big for the
-    partner groups with the longest hashed lists, then k_count) split one
-    work list and run back to back once per step, followed by the small
-    gather of t[] to vertex ids.  Its algorithmic bytes are the forward-list
-    elements the hash intersections read -- each partner group's hashed list
-    once (inserts) and, per forward edge, the list streamed through it
-    (lookups), 4 bytes each, counted exactly by tc_count_work for the split of
-    the edges by whole lists (the kernels weigh what is streamed and leave the
-    top ranks of long lists to bitmaps, so they read less) -- plus the
-    partner ids (4m), both offset arrays (8(n+1)) and, per vertex, t[] in
-    rank space written, gathered and written again (28n)."""
+    The counting phase is one unit: the dense block's product, the bitmap
+    intersections, the partners' streams and the two kernels that count by
+    hashing share one work list and run back to back once per step, followed by
+    the small gather of t[] to vertex ids.  Its algorithmic bytes are what the
+    timed call's intersections read, counted by tc_debug_run_work over the groups
+    and streams of that very call: each partner group's hashed list once
+    (inserts) and, per partner, the part of the list streamed through it
+    (lookups), 4 bytes each, and 512 bytes per partner intersected by bitmaps --
+    plus the partner ids (4 each; without the count, 4m), both offset arrays
+    (8(n+1)) and, per vertex, t[] in rank space written, gathered and written
+    again (28n).  Most of it is served by L2, so `frac` compares a rate of bytes
+    used with the HBM peak; it is not DRAM traffic (see `traffic`)."""
     b = max(1, (max(n, 2) - 1).bit_length())
     passes2 = (b + 7) // 8
     per_kernel = {}
@@ -272,13 +273,19 @@ def roofline(prof: dict, steps: int, m_in: int, m: int, n: int, workload: str,
     if kernel == "k_count":
         kernel = "k_count+k_count_big"
         units = steps
-        lists = 4 * (work["lookups"] + work["inserts"])
-        bytes_per_launch = lists + 4 * m + 8 * (n + 1) + (0 if total_only else 28 * n)
+        pairs, partners = work.get("bitmap_pairs", 0), work.get("partners", m)
+        lists = 4 * (work["lookups"] + work["inserts"]) + 512 * pairs
+        bytes_per_launch = lists + 4 * partners + 8 * (n + 1) + (0 if total_only else 28 * n)
         how = ("one counting phase: 4 B per list element read by the hash intersections "
-               "(lookups %d + inserts %d) + partner ids 4m + offsets 8(n+1)%s"
-               % (work["lookups"], work["inserts"], "" if total_only else " + t[] 28n"))
+               "(lookups %d + inserts %d) + 512 B per bitmap intersection (%d) + partner ids "
+               "(%d) + offsets 8(n+1)%s"
+               % (work["lookups"], work["inserts"], pairs, partners,
+                  "" if total_only else " + t[] 28n"))
         t = ms_total / 1e3 / units
-        extra = {"merge_equivalent_gbs": round(4 * work["merge_work"] / t / 1e9, 1),
+        extra = {"kernels_timed": "k_hub_zero, k_hub_scatter, k_hub_gemm, k_hub_finish, "
+                                  "k_count_bits, k_stream_desc, k_count_big, k_count, "
+                                  "k_gather_counts (those that the call launches)",
+                 "merge_equivalent_gbs": round(4 * work["merge_work"] / t / 1e9, 1),
                  "merge_work_W": work["merge_work"],
                  "compulsory_gbs": round((4 * m + 4 * (n + 1) + (0 if total_only else 8 * n))
                                          / t / 1e9, 1)}
@@ -673,8 +680,12 @@ def run_ours(args, world, rank, local, pg):
     if args.total_only:
         tc.tc_count_per_vertex(s, d, n, stream=stream, t_out=t_out, deg_out=deg_out)
     m = int((deg_out.to(torch.int64).sum() // 2).item())
-    work = tc.tc_count_work(s, d, n)  # untimed: the counting phase's exact work
+    # untimed: the work by whole lists, and what the timed call's kernels do
+    # (a share is dealt by whole lists)
+    work = tc.tc_count_work(s, d, n)
     assert work["edges"] == m and work["triangles"] == T
+    run = work if sharded else tc.tc_debug_run_work(s, d, n, not args.total_only)
+    assert run["triangles"] == T
 
     clocks = ClockSampler(gpu_uuid(dev))
     tc.tc_profile_read(reset=True)
@@ -782,19 +793,23 @@ def run_ours(args, world, rank, local, pg):
                          % (8 * m_in / 1e9, 16 * m_in / 1e9),
                    "parallelism": ("shards%d" % world if sharded else "replicas")
                                   if world > 1 else "single"},
-        "roofline": roofline(prof, args.steps, m_in, m, n, args.workload, work,
-                             args.total_only),
+        "roofline": roofline(prof, args.steps, m_in, m, n, args.workload,
+                             {**work, **run}, args.total_only),
         "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": launches, "clocks": clk,
         "step_ms": step_ms, "phase_ms_per_step": steps_ms, "batched": batched,
         "paper_format": paper_format,
         "paper_table1": paper_table,
-        "counting_work": {"lookups": work["lookups"], "inserts": work["inserts"],
-                          "merge_work_W": work["merge_work"],
+        "counting_work": {"lookups": run["lookups"], "inserts": run["inserts"],
+                          "partners": run.get("partners", m),
+                          "bitmap_pairs": run.get("bitmap_pairs", 0),
+                          "dense_hub_vertices": run["dense_vertices"],
+                          "dense_hub_triangles": run["dense_triangles"],
                           "max_out_degree": work["max_out_degree"],
-                          "dense_hub_vertices": work["dense_vertices"],
-                          "dense_hub_triangles": work["dense_triangles"],
-                          "hub_lookup_share": {str(k): round(v / max(work["lookups"], 1), 4)
-                                               for k, v in work["hub_lookups"].items()}},
+                          "merge_work_W": work["merge_work"],
+                          "by_whole_lists": {
+                              "lookups": work["lookups"], "inserts": work["inserts"],
+                              "hub_lookup_share": {str(k): round(v / max(work["lookups"], 1), 4)
+                                                   for k, v in work["hub_lookups"].items()}}},
     }
     print(json.dumps(line), flush=True)
 
