@@ -3,8 +3,8 @@
  *
  * The paper has no counterpart: these calls exist so that tests can drive
  * the library's error paths without faulting or hanging a GPU, and see what a
- * call's kernels do.  The hooks change process-wide (allocation failures) or
- * per-device (waits) state and are not meant for production use;
+ * call's kernels do.  The hooks change process-wide (allocation failures,
+ * scans) or per-device (waits) state and are not meant for production use;
  * tc_debug_reset() undoes all of them.
  */
 #ifndef TC_DEBUG_H
@@ -39,8 +39,9 @@ tc_status tc_debug_set_wait_limit(uint32_t spin_limit, int32_t unpublished_tile)
 /*
  * The same for the offset scans, the waits that every call has: tile `tile`
  * (4096 vertices each) of the scan of the forward lists (scan 0) or of the
- * partner groups (scan 1) never publishes its status; tile < 0: all of both
- * do (default).  Synchronises the device.
+ * partner groups (scan 1) never publishes its status; tile < 0: all of that
+ * scan do (default).  Process-wide, for calls made and engines created from
+ * now on (an engine keeps what it was created with).
  */
 tc_status tc_debug_set_unpublished_scan(int32_t scan, int32_t tile);
 

@@ -603,13 +603,12 @@ def tc_debug_set_wait_limit(spin_limit: int, unpublished_tile: int = -1, device=
         _check(load_library().tc_debug_set_wait_limit(spin_limit, unpublished_tile))
 
 
-def tc_debug_set_unpublished_scan(scan: int, tile: int, device=None) -> None:
+def tc_debug_set_unpublished_scan(scan: int, tile: int) -> None:
     """Failure-path test hook (include/tc_debug.h): tile `tile` of the offset
     scan of the forward lists (scan 0) or of the partner groups (scan 1) never
-    publishes (tile < 0: every tile of both does)."""
-    torch = _torch()
-    with torch.cuda.device(device if device is not None else torch.cuda.current_device()):
-        _check(load_library().tc_debug_set_unpublished_scan(scan, tile))
+    publishes (tile < 0: every tile does), in calls made and engines created
+    from now on."""
+    _check(load_library().tc_debug_set_unpublished_scan(scan, tile))
 
 
 def tc_debug_fail_allocations(skip: int, count: int) -> None:

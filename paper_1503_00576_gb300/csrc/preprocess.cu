@@ -39,6 +39,7 @@
 // together); here no global sort of the undirected keys is needed: each
 // forward list is sorted on its own afterwards (group.cu), which is where
 // repeated edges meet and are dropped.
+#include <atomic>
 #include <cstdio>
 
 #include "tc_common.cuh"
@@ -50,10 +51,11 @@ constexpr unsigned kFull = 0xffffffffu;
 
 // Bound of every spin-wait of this file, and the tiles that never publish
 // (none by default): of the radix passes, and of the offset scans of the lists
-// and of the groups.  Only the failure-path tests change them.
+// and of the groups (those by a kernel argument: read from device memory it cost
+// a small call 2 us).  Only the failure-path tests change them.
 __device__ uint32_t g_spin_limit = kSpinLimit;
 __device__ uint32_t g_unpublished_tile = kNoTile;
-__device__ uint32_t g_unpublished_scan[2] = {kNoTile, kNoTile};
+std::atomic<uint32_t> g_unpublished_scan[2] = {{kNoTile}, {kNoTile}};
 
 __device__ __forceinline__ unsigned long long ld_volatile_u64(const unsigned long long *p) {
   return *(const volatile unsigned long long *)p;
@@ -720,6 +722,7 @@ struct ScanArgs {
   uint32_t *ticket;
   Ctrl *ctrl;
   uint32_t shard, shards;
+  uint32_t unpublished;   // tile that never publishes its status (kNoTile: none)
 };
 
 template <int KIND>
@@ -777,8 +780,8 @@ k_offsets(const ScanArgs a) {
   const uint64_t toff = block_scan_exclusive<kScanThreads>(sum, s_scratch, &tile_sum);
   if (tid < 32) {
     bool bad;
-    const bool silent = KIND != kScanRecount && tile == g_unpublished_scan[KIND & 1];
-    const uint64_t excl = lookback_warp(a.status, tile, tile_sum, ctrl, &bad, false, silent);
+    const uint64_t excl =
+        lookback_warp(a.status, tile, tile_sum, ctrl, &bad, false, tile == a.unpublished);
     if (tid == 0) {
       s_excl = excl;
       s_abort = bad ? 1u : 0u;
@@ -885,9 +888,7 @@ cudaError_t set_wait_hooks(uint32_t spin_limit, uint32_t unpublished_tile) {
   return e;
 }
 
-cudaError_t set_unpublished_scan(const uint32_t (&tiles)[2]) {
-  return cudaMemcpyToSymbol(g_unpublished_scan, tiles, sizeof(tiles));
-}
+void set_unpublished_scan(int scan, uint32_t tile) { g_unpublished_scan[scan].store(tile); }
 
 static uint32_t canon_grid(uint32_t m_in) {
   // many pairs in flight: the degree atomics wait on L2
@@ -951,6 +952,7 @@ void launch_offsets(const int32_t *counts, int32_t n, int32_t *off, int32_t *vof
   a.status = status;
   a.ticket = ticket;
   a.ctrl = ctrl;
+  a.unpublished = g_unpublished_scan[kScanLists].load(std::memory_order_relaxed);
   launch(k_offsets<kScanLists>, scan_grid(n), kScanThreads, 0, st, a);
 }
 
@@ -960,7 +962,8 @@ void launch_group_offsets(const int32_t *counts, const int32_t *own, int32_t n, 
                           cudaStream_t st, int32_t shard, int32_t shards) {
   tune.warp_max_list = min(max(tune.warp_max_list, 0), kWarpMaxRow);  // warp table capacity
   const ScanArgs a{counts, own,    n,      goff, nullptr,         ldesc,          groups, big_list,
-                   tune,   status, ticket, ctrl, (uint32_t)shard, (uint32_t)shards};
+                   tune,   status, ticket, ctrl, (uint32_t)shard, (uint32_t)shards,
+                   g_unpublished_scan[kScanGroups].load(std::memory_order_relaxed)};
   launch(k_offsets<kScanGroups>, scan_grid(n), kScanThreads, 0, st, a);
 }
 
@@ -973,6 +976,7 @@ void launch_recount(const int32_t *counts, int32_t n, int32_t *off, unsigned lon
   a.status = status;
   a.ticket = ticket;
   a.ctrl = ctrl;
+  a.unpublished = kNoTile;
   launch(k_offsets<kScanRecount>, scan_grid(n), kScanThreads, 0, st, a);
 }
 

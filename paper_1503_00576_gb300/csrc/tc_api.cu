@@ -1231,10 +1231,7 @@ tc_status tc_debug_set_wait_limit(uint32_t spin_limit, int32_t unpublished_tile)
 
 tc_status tc_debug_set_unpublished_scan(int32_t scan, int32_t tile) {
   if (scan < 0 || scan > 1) return set_status(TC_ERR_INVALID_ARG, "scan %d", scan);
-  TC_CUDA(cudaDeviceSynchronize(), "synchronize");
-  uint32_t tiles[2] = {kNoTile, kNoTile};
-  if (tile >= 0) tiles[scan] = (uint32_t)tile;
-  TC_CUDA(set_unpublished_scan(tiles), "scan hook");
+  set_unpublished_scan(scan, tile < 0 ? kNoTile : (uint32_t)tile);
   return set_status(TC_OK);
 }
 
@@ -1284,9 +1281,8 @@ tc_status tc_debug_run_work(const int32_t *src, const int32_t *dst, int64_t m, i
 
 tc_status tc_debug_reset(void) {
   tc_debug_fail_allocations(0, 0);
-  const tc_status s = tc_debug_set_unpublished_scan(0, -1);
-  const tc_status w = tc_debug_set_wait_limit(kSpinLimit, -1);
-  return s != TC_OK ? set_status(s) : w;
+  for (int scan = 0; scan < 2; ++scan) set_unpublished_scan(scan, kNoTile);
+  return tc_debug_set_wait_limit(kSpinLimit, -1);
 }
 
 tc_status tc_last_error(void) { return t_last; }

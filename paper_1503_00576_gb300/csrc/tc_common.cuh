@@ -465,8 +465,9 @@ void launch(void (*kernel)(Params...), uint32_t grid, uint32_t block, size_t sme
 // tile numbered unpublished_tile (kNoTile: none) never publishes its
 // status, so the tiles after it wait on a word that nothing sets.
 cudaError_t set_wait_hooks(uint32_t spin_limit, uint32_t unpublished_tile);
-// The same for a tile of the offset scan of the lists (0) and of the groups (1).
-cudaError_t set_unpublished_scan(const uint32_t (&tiles)[2]);
+// The same for a tile of the offset scan of the lists (0) and of the groups (1),
+// in all launches and captures from now on.
+void set_unpublished_scan(int scan, uint32_t tile);
 
 // ---- launchers (preprocess.cu) ----
 // Undirected keys min << b | max of the pairs (self-loops and pairs with an
