@@ -99,7 +99,7 @@ __device__ __forceinline__ void warp_sort_regs(int32_t (&x)[E]) {
 // Where the list sort leaves its results (see launch_sort_lists).
 struct ListOut {
   int32_t *col4;   // sorted lists, padded with -1 to whole 32-byte blocks
-  int32_t *dlen;   // length of a list that held repeats, after dropping them
+  int32_t *dlen;   // length of a list that held repeats, after dropping them (may be nullptr)
   int32_t *dcorr;  // per rank: repeated edges dropped at that vertex
   int2 *ldesc;     // per vertex: {first col4 word, length without repeats}
   Ctrl *ctrl;
@@ -108,7 +108,8 @@ struct ListOut {
 // What the list sort needs to emit edges (GroupOut) beside the lists.
 struct Emit {
   GroupOut g;
-  const int32_t *len;  // list lengths (with repeats, or without once dropped)
+  const int32_t *len;  // list lengths: with repeats where the list sort emits, so that no
+                       //   warp writes them meanwhile; otherwise without
   int32_t hub_lo;      // lists of vertices from this rank on are counted densely
   int32_t *hot;        // shared counters of the edges emitted to the ranks from
   int32_t hot_lo;      //   hot_lo on (nullptr: none)
@@ -179,7 +180,7 @@ __device__ __forceinline__ void emit_entry(const Emit &o, int32_t u, int32_t du,
 __device__ __forceinline__ void note_repeats(int32_t u, int32_t dropped, int32_t len,
                                              const ListOut &o) {
   atomicAdd(&o.dcorr[u], dropped);
-  o.dlen[u] = len;
+  if (o.dlen) o.dlen[u] = len;
   uint32_t seen;
   asm volatile("ld.global.ca.u32 %0, [%1];" : "=r"(seen) : "l"(&o.ctrl->dups));
   if (!seen) *(volatile uint32_t *)&o.ctrl->dups = 1u;
@@ -428,7 +429,7 @@ k_sort_lists(const int32_t *col, const int32_t *off,
   grid_begin();
   Ctrl *ctrl = o.ctrl;
   if (aborted(ctrl)) return;  // an earlier wait of this call ran out
-  const Emit em{g, o.dlen, ctrl->hub_on ? (int32_t)ctrl->hub_lo : n, nullptr, n};
+  const Emit em{g, g.len, ctrl->hub_on ? (int32_t)ctrl->hub_lo : n, nullptr, n};
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t warps = gridDim.x * kListWarps;
   const uint32_t lt = (1u << lane) - 1u;
@@ -566,7 +567,7 @@ k_sort_long_lists(int32_t *col, const int32_t *off,
   __shared__ int32_t s_own;
   const int tid = threadIdx.x, lane = tid & 31;
   const uint32_t n_cta = ctrl->n_cta_lists, n_warp = ctrl->n_warp_lists;
-  Emit em{g, o.dlen, ctrl->hub_on ? (int32_t)ctrl->hub_lo : n, nullptr, n};
+  Emit em{g, g.len, ctrl->hub_on ? (int32_t)ctrl->hub_lo : n, nullptr, n};
   while (n_cta) {
     if (tid == 0) s_i = atomicAdd(&ctrl->next_cta_list, 1u);
     __syncthreads();
@@ -748,7 +749,7 @@ k_group_keys(const int32_t *row, const int32_t *col4,
   const bool carry_skip = 2 * b <= kSkipShift;
   const bool hub_on = carry_skip && ctrl->hub_on != 0u;
   const int32_t hub_lo = (int32_t)ctrl->hub_lo;
-  const Emit em{GroupOut{nullptr, nullptr, nullptr, b, heavy_ratio_pct}, len, 0, nullptr, 0};
+  const Emit em{GroupOut{nullptr, nullptr, nullptr, nullptr, b, heavy_ratio_pct}, len, 0, nullptr, 0};
   const uint32_t stride = gridDim.x * kGroupThreads;
   // UNROLL edges per thread per round, each step's loads issued for
   // all of them together: the offsets are gathers that depend on the edge
@@ -967,7 +968,7 @@ static uint32_t num_sms() {
 void launch_sort_lists(int32_t *col, const int32_t *off, const int32_t *voff, int32_t n,
                        Ctrl *ctrl, int32_t *col4, int32_t *queue, int32_t *dlen,
                        int32_t *dcorr, int2 *ldesc, const GroupOut *emit, cudaStream_t st) {
-  const ListOut o{col4, dlen, dcorr, ldesc, ctrl};
+  const ListOut o{col4, emit ? nullptr : dlen, dcorr, ldesc, ctrl};
   const uint32_t warps = num_sms() * 8u * kListWarps;
   uint32_t per = 4;
   while (per < 32 && per * warps < (uint32_t)n) per <<= 1;

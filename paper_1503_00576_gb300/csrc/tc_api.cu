@@ -375,7 +375,7 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
   pt.start(TC_PHASE_LISTS);
   int32_t *queue = reinterpret_cast<int32_t *>(vkeys_a);
   int32_t *own = queue + n;  // the rank keys' first buffer holds both
-  const GroupOut emit{in, gcnt, own, b, tune.heavy_ratio_pct};
+  const GroupOut emit{in, gcnt, own, outdeg, b, tune.heavy_ratio_pct};
   launch_sort_lists(col, off, voff, n, ctrl, col4, queue, outdeg, dcorr, ldesc,
                     direct ? &emit : nullptr, st);
   if (!direct)

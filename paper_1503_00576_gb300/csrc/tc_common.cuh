@@ -234,10 +234,12 @@ struct BatchDesc {
 //   kOwnEdge when h = u, the skip field (0 then) being the edge's number among
 //   u's own edges;
 // or kHole: the entry was a repeat, or no triangle can be found there.
-// gcnt[h] counts the edges emitted to h by others, own[u] gets u's own.
+// gcnt[h] counts the edges emitted to h by others, own[u] gets u's own.  len:
+// the list lengths with repeats.
 struct GroupOut {
   uint64_t *gkeys;
   int32_t *gcnt, *own;
+  const int32_t *len;
   int32_t b, heavy_ratio_pct;
 };
 
@@ -556,11 +558,10 @@ cudaError_t launch_hub_count(const int2 *ldesc, const int32_t *col4, int32_t n, 
 // lengths with repeats on entry), each dropped copy adds one to dcorr at
 // both its ends (rank space; zero on entry) and ctrl->dups is set.
 // emit (may be nullptr): the list sort also emits every edge to its partner
-// group (see GroupOut).
+// group (see GroupOut), and leaves dlen alone.
 // queue: n entries; the lists of more than 64 entries, ctrl->n_warp_lists
 // of them from its front and ctrl->n_cta_lists (the longest) from its end
-// down; col is scratch for lists longer than
-// kCtaSortMax.
+// down; col is scratch for lists longer than kCtaSortMax.
 void launch_sort_lists(int32_t *col, const int32_t *off, const int32_t *voff, int32_t n,
                        Ctrl *ctrl, int32_t *col4, int32_t *queue, int32_t *dlen,
                        int32_t *dcorr, int2 *ldesc, const GroupOut *emit, cudaStream_t st);

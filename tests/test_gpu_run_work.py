@@ -93,10 +93,11 @@ class Lists:
         return oracle.forward((self.u[inside] - lo).astype(np.int32),
                               (self.v[inside] - lo).astype(np.int32), size)["T"]
 
-    def work(self, per_vertex, bits, hub=0):
-        """partners, lookups, inserts and bitmap pairs."""
+    def work(self, per_vertex, bits, hub=0, emitted=False):
+        """partners, lookups, inserts and bitmap pairs; emitted: by the list sort,
+        which weighs the other endpoint's list with repeats."""
         u, v, i, n = self.u, self.v, self.i, self.n
-        du, dv = self.len[u], self.len[v]
+        du, dv = self.len[u], (self.raw if emitted else self.len)[v]
         keep = (i + 1 != du) & (dv > 0) & (u < n - hub)
         u, v, i, du, dv = u[keep], v[keep], i[keep], du[keep], dv[keep]
         skip = (i + 1) >> 3
@@ -177,15 +178,19 @@ def threshold_graph(n):
     return a[keep], b[keep], n
 
 
-@pytest.mark.parametrize("n", [9, 64, 250])
-def test_counting_sort_runs_do_the_restated_work(tc, n):
+@pytest.mark.parametrize("n,times", [(9, 1), (64, 1), (250, 1), (127, 2), (60, 4), (28, 9)])
+def test_counting_sort_runs_do_the_restated_work(tc, n, times):
+    """Repeats too: the split goes by lengths that no warp changes meanwhile, so
+    every call's is the same."""
     src, dst, n = threshold_graph(n)
+    src, dst = np.tile(src, times), np.tile(dst, times)
+    assert (n - 1) * times < 256  # one class per degree
     lists = Lists(src, dst, n)
     T = oracle.forward(np.asarray(src, np.int32), np.asarray(dst, np.int32), n)["T"]
-    for per_vertex in (False, True):
+    for per_vertex in (False, True) * 4:
         got = tc.tc_debug_run_work(dev(src), dev(dst), n, per_vertex)
-        assert got == {**lists.work(per_vertex, False), "triangles": T, "dense_triangles": 0,
-                       "dense_vertices": 0}
+        assert got == {**lists.work(per_vertex, False, emitted=True), "triangles": T,
+                       "dense_triangles": 0, "dense_vertices": 0}
 
 
 def test_dense_block_of_counting_sort_runs(tc):
