@@ -273,9 +273,9 @@ tc_status enqueue_core(const int32_t *src, const int32_t *dst, int64_t m_in, int
   // shares and the work counters go by the whole lists' lengths
   const bool whole = shards > 1 || stats == kWholeWork || tune.heavy_ratio_pct != 100 ||
                      2 * b > kSkipShift;
-  // counting sorts by atomics, or radix passes (see kDirectMaxPairs)
-  const bool direct = m_in <= (batch ? kDirectMaxBatchPairs : kDirectMaxPairs) &&
-                      2 * b <= kSkipShift && shards == 1 && stats != kWholeWork && !g_radix_only.load();
+  // counting sorts by atomics, or radix passes
+  const bool direct = counting_sorts(m_in, n, batch != nullptr) && shards == 1 &&
+                      stats != kWholeWork && !g_radix_only.load();
   if (!direct)
     TC_CUDA(cudaMemsetAsync(ws + L.st_sort, 0,
                             sizeof(unsigned long long) * words * (size_t)radix_passes(b), st),

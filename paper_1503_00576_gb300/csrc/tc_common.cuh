@@ -76,6 +76,16 @@ template <bool PV> constexpr int64_t kBitMinPairs = PV ? 1 << 25 : 1 << 18;
 // (the scattered writes leave L2).
 constexpr int64_t kDirectMaxPairs = 20ll << 20;
 constexpr int64_t kDirectMaxBatchPairs = 1ll << 25;
+// ... but for runs of more than kCrowdedPairs pairs with more than kCrowdedMean
+// of them per vertex, mostly pairs given many times: their counters share so few
+// L2 sectors that the places taken from them cost more than the passes (m/n the
+// mean): K_200 x 200 (20,000) 2.94 / 3.86 ms, K_1000 x 8 (4,000) 1.11 / 1.49,
+// K_2000 x 8 (8,000) 2.68 / 3.76, 20,000 edges x 200 (2,000) 0.98 / 1.11 ms,
+// 160,000 x 100 (1,000) 1.66 / 1.83; 6,000 x 66 (660) 0.36 / 0.34, 80,000 x 50
+// (500) 0.50 / 0.48, 320,000 x 50 (500) 1.25 / 1.24, 99,840 pairs of 64 vertices
+// (1,560) 0.22 / 0.21 ms.
+constexpr int64_t kCrowdedPairs = 1 << 18;
+constexpr int64_t kCrowdedMean = 768;
 constexpr int kRankClasses = 1024;
 // Runs whose kernels are launched early (see launch()).  Whole calls, in turn /
 // early: 8,191 pairs 135 / 85 us, 131,072 with clustering 259 / 198 us, R-MAT
@@ -308,6 +318,13 @@ inline int id_bits(int32_t n) {
 // 2^b), the oriented keys (owner bits) and the group keys (group bits).
 inline int radix_passes(int b) { return 3 * ((b + 7) / 8); }
 
+// Whether a run of m pairs and n vertices (a batch: of the union) sorts by
+// counting.
+inline bool counting_sorts(int64_t m, int32_t n, bool batch) {
+  return m <= (batch ? kDirectMaxBatchPairs : kDirectMaxPairs) && 2 * id_bits(n) <= kSkipShift &&
+         (m <= kCrowdedPairs || m <= kCrowdedMean * n);
+}
+
 // Whether a single-graph run of n vertices has the dense hub block.
 inline bool hub_enabled(int32_t n, int b) { return n >= kHubMinVertices && 2 * b <= kSkipShift; }
 
@@ -361,7 +378,7 @@ inline Layout make_layout(int64_t m_in, int32_t n, bool with_hub = false,
   // elements, since each non-empty list adds at most 7
   L.col4 = take(sizeof(int32_t) * (m + 7 * (nv < m ? nv : m)));
   L.bits = per_vertex && L.has_bits ? take((size_t)L.bit_slots * (kBitCols / 4)) : 0;
-  L.has_desc = per_vertex && !lean && m_in <= kDirectMaxPairs;
+  L.has_desc = per_vertex && !lean && counting_sorts(m_in, n, batch);
   L.desc = L.has_desc ? take(sizeof(uint64_t) * m) : 0;
   const bool hub = with_hub && hub_enabled(n, id_bits(n > 0 ? n : 1));
   const size_t H = (size_t)hub_vertices;

@@ -45,5 +45,6 @@ def test_lean_layout_is_no_larger_than_without_counts(tmp_path):
     for m, n, total_only, per_vertex, lean, bits, desc in rows:
         assert lean == total_only <= per_vertex, (m, n)
         assert bits == 0 and desc == 0
-        if n <= m // 64 and (m <= 20 << 20 or m >= 1 << 25):
+        counting = m <= 20 << 20 and (m <= 1 << 18 or m <= 768 * n)
+        if n <= m // 64 and (counting or m >= 1 << 25):
             assert per_vertex > lean, (m, n)
