@@ -20,7 +20,8 @@
 // An atomic and a scattered write per key cost less than three passes while
 // the counters and the array written to stay in L2; past that, a list's
 // entries reach DRAM one 32-byte sector each (kDirectMaxPairs has both
-// sides measured).  R-MAT scale 20, 16.8M pairs: orient 244 us, lists 169,
+// sides measured), and unless very many pairs share very few counters
+// (kCrowdedMean).  R-MAT scale 20, 16.8M pairs: orient 244 us, lists 169,
 // groups 243, classes 12; the radix passes of the three sorts took 690 and
 // the group keys 89.
 #include "tc_common.cuh"

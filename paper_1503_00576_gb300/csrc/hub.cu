@@ -14,9 +14,10 @@
 //   r(i) = sum_j C(i,j) A(i,j) = 2 t_H(i)   (t_H(i): triangles of H at i)
 //   sum_i r(i) = 6 T_H.
 //
-// The hash-set counting (count.cu) skips the edges with both endpoints in
-// H (group.cu marks them), so every triangle is counted once: by the dense
-// block if its lowest vertex is in H, by the hash path otherwise.
+// The edges with both endpoints in H are left out of the partner groups
+// (group.cu; where the groups are dealt to shares, marked to be skipped whole),
+// so every triangle is counted once: by the dense block if its lowest vertex is
+// in H, by hashing or bitmaps otherwise.
 //
 // The product runs on 128 x 128 tiles of C, only those with row block
 // I <= column block J (C and A are symmetric: an off-diagonal tile stands

@@ -1,5 +1,5 @@
 // preprocess.cu -- preprocessing of the forward algorithm on sm_103a.
-// (Calls of up to kDirectMaxPairs pairs replace the rank sort, the orient and
+// (Runs for which counting_sorts() holds replace the rank sort, the orient and
 // sort steps and the group sort by the counting sorts of direct.cu.)
 //
 // Sec. III-B of the paper builds, from an edge array, the sorted forward

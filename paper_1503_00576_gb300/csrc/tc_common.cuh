@@ -22,7 +22,7 @@ enum : uint32_t { kErrIdRange = 1u, kErrTimeout = 2u, kErrInternal = 4u };
 constexpr uint32_t kSpinLimit = 1u << 24;
 constexpr uint32_t kNoTile = 0xffffffffu;  // no tile withholds its status (see set_wait_hooks)
 
-// Sorted forward lists (the padded column array col4).  Lists of up to
+// Sorted forward lists (the padded column array col4).  Lists of up to 2
 // kWarpSortMax entries are sorted by one warp, up to kCtaSortMax by a CTA in
 // shared memory; longer ones (never met in the workloads: they need a dense
 // core of more than 8192 vertices) by a CTA in sorted chunks of kCtaSortMax
@@ -43,10 +43,16 @@ constexpr uint32_t kSkipAll = 0xFFFFu;
 // if it has at least kBitMinPartners partners.  A list's record is (slot + 1)
 // << kBitTbBits | tb, tb the first block that the bitmap stands for; 0: none.
 // Per vertex (PV) an edge costs about three times as much (counts per column
-// and partner), so the lines lie higher there.  Measured on R-MAT graphs (T
-// only / per vertex, ms; 4, 5, 6, 8 and 5, 8, 12, 16, 24 blocks tried): more
-// or fewer blocks change a call by less than 1%; 8192 columns instead of 4096
-// cost 10% more per call for 4% more of the lookups.
+// and partner), so the lines lie higher there.  R-MAT 20 of 44.5M pairs / 21 of
+// 91M / 24 of 180M / 22 of 180M, whole calls in ms:
+//   T only      4 blocks 7.16 15.63 31.19 37.55   8 partners 7.08 15.50 30.15 37.11
+//               6        7.05 15.50 30.16 37.12  16          (the same call)
+//               8        7.05 15.58 30.10 37.03  32          7.06 15.50 30.15 37.13
+//   per vertex  8        8.67 20.20 37.26 47.45  32          8.72 20.13 37.12 47.28
+//              12        8.70 20.09 37.11 47.33  64          (the same call)
+//              16        8.77 20.17 36.89 47.30 128          8.71 20.08 37.08 47.36
+// so only fewer blocks than 6 cost anything; 8192 columns instead of 4096 cost
+// 10% more per call for 4% more of the lookups.
 constexpr int kBitCols = 4096;
 template <bool PV> constexpr int kBitMinBlocks = PV ? 12 : 6;
 template <bool PV> constexpr int kBitMinPartners = PV ? 64 : 16;
@@ -57,23 +63,30 @@ constexpr int kBitTbBits = 11;
 constexpr uint32_t kBitTbMask = (1u << kBitTbBits) - 1;
 constexpr uint32_t kBitMaxSlots = (1u << (32 - kBitTbBits)) - 1;
 // Only for single graphs of at least this many pairs.  T only: below it few
-// lists are that long, and two launches cost more.  Per vertex, without / with
-// them: R-MAT 18 of 10.5M pairs 2.50 / 2.53 ms, 20 of 16.8M 3.30 / 3.46, 20
-// of 44.5M 11.6 / 10.3, 21 of 91M 28.5 / 21.6, 24 of 180M 41.7 / 40.2, 22 of
-// 180M 69.9 / 49.6 (T only, before / with: 16 of 2.5M 0.64 / 0.61 ms, 21 of
-// 91M 22.5 / 16.9).
+// lists are that long, and two launches cost more (R-MAT 16 of 2.5M pairs,
+// without / with them when they came: 0.64 / 0.61 ms, 21 of 91M 22.5 / 16.9).
+// Per vertex, without / with them: R-MAT 18 of 4M pairs 0.88 / 0.93 ms, of 10.5M
+// 2.14 / 2.14, 20 of 16.8M with repeats 3.01 / 3.18, of 25M 4.94 / 4.77, of 33M
+// 7.12 / 6.21, of 44.5M 10.7 / 8.69, 21 of 91M 26.1 / 20.2, 24 of 180M 38.5 /
+// 37.2, 22 of 180M 62.9 / 47.3: where they pay depends on the density, and the
+// line lies where they do on all of these.
 template <bool PV> constexpr int64_t kBitMinPairs = PV ? 1 << 25 : 1 << 18;
 
 // Counting sorts by atomics (direct.cu) instead of radix passes: runs of at
-// most this many pairs (a single graph; a batch) with ids of at most 24 bits,
-// but for shares of a run (their dealing needs the exact vertex order).  Whole
-// calls, radix passes / counting sorts: 8,191 pairs 196 / 134 us, R-MAT 16 of
-// 2.5M 604 / 539 us, a union of 300 small graphs (3.1M) 745 / 581 us, R-MAT 20
-// of 16.8M 3.37 / 3.15 ms, uniform of 16M 2.49 / 2.13 and of 32M 4.82 / 4.55 ms,
-// Barabasi-Albert of 12M 1.85 / 1.59, of 20M 2.85 / 2.68, of 24M 3.35 / 3.32 and
-// of 32M 4.42 / 4.72 ms; 64 graphs of 33M 5.31 / 4.93 ms; ring lattice of 50M
-// 4.91 / 5.05 ms, geometric of 67M 9.4 / 10.6 ms, R-MAT 24 of 180M 39 / 45 ms
-// (the scattered writes leave L2).
+// most this many pairs (a single graph; a batch, an engine by its capacity) with
+// ids of at most 24 bits, but for shares of a run (their dealing needs the exact
+// vertex order).  Whole calls, radix passes / counting sorts: 19,900 pairs 0.15 /
+// 0.11 ms, 320,000 0.20 / 0.14; uniform of 8M 1.35 / 1.06 ms, of 24M 3.65 / 3.30,
+// of 32M 4.81 / 4.67, of 50M 7.46 / 7.80; Barabasi-Albert of 12M 1.75 / 1.53, of
+// 24M 3.29 / 3.07, of 32M 4.32 / 4.18; R-MAT 20 of 16M 2.52 / 2.45, of 32M 4.90 /
+// 4.70, of 44M 6.97 / 6.89 (per vertex 8.57 / 8.61); ring lattice of 32M 3.00 /
+// 2.81, of 50M 4.52 / 4.77; geometric of 24M 3.04 / 2.71, of 32M 4.01 / 3.84, of
+// 67M 8.16 / 8.97 (the scattered writes leave L2).  So the two cross between 32M
+// and 50M pairs; the line for single graphs was drawn before the kernels behind
+// it changed, when Barabasi-Albert of 32M took 4.42 / 4.72 ms.  Batches: 300
+// graphs of 3.3M pairs 0.75 / 0.54 ms, 64 of 33M 4.55 / 4.21, 30 of 42M 5.84 /
+// 5.69, 76 of 48M 6.46 / 6.25, 96 of 62.5M 8.26 / 8.27, 128 of 72M 9.54 / 9.70,
+// 1500 of 66M 9.04 / 8.48: the line lies below where they cross, too.
 constexpr int64_t kDirectMaxPairs = 20ll << 20;
 constexpr int64_t kDirectMaxBatchPairs = 1ll << 25;
 // ... but for runs of more than kCrowdedPairs pairs with more than kCrowdedMean
